@@ -223,21 +223,20 @@ adapt_status_t adapt_matmul_noalloc(int64_t M, int64_t N, int64_t K, adapt_dtype
 
 /* `count` independent GEMMs enqueued on one stream by one call: adapt_matmul(plans[i], A[i], B[i], C[i])
  * for i = 0 .. count-1, in that order, stopping at the first failure.  plans, A, B and C are HOST arrays
- * of `count` entries (the entries of A, B, C are device pointers).  It is the loop a caller would write,
- * moved behind the boundary so that a caller in an interpreted language pays its foreign-call cost once per
- * batch, not once per GEMM; each GEMM is still its own launch(es).  The paper replaces the vendor's
- * MatMul / GroupMM operators in recommendation models (Section 6.5), whose layers issue exactly such
- * lists of small GEMMs of different shapes.
- * A batch of eight or more calls is spread over up to four internal streams between a fork from and a join to
- * cuda_stream (work queued on cuda_stream before the call comes first, work queued after it comes last), so that
- * the launch gaps and the tail of one GEMM fill with the next one's work.  The result is the one of the calls made
- * in order: a call whose output overlaps a buffer that an earlier call of the batch still reads or writes on another
- * internal stream, or whose inputs overlap such an output, waits for that stream first.  Option "batch_streams"
- * (adapt_set_option; 1 to 4, default 4) sets the number of internal streams; with 1 the calls run one after the
- * other on cuda_stream itself.  The internal streams keep workspaces of their own.  Once a batch has run (workspaces
- * grown, tensor maps of its pointers cached) the same batch only launches kernels and records and waits for events, so
- * it can be captured into a CUDA graph through cuda_stream and replayed (1,200 launch-bound GEMMs: 5.1 ms direct,
- * 4.6 ms as a graph). */
+ * of `count` entries (the entries of A, B, C are device pointers).  The paper replaces the vendor's
+ * MatMul / GroupMM operators in recommendation models (Section 6.5), whose layers issue lists of small GEMMs of different
+ * shapes.  The result is the one of the calls made in order, bit for bit:
+ * - Small calls whose plans are of the one-launch family, or of the CUDA-core family with a short K (as adapt_matmul_plan
+ *   returned them), leave together in one grouped launch per 64 calls, data type and pair of layouts.  A call that reads or
+ *   overwrites what a collected one writes, or overwrites what it reads, makes the collected ones leave first.
+ * - From eight calls on the launches are spread over cuda_stream and up to three internal streams between a fork from and a
+ *   join to it (work queued on cuda_stream before the call comes first, work queued after it comes last), so that the launch
+ *   gaps and the tail of one GEMM fill with the next one's work.  A launch whose output overlaps a buffer that an earlier one
+ *   still reads or writes on another stream, or whose inputs overlap such an output, waits for that stream first.  Option
+ *   "batch_streams" (adapt_set_option; 1 to 4, default 4) sets the number of streams; with 1 everything runs on cuda_stream.
+ * The internal streams keep workspaces of their own.  Once a batch has run (workspaces grown, tensor maps of its pointers
+ * cached) the same batch only launches kernels and records and waits for events, so it can be captured into a CUDA graph
+ * through cuda_stream and replayed. */
 adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t* plans, const void* const* A,
                                   const void* const* B, void* const* C, void* cuda_stream);
 
@@ -253,7 +252,8 @@ adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t* plans, co
  * of the warp-level and one-launch families run on the CUDA-core kernel for this call.  K == 0 gives beta * D.
  *
  * adapt_matmul_strided_batch:  `batch` GEMMs of the plan's shape on operands stride_a, stride_b, stride_c ELEMENTS apart
- * (a stride of 0 shares that input across the batch; stride_c must be at least M * N), enqueued in batch order on the stream. */
+ * (a stride of 0 shares that input across the batch; stride_c must be at least M * N).  The result is the one of the entries run in
+ * batch order; entries that do not depend on one another (no output overlaps an input) share one launch where that is faster. */
 adapt_status_t adapt_addmm(adapt_handle_t plan, const void* A, const void* B, const void* D, int d_is_vector,
                            float alpha, float beta, void* C, void* cuda_stream);
 adapt_status_t adapt_matmul_strided_batch(adapt_handle_t plan, const void* A, int64_t stride_a, const void* B, int64_t stride_b,

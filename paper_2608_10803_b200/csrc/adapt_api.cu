@@ -20,6 +20,7 @@
 #include "aux_kernels.cuh"
 #include "skinny_gemm.cuh"
 #include "cluster_gemm.cuh"
+#include "group_gemm.cuh"
 #include "umma_gemm.cuh"
 
 using namespace adapt;
@@ -749,6 +750,7 @@ extern "C" adapt_status_t adapt_init(int device)
         (void)cudaGetLastError();
     }
     CUDA_TRY(cluster_set_attributes());
+    CUDA_TRY(group_set_attributes());
     S.machine.max_cluster = cluster_max_size();
     S.device = device;
     S.inited = true;
@@ -1282,7 +1284,7 @@ adapt_status_t run_simt(State& S, Plan* pl, const void* A, const void* B, void* 
 
 adapt_status_t run_cluster(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream)
 {
-    if (launch_cluster(pl->s, pl->c, A, B, C, S.d_status, stream, S.prefetch) != ADAPT_OK) return fail(ADAPT_ERR_CUDA, "cluster kernel launch failed%s");
+    if (launch_cluster(pl->s, pl->c, A, B, C, stream, S.prefetch) != ADAPT_OK) return fail(ADAPT_ERR_CUDA, "cluster kernel launch failed%s");
     S.launches.fetch_add(1, std::memory_order_relaxed);
     CUDA_TRY(cudaGetLastError());
     return ADAPT_OK;
@@ -1379,12 +1381,56 @@ extern "C" adapt_status_t adapt_addmm(adapt_handle_t plan, const void* A, const 
     return run_simt_splits(S, s, (int)pk, A, B, C, stream, &ep);
 }
 
+namespace {
+
+// A strided batch of small GEMMs in one grouped launch.  *done stays false when the batch is to run entry by entry instead:
+// plans of other families, entries that depend on one another (an output that overlaps any input of the batch), arguments
+// that the single call refuses.
+adapt_status_t run_strided_grouped(State& S, Plan* pl, const void* A, int64_t sa, const void* B, int64_t sb, void* C, int64_t sc,
+                                   int64_t batch, cudaStream_t stream, bool* done)
+{
+    const Shape& s = pl->s;
+    if (!S.inited || pl->noop || pl->zero_fill || !A || !B || !C || (((uintptr_t)A | (uintptr_t)B | (uintptr_t)C) & 1)) return ADAPT_OK;
+    if (pl->c.family != ADAPT_FAM_CLUSTER && pl->c.family != ADAPT_FAM_SIMT) return ADAPT_OK;
+    // (the sizes below are a few GB at most: the plan's tiles fit the machine about twice, K is bounded by the chain)
+    const int64_t tiles = (int64_t)pl->c.P_m * pl->c.P_n;
+    if (batch > ((int64_t)1 << 24) || batch * tiles > ((int64_t)1 << 26) || std::max(sa, std::max(sb, sc)) > ((int64_t)1 << 36)) return ADAPT_OK;
+    const size_t nA = (size_t)((batch - 1) * sa + s.M * s.K) * 2, nB = (size_t)((batch - 1) * sb + s.K * s.N) * 2;
+    const size_t nC = (size_t)((batch - 1) * sc + s.M * s.N) * 2;
+    if (overlaps(C, nC, A, nA) || overlaps(C, nC, B, nB)) return ADAPT_OK;
+    Config c = pl->c;
+    if (c.family == ADAPT_FAM_CLUSTER ? s.K > 1 << 20 : !group_eligible(s, c)) return ADAPT_OK;
+    GroupParams p;
+    const int chain = group_item(s, c, A, B, C, &p.item[0]);
+    // rounds of two CTAs per SM, 1.5 us and 0.6 us per stage each, against the calls one by one
+    const double rounds = (double)ceil_div(batch * tiles, 2 * (int64_t)S.machine.n_sm);
+    if (3.0 + rounds * (1.5 + 0.6 * chain) > (double)batch * std::max(1.5, pl->c.predicted_us - 1.0)) return ADAPT_OK;
+    p.item[0].tile_end = (int)(batch * tiles);
+    p.count = 1;
+    p.ring = cluster_seq_ring(chain);
+    p.k_max = (int)s.K;
+    p.prefetch = S.prefetch;
+    p.dtype = s.dtype;
+    p.sa = sa; p.sb = sb; p.sc = sc;
+    *done = true;
+    CUDA_TRY(launch_group(p, s.layoutA == ADAPT_ROW_MAJOR, s.layoutB == ADAPT_COL_MAJOR, stream));
+    S.launches.fetch_add(1, std::memory_order_relaxed);
+    return ADAPT_OK;
+}
+
+}  // namespace
+
 extern "C" adapt_status_t adapt_matmul_strided_batch(adapt_handle_t plan, const void* A, int64_t stride_a, const void* B,
                                                      int64_t stride_b, void* C, int64_t stride_c, int64_t batch, void* cuda_stream)
 {
     if (batch < 0 || stride_a < 0 || stride_b < 0 || stride_c < 0) return fail(ADAPT_ERR_INVALID_ARG, "negative batch count or stride%s");
     if (!plan) return fail(ADAPT_ERR_INVALID_ARG, "null plan%s");
     if (batch > 1 && !plan->noop && stride_c < plan->s.M * plan->s.N) return fail(ADAPT_ERR_INVALID_ARG, "outputs of the batch overlap%s");
+    if (batch > 1) {
+        bool done = false;
+        const adapt_status_t r = run_strided_grouped(st(), plan, A, stride_a, B, stride_b, C, stride_c, batch, (cudaStream_t)cuda_stream, &done);
+        if (done || r != ADAPT_OK) return r;
+    }
     for (int64_t i = 0; i < batch; ++i) {
         const adapt_status_t r = adapt_matmul(plan, (const unsigned short*)A + i * stride_a, (const unsigned short*)B + i * stride_b,
                                               (unsigned short*)C + i * stride_c, cuda_stream);
@@ -1462,91 +1508,204 @@ extern "C" adapt_status_t adapt_matmul_host(adapt_handle_t plan, const void* A_h
 // ---------------------------------------------------------------------------------------------
 // batched call, measurement support, self-test
 // ---------------------------------------------------------------------------------------------
+namespace {
+
+struct Range { uintptr_t lo, hi; };
+inline bool hits(const std::vector<Range>& v, uintptr_t lo, uintptr_t hi)
+{
+    bool any = false;
+    for (const Range& r : v) any |= (lo < r.hi) & (r.lo < hi);
+    return any;
+}
+
+// Calls of a batch that wait for their grouped launch: independent of one another, one dtype and pair of layouts per launch.
+struct PendingGroup {
+    struct Entry { GroupItem item; int chain, variant; };
+    std::vector<Entry> entries;
+    std::vector<Range> reads, writes;
+    double predicted_us = 0.0;
+    bool conflicts(const Range& a, const Range& b, const Range& c) const
+    {
+        return !entries.empty() && (hits(writes, c.lo, c.hi) || hits(reads, c.lo, c.hi) || hits(writes, a.lo, a.hi) || hits(writes, b.lo, b.hi));
+    }
+    void clear() { entries.clear(); reads.clear(); writes.clear(); predicted_us = 0.0; }
+};
+
+adapt_status_t launch_pending(State& S, PendingGroup& g, cudaStream_t stream)
+{
+    // longest chains first: what starts last is short
+    std::stable_sort(g.entries.begin(), g.entries.end(), [](const PendingGroup::Entry& x, const PendingGroup::Entry& y) { return x.chain > y.chain; });
+    GroupParams p;
+    p.prefetch = S.prefetch;
+    p.sa = p.sb = p.sc = 0;
+    for (int variant = 0; variant < 8; ++variant) {         // bit 0: dtype, 1: A row-major, 2: B column-major
+        p.count = 0;
+        p.ring = 1;
+        p.k_max = 0;
+        int64_t end = 0;
+        auto flush = [&]() -> adapt_status_t {
+            if (p.count == 0) return ADAPT_OK;
+            p.dtype = variant & 1;
+            CUDA_TRY(launch_group(p, (variant & 2) != 0, (variant & 4) != 0, stream));
+            S.launches.fetch_add(1, std::memory_order_relaxed);
+            p.count = 0;
+            p.ring = 1;
+            p.k_max = 0;
+            end = 0;
+            return ADAPT_OK;
+        };
+        for (const PendingGroup::Entry& e : g.entries) {
+            if (e.variant != variant) continue;
+            p.item[p.count] = e.item;
+            end += e.item.tiles;
+            p.item[p.count].tile_end = (int)end;
+            p.ring = std::max(p.ring, cluster_seq_ring(e.chain));
+            p.k_max = std::max(p.k_max, e.item.K);
+            if (++p.count == kGroupMax) {
+                const adapt_status_t r = flush();
+                if (r != ADAPT_OK) return r;
+            }
+        }
+        const adapt_status_t r = flush();
+        if (r != ADAPT_OK) return r;
+    }
+    return ADAPT_OK;
+}
+
+}  // namespace
+
 extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t* plans, const void* const* A,
                                              const void* const* B, void* const* C, void* cuda_stream)
 {
     if (count < 0 || (count > 0 && (!plans || !A || !B || !C))) return fail(ADAPT_ERR_INVALID_ARG, "null array%s");
     State& S = st();
-    if (count < 8 || S.batch_lanes < 2 || !S.inited) {
+    cudaStream_t user = (cudaStream_t)cuda_stream;
+    if (count < 2 || !S.inited) {
         for (int64_t i = 0; i < count; ++i) {
             const adapt_status_t r = adapt_matmul(plans[i], A[i], B[i], C[i], cuda_stream);
             if (r != ADAPT_OK) return r;
         }
         return ADAPT_OK;
     }
-    // Lanes.  The calls of a batch are handed in turn to the lane with the least predicted work queued, so that the
-    // launch gaps and the tail of one call fill with the next call's work.  The result is the one of running the calls in
-    // order: a call whose output overlaps what the other lane still reads or writes, or whose inputs overlap what it
-    // writes, first waits for that lane; a lane remembers the buffers of its last 16 calls, and when that memory is
-    // full all other lanes are made to wait for it.  A stream-K call runs with nothing beside it: its CTAs wait for one another and
-    // must all be resident, which two such kernels sharing the SMs could deny each other.
-    std::lock_guard<std::mutex> batch_lock(S.batch_mu);
+    // Small calls (plans of the one-launch and CUDA-core families, as adapt_matmul_plan returned them) are collected and
+    // leave together in one grouped launch; the others are launched as they come.  A call is only collected, and another
+    // only launched past the collected ones, while none of its buffers meets theirs in a way that order would matter.
+    auto grouped = [&](const Plan* pl) { return pl && pl->selected && !pl->noop && !pl->zero_fill && group_eligible(pl->s, pl->c); };
+    int64_t singles = 0;
+    for (int64_t i = 0; i < count; ++i) singles += grouped(plans[i]) ? 0 : 1;
+    // Lanes.  Lane 0 is the caller's stream, the others are internal streams between a fork from and a join to it, used
+    // from eight calls on and no more of them than there are launches to overlap.  A launch goes to the lane with the least
+    // predicted work queued, so that the launch gaps and the tail of one call fill with the next call's work.  The result is
+    // the one of running the calls in order: a call whose output overlaps what another lane still reads or writes, or whose
+    // inputs overlap what it writes, first waits for that lane; a lane remembers the buffers of its last 16 calls, and when that
+    // memory is full all other lanes are made to wait for it.  A stream-K call runs with nothing beside it: its CTAs wait
+    // for one another and must all be resident, which two such kernels sharing the SMs could deny each other.
+    const int NL = count < 8 ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(S.batch_lanes, singles + (singles < count ? 1 : 0)));
+    std::unique_lock<std::mutex> batch_lock(S.batch_mu, std::defer_lock);
     State::BatchLanes& L = S.lanes;
-    if (!L.ready) {
-        for (int l = 0; l < 4; ++l) {
-            CUDA_TRY(cudaStreamCreateWithFlags(&L.s[l], cudaStreamNonBlocking));
-            CUDA_TRY(cudaEventCreateWithFlags(&L.join[l], cudaEventDisableTiming));
-            CUDA_TRY(cudaEventCreateWithFlags(&L.cross[l], cudaEventDisableTiming));
+    cudaStream_t stream[4] = {user, nullptr, nullptr, nullptr};
+    if (NL > 1) {
+        batch_lock.lock();
+        if (!L.ready) {
+            for (int l = 0; l < 4; ++l) {
+                CUDA_TRY(cudaStreamCreateWithFlags(&L.s[l], cudaStreamNonBlocking));
+                CUDA_TRY(cudaEventCreateWithFlags(&L.join[l], cudaEventDisableTiming));
+                CUDA_TRY(cudaEventCreateWithFlags(&L.cross[l], cudaEventDisableTiming));
+            }
+            CUDA_TRY(cudaEventCreateWithFlags(&L.fork, cudaEventDisableTiming));
+            L.ready = true;
         }
-        CUDA_TRY(cudaEventCreateWithFlags(&L.fork, cudaEventDisableTiming));
-        L.ready = true;
+        CUDA_TRY(cudaEventRecord(L.fork, user));
+        for (int l = 1; l < NL; ++l) {
+            stream[l] = L.s[l];
+            CUDA_TRY(cudaStreamWaitEvent(L.s[l], L.fork, 0));
+        }
     }
-    const int NL = S.batch_lanes;
-    cudaStream_t user = (cudaStream_t)cuda_stream;
-    CUDA_TRY(cudaEventRecord(L.fork, user));
-    for (int l = 0; l < NL; ++l) CUDA_TRY(cudaStreamWaitEvent(L.s[l], L.fork, 0));
-    struct Range { uintptr_t lo, hi; };
     constexpr size_t kLaneMemory = 32;
     std::vector<Range> reads[4], writes[4];
     double queued[4] = {0.0, 0.0, 0.0, 0.0};
-    auto hits = [](const std::vector<Range>& v, uintptr_t lo, uintptr_t hi) {
-        for (const Range& r : v) if (lo < r.hi && r.lo < hi) return true;
-        return false;
-    };
     auto wait_for = [&](int lane, int other) -> adapt_status_t {      // `lane` continues after everything queued on `other`
-        CUDA_TRY(cudaEventRecord(L.cross[other], L.s[other]));
-        CUDA_TRY(cudaStreamWaitEvent(L.s[lane], L.cross[other], 0));
+        CUDA_TRY(cudaEventRecord(L.cross[other], stream[other]));
+        CUDA_TRY(cudaStreamWaitEvent(stream[lane], L.cross[other], 0));
         return ADAPT_OK;
+    };
+    // Chooses the lane of a launch that reads and writes the given buffers and makes it wait for the lanes it depends on.
+    auto enter = [&](const Range* rd, size_t n_rd, const Range* wr, size_t n_wr, bool alone, int* out) -> adapt_status_t {
+        int lane = 0;
+        for (int l = 1; l < NL; ++l) if (queued[l] < queued[lane]) lane = l;
+        *out = lane;
+        for (int o = 0; o < NL; ++o) {
+            if (o == lane) continue;
+            bool dep = alone;
+            for (size_t j = 0; j < n_wr && !dep; ++j) dep = hits(reads[o], wr[j].lo, wr[j].hi) || hits(writes[o], wr[j].lo, wr[j].hi);
+            for (size_t j = 0; j < n_rd && !dep; ++j) dep = hits(writes[o], rd[j].lo, rd[j].hi);
+            // everything lane o has queued comes first; what o did before is then ordered before all of this lane's
+            // later calls as well, but the other lanes still have to see it: keep o's memory
+            if (dep) { const adapt_status_t r = wait_for(lane, o); if (r != ADAPT_OK) return r; }
+        }
+        if (NL > 1 && reads[lane].size() >= kLaneMemory) {
+            // this lane's memory is full: every other lane waits for it, and it starts a new memory
+            for (int o = 0; o < NL; ++o)
+                if (o != lane) { const adapt_status_t r = wait_for(o, lane); if (r != ADAPT_OK) return r; }
+            reads[lane].clear();
+            writes[lane].clear();
+        }
+        return ADAPT_OK;
+    };
+    auto leave = [&](int lane, const Range* rd, size_t n_rd, const Range* wr, size_t n_wr, double us) {
+        queued[lane] += std::max(1.0, us);
+        if (NL == 1) return;
+        reads[lane].insert(reads[lane].end(), rd, rd + n_rd);
+        writes[lane].insert(writes[lane].end(), wr, wr + n_wr);
+    };
+    PendingGroup group;
+    auto flush_group = [&]() -> adapt_status_t {
+        if (group.entries.empty()) return ADAPT_OK;
+        int lane = 0;
+        adapt_status_t r = enter(group.reads.data(), group.reads.size(), group.writes.data(), group.writes.size(), false, &lane);
+        if (r != ADAPT_OK) return r;
+        r = launch_pending(S, group, stream[lane]);
+        leave(lane, group.reads.data(), group.reads.size(), group.writes.data(), group.writes.size(), group.predicted_us);
+        group.clear();
+        return r;
     };
     adapt_status_t status = ADAPT_OK;
     for (int64_t i = 0; i < count && status == ADAPT_OK; ++i) {
         Plan* pl = plans[i];
-        if (!pl) { status = fail(ADAPT_ERR_INVALID_ARG, "null plan%s"); break; }
+        if (!pl) { status = flush_group(); if (status == ADAPT_OK) status = fail(ADAPT_ERR_INVALID_ARG, "null plan%s"); break; }
         const Shape& sh = pl->s;
-        const uintptr_t a0 = (uintptr_t)A[i], b0 = (uintptr_t)B[i], c0 = (uintptr_t)C[i];
-        const uintptr_t a1 = a0 + (uintptr_t)sh.M * sh.K * 2, b1 = b0 + (uintptr_t)sh.K * sh.N * 2, c1 = c0 + (uintptr_t)sh.M * sh.N * 2;
-        int lane = 0;
-        for (int l = 1; l < NL; ++l) if (queued[l] < queued[lane]) lane = l;
+        const Range a = {(uintptr_t)A[i], (uintptr_t)A[i] + (uintptr_t)sh.M * sh.K * 2}, b = {(uintptr_t)B[i], (uintptr_t)B[i] + (uintptr_t)sh.K * sh.N * 2};
+        const Range c = {(uintptr_t)C[i], (uintptr_t)C[i] + (uintptr_t)sh.M * sh.N * 2};
+        if (group.conflicts(a, b, c) && (status = flush_group()) != ADAPT_OK) break;
+        const bool sound = A[i] && B[i] && C[i] && (((uintptr_t)A[i] | (uintptr_t)B[i] | (uintptr_t)C[i]) & 1) == 0 &&
+                           !(c.lo < a.hi && a.lo < c.hi) && !(c.lo < b.hi && b.lo < c.hi);
+        if (sound && grouped(pl)) {
+            PendingGroup::Entry e;
+            e.chain = group_item(sh, pl->c, A[i], B[i], C[i], &e.item);
+            e.variant = (sh.dtype != 0 ? 1 : 0) | (sh.layoutA == ADAPT_ROW_MAJOR ? 2 : 0) | (sh.layoutB == ADAPT_COL_MAJOR ? 4 : 0);
+            group.entries.push_back(e);
+            group.reads.push_back(a);
+            group.reads.push_back(b);
+            group.writes.push_back(c);
+            group.predicted_us += 0.25 * pl->c.predicted_us;
+            if (group.entries.size() >= kGroupMax) status = flush_group();
+            continue;
+        }
+        if (!sound && (status = flush_group()) != ADAPT_OK) break;      // the calls before one that is refused are enqueued
+        const Range rd[2] = {a, b};
         const bool alone = pl->c.streamk != 0;
-        for (int o = 0; o < NL && status == ADAPT_OK; ++o) {
-            if (o == lane) continue;
-            if (alone || hits(reads[o], c0, c1) || hits(writes[o], c0, c1) || hits(writes[o], a0, a1) || hits(writes[o], b0, b1)) {
-                // everything lane o has queued comes first; what o did before is then ordered before all of this lane's
-                // later calls as well, but the other lanes still have to see it: keep o's memory
-                status = wait_for(lane, o);
-            }
-        }
+        int lane = 0;
+        if ((status = enter(rd, 2, &c, 1, alone, &lane)) != ADAPT_OK) break;
+        status = adapt_matmul(pl, A[i], B[i], C[i], (void*)stream[lane]);
         if (status != ADAPT_OK) break;
-        if (reads[lane].size() >= kLaneMemory) {
-            // this lane's memory is full: every other lane waits for it, and it starts a new memory
-            for (int o = 0; o < NL && status == ADAPT_OK; ++o)
-                if (o != lane) status = wait_for(o, lane);
-            if (status != ADAPT_OK) break;
-            reads[lane].clear();
-            writes[lane].clear();
-        }
-        status = adapt_matmul(pl, A[i], B[i], C[i], (void*)L.s[lane]);
-        if (status != ADAPT_OK) break;
-        reads[lane].push_back({a0, a1});
-        reads[lane].push_back({b0, b1});
-        writes[lane].push_back({c0, c1});
-        queued[lane] += std::max(1.0, pl->c.predicted_us);
+        leave(lane, rd, 2, &c, 1, pl->c.predicted_us);
         if (alone)
             for (int o = 0; o < NL && status == ADAPT_OK; ++o)
                 if (o != lane) status = wait_for(o, lane);
     }
+    if (status == ADAPT_OK) status = flush_group();
     // join, also after an error: the caller's stream continues after whatever was queued
-    for (int l = 0; l < NL; ++l) {
+    for (int l = 1; l < NL; ++l) {
         if (cudaEventRecord(L.join[l], L.s[l]) == cudaSuccess) (void)cudaStreamWaitEvent(user, L.join[l], 0);
     }
     return status;

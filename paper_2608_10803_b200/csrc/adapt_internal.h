@@ -203,11 +203,15 @@ const Calib& default_calib();
 // Shared-memory layout of the tcgen05 kernels, used by the capacity check and by the launcher:
 // S stages of (A: box rows x 64, B: BN/cluster x 64) 16-bit, a barrier block, the epilogue staging
 // (8 KB per epilogue warp, only when the kernel stores the 16-bit C), and slack to align the stages to 1024 B.
-// One-launch cluster kernel: a ring of raw stages (64 rows of 144 bytes per operand) plus two shifted stages.
+// One-launch cluster kernel: a ring of stages (64 rows of 144 bytes per operand).
 // The ring is as deep as the CTA's k range needs, capped so that the CTAs that share an SM all fit.
 constexpr int kClusterStageBytes = 2 * 64 * 144;
 constexpr int kClusterMaxRing = 6;
-inline int cluster_smem_bytes(int ring) { return (ring + 2) * kClusterStageBytes + 128; }   // + two shifted stages, barriers
+inline int cluster_smem_bytes(int ring) { return ring * kClusterStageBytes; }
+// A tile of one CTA: two groups of warps with a ring each, of `chain` stages at most (three: two CTAs per SM).
+constexpr int kClusterSeqRing = 3;
+inline int cluster_seq_ring(int chain) { return std::max(1, std::min(kClusterSeqRing, chain)); }
+inline int cluster_seq_smem_bytes(int ring) { return 2 * ring * kClusterStageBytes; }
 // Clusters of a size the machine runs at a time with one CTA per SM (a cluster is placed inside one GPC, so
 // the larger sizes leave SMs unused): what cudaOccupancyMaxActiveClusters reports on a B200 for this kernel
 // with its deepest ring (148, 74, 33, 15, 7), scaled to other SM counts.  With two CTAs per SM (rings of up

@@ -266,15 +266,12 @@ struct SimtParams {
     float* partial;
 };
 
-__global__ void __launch_bounds__(256)
-simt_gemm_kernel(const unsigned short* __restrict__ A, const unsigned short* __restrict__ B, const SimtParams p)
+// One 64 x 64 tile at (m0, n0), k split `split`; sA and sB are 16 x 68 floats of shared memory each.
+typedef float SimtStage[16][64 + 4];
+__device__ __forceinline__ void simt_tile_body(const unsigned short* __restrict__ A, const unsigned short* __restrict__ B, const SimtParams& p,
+                                               int m0, int n0, int split, SimtStage& sA, SimtStage& sB)
 {
-    __shared__ float sA[16][64 + 4];
-    __shared__ float sB[16][64 + 4];
-    pdl_launch_dependents();
     const int tid = threadIdx.x;
-    const int m0 = (int)(blockIdx.x / p.P_n) * 64, n0 = (int)(blockIdx.x % p.P_n) * 64;
-    const int split = blockIdx.y;
     const int k_begin = split * p.kb_per_split * 16;
     const int k_end = min(p.K, k_begin + p.kb_per_split * 16);
     // Ahead of the wait for the kernel before this one on the stream: ask L2 for the lines the first two k steps
@@ -348,6 +345,14 @@ simt_gemm_kernel(const unsigned short* __restrict__ A, const unsigned short* __r
             else p.partial[((int64_t)split * p.M + m) * p.Np + n] = acc[i][j];
         }
     }
+}
+
+__global__ void __launch_bounds__(256)
+simt_gemm_kernel(const unsigned short* __restrict__ A, const unsigned short* __restrict__ B, const SimtParams p)
+{
+    __shared__ SimtStage sA, sB;
+    pdl_launch_dependents();
+    simt_tile_body(A, B, p, (int)(blockIdx.x / p.P_n) * 64, (int)(blockIdx.x % p.P_n) * 64, (int)blockIdx.y, sA, sB);
 }
 
 // ---- measurement and self-test kernels ---------------------------------------------------------------

@@ -1,0 +1,159 @@
+// Many small GEMMs in ONE launch: the lists of adapt_matmul_batch and the entries of adapt_matmul_strided_batch.
+//
+// A GEMM of a few microseconds is mostly launch, first trip to memory and drain; one launch each leaves the chip idle
+// between them (48 layers of 16 .. 1024 a side: 97 us on four streams, two microseconds a call, for 16 MB of operands).
+// Here the 64 x 64 tiles of all entries run side by side, one per CTA.  An entry keeps the arithmetic of its own plan:
+//   pieces > 0: the one-launch cluster kernel's tiles.  The CTA walks the plan's pieces of the k range and adds
+//               their sums in the same order: the bits of the call made alone, where each piece has a CTA of its own.
+//               (Clusters of four CTAs with the pieces spread over them took 53 us for those 48 layers, one CTA per tile 40 us:
+//               the exchange of the partial tiles cost more than the shorter chains saved.)
+//   pieces = 0: the CUDA-core kernel's tiles (a few 16-k steps).
+// The list travels in the kernel's parameters, so nothing is copied to the device and the launch can be captured.
+#pragma once
+
+#include "aux_kernels.cuh"
+#include "cluster_gemm.cuh"
+
+namespace adapt {
+
+constexpr int kGroupMax = 64;           // entries per launch (the parameters stay below 4 KB)
+
+struct GroupItem {
+    const unsigned short* A;
+    const unsigned short* B;
+    unsigned short* C;
+    int M, N, K;
+    int P_n;
+    int pieces;                         // pieces of the k range; 0: CUDA-core tiles
+    int k_per_piece;
+    int tiles;                          // 64 x 64 tiles of one entry
+    int tile_end;                       // tiles of this and all earlier items
+};
+struct GroupParams {
+    int count;
+    int ring;
+    int prefetch;
+    int dtype;
+    int k_max;                          // largest K of the list
+    int64_t sa, sb, sc;                 // strided batch: item 0 stands for all entries, sa, sb, sc elements apart
+    GroupItem item[kGroupMax];
+};
+static_assert(sizeof(GroupParams) <= 4096, "kernel parameters");
+
+// What bounds it: for a list with a deep entry the chain of that entry's stages (0.33 us per aligned 64 k values and group of
+// warps, 0.6 off 16-byte boundaries), else the shared-memory port.  The deepest entries come first and the ring is no deeper
+// than the list needs.  48 layers of 16 .. 1024 a side: 97 us one launch each on four streams, 31 us (21 us without the one
+// layer that keeps a launch of its own); 96 products of 128 x 128 x 64: 266 us one launch each, 4.4 us.
+// SHORT: every item has K <= 64 (one stage): no two-group tiles, so fewer registers and three CTAs per SM instead of two
+// (96 products of 128 x 128 x 64: 6.6 us with the general kernel, 4.4 with this one).
+template <bool A_KC, bool B_KC, bool BF16, bool SHORT>
+__global__ void __launch_bounds__(kClusterThreads, SHORT ? 3 : 2)
+group_gemm_kernel(const __grid_constant__ GroupParams p)
+{
+    extern __shared__ __align__(128) unsigned char s_dyn[];
+    pdl_launch_dependents();
+    const int t_all = (int)blockIdx.x;
+    int lo = 0, hi = p.count - 1;                           // the first item whose tiles end beyond this one
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (t_all < p.item[mid].tile_end) hi = mid; else lo = mid + 1;
+    }
+    const GroupItem& it = p.item[lo];
+    const int local = t_all - (lo > 0 ? p.item[lo - 1].tile_end : 0);
+    const int entry = local / it.tiles, tile = local - entry * it.tiles;
+    const int m0 = (tile / it.P_n) * kClusterTile, n0 = (tile % it.P_n) * kClusterTile;
+    const unsigned short* A = it.A + entry * p.sa;
+    const unsigned short* B = it.B + entry * p.sb;
+    unsigned short* C = it.C + entry * p.sc;
+    if (it.pieces == 0) {
+        SimtParams q;
+        q.M = it.M; q.N = it.N; q.K = it.K;
+        q.a_sm = A_KC ? it.K : 1; q.a_sk = A_KC ? 1 : it.M;
+        q.b_sk = B_KC ? 1 : it.N; q.b_sn = B_KC ? it.K : 1;
+        q.P_n = it.P_n; q.P_k = 1; q.kb_per_split = (it.K + 15) / 16;
+        q.Np = 0; q.dtype = BF16 ? 1 : 0; q.prefetch = 0;
+        q.C = C; q.partial = nullptr;
+        SimtStage* sm = reinterpret_cast<SimtStage*>(s_dyn);
+        simt_tile_body(A, B, q, m0, n0, 0, sm[0], sm[1]);
+        return;
+    }
+    ClusterParams q;
+    q.A = A; q.B = B; q.C = C;
+    q.M = it.M; q.N = it.N; q.K = it.K;
+    q.lda = A_KC ? it.K : it.M;
+    q.ldb = B_KC ? it.K : it.N;
+    q.P_n = it.P_n;
+    q.CS = it.pieces;
+    q.k_per_cta = it.k_per_piece;
+    q.ring = p.ring;
+    q.prefetch = p.prefetch;
+    q.aligned = (rows_aligned16(A, q.lda) ? 1 : 0) | (rows_aligned16(B, q.ldb) ? 2 : 0);
+    q.ep.D = nullptr; q.ep.d_is_vector = 0; q.ep.alpha = 1.f; q.ep.beta = 0.f;
+    cluster_tile_body<A_KC, B_KC, BF16, !SHORT>(q, m0, n0, s_dyn);
+}
+
+typedef void (*GroupKernel)(const GroupParams);
+
+template <bool SHORT>
+inline GroupKernel group_pick(bool a_kc, bool b_kc, bool bf16)
+{
+    if (bf16) {
+        if (a_kc) return b_kc ? group_gemm_kernel<true, true, true, SHORT> : group_gemm_kernel<true, false, true, SHORT>;
+        return b_kc ? group_gemm_kernel<false, true, true, SHORT> : group_gemm_kernel<false, false, true, SHORT>;
+    }
+    if (a_kc) return b_kc ? group_gemm_kernel<true, true, false, SHORT> : group_gemm_kernel<true, false, false, SHORT>;
+    return b_kc ? group_gemm_kernel<false, true, false, SHORT> : group_gemm_kernel<false, false, false, SHORT>;
+}
+
+inline cudaError_t group_set_attributes()
+{
+    for (int v = 0; v < 8; ++v) {
+        cudaError_t e = cudaFuncSetAttribute(group_pick<false>(v & 1, v & 2, v & 4), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             cluster_seq_smem_bytes(kClusterSeqRing));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// Can an entry with this configuration run in the grouped launch?  The cluster kernel's tiles: the k range must not be a long
+// chain (24 stages are about 10 us).  CUDA-core tiles: no k split and a few steps.
+inline bool group_eligible(const Shape& s, const Config& c)
+{
+    if (c.family == ADAPT_FAM_SIMT) return c.P_k == 1 && s.K <= 64 && (int64_t)c.P_m * c.P_n <= 512;
+    return c.family == ADAPT_FAM_CLUSTER && c.cluster * ceil_div(round_up(ceil_div(s.K, c.cluster), 16), kClusterKS) <= 24;
+}
+
+// Fills everything of an item but tile_end; returns its chain: the stages one group of warps of a tile walks.
+inline int group_item(const Shape& s, const Config& c, const void* A, const void* B, void* C, GroupItem* it)
+{
+    it->A = (const unsigned short*)A;
+    it->B = (const unsigned short*)B;
+    it->C = (unsigned short*)C;
+    it->M = (int)s.M; it->N = (int)s.N; it->K = (int)s.K;
+    it->P_n = c.P_n;
+    it->tiles = c.P_m * c.P_n;
+    const bool simt = c.family == ADAPT_FAM_SIMT;
+    it->pieces = simt ? 0 : c.cluster;
+    it->k_per_piece = simt ? 0 : (int)round_up(ceil_div(s.K, c.cluster), 16);
+    return simt ? 1 : it->pieces == 1 ? (int)ceil_div(s.K, 2 * kClusterKS) : (it->pieces / 2) * (int)ceil_div(it->k_per_piece, kClusterKS);
+}
+
+// One launch; p holds `count` items with their tile_end, k_max, ring and strides set.
+inline cudaError_t launch_group(GroupParams& p, bool a_kc, bool b_kc, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)p.item[p.count - 1].tile_end, 1, 1);
+    cfg.blockDim = dim3(kClusterThreads, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)(p.k_max <= kClusterKS ? cluster_smem_bytes(1) : cluster_seq_smem_bytes(p.ring));
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    pdl_attribute(&attr[0]);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    void* args[1] = {&p};
+    const size_t bytes[1] = {sizeof(p)};
+    return launch_exc(&cfg, (const void*)(p.k_max <= kClusterKS ? group_pick<true>(a_kc, b_kc, p.dtype != 0) : group_pick<false>(a_kc, b_kc, p.dtype != 0)), args, bytes, 1);
+}
+
+}  // namespace adapt

@@ -1,0 +1,135 @@
+"""Grouped launches: lists of small GEMMs and strided batches that leave as one launch give the bits of the calls made alone
+(lists), and the oracle's exact result on integers (strided batches)."""
+import random
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import gemm as og
+from paper_2608_10803_b200 import binding as ab
+from paper_2608_10803_b200 import synth
+
+from gpu_util import init
+
+pytestmark = pytest.mark.gpu
+
+
+def stream():
+    return torch.cuda.current_stream().cuda_stream
+
+
+def offset_operand(rows, cols, seed, dtype, offset):
+    """A dense operand whose first element sits `offset` elements behind an aligned address."""
+    flat = torch.empty(rows * cols + offset, dtype=synth.torch_dtype(dtype), device="cuda")
+    flat[offset:] = synth.draw_operand(rows, cols, synth.U11, seed, dtype, "cuda").reshape(-1)
+    return flat[offset:]
+
+
+@pytest.mark.parametrize("layouts", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("offset", [0, 1, 8])
+def test_grouped_list_gives_the_bits_of_single_calls(layouts, offset):
+    """Every split of the one-launch plans (1 to 16 pieces), CUDA-core plans, tile edges, both types in one list, and a list
+    longer than one launch takes."""
+    init()
+    r = random.Random(5 + offset)
+    dims = [1, 3, 16, 33, 63, 64, 65, 100, 128, 200, 257]
+    shapes = [(r.choice(dims), r.choice(dims), r.choice([1, 5, 16, 31, 64, 65, 130, 250, 400, 787, 1014])) for _ in range(90)]
+    shapes += [(64, 64, 1024), (17, 30, 900), (65, 129, 513), (4, 1000, 1000), (300, 300, 64)]
+    calls = []
+    for i, (M, N, K) in enumerate(shapes):
+        dt = ab.F16 if i % 3 else ab.BF16
+        A, B = offset_operand(M, K, 2 * i, dt, offset), offset_operand(K, N, 2 * i + 1, dt, offset)
+        C1, C2 = (torch.full((M * N + offset,), float("nan"), dtype=A.dtype, device="cuda")[offset:] for _ in range(2))
+        calls.append((ab.adapt_matmul_plan(M, N, K, dt, *layouts), A, B, C1, C2))
+    for p, A, B, C1, _ in calls:
+        ab.adapt_matmul(p, A.data_ptr(), B.data_ptr(), C1.data_ptr(), stream())
+    torch.cuda.synchronize()
+    launches = ab.adapt_launch_count()
+    ab.adapt_matmul_batch([c[0] for c in calls], *([c[j].data_ptr() for c in calls] for j in (1, 2, 4)), stream())
+    torch.cuda.synchronize()
+    assert ab.adapt_launch_count() - launches < len(calls) // 2
+    ab.adapt_poll_device_status(stream())
+    pieces = set()
+    for (p, _, _, C1, C2), shape in zip(calls, shapes):
+        pieces.add(ab.adapt_plan_info(p).cluster)
+        assert torch.equal(C1.view(torch.int16), C2.view(torch.int16)), shape
+    assert {1, 4, 8} <= pieces
+
+
+def test_grouped_list_keeps_the_order_of_dependent_calls():
+    """Calls that read what an earlier call of the list wrote, overwrite what it read, or write the same output."""
+    init()
+    n, dt = 96, ab.F16
+    plan = ab.adapt_matmul_plan(n, n, n, dt)
+    eye = torch.eye(n, dtype=torch.float16, device="cuda")
+    X = [synth.position_coded(n, n, dt, 3, "cuda").contiguous() for _ in range(2)] + [torch.zeros((n, n), dtype=torch.float16, device="cuda") for _ in range(3)]
+    roll = torch.roll(eye, 1, 1).contiguous()
+    # X2 = X0 R, X3 = X2 R, X0 = X1 I (overwrites an input), X4 = X0 R, X4 = X3 I (overwrites an output)
+    steps = [(0, roll, 2), (2, roll, 3), (1, eye, 0), (0, roll, 4), (3, eye, 4)]
+    want = [x.clone() for x in X]
+    for a, b, c in steps:
+        want[c] = want[a] @ b
+    ab.adapt_matmul_batch([plan] * 5, [X[a].data_ptr() for a, _, _ in steps], [b.data_ptr() for _, b, _ in steps],
+                          [X[c].data_ptr() for _, _, c in steps], stream())
+    torch.cuda.synchronize()
+    for x, w in zip(X, want):
+        assert torch.equal(x, w)
+
+
+def test_grouped_list_enqueues_the_calls_before_a_refused_one():
+    init()
+    plan = ab.adapt_matmul_plan(40, 24, 32, ab.F16)
+    A, B = torch.ones((40, 32), dtype=torch.float16, device="cuda"), torch.ones((32, 24), dtype=torch.float16, device="cuda")
+    C = torch.zeros((3, 40, 24), dtype=torch.float16, device="cuda")
+    with pytest.raises(ab.AdaptError) as e:
+        ab.adapt_matmul_batch([plan] * 3, [A.data_ptr()] * 3, [B.data_ptr(), 0, B.data_ptr()], [C[i].data_ptr() for i in range(3)], stream())
+    torch.cuda.synchronize()
+    assert e.value.status == ab.ERR_INVALID_ARG and bool((C[0] == 32).all()) and not C[1:].any()
+
+
+def check_strided(M, N, K, batch, dtype, lA=0, lB=0, shared_a=False, shared_b=False, gap=(0, 0, 0), offset=0, plan=None):
+    init()
+    na, nb, nc = M * K + gap[0], K * N + gap[1], M * N + gap[2]
+    def operand(count, each, seed):
+        flat = torch.empty(count * each + offset, dtype=synth.torch_dtype(dtype), device="cuda")
+        flat[offset:] = synth.draw_operand(count, each, ("integer", -4, 4), seed, dtype, "cuda").reshape(-1)
+        return flat[offset:]
+    A, B = operand(1 if shared_a else batch, na, 71), operand(1 if shared_b else batch, nb, 72)
+    C = torch.full((batch * nc + offset,), 77.0, dtype=A.dtype, device="cuda")[offset:]
+    plan = plan or ab.adapt_matmul_plan(M, N, K, dtype, lA, lB)
+    ab.adapt_matmul_strided_batch(plan, A.data_ptr(), 0 if shared_a else na, B.data_ptr(), 0 if shared_b else nb, C.data_ptr(), nc, batch, stream())
+    torch.cuda.synchronize()
+    ab.adapt_poll_device_status(stream())
+    for b in range(batch):
+        a_, b_ = A[0 if shared_a else b * na:][:M * K], B[0 if shared_b else b * nb:][:K * N]
+        _, C16 = og.gemm(synth.bits(a_), synth.bits(b_), M, N, K, dtype, lA, lB)
+        got = C[b * nc:(b + 1) * nc]
+        assert np.array_equal(synth.bits(got[:M * N]).reshape(C16.shape), C16), (M, N, K, b)
+        assert bool((got[M * N:] == 77).all()), "the gap between two outputs was written"
+
+
+@pytest.mark.parametrize("dtype", [ab.F16, ab.BF16])
+@pytest.mark.parametrize("shape", [(128, 128, 64, 5), (64, 64, 64, 3), (65, 33, 130, 7), (8, 8, 8, 40), (1, 1, 1, 9), (16, 264, 96, 6), (129, 257, 72, 4),
+                                   (40, 1000, 200, 3), (256, 128, 520, 2), (48, 80, 1024, 2), (320, 192, 128, 9), (8, 17, 33, 300)])
+def test_strided_batch_exact_in_every_layout(shape, dtype):
+    M, N, K, batch = shape
+    for lA, lB in ((0, 0), (0, 1), (1, 0), (1, 1)):
+        check_strided(M, N, K, batch, dtype, lA, lB)
+    check_strided(M, N, K, batch, dtype, shared_b=True, gap=(3, 0, 5))
+    check_strided(M, N, K, batch, dtype, 0, 1, shared_a=True, gap=(0, 8, 16))
+    check_strided(M, N, K, batch, dtype, gap=(1, 1, 1), offset=1)
+
+
+def test_strided_batch_whose_entries_feed_one_another_runs_in_order():
+    """Entry i writes the operand that entry i + 1 reads."""
+    init()
+    n, batch = 64, 6
+    X = torch.zeros((batch + 1, n, n), dtype=torch.float16, device="cuda")
+    X[0] = synth.position_coded(n, n, ab.F16, 3, "cuda")
+    roll = torch.roll(torch.eye(n, dtype=torch.float16, device="cuda"), 1, 1).contiguous()
+    plan = ab.adapt_matmul_plan(n, n, n, ab.F16)
+    ab.adapt_matmul_strided_batch(plan, X.data_ptr(), n * n, roll.data_ptr(), 0, X[1].data_ptr(), n * n, batch, stream())
+    torch.cuda.synchronize()
+    for i in range(batch):
+        assert torch.equal(X[i + 1], X[i] @ roll)
