@@ -247,9 +247,9 @@ adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t* plans, co
  * the addition done in fp32 on the accumulated sum, and ONE round-to-nearest-even cast to the 16-bit output.  D (DEVICE,
  * same 16-bit type) is an M x N row-major matrix (d_is_vector == 0) or one row of N values added to every output row
  * (d_is_vector != 0, a bias).  C may be D itself (in-place beta * C + alpha * A * B); it must not overlap A, B, or D in
- * any other way.  The GEMM kernels leave their fp32 sums in the workspace (as a split-K call does) and the fixed-order
- * reduction kernel applies alpha, beta and D before the cast, so the result is as reproducible as adapt_matmul's; plans
- * of the warp-level and one-launch families run on the CUDA-core kernel for this call.  K == 0 gives beta * D.
+ * any other way.  The kernel that stores the 16-bit output applies alpha, beta and D before the cast (the GEMM kernel itself,
+ * or the fixed-order reduction kernel of a plan with k splits), so the result is as reproducible as adapt_matmul's.
+ * K == 0 gives beta * D.
  *
  * adapt_matmul_strided_batch:  `batch` GEMMs of the plan's shape on operands stride_a, stride_b, stride_c ELEMENTS apart
  * (a stride of 0 shares that input across the batch; stride_c must be at least M * N).  The result is the one of the entries run in

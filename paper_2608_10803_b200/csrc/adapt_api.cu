@@ -563,15 +563,15 @@ extern "C" int64_t adapt_plan_many(int64_t count, const int64_t* dims, const int
 // ---------------------------------------------------------------------------------------------
 typedef const void* UmmaKernel;     // the parameter pack's type depends on the kernel mode: launched through cudaLaunchKernelExC
 
-template <int CG>
+template <int CG, bool EPI>
 static UmmaKernel umma_lookup(int BN, bool a_mn, bool b_mn)
 {
 #define ADAPT_PICK(bn)                                                               \
     if (BN == bn) {                                                                  \
-        if (!a_mn && !b_mn) return (const void*)umma_gemm_kernel<bn, false, false, CG, 0>;    \
-        if (!a_mn && b_mn) return (const void*)umma_gemm_kernel<bn, false, true, CG, 0>;      \
-        if (a_mn && !b_mn) return (const void*)umma_gemm_kernel<bn, true, false, CG, 0>;      \
-        return (const void*)umma_gemm_kernel<bn, true, true, CG, 0>;                          \
+        if (!a_mn && !b_mn) return (const void*)umma_gemm_kernel<bn, false, false, CG, 0, false, false, EPI>;    \
+        if (!a_mn && b_mn) return (const void*)umma_gemm_kernel<bn, false, true, CG, 0, false, false, EPI>;      \
+        if (a_mn && !b_mn) return (const void*)umma_gemm_kernel<bn, true, false, CG, 0, false, false, EPI>;      \
+        return (const void*)umma_gemm_kernel<bn, true, true, CG, 0, false, false, EPI>;                          \
     }
     if constexpr (CG == 1) { ADAPT_PICK(64) }
     ADAPT_PICK(128)
@@ -619,7 +619,37 @@ static UmmaKernel launch_map_umma_sk(int family, int BN, bool a_mn, bool b_mn)
     return family == ADAPT_FAM_UMMA_1CTA ? umma_lookup_sk<1>(BN, a_mn, b_mn) : umma_lookup_sk<2>(BN, a_mn, b_mn);
 }
 
-static UmmaKernel launch_map_umma(int family, int BN, bool a_mn, bool b_mn, int mode = 0, bool fused = false)
+template <bool EPI>
+static UmmaKernel launch_map_umma_plain(int family, int BN, bool a_mn, bool b_mn, int mode)
+{
+    if (mode == 1 && family == ADAPT_FAM_UMMA_2CTA) {     // 256 rows of one row class per SM pair
+        if (BN == 128) return (const void*)umma_gemm_kernel<128, false, true, 2, 1, false, false, EPI>;
+        if (BN == 256) return (const void*)umma_gemm_kernel<256, false, true, 2, 1, false, false, EPI>;
+        if (BN == 144) return (const void*)umma_gemm_kernel<144, false, true, 2, 1, false, false, EPI>;    // 128 / 192 owned + 16 halo columns, 16 row classes
+        if (BN == 208) return (const void*)umma_gemm_kernel<208, false, true, 2, 1, false, false, EPI>;
+        return nullptr;
+    }
+    if (mode == 1) {                     // row-major A read through per-row-class maps (1-CTA tiles, row-major B)
+        if (BN == 64) return (const void*)umma_gemm_kernel<64, false, true, 1, 1, false, false, EPI>;
+        if (BN == 128) return (const void*)umma_gemm_kernel<128, false, true, 1, 1, false, false, EPI>;
+        if (BN == 256) return (const void*)umma_gemm_kernel<256, false, true, 1, 1, false, false, EPI>;
+        if (BN == 80) return (const void*)umma_gemm_kernel<80, false, true, 1, 1, false, false, EPI>;      // 64 / 128 / 192 owned + 16 halo columns
+        if (BN == 144) return (const void*)umma_gemm_kernel<144, false, true, 1, 1, false, false, EPI>;
+        if (BN == 208) return (const void*)umma_gemm_kernel<208, false, true, 1, 1, false, false, EPI>;
+        return nullptr;
+    }
+    if (mode == 2) {                     // B through per-k-class maps: eight accumulators (BN = 64), or classes as k splits
+        if (BN == 64) return (const void*)umma_gemm_kernel<64, false, true, 1, 2, false, false, EPI>;
+        if (BN == 128) return (const void*)umma_gemm_kernel<128, false, true, 1, 3>;
+        if (BN == 256) return family == ADAPT_FAM_UMMA_2CTA ? (const void*)umma_gemm_kernel<256, false, true, 2, 3>
+                                                             : (const void*)umma_gemm_kernel<256, false, true, 1, 3>;
+        return nullptr;
+    }
+    return family == ADAPT_FAM_UMMA_1CTA ? umma_lookup<1, EPI>(BN, a_mn, b_mn) : umma_lookup<2, EPI>(BN, a_mn, b_mn);
+}
+
+// epi: the instantiation that adds beta * D itself (fused kernels take it at run time; k classes as k splits have none)
+static UmmaKernel launch_map_umma(int family, int BN, bool a_mn, bool b_mn, int mode = 0, bool fused = false, bool epi = false)
 {
     if (fused) {
         if (family != ADAPT_FAM_UMMA_1CTA) return nullptr;
@@ -634,30 +664,7 @@ static UmmaKernel launch_map_umma(int family, int BN, bool a_mn, bool b_mn, int 
         if (BN == 256) return (const void*)umma_gemm_kernel<256, false, true, 1, 3, true>;
         return nullptr;
     }
-    if (mode == 1 && family == ADAPT_FAM_UMMA_2CTA) {     // 256 rows of one row class per SM pair
-        if (BN == 128) return (const void*)umma_gemm_kernel<128, false, true, 2, 1>;
-        if (BN == 256) return (const void*)umma_gemm_kernel<256, false, true, 2, 1>;
-        if (BN == 144) return (const void*)umma_gemm_kernel<144, false, true, 2, 1>;    // 128 / 192 owned + 16 halo columns, 16 row classes
-        if (BN == 208) return (const void*)umma_gemm_kernel<208, false, true, 2, 1>;
-        return nullptr;
-    }
-    if (mode == 1) {                     // row-major A read through per-row-class maps (1-CTA tiles, row-major B)
-        if (BN == 64) return (const void*)umma_gemm_kernel<64, false, true, 1, 1>;
-        if (BN == 128) return (const void*)umma_gemm_kernel<128, false, true, 1, 1>;
-        if (BN == 256) return (const void*)umma_gemm_kernel<256, false, true, 1, 1>;
-        if (BN == 80) return (const void*)umma_gemm_kernel<80, false, true, 1, 1>;      // 64 / 128 / 192 owned + 16 halo columns
-        if (BN == 144) return (const void*)umma_gemm_kernel<144, false, true, 1, 1>;
-        if (BN == 208) return (const void*)umma_gemm_kernel<208, false, true, 1, 1>;
-        return nullptr;
-    }
-    if (mode == 2) {                     // B through per-k-class maps: eight accumulators (BN = 64), or classes as k splits
-        if (BN == 64) return (const void*)umma_gemm_kernel<64, false, true, 1, 2>;
-        if (BN == 128) return (const void*)umma_gemm_kernel<128, false, true, 1, 3>;
-        if (BN == 256) return family == ADAPT_FAM_UMMA_2CTA ? (const void*)umma_gemm_kernel<256, false, true, 2, 3>
-                                                             : (const void*)umma_gemm_kernel<256, false, true, 1, 3>;
-        return nullptr;
-    }
-    return family == ADAPT_FAM_UMMA_1CTA ? umma_lookup<1>(BN, a_mn, b_mn) : umma_lookup<2>(BN, a_mn, b_mn);
+    return epi ? launch_map_umma_plain<true>(family, BN, a_mn, b_mn, mode) : launch_map_umma_plain<false>(family, BN, a_mn, b_mn, mode);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -692,25 +699,14 @@ extern "C" adapt_status_t adapt_init(int device)
     CUDA_TRY(cudaMemset(S.d_trace, 0, 8 * 60002));
 #endif
     // opt every tensor-core kernel into the full shared-memory carve-out
-    for (int fam = ADAPT_FAM_UMMA_1CTA; fam <= ADAPT_FAM_UMMA_2CTA; ++fam)
-        for (int BN : {64, 128, 256})
-            for (int a = 0; a < 2; ++a)
-                for (int b = 0; b < 2; ++b) {
-                    UmmaKernel k = launch_map_umma(fam, BN, a != 0, b != 0);
-                    if (!k) continue;
-                    CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
-                }
-    for (int BN : {64, 128, 256, 80, 144, 208})
-        CUDA_TRY(cudaFuncSetAttribute(launch_map_umma(ADAPT_FAM_UMMA_1CTA, BN, false, true, 1),
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
-    for (int BN : {64, 128, 256})
-        CUDA_TRY(cudaFuncSetAttribute(launch_map_umma(ADAPT_FAM_UMMA_1CTA, BN, false, true, 2),
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
-    CUDA_TRY(cudaFuncSetAttribute(launch_map_umma(ADAPT_FAM_UMMA_2CTA, 256, false, true, 2),
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
-    for (int BN : {128, 256, 144, 208})
-        CUDA_TRY(cudaFuncSetAttribute(launch_map_umma(ADAPT_FAM_UMMA_2CTA, BN, false, true, 1),
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
+    for (int epi = 0; epi < 2; ++epi)
+        for (int fam = ADAPT_FAM_UMMA_1CTA; fam <= ADAPT_FAM_UMMA_2CTA; ++fam)
+            for (int mode = 0; mode < 3; ++mode)
+                for (int BN : {64, 128, 256, 80, 144, 208})
+                    for (int v = 0; v < (mode == 0 ? 4 : 1); ++v) {
+                        UmmaKernel k = launch_map_umma(fam, BN, (v & 1) != 0, mode != 0 || (v & 2) != 0, mode, false, epi != 0);
+                        if (k) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
+                    }
     for (int BN : {64, 128, 256}) {
         for (int a = 0; a < 2; ++a)
             for (int b = 0; b < 2; ++b)
@@ -989,9 +985,7 @@ adapt_status_t launch_pad2(State& S, const void* srcA, void* dstA, int64_t outer
 adapt_status_t launch_reduce(State& S, const float* partial, void* C, int64_t M, int64_t N, int P_k, int dtype, cudaStream_t stream,
                              const ReduceEpilogue* epi = nullptr)
 {
-    ReduceEpilogue ep;
-    ep.D = nullptr; ep.d_is_vector = 0; ep.alpha = 1.f; ep.beta = 0.f;
-    if (epi) ep = *epi;
+    const ReduceEpilogue ep = epi ? *epi : no_epilogue();
     const int64_t Np = partial_pitch(N);
     const int64_t work = M * (Np / 4);
     const int blocks = (int)std::min<int64_t>(ceil_div(work, 256), (int64_t)S.machine.n_sm * 8);
@@ -1052,9 +1046,11 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
     p.num_units = p.P_m * p.P_n * p.P_k;
 
     // the plan's fused reduction stands unless a fallback changed the tiling (then: partials in the workspace)
-    // (a fused-add epilogue runs in the reduction kernel: the GEMM then always leaves fp32 partials in the workspace)
-    const bool fused = !epi && c.fused != 0 && p.P_k == c.P_k && !(c.srcB == ADAPT_SRC_TMA_CLASSES && !kclsB);
-    const size_t szP = ((p.P_k > 1 || epi) && !fused) ? (size_t)round_up((int64_t)p.P_k * s.M * partial_pitch(s.N) * 4, 256) : 0;
+    const bool fused = c.fused != 0 && p.P_k == c.P_k && !(c.srcB == ADAPT_SRC_TMA_CLASSES && !kclsB);
+    // a fused add runs where the 16-bit output is stored: here, or with unfused k splits in the reduction kernel
+    const bool partials = p.P_k > 1 && !fused;
+    p.ep = epi && !partials ? *epi : no_epilogue();
+    const size_t szP = partials ? (size_t)round_up((int64_t)p.P_k * s.M * partial_pitch(s.N) * 4, 256) : 0;
     // stream-K stands unless a fallback changed the tiling; one fp32 partial tile per CTA
     const bool streamk = !epi && c.streamk != 0 && p.P_k == 1 && !classesA && !kclsB;
     const int sk_slots = S.machine.n_sm / c.cluster;
@@ -1088,7 +1084,7 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
         if ((r = launch_pad(S, B, w8 + szA, outB, inB, pitchB, stream)) != ADAPT_OK) return r;
         b_src = w8 + szA;
     }
-    float* partial = ((p.P_k > 1 || epi) && !fused) ? (float*)(w8 + szA + szB) : nullptr;
+    float* partial = partials ? (float*)(w8 + szA + szB) : nullptr;
 
     // K-major operand: one box of 64 k x (rows this CTA owns); MN-major operand: boxes of 64 x 64
     if (classesA) {
@@ -1121,7 +1117,7 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
     p.part_hint = (p.P_k > 1 && szP <= ((size_t)100 << 20)) ? 1 : 0;
     memset(p.c_sigma, 0, sizeof(p.c_sigma));
     memset(p.c_extent, 0, sizeof(p.c_extent));
-    if (p.P_k == 1 && !epi && !kclsB && (halo ? ((uintptr_t)C & 15) == 0 : (((uintptr_t)C & 31) == 0 && s.N % 16 == 0))) {
+    if (p.P_k == 1 && !kclsB && (halo ? ((uintptr_t)C & 15) == 0 : (((uintptr_t)C & 31) == 0 && s.N % 16 == 0))) {
         if (classesA) {
             if ((r = cached_class_maps(S, pl, kMapC, C, s.M, s.N, 32, ncls, 32, true, maps.c, p.c_sigma, p.c_extent)) != ADAPT_OK)
                 return r;
@@ -1141,7 +1137,6 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
     p.prefetch = S.prefetch;
     p.shuffle_k = S.shuffle_k;
     p.ncls_log2 = ncls == 16 ? 4 : (ncls == 8 ? 3 : (ncls == 4 ? 2 : 1));
-    p.force_partial = epi ? 1 : 0;
     p.a_shift_any = 0;
     for (int j = 0; j < 16; ++j) p.a_shift_any |= p.a_sigma[j];
     if (p.a_shift_any) p.a_shift_any = 1;
@@ -1180,7 +1175,7 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
 #endif
 
     UmmaKernel k = streamk ? launch_map_umma_sk(c.family, c.BN, a_mn, b_mn)
-                           : launch_map_umma(c.family, c.BN, a_mn, b_mn, classesA ? 1 : (kclsB ? 2 : 0), fused);
+                           : launch_map_umma(c.family, c.BN, a_mn, b_mn, classesA ? 1 : (kclsB ? 2 : 0), fused, p.ep.D != nullptr);
     if (!k) return fail(ADAPT_ERR_UNSUPPORTED, "no compiled kernel for this tiling key%s");
     const int slots = fused ? umma_cluster_slots(S.machine, p.P_k) : S.machine.n_sm / cg;
     const int launch_cluster = fused ? p.P_k : cg;            // fused split-K: the splits of a tile are one cluster
@@ -1220,16 +1215,15 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
     }
     CUDA_TRY(launch_exc(&cfg, k, args, arg_bytes, 2));
     S.launches.fetch_add(1, std::memory_order_relaxed);
-    if ((p.P_k > 1 || epi) && !fused) return launch_reduce(S, partial, C, s.M, s.N, p.P_k, s.dtype, stream, epi);
+    if (partials) return launch_reduce(S, partial, C, s.M, s.N, p.P_k, s.dtype, stream, epi);
     return ADAPT_OK;
 }
 
-// The CUDA-core kernel with an explicit split count (the plan's own family, and the stand-in of the families that have
-// no fp32 partial path when a fused-add epilogue is asked for).
-adapt_status_t run_simt_splits(State& S, const Shape& s, int P_k, const void* A, const void* B, void* C, cudaStream_t stream,
-                               const ReduceEpilogue* epi)
+adapt_status_t run_simt(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi = nullptr)
 {
-    const bool partials = P_k > 1 || epi;
+    const Shape& s = pl->s;
+    const int P_k = pl->c.P_k;
+    const bool partials = P_k > 1;
     const size_t szP = partials ? (size_t)round_up((int64_t)P_k * s.M * partial_pitch(s.N) * 4, 256) : 0;
     void* ws = nullptr;
     adapt_status_t r = get_workspace(S, stream, szP, &ws);
@@ -1239,7 +1233,8 @@ adapt_status_t run_simt_splits(State& S, const Shape& s, int P_k, const void* A,
     if (s.layoutA == ADAPT_ROW_MAJOR) { p.a_sm = s.K; p.a_sk = 1; } else { p.a_sm = 1; p.a_sk = s.M; }
     if (s.layoutB == ADAPT_ROW_MAJOR) { p.b_sk = s.N; p.b_sn = 1; } else { p.b_sk = 1; p.b_sn = s.K; }
     p.P_n = (int)ceil_div(s.N, 64);
-    p.P_k = partials ? std::max(P_k, 2) : 1;                  // any value > 1 makes the kernel write fp32 partials
+    p.P_k = P_k;
+    p.ep = epi && !partials ? *epi : no_epilogue();
     p.Np = (int)partial_pitch(s.N);
     p.kb_per_split = (int)ceil_div(ceil_div(s.K, 16), P_k);
     p.dtype = s.dtype;
@@ -1254,7 +1249,15 @@ adapt_status_t run_simt_splits(State& S, const Shape& s, int P_k, const void* A,
     return ADAPT_OK;
 }
 
-adapt_status_t run_simt(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream)
+adapt_status_t run_cluster(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi = nullptr)
+{
+    if (launch_cluster(pl->s, pl->c, A, B, C, stream, S.prefetch, epi) != ADAPT_OK) return fail(ADAPT_ERR_CUDA, "cluster kernel launch failed%s");
+    S.launches.fetch_add(1, std::memory_order_relaxed);
+    CUDA_TRY(cudaGetLastError());
+    return ADAPT_OK;
+}
+
+adapt_status_t run_skinny(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi = nullptr)
 {
     const Shape& s = pl->s;
     const Config& c = pl->c;
@@ -1262,48 +1265,24 @@ adapt_status_t run_simt(State& S, Plan* pl, const void* A, const void* B, void* 
     void* ws = nullptr;
     adapt_status_t r = get_workspace(S, stream, szP, &ws);
     if (r != ADAPT_OK) return r;
-    SimtParams p;
-    p.M = (int)s.M; p.N = (int)s.N; p.K = (int)s.K;
-    if (s.layoutA == ADAPT_ROW_MAJOR) { p.a_sm = s.K; p.a_sk = 1; } else { p.a_sm = 1; p.a_sk = s.M; }
-    if (s.layoutB == ADAPT_ROW_MAJOR) { p.b_sk = s.N; p.b_sn = 1; } else { p.b_sk = 1; p.b_sn = s.K; }
-    p.P_n = c.P_n;
-    p.P_k = c.P_k;
-    p.Np = (int)partial_pitch(s.N);
-    p.kb_per_split = (int)ceil_div(ceil_div(s.K, 16), c.P_k);
-    p.dtype = s.dtype;
-    p.prefetch = S.prefetch;
-    p.C = (unsigned short*)C;
-    p.partial = (float*)ws;
-    dim3 grid((unsigned)((int64_t)c.P_m * c.P_n), (unsigned)c.P_k, 1);
-    CUDA_TRY(launch_pdl(simt_gemm_kernel, grid, dim3(256), 0, stream, (const unsigned short*)A, (const unsigned short*)B, p));
-    S.launches.fetch_add(1, std::memory_order_relaxed);
-    CUDA_TRY(cudaGetLastError());
-    if (c.P_k > 1) return launch_reduce(S, (const float*)ws, C, s.M, s.N, c.P_k, s.dtype, stream);
-    return ADAPT_OK;
-}
-
-adapt_status_t run_cluster(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream)
-{
-    if (launch_cluster(pl->s, pl->c, A, B, C, stream, S.prefetch) != ADAPT_OK) return fail(ADAPT_ERR_CUDA, "cluster kernel launch failed%s");
-    S.launches.fetch_add(1, std::memory_order_relaxed);
-    CUDA_TRY(cudaGetLastError());
-    return ADAPT_OK;
-}
-
-adapt_status_t run_skinny(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream)
-{
-    const Shape& s = pl->s;
-    const Config& c = pl->c;
-    const size_t szP = c.P_k > 1 ? (size_t)round_up((int64_t)c.P_k * s.M * partial_pitch(s.N) * 4, 256) : 0;
-    void* ws = nullptr;
-    adapt_status_t r = get_workspace(S, stream, szP, &ws);
-    if (r != ADAPT_OK) return r;
-    r = launch_skinny(s, c, A, B, C, (float*)ws, stream);
+    r = launch_skinny(s, c, A, B, C, (float*)ws, stream, epi);
     if (r != ADAPT_OK) return fail(r, "skinny kernel launch failed%s");
     S.launches.fetch_add(1, std::memory_order_relaxed);
     CUDA_TRY(cudaGetLastError());
-    if (c.P_k > 1) return launch_reduce(S, (const float*)ws, C, s.M, s.N, c.P_k, s.dtype, stream);
+    if (c.P_k > 1) return launch_reduce(S, (const float*)ws, C, s.M, s.N, c.P_k, s.dtype, stream, epi);
     return ADAPT_OK;
+}
+
+adapt_status_t run_plan(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi)
+{
+    switch (pl->c.family) {
+        case ADAPT_FAM_UMMA_1CTA:
+        case ADAPT_FAM_UMMA_2CTA: return run_umma(S, pl, A, B, C, stream, epi);
+        case ADAPT_FAM_SKINNY: return run_skinny(S, pl, A, B, C, stream, epi);
+        case ADAPT_FAM_SIMT: return run_simt(S, pl, A, B, C, stream, epi);
+        case ADAPT_FAM_CLUSTER: return run_cluster(S, pl, A, B, C, stream, epi);
+    }
+    return fail(ADAPT_ERR_UNSUPPORTED, "unknown kernel family%s");
 }
 
 bool overlaps(const void* a, size_t an, const void* b, size_t bn)
@@ -1332,14 +1311,7 @@ extern "C" adapt_status_t adapt_matmul(adapt_handle_t plan, const void* A, const
     if (((uintptr_t)A | (uintptr_t)B | (uintptr_t)C) & 1) return fail(ADAPT_ERR_INVALID_ARG, "operands must be 2-byte aligned%s");
     const size_t nA = (size_t)s.M * s.K * 2, nB = (size_t)s.K * s.N * 2, nC = (size_t)s.M * s.N * 2;
     if (overlaps(C, nC, A, nA) || overlaps(C, nC, B, nB)) return fail(ADAPT_ERR_INVALID_ARG, "C overlaps an input%s");
-    switch (pl->c.family) {
-        case ADAPT_FAM_UMMA_1CTA:
-        case ADAPT_FAM_UMMA_2CTA: return run_umma(S, pl, A, B, C, stream);
-        case ADAPT_FAM_SKINNY: return run_skinny(S, pl, A, B, C, stream);
-        case ADAPT_FAM_SIMT: return run_simt(S, pl, A, B, C, stream);
-        case ADAPT_FAM_CLUSTER: return run_cluster(S, pl, A, B, C, stream);
-    }
-    return fail(ADAPT_ERR_UNSUPPORTED, "unknown kernel family%s");
+    return run_plan(S, pl, A, B, C, stream, nullptr);
 }
 
 extern "C" adapt_status_t adapt_addmm(adapt_handle_t plan, const void* A, const void* B, const void* D, int d_is_vector,
@@ -1367,18 +1339,7 @@ extern "C" adapt_status_t adapt_addmm(adapt_handle_t plan, const void* A, const 
         // K == 0: the product is zero; the reduction kernel over zero partial slabs leaves beta * D
         return launch_reduce(S, nullptr, C, s.M, s.N, 0, s.dtype, stream, &ep);
     }
-    switch (pl->c.family) {
-        case ADAPT_FAM_UMMA_1CTA:
-        case ADAPT_FAM_UMMA_2CTA: return run_umma(S, pl, A, B, C, stream, &ep);
-        default: break;
-    }
-    // the warp-level and one-launch families have no fp32 partial path: the CUDA-core kernel stands in, with enough k
-    // splits to fill the machine (their shapes are small or skinny)
-    const int64_t tiles = ceil_div(s.M, 64) * ceil_div(s.N, 64), ksteps = ceil_div(s.K, 16);
-    int64_t pk = pl->c.family == ADAPT_FAM_SIMT ? pl->c.P_k : std::max<int64_t>(1, std::min<int64_t>((4 * (int64_t)S.machine.n_sm) / tiles, ksteps / 4));
-    pk = std::max<int64_t>(1, std::min<int64_t>(pk, 256));
-    pk = ceil_div(ksteps, ceil_div(ksteps, pk));               // no empty split
-    return run_simt_splits(S, s, (int)pk, A, B, C, stream, &ep);
+    return run_plan(S, pl, A, B, C, stream, &ep);
 }
 
 namespace {

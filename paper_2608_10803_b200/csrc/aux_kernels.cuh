@@ -26,6 +26,25 @@ __device__ __forceinline__ unsigned short float_to_16(float a, int dtype)
     return *reinterpret_cast<unsigned short*>(&h);
 }
 
+// Fused-add epilogue (the AddMM operator): out = alpha * sum + beta * D in fp32 before the single cast, D either a
+// full M x N 16-bit matrix or one row of N values added to every row.  D == nullptr: plain sum.
+struct ReduceEpilogue {
+    const unsigned short* D;
+    int d_is_vector;
+    float alpha, beta;
+};
+inline ReduceEpilogue no_epilogue()
+{
+    ReduceEpilogue e;
+    e.D = nullptr; e.d_is_vector = 0; e.alpha = 1.f; e.beta = 0.f;
+    return e;
+}
+__device__ __forceinline__ float fused_add(const ReduceEpilogue& e, float v, int m, int n, int N, int dtype)
+{
+    if (!e.D) return v;
+    return fmaf(e.beta, load16_as_float(e.D + (e.d_is_vector ? (int64_t)n : (int64_t)m * N + n), dtype), e.alpha * v);
+}
+
 // ---- Padding: re-pitch a dense [outer][inner] 16-bit matrix to [outer][pitch], pitch % 8 == 0 ----
 // One thread produces one 16-byte chunk of the destination.  The pad columns are written as zeros:
 // the tensor map of a narrow operand (inner < 64, pitch a 32-byte multiple) covers them, so that
@@ -196,13 +215,6 @@ regroup_a_kernel(const unsigned short* __restrict__ A, unsigned short* __restric
 // The order is fixed, so the result does not depend on which CTA finished first.  Partials are
 // stored [P_k][M][Np] with Np = N rounded up to 8, so every row starts on a 32-byte boundary and
 // one thread reduces four consecutive columns with 16-byte loads.
-// Optional fused-add epilogue (the AddMM operator): out = alpha * sum + beta * D in fp32 before the single cast, D either a
-// full M x N 16-bit matrix or one row of N values added to every row.  D == nullptr: plain sum.
-struct ReduceEpilogue {
-    const unsigned short* D;
-    int d_is_vector;
-    float alpha, beta;
-};
 __global__ void __launch_bounds__(256)
 splitk_reduce_kernel(const float* __restrict__ partial, unsigned short* __restrict__ C,
                      int M, int N, int Np, int P_k, int dtype, const ReduceEpilogue ep)
@@ -264,6 +276,7 @@ struct SimtParams {
     int prefetch;                // L2 prefetch of the first k steps ahead of the dependency wait
     unsigned short* C;
     float* partial;
+    ReduceEpilogue ep;           // P_k == 1 only
 };
 
 // One 64 x 64 tile at (m0, n0), k split `split`; sA and sB are 16 x 68 floats of shared memory each.
@@ -341,7 +354,7 @@ __device__ __forceinline__ void simt_tile_body(const unsigned short* __restrict_
         for (int j = 0; j < 4; ++j) {
             const int n = n0 + tx * 4 + j;
             if (n >= p.N) continue;
-            if (p.P_k == 1) p.C[(int64_t)m * p.N + n] = float_to_16(acc[i][j], p.dtype);
+            if (p.P_k == 1) p.C[(int64_t)m * p.N + n] = float_to_16(fused_add(p.ep, acc[i][j], m, n, p.N, p.dtype), p.dtype);
             else p.partial[((int64_t)split * p.M + m) * p.Np + n] = acc[i][j];
         }
     }

@@ -313,11 +313,7 @@ __device__ __forceinline__ void cluster_tile_body(const ClusterParams& p, int m0
         }
     }
     // the fused add: alpha * sum + beta * D in fp32, before the cast
-    auto finish = [&](float v, int m, int n) -> float {
-        if (!p.ep.D) return v;
-        const unsigned short* d = p.ep.D + (p.ep.d_is_vector ? (int64_t)n : (int64_t)m * p.N + n);
-        return fmaf(p.ep.beta, load16_as_float(d, BF16 ? 1 : 0), p.ep.alpha * v);
-    };
+    auto finish = [&](float v, int m, int n) -> float { return fused_add(p.ep, v, m, n, p.N, BF16 ? 1 : 0); };
 
     // rounds and stores this thread's accumulators, or (both) the half of them that its group stores with the other group's sums
     // added from shared memory; a lane holds pairs of neighbouring columns
@@ -515,8 +511,7 @@ inline adapt_status_t launch_cluster(const Shape& s, const Config& c, const void
     p.ring = seq ? cluster_seq_ring((int)ceil_div(s.K, 2 * kClusterKS)) : c.stages;
     p.prefetch = prefetch;
     p.aligned = (rows_aligned16(A, p.lda) ? 1 : 0) | (rows_aligned16(B, p.ldb) ? 2 : 0);
-    p.ep.D = nullptr; p.ep.d_is_vector = 0; p.ep.alpha = 1.f; p.ep.beta = 0.f;
-    if (epi) p.ep = *epi;
+    p.ep = epi ? *epi : no_epilogue();
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)((int64_t)c.P_m * c.P_n * c.cluster), 1, 1);

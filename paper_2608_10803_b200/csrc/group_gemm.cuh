@@ -72,7 +72,7 @@ group_gemm_kernel(const __grid_constant__ GroupParams p)
         q.b_sk = B_KC ? 1 : it.N; q.b_sn = B_KC ? it.K : 1;
         q.P_n = it.P_n; q.P_k = 1; q.kb_per_split = (it.K + 15) / 16;
         q.Np = 0; q.dtype = BF16 ? 1 : 0; q.prefetch = 0;
-        q.C = C; q.partial = nullptr;
+        q.C = C; q.partial = nullptr; q.ep.D = nullptr;
         SimtStage* sm = reinterpret_cast<SimtStage*>(s_dyn);
         simt_tile_body(A, B, q, m0, n0, 0, sm[0], sm[1]);
         return;
@@ -88,7 +88,7 @@ group_gemm_kernel(const __grid_constant__ GroupParams p)
     q.ring = p.ring;
     q.prefetch = p.prefetch;
     q.aligned = (rows_aligned16(A, q.lda) ? 1 : 0) | (rows_aligned16(B, q.ldb) ? 2 : 0);
-    q.ep.D = nullptr; q.ep.d_is_vector = 0; q.ep.alpha = 1.f; q.ep.beta = 0.f;
+    q.ep.D = nullptr;
     cluster_tile_body<A_KC, B_KC, BF16, !SHORT>(q, m0, n0, s_dyn);
 }
 

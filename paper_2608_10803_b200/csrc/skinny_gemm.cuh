@@ -27,6 +27,7 @@
 #include <cuda_bf16.h>
 
 #include "adapt_internal.h"
+#include "aux_kernels.cuh"        // 16-bit conversions, fused-add parameters
 #include "launch_pdl.cuh"
 
 namespace adapt {
@@ -53,6 +54,8 @@ struct SkinnyParams {
     int64_t out_ss, out_sr;          // element strides of the output along s and r
     int64_t part_ss, part_sr;        // element strides of the fp32 partial along s and r
     int64_t part_slab;               // elements per split: M * Np
+    int N, n_streamed;               // output columns; 1: the streamed side is n, 0: it is m
+    ReduceEpilogue ep;               // used when P_k == 1
 };
 
 // Eight consecutive 16-bit elements from a 2-byte aligned address, branch-free.
@@ -251,10 +254,9 @@ skinny_gemm_kernel(const SkinnyParams p)
             float sum = 0.f;
             for (int w = 0; w < WK; ++w) sum += s_out[(w * warps_r + w0) * (16 * 64) + s * 64 + rr];
             if (p.P_k == 1) {
-                unsigned short h;
-                if (BF16) { __nv_bfloat16 b = __float2bfloat16_rn(sum); h = *reinterpret_cast<unsigned short*>(&b); }
-                else { __half b = __float2half_rn(sum); h = *reinterpret_cast<unsigned short*>(&b); }
-                p.C[(int64_t)s * p.out_ss + (int64_t)r * p.out_sr] = h;
+                // the streamed side is n or m
+                const float out = fused_add(p.ep, sum, p.n_streamed ? s : r, p.n_streamed ? r : s, p.N, BF16 ? 1 : 0);
+                p.C[(int64_t)s * p.out_ss + (int64_t)r * p.out_sr] = float_to_16(out, BF16 ? 1 : 0);
             } else {
                 p.partial[(int64_t)split * p.part_slab + (int64_t)s * p.part_ss + (int64_t)r * p.part_sr] = sum;
             }
@@ -311,10 +313,9 @@ skinny_gemm_kernel(const SkinnyParams p)
                 if (s >= p.ms || rr >= p.R) continue;
                 const float sum = acc[0][i] + acc[1][i];
                 if (p.P_k == 1) {
-                    unsigned short h;
-                    if (BF16) { __nv_bfloat16 b = __float2bfloat16_rn(sum); h = *reinterpret_cast<unsigned short*>(&b); }
-                    else { __half b = __float2half_rn(sum); h = *reinterpret_cast<unsigned short*>(&b); }
-                    p.C[(int64_t)s * p.out_ss + (int64_t)rr * p.out_sr] = h;
+                    // the streamed side is n or m
+                    const float out = fused_add(p.ep, sum, p.n_streamed ? s : rr, p.n_streamed ? rr : s, p.N, BF16 ? 1 : 0);
+                    p.C[(int64_t)s * p.out_ss + (int64_t)rr * p.out_sr] = float_to_16(out, BF16 ? 1 : 0);
                 } else {
                     p.partial[(int64_t)split * p.part_slab + (int64_t)s * p.part_ss + (int64_t)rr * p.part_sr] = sum;
                 }
@@ -334,12 +335,13 @@ inline SkinnyKernel skinny_pick(bool bf16, bool aligned)
 
 // Host launcher: maps (M, N, K, layouts) onto the canonical form above.
 inline adapt_status_t launch_skinny(const Shape& s, const Config& c, const void* A, const void* B, void* C,
-                                    float* partial, cudaStream_t stream)
+                                    float* partial, cudaStream_t stream, const ReduceEpilogue* epi = nullptr)
 {
     SkinnyParams p;
     bool kc;
     if (s.M <= 16 && (s.M <= s.N || s.N > 16)) {
         // Small = A, streamed = B
+        p.n_streamed = 1;
         p.Small = (const unsigned short*)A;
         p.Str = (const unsigned short*)B;
         p.ms = (int)s.M; p.R = (int)s.N;
@@ -350,6 +352,7 @@ inline adapt_status_t launch_skinny(const Shape& s, const Config& c, const void*
         p.part_ss = partial_pitch(s.N); p.part_sr = 1;
     } else {
         // Small = B^T, streamed = A^T
+        p.n_streamed = 0;
         p.Small = (const unsigned short*)B;
         p.Str = (const unsigned short*)A;
         p.ms = (int)s.N; p.R = (int)s.M;
@@ -362,6 +365,8 @@ inline adapt_status_t launch_skinny(const Shape& s, const Config& c, const void*
     p.K = (int)s.K;
     p.BNs = c.BN;
     p.P_k = c.P_k;
+    p.N = (int)s.N;
+    p.ep = epi && c.P_k == 1 ? *epi : no_epilogue();        // with k splits the reduction kernel adds D
     // splits are whole multiples of the staging chunk so that no chunk straddles two splits
     const int64_t chunks = ceil_div(s.K, kSkinnyKChunk);
     p.k_per_split = (int)(ceil_div(chunks, c.P_k) * kSkinnyKChunk);

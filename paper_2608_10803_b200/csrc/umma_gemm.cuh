@@ -23,6 +23,7 @@
 #include <cuda_bf16.h>
 
 #include "adapt_internal.h"
+#include "aux_kernels.cuh"        // fused-add parameters
 #include "ptx_sm100.cuh"
 #include "launch_pdl.cuh"
 
@@ -54,7 +55,6 @@ struct UmmaParams {
     int c_mode;                      // 16-bit output: 0 = stores by the epilogue threads (any N, any alignment),
                                      // 1 = TMA stores through the maps of C (rows of C, or of the tile's row class,
                                      //     start on 32-byte boundaries; class tiles with 16 halo columns shift them there)
-    int force_partial;               // write fp32 partials also with P_k = 1 (a fused-add epilogue follows in the reduction kernel)
     int shuffle_k;                   // ShuffleK (Table 2): a tile starts its k range at a k-block that depends on the tile, so the CTAs of a wave
                                      // do not all ask for the same k slice of a shared operand at the same moment (plain tiles only)
     int prefetch;                    // ask L2 for the first unit's operand boxes before waiting for the kernel ahead on the stream
@@ -74,6 +74,7 @@ struct UmmaParams {
     int x_rows, x_pitch;             // fused split-K: rows and row pitch (fp32 elements) of the partial tile each CTA of the
                                      // cluster keeps in its shared memory for the exchange
     int ncls_log2;                   // halo class tiles: log2 of the number of row classes (1 .. 4)
+    ReduceEpilogue ep;               // fused add (AddMM) where the kernel stores the 16-bit output itself; D == nullptr: none
     unsigned int* status;            // device status word: bit 0 = a bounded wait expired
     unsigned long long* trace;       // timestamp trace of one CTA (diagnostic builds only), else null
     int trace_cta;
@@ -240,6 +241,32 @@ __device__ __forceinline__ void store_run16(unsigned short* dst, int count, cons
     }
 }
 
+// r[i] = alpha * r[i] + beta * D[row][n + i] for the columns below `end` (AddMM, in fp32 before the cast); a row that does not
+// exist (!row_ok) is left alone.  A row of D is read as 16-byte pieces where they are aligned and whole: a thread owns 32
+// consecutive columns, two whole sectors when N % 16 == 0; a bias is the same address for all lanes.
+// Adding D here instead of in the reduction kernel saves the trip of the fp32 sums through memory (2048 x 4096 x 4096 with a
+// bias: 33 MB out and back and a launch).
+template <int COUNT>
+__device__ __forceinline__ void epilogue_add(const ReduceEpilogue& e, uint32_t (&r)[COUNT], int row, int n, int end, int N, bool row_ok, int dtype)
+{
+    if (!row_ok) return;
+    const unsigned short* d = e.D + (e.d_is_vector ? (int64_t)n : (int64_t)row * N + n);
+    const bool whole = (reinterpret_cast<uintptr_t>(d) & 15) == 0;
+#pragma unroll
+    for (int c = 0; c < COUNT; c += 8) {
+        unsigned short v[8];
+        if (whole && n + c + 8 <= end) {
+            *reinterpret_cast<uint4*>(v) = *reinterpret_cast<const uint4*>(d + c);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = n + c + i < end ? d[c + i] : (unsigned short)0;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            r[c + i] = __float_as_uint(fmaf(e.beta, load16_as_float(&v[i], dtype), e.alpha * __uint_as_float(r[c + i])));
+    }
+}
+
 // A_CLS ("row classes", the Padding module without a copy): A is row-major with K % 8 != 0, so its
 // rows are not 16-byte aligned and one tensor map cannot describe it.  Rows r and r + 8 do start
 // at the same offset from a 16-byte boundary (their distance is 16*K bytes), so the rows of one
@@ -279,7 +306,10 @@ __device__ __forceinline__ void store_run16(unsigned short* dst, int count, cons
 // following slots computed FIRST; the slot adds their partials to its accumulator in ascending k order and stores the
 // tile.  The assignment and the order of the additions are fixed by the shape, so the result is too.  Every wait on a
 // flag is bounded like the barrier waits.
-template <int BN, bool A_MN, bool B_MN, int CG, int MODE, bool FUSE = false, bool SK = false>
+//
+// EPI: the kernel adds beta * D itself (instantiations of their own: the test alone, on top of the halo tiles' code, made
+// 20000 x 20001 x 12 without a D 5 % slower).  The fused reduction's output loop takes p.ep at run time.
+template <int BN, bool A_MN, bool B_MN, int CG, int MODE, bool FUSE = false, bool SK = false, bool EPI = false>
 __global__ void __launch_bounds__(kUmmaThreads, 1)
 umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams p)
 {
@@ -296,6 +326,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
     // units of the shifted rows instead of columns, so they compute 16 columns more than they own (see
     // the epilogue); they use 16 row classes, since rows 16 apart share their offset from such a boundary
     constexpr bool HALO = A_CLS && (BN % 64 != 0);
+    static_assert(!EPI || (!FUSE && !SK && MODE != 3), "kernels that store the 16-bit output from their own accumulator");
     static_assert(BN % 64 == 0 || (A_CLS && (BN - 16) % 64 == 0), "BN is a multiple of 64, plus 16 halo columns for class tiles");
     // row classes of a class tile (rows NCLS*128*g + j + NCLS*i): 8, or for halo tiles as many as C's rows need to share
     // their offset from a 32-byte boundary (16 for an odd N, 8, 4 or 2 for an even one: p.ncls_log2)
@@ -885,6 +916,13 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                         sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
                     }
                     const int n = n0 + 4 * g;
+                    if (p.ep.D) {
+                        const int m = row_base + row_step * rr;
+                        sum.x = fused_add(p.ep, sum.x, m, n, p.N, p.dtype);
+                        if (n + 1 < p.N) sum.y = fused_add(p.ep, sum.y, m, n + 1, p.N, p.dtype);
+                        if (n + 2 < p.N) sum.z = fused_add(p.ep, sum.z, m, n + 2, p.N, p.dtype);
+                        if (n + 3 < p.N) sum.w = fused_add(p.ep, sum.w, m, n + 3, p.N, p.dtype);
+                    }
                     unsigned short* dst = c16 + (size_t)(row_base + row_step * rr) * p.N + n;
                     if (n + 4 <= p.N && (reinterpret_cast<uintptr_t>(dst) & 7) == 0) {
                         *reinterpret_cast<uint2*>(dst) = make_uint2(pack16(sum.x, sum.y, p.dtype), pack16(sum.z, sum.w, p.dtype));
@@ -898,7 +936,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                 // done reading every rank's partial: each may overwrite it for its next tile
                 __syncwarp();
                 if (lane < p.P_k) ptx::mbar_arrive_cluster(xempty_bar, (uint32_t)lane);
-            } else if (p.P_k == 1 && !p.force_partial) {
+            } else if (p.P_k == 1) {
                 // 16-bit output, any N and any base alignment.  A thread converts 64 columns of its row
                 // and stages them in shared memory shifted by the row's misalignment in C, so that
                 // 16-byte aligned chunks of a staged row are 16-byte aligned chunks of C.  The warp then
@@ -956,6 +994,10 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                                 ptx::tmem_ld_32x8(t_row + (uint32_t)col, e0);
                                 ptx::tmem_ld_32x8(t_row + (uint32_t)(col + 8), e1);
                                 ptx::tmem_ld_wait();
+                                if (EPI) {
+                                    epilogue_add(p.ep, e0, row, n_first, n_first + count, p.N, row_ok, p.dtype);
+                                    if (count > 8) epilogue_add(p.ep, e1, row, n_first + 8, n_first + count, p.N, row_ok, p.dtype);
+                                }
                                 if (row_ok) store_run16(crow + n_first, count, e0, e1, p.dtype);
                             }
                         }
@@ -973,6 +1015,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                                 ptx::tmem_ld_32x32(t_row + (uint32_t)(off + 64 * pass + 32 * h), r);
                                 ptx::tmem_ld_wait();
                                 if (SK && w.kind == 2) sk_fixup(r, 64 * pass + 32 * h);
+                                if (EPI) epilogue_add(p.ep, r, row, x - sig + 32 * h, p.N, p.N, row_ok, p.dtype);
                                 if ((pass == PASSES - 1 || x + 64 >= x_end) && (h == 1 || ncols <= 32)) {
                                     // the tile's last read of the accumulator: hand the buffer back now, so the MMA
                                     // of the tile after next starts while this pass is still being packed and stored
@@ -1032,6 +1075,10 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                                 sk_fixup(r0, c0);
                                 if (ncols > 32) sk_fixup(r1, c0 + 32);
                             }
+                        }
+                        if (EPI) {
+                            epilogue_add(p.ep, r0, row, n0 + c0, n0 + tile_cols, p.N, row_ok, p.dtype);
+                            if (ncols > 32) epilogue_add(p.ep, r1, row, n0 + c0 + 32, n0 + tile_cols, p.N, row_ok, p.dtype);
                         }
                         if (warp == 2 && lane == 0) ADAPT_TRACE(5, unit);
                         __syncwarp();                                    // the previous pass has been written out
