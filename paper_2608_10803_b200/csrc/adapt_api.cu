@@ -988,8 +988,9 @@ adapt_status_t launch_reduce(State& S, const float* partial, void* C, int64_t M,
     const ReduceEpilogue ep = epi ? *epi : no_epilogue();
     const int64_t Np = partial_pitch(N);
     const int64_t work = M * (Np / 4);
-    const int blocks = (int)std::min<int64_t>(ceil_div(work, 256), (int64_t)S.machine.n_sm * 8);
-    CUDA_TRY(launch_pdl(splitk_reduce_kernel, dim3(blocks), dim3(256), 0, stream, (const float*)partial, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)P_k, (int)dtype, ep));
+    const int groups = reduce_groups(work, P_k, S.machine.n_sm);
+    const int blocks = (int)std::min<int64_t>(ceil_div(work, 256 / groups), (int64_t)S.machine.n_sm * 8);
+    CUDA_TRY(launch_pdl(splitk_reduce_kernel, dim3(blocks), dim3(256), 0, stream, (const float*)partial, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)P_k, (int)dtype, ep, groups));
     S.launches.fetch_add(1, std::memory_order_relaxed);
     CUDA_TRY(cudaGetLastError());
     return ADAPT_OK;
@@ -1925,6 +1926,7 @@ extern "C" adapt_status_t adapt_matmul_noalloc(int64_t M, int64_t N, int64_t K, 
 
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     SimtParams p;
+    p.ep = no_epilogue();
     p.M = (int)M; p.N = (int)N; p.K = (int)K;
     if (layoutA == ADAPT_ROW_MAJOR) { p.a_sm = K; p.a_sk = 1; } else { p.a_sm = 1; p.a_sk = M; }
     if (layoutB == ADAPT_ROW_MAJOR) { p.b_sk = N; p.b_sn = 1; } else { p.b_sk = 1; p.b_sn = K; }
@@ -1941,8 +1943,9 @@ extern "C" adapt_status_t adapt_matmul_noalloc(int64_t M, int64_t N, int64_t K, 
     CUDA_TRY(launch_pdl(simt_gemm_kernel, grid, dim3(256), 0, stream, (const unsigned short*)A, (const unsigned short*)B, p));
     CUDA_TRY(cudaGetLastError());
     const int64_t work = M * (Np / 4);
-    const int blocks = (int)std::min<int64_t>(ceil_div(work, 256), 148 * 8);
-    CUDA_TRY(launch_pdl(splitk_reduce_kernel, dim3(blocks), dim3(256), 0, stream, (const float*)scratch, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)pk, (int)dtype, ReduceEpilogue{nullptr, 0, 1.f, 0.f}));
+    const int groups = reduce_groups(work, (int)pk, 148);
+    const int blocks = (int)std::min<int64_t>(ceil_div(work, 256 / groups), 148 * 8);
+    CUDA_TRY(launch_pdl(splitk_reduce_kernel, dim3(blocks), dim3(256), 0, stream, (const float*)scratch, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)pk, (int)dtype, no_epilogue(), groups));
     CUDA_TRY(cudaGetLastError());
     st().launches.fetch_add(2, std::memory_order_relaxed);
     return ADAPT_OK;

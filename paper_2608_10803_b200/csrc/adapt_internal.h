@@ -198,6 +198,15 @@ inline bool class_tiles_copy_a(const Shape& s) { return s.K < 64 && !tma_friendl
 // copy every view is aligned and nothing shifts.
 inline int64_t class_k_slack(const Shape& s) { return (s.K % 8 != 0 && !class_tiles_copy_a(s)) ? 7 : 0; }
 
+// Threads that share the splits of one output (four columns) in the reduction kernel: as many as bring a thread's share down to one
+// batch of eight splits, up to 16, while all threads fit the machine at once.
+inline int reduce_groups(int64_t outputs, int P_k, int n_sm)
+{
+    int g = 1;
+    while (g < 16 && P_k > 8 * g && outputs * g * 2 <= (int64_t)n_sm * 2048) g *= 2;
+    return g;
+}
+
 const Calib& default_calib();
 
 // Shared-memory layout of the tcgen05 kernels, used by the capacity check and by the launcher:

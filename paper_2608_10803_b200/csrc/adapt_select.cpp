@@ -179,7 +179,7 @@ static void model_prologue(const Shape& s, Config& c, const Calib& cal)
 
 // Epilogue (Eq. 11): cross-CTA reduction of the fp32 partials (Eq. 4's extra 4*M*N*P_k bytes are
 // written by the main loop and read back here), then the single 16-bit write.
-static void model_epilogue(const Shape& s, Config& c, const Calib& cal)
+static void model_epilogue(const Shape& s, Config& c, const Calib& cal, int n_sm)
 {
     c.t_epi_us = 0;
     c.ws_partial = 0;
@@ -201,8 +201,9 @@ static void model_epilogue(const Shape& s, Config& c, const Calib& cal)
         double part = 4.0 * MN * c.P_k;
         // partials that fit in L2 are read back at L2 speed; model that as half the HBM cost
         const double factor = part <= kL2Bytes ? 0.5 : 1.0;
-        // the reduction kernel walks the P_k slabs eight at a time: one dependent trip to L2 / HBM per batch
-        c.t_epi_us = cal.reduce_launch_us + copy_time_us(part * factor + 2.0 * MN, cal) + cal.reduce_batch_us * (double)ceil_div(c.P_k, 8);
+        // a thread of the reduction kernel walks its share of the P_k slabs eight at a time: one dependent trip to L2 / HBM per batch
+        const int groups = reduce_groups(s.M * partial_pitch(s.N) / 4, c.P_k, n_sm);
+        c.t_epi_us = cal.reduce_launch_us + copy_time_us(part * factor + 2.0 * MN, cal) + cal.reduce_batch_us * (double)ceil_div(ceil_div(c.P_k, groups), 8);
         c.hbm_bytes += part * (1.0 + factor);
     }
 }
@@ -314,7 +315,7 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
     if (halo && c.P_k == 1)
         pipe += 2.0 * cal.halo_edge_tile_us * (double)c.P_m / (double)std::min<int64_t>(m.n_sm, (int64_t)c.P_m * c.P_n);
     model_prologue(s, c, cal);
-    model_epilogue(s, c, cal);
+    model_epilogue(s, c, cal, m.n_sm);
     // strided row-class views stream A at a lower rate than a dense tensor (measured 3.5-4.1 TB/s)
     // (k classes as splits: the rate falls as the regrouped A, re-read by every column of tiles, grows beside the B
     // stream: 0.93 of the copy rate at M = 1, 0.80 at M = 30, 0.70 at M = 80; with the eight classes of a tile as
@@ -380,7 +381,7 @@ static void model_skinny(const Shape& s, const Machine& m, const Calib& cal, Con
         const int64_t k_split = ceil_div(s.K, c.P_k);
         t_cta = std::max(t_cta, cal.skinny_pass_us * (double)(c.BN / 64) * (double)ceil_div(k_split, kSkinnyKChunk));
     }
-    model_epilogue(s, c, cal);
+    model_epilogue(s, c, cal, m.n_sm);
     const double t_alu = macs / cal.skinny_mac_rate * 1e6;
     c.t_pro_us = 0;
     c.t_main_us = cal.skinny_fixed_us + std::max(t_alu, (double)Q * t_cta);
@@ -402,7 +403,7 @@ static void model_simt(const Shape& s, const Machine& m, const Calib& cal, Confi
     const double crowd = std::min(4.0, (double)units / m.n_sm);
     const double t_step = std::max(cal.simt_step_us, crowd * 2.0 * 64 * 64 * 16 / (cal.simt_flops / m.n_sm) * 1e6);
     const double t_tile = steps * t_step + cal.simt_fixed_us;
-    model_epilogue(s, c, cal);
+    model_epilogue(s, c, cal, m.n_sm);
     // element-wise 2-byte loads and stores: about a seventh of the HBM rate when memory-bound
     const double t_hbm = c.hbm_bytes / (cal.hbm_bw * cal.simt_bw_eff) * 1e6 - c.t_epi_us;
     c.t_pro_us = 0;

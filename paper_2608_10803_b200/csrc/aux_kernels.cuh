@@ -211,35 +211,55 @@ regroup_a_kernel(const unsigned short* __restrict__ A, unsigned short* __restric
     }
 }
 
-// ---- split-K reduction: C = RN16( sum_{p = 0..P_k-1} partial[p] ), ascending p, fp32 ---------------
-// The order is fixed, so the result does not depend on which CTA finished first.  Partials are
-// stored [P_k][M][Np] with Np = N rounded up to 8, so every row starts on a 32-byte boundary and
-// one thread reduces four consecutive columns with 16-byte loads.
+// ---- split-K reduction: C = RN16( sum_{p = 0..P_k-1} partial[p] ), fp32 ---------------
+// Partials are stored [P_k][M][Np] with Np = N rounded up to 8, so every row starts on a 32-byte boundary and
+// one thread reduces four consecutive columns with 16-byte loads, eight splits in flight.
+// A small output with many splits leaves most of the chip idle while each thread walks its splits batch by batch (one trip to L2
+// per eight): there the splits are shared by `groups` threads (a power of two), each adding a run of consecutive splits in
+// ascending order; the runs' sums are then added in ascending order too.  The order depends on the shape only.
+// (256 x 256 x 262144, P_k = 64: eight batches 59.5 us for the call, one batch 55.2 us; 34 x 21 x 34323: 16.5 and 11.4 us.)
 __global__ void __launch_bounds__(256)
 splitk_reduce_kernel(const float* __restrict__ partial, unsigned short* __restrict__ C,
-                     int M, int N, int Np, int P_k, int dtype, const ReduceEpilogue ep)
+                     int M, int N, int Np, int P_k, int dtype, const ReduceEpilogue ep, int groups)
 {
+    __shared__ float4 s_sum[256];
     pdl_launch_dependents();
     pdl_wait();
-    const int groups = Np >> 2;
-    const int64_t total = (int64_t)M * groups;
+    const int quads = Np >> 2;                              // columns in fours
+    const int64_t total = (int64_t)M * quads;
     const int64_t slab = (int64_t)M * Np;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-        const int m = (int)(i / groups);
-        const int n = (int)(i - (int64_t)m * groups) * 4;
-        const float* src = partial + (int64_t)m * Np + n;
-        // loads are issued eight splits at a time; the additions stay in ascending split order
+    const int width = 256 / groups;                         // outputs (fours of columns) per block and step
+    const int sub = threadIdx.x / width, lane = threadIdx.x - sub * width;
+    const int per = (P_k + groups - 1) / groups;
+    const int p_begin = sub * per, p_end = min(P_k, p_begin + per);
+    for (int64_t base = (int64_t)blockIdx.x * width; base < total; base += (int64_t)gridDim.x * width) {
+        const int64_t i = base + lane;
+        const int m = (int)(i / quads);
+        const int n = (int)(i - (int64_t)m * quads) * 4;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int p0 = 0; p0 < P_k; p0 += 8) {
-            float4 v[8];
+        if (i < total) {
+            const float* src = partial + (int64_t)m * Np + n;
+            for (int p0 = p_begin; p0 < p_end; p0 += 8) {
+                float4 v[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (p0 + j < P_k) v[j] = __ldcs(reinterpret_cast<const float4*>(src + (int64_t)(p0 + j) * slab));
+                for (int j = 0; j < 8; ++j)
+                    if (p0 + j < p_end) v[j] = __ldcs(reinterpret_cast<const float4*>(src + (int64_t)(p0 + j) * slab));
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-                if (p0 + j < P_k) { acc.x += v[j].x; acc.y += v[j].y; acc.z += v[j].z; acc.w += v[j].w; }
+                for (int j = 0; j < 8; ++j)
+                    if (p0 + j < p_end) { acc.x += v[j].x; acc.y += v[j].y; acc.z += v[j].z; acc.w += v[j].w; }
+            }
         }
+        if (groups > 1) {
+            __syncthreads();                                // the sums of the step before have been read
+            s_sum[threadIdx.x] = acc;
+            __syncthreads();
+            if (sub != 0) continue;
+            for (int j = 1; j < groups; ++j) {
+                const float4 v = s_sum[j * width + lane];
+                acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+            }
+        }
+        if (i >= total) continue;
         if (ep.D) {
             const unsigned short* d = ep.D + (ep.d_is_vector ? (int64_t)n : (int64_t)m * N + n);
             float v[4] = {acc.x, acc.y, acc.z, acc.w};
