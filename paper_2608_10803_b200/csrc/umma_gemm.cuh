@@ -73,6 +73,9 @@ struct UmmaParams {
     unsigned int sk_epoch;           // this launch's epoch (unique per workspace)
     int x_rows, x_pitch;             // fused split-K: rows and row pitch (fp32 elements) of the partial tile each CTA of the
                                      // cluster keeps in its shared memory for the exchange
+    int tiles_per_entry;             // strided batch (MODE 4): P_m * P_n; units are numbered entry by entry
+    int a_entry, b_entry;            // ... 1: every entry has an A (B) of its own, 0: all share one
+    int64_t c_entry;                 // ... elements from an entry's C to the next one's
     int ncls_log2;                   // halo class tiles: log2 of the number of row classes (1 .. 4)
     ReduceEpilogue ep;               // fused add (AddMM) where the kernel stores the 16-bit output itself; D == nullptr: none
     unsigned int* status;            // device status word: bit 0 = a bounded wait expired
@@ -100,7 +103,7 @@ struct UmmaParams {
 template <int MODE>
 struct TmapPackT {
     CUtensorMap a[MODE == 1 ? 16 : 1];
-    CUtensorMap b[MODE >= 2 ? 8 : 1];
+    CUtensorMap b[MODE == 2 || MODE == 3 ? 8 : 1];
     CUtensorMap c[MODE == 1 ? 16 : 1];
 };
 
@@ -130,20 +133,23 @@ __device__ __forceinline__ void decode_unit(const UmmaParams& p, int unit, int& 
 // kind 2 (stream-K): the start of a tile whose later k ranges `npeers` following slots contribute.
 struct WorkItem {
     int unit, mb, nb, split, kb0, kb1, kind, npeers;
+    int entry;                       // of a strided batch
 };
 
 // The it-th work item of slot `slot` (of `n_slots`).  Without stream-K: unit slot + it * n_slots.  With stream-K
 // (Section 4.2's StreamK remark, made deterministic): first the slot's share of the stream-K tiles (at most two
 // ranges: the end of one tile, then the start of the next), then whole tiles sk_tiles + slot + j * n_slots.
-template <bool SK, bool B_SPLIT>
+template <bool SK, bool B_SPLIT, bool BATCH = false>
 __device__ __forceinline__ bool next_item(const UmmaParams& p, int slot, int n_slots, int it, WorkItem& w)
 {
     w.kind = 0;
     w.npeers = 0;
+    w.entry = 0;
     if (!SK) {
         w.unit = slot + it * n_slots;
         if (w.unit >= p.num_units) return false;
-        decode_unit(p, w.unit, w.mb, w.nb, w.split);
+        if (BATCH) w.entry = w.unit / p.tiles_per_entry;
+        decode_unit(p, BATCH ? w.unit - w.entry * p.tiles_per_entry : w.unit, w.mb, w.nb, w.split);
         w.kb0 = (B_SPLIT ? (w.split >> 3) : w.split) * p.kb_per_split;
         w.kb1 = min(p.kb_total, w.kb0 + p.kb_per_split);
         return true;
@@ -307,6 +313,9 @@ __device__ __forceinline__ void epilogue_add(const ReduceEpilogue& e, uint32_t (
 // tile.  The assignment and the order of the additions are fixed by the shape, so the result is too.  Every wait on a
 // flag is bounded like the barrier waits.
 //
+// BATCH (MODE 4): the tiles of all entries of a strided batch in one launch, plain tiles through 3D maps whose outermost
+// dimension is the entry.
+//
 // EPI: the kernel adds beta * D itself (instantiations of their own: the test alone, on top of the halo tiles' code, made
 // 20000 x 20001 x 12 without a D 5 % slower).  The fused reduction's output loop takes p.ep at run time.
 template <int BN, bool A_MN, bool B_MN, int CG, int MODE, bool FUSE = false, bool SK = false, bool EPI = false>
@@ -319,7 +328,9 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
     constexpr bool A_CLS = MODE == 1;
     constexpr bool B_CLS = MODE == 2;
     constexpr bool B_SPLIT = MODE == 3;                   // k classes as k splits (see below)
-    static_assert(MODE == 0 || (!A_MN && B_MN), "class modes: K-major A, row-major B");
+    constexpr bool BATCH = MODE == 4;
+    static_assert(MODE == 0 || BATCH || (!A_MN && B_MN), "class modes: K-major A, row-major B");
+    static_assert(!BATCH || (CG == 1 && !FUSE && !EPI), "strided batches: 1-CTA tiles");
     static_assert(MODE != 2 || CG == 1, "tiles with eight class accumulators: one CTA per tile");
     static_assert(!B_CLS || BN == 64, "k-class mode uses 64-column windows");
     // HALO: class tiles for a C whose rows do not start on 32-byte boundaries (N % 16 != 0) own 32-byte
@@ -442,7 +453,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
         constexpr int NREQ_A = A_MN ? 2 : 1;
         constexpr int NREQ = NREQ_A + (B_MN ? B_BOXES : 1);
         WorkItem w;
-        if (lane < NREQ && next_item<SK, B_SPLIT>(p, unit0, unit_step, 0, w)) {
+        if (lane < NREQ && next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, 0, w)) {
             const int cls = A_CLS ? (w.mb & (NCLS - 1)) : 0;
             const int row0 = A_CLS ? (w.mb >> NSH) * (128 * CG) + (int)cta_rank * 128 : w.mb * (128 * CG) + (int)cta_rank * 128;
             const int kshift = A_CLS ? p.a_sigma[cls] : 0;
@@ -451,7 +462,10 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
             const int jb = lane - NREQ_A;
             for (int kb = w.kb0; kb < w.kb1 && kb < w.kb0 + S; ++kb) {
                 const int k0 = kb * kUmmaBK;
-                if (lane < NREQ_A) {
+                if (BATCH) {
+                    if (lane < NREQ_A) ptx::tma_prefetch_3d(&maps.a[0], A_MN ? row0 + lane * 64 : k0, A_MN ? k0 : row0, w.entry * p.a_entry);
+                    else ptx::tma_prefetch_3d(&maps.b[0], B_MN ? col0 + jb * 64 : k0, B_MN ? k0 : col0, w.entry * p.b_entry);
+                } else if (lane < NREQ_A) {
                     if (!A_MN) ptx::tma_prefetch_2d(&maps.a[cls], k0 + a_k_off, row0);
                     else ptx::tma_prefetch_2d(&maps.a[cls], row0 + lane * 64, k0);
                 } else {
@@ -494,7 +508,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
             const int jb = lane - NREQ_A;                                     // B box of this lane
             for (int it = 0; ok; ++it) {
                 WorkItem w;
-                if (!next_item<SK, B_SPLIT>(p, unit0, unit_step, it, w)) break;
+                if (!next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w)) break;
                 const int unit = w.unit, mb = w.mb, nb = w.nb, split = w.split, kb0 = w.kb0, kb1 = w.kb1;
                 // A rows of this CTA: consecutive rows, or in class mode rows 1024*g + j + 8*i read through
                 // map j at class-row index 128*g
@@ -563,6 +577,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                         else { dst = sB; x = k0; y = col0; }
                     }
                     if (A_CLS && CG == 2 && is_a && kb == 0 && kshift > 0) load(dst, tm, afull_own + 8u * stage, x, y);   // this CTA's own barrier
+                    else if (BATCH) ptx::tma_load_3d(dst, tm, fb, x, y, w.entry * (is_a ? p.a_entry : p.b_entry));
                     else load(dst, tm, fb, x, y);
                     if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
@@ -618,7 +633,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
             bool ok = true;
             for (int it = 0; ok; ++it) {
                 WorkItem w;
-                if (!next_item<SK, B_SPLIT>(p, unit0, unit_step, it, w)) break;
+                if (!next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w)) break;
                 const int sigma = p.a_sigma[w.mb & (NCLS - 1)];
                 if (w.kb0 == 0 && w.kb1 > 0 && sigma > 0) {
                     if (!mma_wait(afull_bar + 8u * stage, (aphase >> stage) & 1u)) { ok = false; break; }
@@ -643,7 +658,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
             bool ok = true;
             for (int it = 0; ok; ++it) {
                 WorkItem w;
-                if (!next_item<SK, B_SPLIT>(p, unit0, unit_step, it, w)) break;
+                if (!next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w)) break;
                 const int unit = w.unit, mb = w.mb, nb = w.nb, split = w.split, kb0 = w.kb0, kb1 = w.kb1;
                 (void)unit; (void)nb; (void)split;
                 if (warp_wide && kb0 == 0 && kb1 > 0) {
@@ -745,10 +760,10 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
         bool ok = true;
         uint8_t* stg = stage_out + (warp - 2) * kUmmaWarpStagingBytes + lane * kUmmaStageRowBytes;   // this thread's staging row
         unsigned short* srow = reinterpret_cast<unsigned short*>(stg);
-        const uintptr_t c_base = reinterpret_cast<uintptr_t>(p.C);
         for (int it = 0; ok; ++it, ++seq) {
             WorkItem w;
-            if (!next_item<SK, B_SPLIT>(p, unit0, unit_step, it, w)) break;
+            if (!next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w)) break;
+            const uintptr_t c_base = reinterpret_cast<uintptr_t>(p.C) + (BATCH ? 2ull * (uintptr_t)(w.entry * p.c_entry) : 0);
             const int unit = w.unit, mb = w.mb, nb = w.nb, split = w.split;
             (void)unit;
             if (!ptx::mbar_wait(tfull_bar + 8u * buf, buf_phase, abort_flag)) { ok = false; break; }
@@ -1041,7 +1056,8 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                             ptx::fence_proxy_async_smem();
                             __syncwarp();
                             if (lane == 0) {
-                                if (p.c_hint) ptx::tma_store_2d_hint(tmC, ptx::smem_u32(box), x, y0, c_policy);
+                                if (BATCH) ptx::tma_store_3d(tmC, ptx::smem_u32(box), x, y0, w.entry);
+                                else if (p.c_hint) ptx::tma_store_2d_hint(tmC, ptx::smem_u32(box), x, y0, c_policy);
                                 else ptx::tma_store_2d(tmC, ptx::smem_u32(box), x, y0);
                                 ptx::bulk_commit();
                                 if (warp == 2) ADAPT_TRACE(6, unit);
