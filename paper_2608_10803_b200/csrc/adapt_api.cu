@@ -1530,11 +1530,10 @@ adapt_status_t run_strided_batch(State& S, Plan* pl, const void* A, int64_t sa, 
     GroupParams p;
     Config one = c;
     if (c.family == ADAPT_FAM_CLUSTER) one.cluster = 1;      // the entries fill the machine: no pieces
-    const int chain = group_item(s, one, A, B, C, &p.item[0]);
-    p.item[0].tile_end = (int)(batch * tiles);
-    p.count = 1;
-    p.ring = cluster_seq_ring(chain);
-    p.k_max = (int)s.K;
+    GroupItem it;
+    const int chain = group_item(s, one, A, B, C, &it);
+    group_clear(p);
+    group_add(p, it, chain, batch);
     p.prefetch = S.prefetch;
     p.dtype = s.dtype;
     p.sa = sa; p.sb = sb; p.sc = sc;
@@ -1664,29 +1663,19 @@ adapt_status_t launch_pending(State& S, PendingGroup& g, cudaStream_t stream)
     p.prefetch = S.prefetch;
     p.sa = p.sb = p.sc = 0;
     for (int variant = 0; variant < 8; ++variant) {         // bit 0: dtype, 1: A row-major, 2: B column-major
-        p.count = 0;
-        p.ring = 1;
-        p.k_max = 0;
-        int64_t end = 0;
+        group_clear(p);
         auto flush = [&]() -> adapt_status_t {
             if (p.count == 0) return ADAPT_OK;
             p.dtype = variant & 1;
             CUDA_TRY(launch_group(p, (variant & 2) != 0, (variant & 4) != 0, stream));
             S.launches.fetch_add(1, std::memory_order_relaxed);
-            p.count = 0;
-            p.ring = 1;
-            p.k_max = 0;
-            end = 0;
+            group_clear(p);
             return ADAPT_OK;
         };
         for (const PendingGroup::Entry& e : g.entries) {
             if (e.variant != variant) continue;
-            p.item[p.count] = e.item;
-            end += e.item.tiles;
-            p.item[p.count].tile_end = (int)end;
-            p.ring = std::max(p.ring, cluster_seq_ring(e.chain));
-            p.k_max = std::max(p.k_max, e.item.K);
-            if (++p.count == kGroupMax) {
+            group_add(p, e.item, e.chain);
+            if (p.count == kGroupMax) {
                 const adapt_status_t r = flush();
                 if (r != ADAPT_OK) return r;
             }

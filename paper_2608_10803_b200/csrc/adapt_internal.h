@@ -214,6 +214,7 @@ const Calib& default_calib();
 // (8 KB per epilogue warp, only when the kernel stores the 16-bit C), and slack to align the stages to 1024 B.
 // One-launch cluster kernel: a ring of stages (64 rows of 144 bytes per operand).
 // The ring is as deep as the CTA's k range needs, capped so that the CTAs that share an SM all fit.
+constexpr int kClusterKS = 64;          // k values per stage
 constexpr int kClusterStageBytes = 2 * 64 * 144;
 constexpr int kClusterMaxRing = 6;
 inline int cluster_smem_bytes(int ring) { return ring * kClusterStageBytes; }

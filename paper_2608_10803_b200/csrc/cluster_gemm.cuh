@@ -41,7 +41,6 @@ namespace adapt {
 
 constexpr int kClusterThreads = 256;
 constexpr int kClusterTile = 64;        // output tile edge
-constexpr int kClusterKS = 64;          // k values per stage
 constexpr int kClusterPitch = 72;       // 16-bit elements per staged row: 144 B, conflict-free for ldmatrix
 constexpr int kClusterCPitch = 72;      // fp32 elements per row of the exchanged partial tile
 static_assert(kClusterStageBytes == 2 * 64 * kClusterPitch * 2, "a stage is 64 rows of each operand");

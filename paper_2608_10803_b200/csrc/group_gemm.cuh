@@ -13,38 +13,15 @@
 
 #include "aux_kernels.cuh"
 #include "cluster_gemm.cuh"
+#include "group_plan.h"
 
 namespace adapt {
-
-constexpr int kGroupMax = 64;           // entries per launch (the parameters stay below 4 KB)
-
-struct GroupItem {
-    const unsigned short* A;
-    const unsigned short* B;
-    unsigned short* C;
-    int M, N, K;
-    int P_n;
-    int pieces;                         // pieces of the k range; 0: CUDA-core tiles
-    int k_per_piece;
-    int tiles;                          // 64 x 64 tiles of one entry
-    int tile_end;                       // tiles of this and all earlier items
-};
-struct GroupParams {
-    int count;
-    int ring;
-    int prefetch;
-    int dtype;
-    int k_max;                          // largest K of the list
-    int64_t sa, sb, sc;                 // strided batch: item 0 stands for all entries, sa, sb, sc elements apart
-    GroupItem item[kGroupMax];
-};
-static_assert(sizeof(GroupParams) <= 4096, "kernel parameters");
 
 // What bounds it: for a list with a deep entry the chain of that entry's stages (0.33 us per aligned 64 k values and group of
 // warps, 0.6 off 16-byte boundaries), else the shared-memory port.  The deepest entries come first and the ring is no deeper
 // than the list needs.  48 layers of 16 .. 1024 a side: 97 us one launch each on four streams, 31 us (21 us without the one
 // layer that keeps a launch of its own); 96 products of 128 x 128 x 64: 266 us one launch each, 4.4 us.
-// SHORT: every item has K <= 64 (one stage): no two-group tiles, so fewer registers and three CTAs per SM instead of two
+// SHORT: every item has K <= 64 in one piece (one stage): no two-group tiles, so fewer registers and three CTAs per SM instead of two
 // (96 products of 128 x 128 x 64: 6.6 us with the general kernel, 4.4 with this one).
 template <bool A_KC, bool B_KC, bool BF16, bool SHORT>
 __global__ void __launch_bounds__(kClusterThreads, SHORT ? 3 : 2)
@@ -115,37 +92,15 @@ inline cudaError_t group_set_attributes()
     return cudaSuccess;
 }
 
-// Can an entry with this configuration run in the grouped launch?  The cluster kernel's tiles: the k range must not be a long
-// chain (24 stages are about 10 us).  CUDA-core tiles: no k split and a few steps.
-inline bool group_eligible(const Shape& s, const Config& c)
-{
-    if (c.family == ADAPT_FAM_SIMT) return c.P_k == 1 && s.K <= 64 && (int64_t)c.P_m * c.P_n <= 512;
-    return c.family == ADAPT_FAM_CLUSTER && c.cluster * ceil_div(round_up(ceil_div(s.K, c.cluster), 16), kClusterKS) <= 24;
-}
-
-// Fills everything of an item but tile_end; returns its chain: the stages one group of warps of a tile walks.
-inline int group_item(const Shape& s, const Config& c, const void* A, const void* B, void* C, GroupItem* it)
-{
-    it->A = (const unsigned short*)A;
-    it->B = (const unsigned short*)B;
-    it->C = (unsigned short*)C;
-    it->M = (int)s.M; it->N = (int)s.N; it->K = (int)s.K;
-    it->P_n = c.P_n;
-    it->tiles = c.P_m * c.P_n;
-    const bool simt = c.family == ADAPT_FAM_SIMT;
-    it->pieces = simt ? 0 : c.cluster;
-    it->k_per_piece = simt ? 0 : (int)round_up(ceil_div(s.K, c.cluster), 16);
-    return simt ? 1 : it->pieces == 1 ? (int)ceil_div(s.K, 2 * kClusterKS) : (it->pieces / 2) * (int)ceil_div(it->k_per_piece, kClusterKS);
-}
-
-// One launch; p holds `count` items with their tile_end, k_max, ring and strides set.
+// One launch; p holds the items (group_add) and the strides.
 inline cudaError_t launch_group(GroupParams& p, bool a_kc, bool b_kc, cudaStream_t stream)
 {
+    const GroupForm form = group_form(p);
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)p.item[p.count - 1].tile_end, 1, 1);
     cfg.blockDim = dim3(kClusterThreads, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)(p.k_max <= kClusterKS ? cluster_smem_bytes(1) : cluster_seq_smem_bytes(p.ring));
+    cfg.dynamicSmemBytes = (size_t)form.smem_bytes;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     pdl_attribute(&attr[0]);
@@ -153,7 +108,7 @@ inline cudaError_t launch_group(GroupParams& p, bool a_kc, bool b_kc, cudaStream
     cfg.numAttrs = 1;
     void* args[1] = {&p};
     const size_t bytes[1] = {sizeof(p)};
-    return launch_exc(&cfg, (const void*)(p.k_max <= kClusterKS ? group_pick<true>(a_kc, b_kc, p.dtype != 0) : group_pick<false>(a_kc, b_kc, p.dtype != 0)), args, bytes, 1);
+    return launch_exc(&cfg, (const void*)(form.short_k ? group_pick<true>(a_kc, b_kc, p.dtype != 0) : group_pick<false>(a_kc, b_kc, p.dtype != 0)), args, bytes, 1);
 }
 
 }  // namespace adapt

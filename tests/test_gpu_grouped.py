@@ -133,3 +133,38 @@ def test_strided_batch_whose_entries_feed_one_another_runs_in_order():
     torch.cuda.synchronize()
     for i in range(batch):
         assert torch.equal(X[i + 1], X[i] @ roll)
+
+
+def installed_plans(tmp_path, shapes, want):
+    """Plans of a table that names, for every (M, N, K, dtype), the first candidate that `want` accepts."""
+    path = tmp_path / "plans.txt"
+    assert ab.adapt_plan_table_save(str(path)) >= 0
+    lines = [path.read_text().splitlines()[0]]
+    for M, N, K, dt in shapes:
+        c = next(c for c in ab.adapt_plan_candidates(M, N, K, dt) if want(c))
+        lines.append(f"{M} {N} {K} {dt} 0 0 {c.tiling_key:016x}")
+    path.write_text("\n".join(lines) + "\n")
+    assert ab.adapt_plan_table_load(str(path)) == len(shapes), "a shape had a plan before"
+    return [ab.adapt_matmul_plan(*s) for s in shapes]
+
+
+@pytest.mark.parametrize("pieces", [2, 4])
+def test_list_of_short_k_plans_that_a_table_cut_into_pieces(tmp_path, pieces):
+    """All K <= 64, so that nothing but the number of pieces tells the launch which kernel it needs."""
+    ab.adapt_shutdown()
+    init()
+    shapes = [(128, 128, 64, ab.F16), (65, 127, 64, ab.F16), (61, 200, 63, ab.F16)] + ([(128, 64, 32, ab.F16), (3, 70, 48, ab.F16)] if pieces == 2 else [])
+    plans = installed_plans(tmp_path, shapes, lambda c: c.family == ab.FAM_CLUSTER and c.cluster == pieces)
+    A = [synth.draw_operand(M, K, synth.U11, 2 * i, dt, "cuda") for i, (M, N, K, dt) in enumerate(shapes)]
+    B = [synth.draw_operand(K, N, synth.U11, 2 * i + 1, dt, "cuda") for i, (M, N, K, dt) in enumerate(shapes)]
+    alone, listed = ([torch.full((M, N), float("nan"), dtype=torch.float16, device="cuda") for M, N, _, _ in shapes] for _ in range(2))
+    for p, a, b, c in zip(plans, A, B, alone):
+        ab.adapt_matmul(p, a.data_ptr(), b.data_ptr(), c.data_ptr(), stream())
+    before = ab.adapt_launch_count()
+    ab.adapt_matmul_batch(plans, *([t.data_ptr() for t in x] for x in (A, B, listed)), stream())
+    torch.cuda.synchronize()
+    ab.adapt_poll_device_status(stream())
+    assert ab.adapt_launch_count() - before == 1
+    for x, y, s in zip(alone, listed, shapes):
+        assert torch.equal(x.view(torch.int16), y.view(torch.int16)), s
+    ab.adapt_shutdown()
