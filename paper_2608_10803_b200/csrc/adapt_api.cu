@@ -21,6 +21,7 @@
 #include "skinny_gemm.cuh"
 #include "cluster_gemm.cuh"
 #include "group_gemm.cuh"
+#include "batch_schedule.h"
 #include "umma_gemm.cuh"
 
 using namespace adapt;
@@ -1634,57 +1635,63 @@ extern "C" adapt_status_t adapt_matmul_host(adapt_handle_t plan, const void* A_h
 // ---------------------------------------------------------------------------------------------
 namespace {
 
-struct Range { uintptr_t lo, hi; };
-inline bool hits(const std::vector<Range>& v, uintptr_t lo, uintptr_t hi)
-{
-    bool any = false;
-    for (const Range& r : v) any |= (lo < r.hi) & (r.lo < hi);
-    return any;
-}
+// What run_batch launches, on the streams of its lanes.
+struct BatchOps {
+    State& S;
+    const adapt_handle_t* plans;
+    const void* const* A;
+    const void* const* B;
+    void* const* C;
+    cudaStream_t stream[kBatchLanesMax];
 
-// Calls of a batch that wait for their grouped launch: independent of one another, one dtype and pair of layouts per launch.
-struct PendingGroup {
-    struct Entry { GroupItem item; int chain, variant; };
-    std::vector<Entry> entries;
-    std::vector<Range> reads, writes;
-    double predicted_us = 0.0;
-    bool conflicts(const Range& a, const Range& b, const Range& c) const
+    adapt_status_t single(int64_t i, int lane) { return adapt_matmul(plans[i], A[i], B[i], C[i], (void*)stream[lane]); }
+    adapt_status_t wait(int lane, int other)
     {
-        return !entries.empty() && (hits(writes, c.lo, c.hi) || hits(reads, c.lo, c.hi) || hits(writes, a.lo, a.hi) || hits(writes, b.lo, b.hi));
+        CUDA_TRY(cudaEventRecord(S.lanes.cross[other], stream[other]));
+        CUDA_TRY(cudaStreamWaitEvent(stream[lane], S.lanes.cross[other], 0));
+        return ADAPT_OK;
     }
-    void clear() { entries.clear(); reads.clear(); writes.clear(); predicted_us = 0.0; }
-};
-
-adapt_status_t launch_pending(State& S, PendingGroup& g, cudaStream_t stream)
-{
-    // longest chains first: what starts last is short
-    std::stable_sort(g.entries.begin(), g.entries.end(), [](const PendingGroup::Entry& x, const PendingGroup::Entry& y) { return x.chain > y.chain; });
-    GroupParams p;
-    p.prefetch = S.prefetch;
-    p.sa = p.sb = p.sc = 0;
-    for (int variant = 0; variant < 8; ++variant) {         // bit 0: dtype, 1: A row-major, 2: B column-major
-        group_clear(p);
-        auto flush = [&]() -> adapt_status_t {
-            if (p.count == 0) return ADAPT_OK;
-            p.dtype = variant & 1;
-            CUDA_TRY(launch_group(p, (variant & 2) != 0, (variant & 4) != 0, stream));
-            S.launches.fetch_add(1, std::memory_order_relaxed);
-            group_clear(p);
-            return ADAPT_OK;
-        };
-        for (const PendingGroup::Entry& e : g.entries) {
-            if (e.variant != variant) continue;
-            group_add(p, e.item, e.chain);
-            if (p.count == kGroupMax) {
-                const adapt_status_t r = flush();
-                if (r != ADAPT_OK) return r;
-            }
+    // Independent calls: one launch per kGroupMax calls, data type and pair of layouts.
+    adapt_status_t group(const std::vector<int64_t>& calls, int lane)
+    {
+        struct Entry { GroupItem item; int chain, variant; };
+        std::vector<Entry> entries;
+        for (int64_t i : calls) {
+            const Shape& s = plans[i]->s;
+            Entry e;
+            e.chain = group_item(s, plans[i]->c, A[i], B[i], C[i], &e.item);
+            e.variant = (s.dtype != 0 ? 1 : 0) | (s.layoutA == ADAPT_ROW_MAJOR ? 2 : 0) | (s.layoutB == ADAPT_COL_MAJOR ? 4 : 0);
+            entries.push_back(e);
         }
-        const adapt_status_t r = flush();
-        if (r != ADAPT_OK) return r;
+        // longest chains first: what starts last is short
+        std::stable_sort(entries.begin(), entries.end(), [](const Entry& x, const Entry& y) { return x.chain > y.chain; });
+        GroupParams p;
+        p.prefetch = S.prefetch;
+        p.sa = p.sb = p.sc = 0;
+        for (int variant = 0; variant < 8; ++variant) {     // bit 0: dtype, 1: A row-major, 2: B column-major
+            group_clear(p);
+            auto launch = [&]() -> adapt_status_t {
+                if (p.count == 0) return ADAPT_OK;
+                p.dtype = variant & 1;
+                CUDA_TRY(launch_group(p, (variant & 2) != 0, (variant & 4) != 0, stream[lane]));
+                S.launches.fetch_add(1, std::memory_order_relaxed);
+                group_clear(p);
+                return ADAPT_OK;
+            };
+            for (const Entry& e : entries) {
+                if (e.variant != variant) continue;
+                group_add(p, e.item, e.chain);
+                if (p.count == kGroupMax) {
+                    const adapt_status_t r = launch();
+                    if (r != ADAPT_OK) return r;
+                }
+            }
+            const adapt_status_t r = launch();
+            if (r != ADAPT_OK) return r;
+        }
+        return ADAPT_OK;
     }
-    return ADAPT_OK;
-}
+};
 
 }  // namespace
 
@@ -1701,23 +1708,16 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
         }
         return ADAPT_OK;
     }
-    // Small calls (plans of the one-launch and CUDA-core families, as adapt_matmul_plan returned them) are collected and
-    // leave together in one grouped launch; the others are launched as they come.  A call is only collected, and another
-    // only launched past the collected ones, while none of its buffers meets theirs in a way that order would matter.
+    // Small calls (plans of the one-launch and CUDA-core families, as adapt_matmul_plan returned them) leave in grouped launches.
     auto grouped = [&](const Plan* pl) { return pl && pl->selected && !pl->noop && !pl->zero_fill && group_eligible(pl->s, pl->c); };
     int64_t singles = 0;
     for (int64_t i = 0; i < count; ++i) singles += grouped(plans[i]) ? 0 : 1;
-    // Lanes.  Lane 0 is the caller's stream, the others are internal streams between a fork from and a join to it, used
-    // from eight calls on and no more of them than there are launches to overlap.  A launch goes to the lane with the least
-    // predicted work queued, so that the launch gaps and the tail of one call fill with the next call's work.  The result is
-    // the one of running the calls in order: a call whose output overlaps what another lane still reads or writes, or whose
-    // inputs overlap what it writes, first waits for that lane; a lane remembers the buffers of its last 16 calls, and when that
-    // memory is full all other lanes are made to wait for it.  A stream-K call runs with nothing beside it: its CTAs wait
-    // for one another and must all be resident, which two such kernels sharing the SMs could deny each other.
+    // Lane 0 is the caller's stream, the others are internal streams between a fork from and a join to it, used from eight
+    // calls on and no more of them than there are launches to overlap.
     const int NL = count < 8 ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(S.batch_lanes, singles + (singles < count ? 1 : 0)));
     std::unique_lock<std::mutex> batch_lock(S.batch_mu, std::defer_lock);
     State::BatchLanes& L = S.lanes;
-    cudaStream_t stream[4] = {user, nullptr, nullptr, nullptr};
+    BatchOps ops = {S, plans, A, B, C, {user, nullptr, nullptr, nullptr}};
     if (NL > 1) {
         batch_lock.lock();
         if (!L.ready) {
@@ -1731,93 +1731,27 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
         }
         CUDA_TRY(cudaEventRecord(L.fork, user));
         for (int l = 1; l < NL; ++l) {
-            stream[l] = L.s[l];
+            ops.stream[l] = L.s[l];
             CUDA_TRY(cudaStreamWaitEvent(L.s[l], L.fork, 0));
         }
     }
-    constexpr size_t kLaneMemory = 32;
-    std::vector<Range> reads[4], writes[4];
-    double queued[4] = {0.0, 0.0, 0.0, 0.0};
-    auto wait_for = [&](int lane, int other) -> adapt_status_t {      // `lane` continues after everything queued on `other`
-        CUDA_TRY(cudaEventRecord(L.cross[other], stream[other]));
-        CUDA_TRY(cudaStreamWaitEvent(stream[lane], L.cross[other], 0));
-        return ADAPT_OK;
+    auto call_of = [&](int64_t i) -> BatchCall {
+        const Plan* pl = plans[i];
+        BatchCall k = {};
+        k.unsound = !pl;
+        if (!pl) return k;
+        const Shape& s = pl->s;
+        k.a = {(uintptr_t)A[i], (uintptr_t)A[i] + (uintptr_t)s.M * s.K * 2};
+        k.b = {(uintptr_t)B[i], (uintptr_t)B[i] + (uintptr_t)s.K * s.N * 2};
+        k.c = {(uintptr_t)C[i], (uintptr_t)C[i] + (uintptr_t)s.M * s.N * 2};
+        k.unsound = !A[i] || !B[i] || !C[i] || (((uintptr_t)A[i] | (uintptr_t)B[i] | (uintptr_t)C[i]) & 1) != 0 || (k.c.lo < k.a.hi && k.a.lo < k.c.hi) ||
+                    (k.c.lo < k.b.hi && k.b.lo < k.c.hi);
+        k.groupable = grouped(pl);
+        k.alone = pl->c.streamk != 0;
+        k.us = pl->c.predicted_us;
+        return k;
     };
-    // Chooses the lane of a launch that reads and writes the given buffers and makes it wait for the lanes it depends on.
-    auto enter = [&](const Range* rd, size_t n_rd, const Range* wr, size_t n_wr, bool alone, int* out) -> adapt_status_t {
-        int lane = 0;
-        for (int l = 1; l < NL; ++l) if (queued[l] < queued[lane]) lane = l;
-        *out = lane;
-        for (int o = 0; o < NL; ++o) {
-            if (o == lane) continue;
-            bool dep = alone;
-            for (size_t j = 0; j < n_wr && !dep; ++j) dep = hits(reads[o], wr[j].lo, wr[j].hi) || hits(writes[o], wr[j].lo, wr[j].hi);
-            for (size_t j = 0; j < n_rd && !dep; ++j) dep = hits(writes[o], rd[j].lo, rd[j].hi);
-            // everything lane o has queued comes first; what o did before is then ordered before all of this lane's
-            // later calls as well, but the other lanes still have to see it: keep o's memory
-            if (dep) { const adapt_status_t r = wait_for(lane, o); if (r != ADAPT_OK) return r; }
-        }
-        if (NL > 1 && reads[lane].size() >= kLaneMemory) {
-            // this lane's memory is full: every other lane waits for it, and it starts a new memory
-            for (int o = 0; o < NL; ++o)
-                if (o != lane) { const adapt_status_t r = wait_for(o, lane); if (r != ADAPT_OK) return r; }
-            reads[lane].clear();
-            writes[lane].clear();
-        }
-        return ADAPT_OK;
-    };
-    auto leave = [&](int lane, const Range* rd, size_t n_rd, const Range* wr, size_t n_wr, double us) {
-        queued[lane] += std::max(1.0, us);
-        if (NL == 1) return;
-        reads[lane].insert(reads[lane].end(), rd, rd + n_rd);
-        writes[lane].insert(writes[lane].end(), wr, wr + n_wr);
-    };
-    PendingGroup group;
-    auto flush_group = [&]() -> adapt_status_t {
-        if (group.entries.empty()) return ADAPT_OK;
-        int lane = 0;
-        adapt_status_t r = enter(group.reads.data(), group.reads.size(), group.writes.data(), group.writes.size(), false, &lane);
-        if (r != ADAPT_OK) return r;
-        r = launch_pending(S, group, stream[lane]);
-        leave(lane, group.reads.data(), group.reads.size(), group.writes.data(), group.writes.size(), group.predicted_us);
-        group.clear();
-        return r;
-    };
-    adapt_status_t status = ADAPT_OK;
-    for (int64_t i = 0; i < count && status == ADAPT_OK; ++i) {
-        Plan* pl = plans[i];
-        if (!pl) { status = flush_group(); if (status == ADAPT_OK) status = fail(ADAPT_ERR_INVALID_ARG, "null plan%s"); break; }
-        const Shape& sh = pl->s;
-        const Range a = {(uintptr_t)A[i], (uintptr_t)A[i] + (uintptr_t)sh.M * sh.K * 2}, b = {(uintptr_t)B[i], (uintptr_t)B[i] + (uintptr_t)sh.K * sh.N * 2};
-        const Range c = {(uintptr_t)C[i], (uintptr_t)C[i] + (uintptr_t)sh.M * sh.N * 2};
-        if (group.conflicts(a, b, c) && (status = flush_group()) != ADAPT_OK) break;
-        const bool sound = A[i] && B[i] && C[i] && (((uintptr_t)A[i] | (uintptr_t)B[i] | (uintptr_t)C[i]) & 1) == 0 &&
-                           !(c.lo < a.hi && a.lo < c.hi) && !(c.lo < b.hi && b.lo < c.hi);
-        if (sound && grouped(pl)) {
-            PendingGroup::Entry e;
-            e.chain = group_item(sh, pl->c, A[i], B[i], C[i], &e.item);
-            e.variant = (sh.dtype != 0 ? 1 : 0) | (sh.layoutA == ADAPT_ROW_MAJOR ? 2 : 0) | (sh.layoutB == ADAPT_COL_MAJOR ? 4 : 0);
-            group.entries.push_back(e);
-            group.reads.push_back(a);
-            group.reads.push_back(b);
-            group.writes.push_back(c);
-            group.predicted_us += 0.25 * pl->c.predicted_us;
-            if (group.entries.size() >= kGroupMax) status = flush_group();
-            continue;
-        }
-        if (!sound && (status = flush_group()) != ADAPT_OK) break;      // the calls before one that is refused are enqueued
-        const Range rd[2] = {a, b};
-        const bool alone = pl->c.streamk != 0;
-        int lane = 0;
-        if ((status = enter(rd, 2, &c, 1, alone, &lane)) != ADAPT_OK) break;
-        status = adapt_matmul(pl, A[i], B[i], C[i], (void*)stream[lane]);
-        if (status != ADAPT_OK) break;
-        leave(lane, rd, 2, &c, 1, pl->c.predicted_us);
-        if (alone)
-            for (int o = 0; o < NL && status == ADAPT_OK; ++o)
-                if (o != lane) status = wait_for(o, lane);
-    }
-    if (status == ADAPT_OK) status = flush_group();
+    const adapt_status_t status = run_batch(count, NL, call_of, ops);
     // join, also after an error: the caller's stream continues after whatever was queued
     for (int l = 1; l < NL; ++l) {
         if (cudaEventRecord(L.join[l], L.s[l]) == cudaSuccess) (void)cudaStreamWaitEvent(user, L.join[l], 0);

@@ -1,0 +1,103 @@
+"""The order of the launches of a list, compiled on its own and run over random lists on simulated streams: two calls of which one writes
+what the other reads or writes are ordered as in the list, every call before a failing one is launched, and nothing runs beside a call
+that must be alone."""
+import os
+
+from test_host_group_plan import build_and_run
+
+PROGRAM = r"""
+#include <cstdio>
+#include <cstdlib>
+#include <random>
+#include "batch_schedule.h"
+using namespace adapt;
+
+struct Ops {
+    int64_t count;
+    int64_t failing;                                    // the call that returns an error, or -1
+    std::vector<std::vector<char>> lane;                // per lane: the calls that come before whatever it runs next
+    std::vector<std::vector<char>> before;              // per launched call: the calls that come before it
+    std::vector<int> launched;
+    int waits = 0, largest = 0;
+    std::vector<BatchCall> call;
+    void run(int64_t i, int l) { before[i] = lane[l]; ++launched[i]; }
+    adapt_status_t single(int64_t i, int l)
+    {
+        if (i == failing) return ADAPT_ERR_NOMEM;
+        run(i, l);
+        lane[l][i] = 1;
+        return ADAPT_OK;
+    }
+    adapt_status_t group(const std::vector<int64_t>& calls, int l)
+    {
+        largest = std::max<int>(largest, (int)calls.size());
+        for (int64_t i : calls) run(i, l);
+        for (int64_t i : calls) lane[l][i] = 1;
+        return ADAPT_OK;
+    }
+    adapt_status_t wait(int l, int other)
+    {
+        ++waits;
+        for (int64_t i = 0; i < count; ++i) lane[l][i] |= lane[other][i];
+        return ADAPT_OK;
+    }
+};
+
+static bool meet(const Range& x, const Range& y) { return x.lo < y.hi && y.lo < x.hi; }
+
+int main()
+{
+    std::mt19937 rng(7);
+    auto pick = [&](int n) { return (int)(rng() % (unsigned)n); };
+    long waits = 0, grouped = 0, failures = 0, ordered = 0;
+    for (int trial = 0; trial < 2000; ++trial) {
+        const int count = 1 + pick(trial % 3 ? 40 : 200), lanes = 1 + pick(kBatchLanesMax), buffers = 8 + pick(trial % 5 ? 30 : 600);
+        const int small = pick(101), failing = pick(3) ? -1 : pick(count);
+        Ops o;
+        o.count = count;
+        o.failing = -1;
+        o.lane.assign(lanes, std::vector<char>(count, 0));
+        o.before.resize(count);
+        o.launched.assign(count, 0);
+        for (int i = 0; i < count; ++i) {
+            BatchCall k = {};
+            auto range = [&]() -> Range { const uintptr_t at = 16 * (1 + pick(buffers)); return {at, at + 8u + 16u * pick(2)}; };
+            k.a = range();
+            k.b = range();
+            do k.c = range(); while (meet(k.c, k.a) || meet(k.c, k.b));
+            k.groupable = pick(100) < small;
+            k.alone = !k.groupable && pick(12) == 0;
+            k.us = 1 + pick(20);
+            k.unsound = pick(60) == 0;
+            if (i == failing && (!k.groupable || k.unsound)) o.failing = i;
+            o.call.push_back(k);
+        }
+        const adapt_status_t status = run_batch(count, lanes, [&](int64_t i) { return o.call[i]; }, o);
+        const int64_t end = o.failing < 0 ? count : o.failing;
+        bool ok = status == (o.failing < 0 ? ADAPT_OK : ADAPT_ERR_NOMEM);
+        for (int i = 0; i < count; ++i) ok &= o.launched[i] == (i < end ? 1 : 0);
+        for (int j = 0; ok && j < end; ++j)
+            for (int i = 0; i < j; ++i) {
+                const BatchCall &x = o.call[i], &y = o.call[j];
+                const bool order = meet(x.c, y.a) || meet(x.c, y.b) || meet(x.c, y.c) || meet(x.a, y.c) || meet(x.b, y.c);
+                if (order) ok &= o.before[j][i] != 0, ++ordered;
+                if (x.alone || y.alone) ok &= o.before[j][i] || o.before[i][j];
+            }
+        ok &= o.largest <= 8 * kGroupMax;
+        waits += o.waits;
+        grouped += o.largest > 1;
+        failures += o.failing >= 0;
+        if (!ok) {
+            printf("trial %d: %d calls on %d lanes, failing %lld, status %d\n", trial, count, lanes, (long long)o.failing, (int)status);
+            return 1;
+        }
+    }
+    printf("%ld waits, %ld lists with groups, %ld failing lists, %ld ordered pairs\n", waits, grouped, failures, ordered);
+    return !(waits > 3000 && grouped > 1000 && failures > 150 && ordered > 10000);
+}
+"""
+
+
+def test_lists_keep_their_order_on_any_number_of_streams(tmp_path):
+    r = build_and_run(tmp_path, PROGRAM)
+    assert r.returncode == 0, r.stdout + r.stderr
