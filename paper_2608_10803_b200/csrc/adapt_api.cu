@@ -22,6 +22,7 @@
 #include "cluster_gemm.cuh"
 #include "group_gemm.cuh"
 #include "batch_schedule.h"
+#include "batch_route.h"
 #include "umma_gemm.cuh"
 
 using namespace adapt;
@@ -841,6 +842,28 @@ extern "C" adapt_status_t adapt_poll_device_status(void* cuda_stream)
 // ---------------------------------------------------------------------------------------------
 namespace {
 
+// Replaces a stream's workspace by one of at least `bytes` (the caller holds S.mu).
+adapt_status_t grow_workspace(State::Workspace& w, size_t bytes, cudaStream_t stream, cudaError_t* alloc_error)
+{
+    *alloc_error = cudaSuccess;
+    if (w.ptr) {
+        CUDA_TRY(cudaStreamSynchronize(stream));
+        CUDA_TRY(cudaFree(w.ptr));
+        w.ptr = nullptr;
+        w.bytes = 0;
+    }
+    const size_t want = (size_t)round_up((int64_t)bytes + (bytes >> 3), 1 << 20);
+    *alloc_error = cudaMalloc(&w.ptr, want);
+    if (*alloc_error != cudaSuccess) {
+        (void)cudaGetLastError();
+        w.ptr = nullptr;
+        return ADAPT_ERR_NOMEM;
+    }
+    w.bytes = want;
+    CUDA_TRY(cudaMemsetAsync(w.ptr, 0, kUmmaFlagBytes, stream));
+    return ADAPT_OK;
+}
+
 // The stream's workspace, at least `bytes` large.  Its first kUmmaFlagBytes are the stream-K flag words: zeroed when the
 // workspace is allocated, afterwards only ever set to the epoch of a launch, and *epoch (if asked for) is a value no
 // earlier launch on this workspace has used.  The caller's regions start at *out (after the flags).
@@ -856,24 +879,37 @@ adapt_status_t get_workspace(State& S, cudaStream_t stream, size_t bytes, void**
         *epoch = w.epoch;
     }
     if (w.bytes < bytes) {
-        if (w.ptr) {
-            CUDA_TRY(cudaStreamSynchronize(stream));
-            CUDA_TRY(cudaFree(w.ptr));
-            w.ptr = nullptr;
-            w.bytes = 0;
-        }
-        const size_t want = (size_t)round_up((int64_t)bytes + (bytes >> 3), 1 << 20);
-        cudaError_t e = cudaMalloc(&w.ptr, want);
-        if (e != cudaSuccess) {
-            (void)cudaGetLastError();
-            w.ptr = nullptr;
-            return fail(ADAPT_ERR_NOMEM, "workspace allocation failed: %s", cudaGetErrorString(e));
-        }
-        w.bytes = want;
-        CUDA_TRY(cudaMemsetAsync(w.ptr, 0, kUmmaFlagBytes, stream));
+        cudaError_t e;
+        const adapt_status_t r = grow_workspace(w, bytes, stream, &e);
+        if (r == ADAPT_ERR_NOMEM) return fail(r, "workspace allocation failed: %s", cudaGetErrorString(e));
+        if (r != ADAPT_OK) return r;
     }
     *out = (uint8_t*)w.ptr + kUmmaFlagBytes;
     if (flags) *flags = w.ptr;
+    return ADAPT_OK;
+}
+
+// The same for a launch that has a substitute without this workspace: *out stays null when it would have to grow inside a stream
+// capture, or cannot.
+adapt_status_t try_workspace(State& S, cudaStream_t stream, size_t bytes, void** out)
+{
+    *out = nullptr;
+    bytes += kUmmaFlagBytes;
+    std::lock_guard<std::mutex> lock(S.mu);
+    State::Workspace& w = S.ws[stream];
+    if (w.bytes < bytes) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) {
+            (void)cudaGetLastError();
+            return ADAPT_OK;
+        }
+        if (capture != cudaStreamCaptureStatusNone) return ADAPT_OK;
+        cudaError_t e;
+        const adapt_status_t r = grow_workspace(w, bytes, stream, &e);
+        if (r == ADAPT_ERR_NOMEM) return ADAPT_OK;
+        if (r != ADAPT_OK) return r;
+    }
+    *out = (uint8_t*)w.ptr + kUmmaFlagBytes;
     return ADAPT_OK;
 }
 
@@ -900,9 +936,9 @@ adapt_status_t encode_map(State& S, CUtensorMap* map, const void* base, int dtyp
     return ADAPT_OK;
 }
 
-// 3D map over `entries` such matrices, `stride` elements apart.
-adapt_status_t encode_map3(State& S, CUtensorMap* map, const void* base, int dtype, int64_t inner, int64_t outer, int64_t pitch,
-                           int64_t entries, int64_t stride, int box_inner, int box_outer)
+// 3D map over `entries` such matrices, `stride` elements apart; false if the driver does not take this geometry.
+bool encode_map3(State& S, CUtensorMap* map, const void* base, int dtype, int64_t inner, int64_t outer, int64_t pitch,
+                 int64_t entries, int64_t stride, int box_inner, int box_outer)
 {
     const cuuint64_t gdim[3] = {(cuuint64_t)inner, (cuuint64_t)outer, (cuuint64_t)entries};
     const cuuint64_t gstride[2] = {(cuuint64_t)pitch * 2, (cuuint64_t)stride * 2};
@@ -911,13 +947,8 @@ adapt_status_t encode_map3(State& S, CUtensorMap* map, const void* base, int dty
     const CUresult r = S.encode(map, dtype == 0 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
                                 const_cast<void*>(base), gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        char buf[32];
-        snprintf(buf, sizeof(buf), "%d", (int)r);
-        return fail(ADAPT_ERR_CUDA, "cuTensorMapEncodeTiled failed with CUresult %s", buf);
-    }
     S.map_encodes.fetch_add(1, std::memory_order_relaxed);
-    return ADAPT_OK;
+    return r == CUDA_SUCCESS;
 }
 
 // The slot a new encoding goes to: a fresh one while fewer than kMapSlots exist, then round-robin.
@@ -1386,91 +1417,48 @@ extern "C" adapt_status_t adapt_addmm(adapt_handle_t plan, const void* A, const 
 
 namespace {
 
-// An operand of a strided batch as the tensor-core kernel reads it: in place, or (rows or entries off 16-byte boundaries, narrow
-// rows) over one re-pitched copy of all entries, which takes entries that lie back to back.
-struct BatchOperand {
-    const void* src;
-    int64_t inner, outer, entries, stride;     // of the caller's matrices (entries = 1: shared by the batch)
-    bool copy, ok;
-    int64_t pitch, entry_stride;               // of what TMA reads
-    size_t bytes;                              // of the copy
-    BatchOperand(const void* p, int64_t in, int64_t out, int64_t batch, int64_t st)
-        : src(p), inner(in), outer(out), entries(st == 0 ? 1 : batch), stride(st == 0 ? in * out : st)
-    {
-        copy = !tma_friendly(inner) || ((uintptr_t)p & 15) != 0 || (entries > 1 && stride % 8 != 0);
-        ok = !copy || stride == inner * outer;
-        pitch = copy ? padded_pitch(inner) : inner;
-        entry_stride = copy || entries == 1 ? pitch * outer : stride;
-        bytes = copy ? (size_t)round_up(entries * outer * pitch * 2, 256) : 0;
-    }
-};
-
-// How a strided batch runs: entry by entry, or in one launch on the grouped kernel's or the tensor-core kernel's tiles.
-enum { kBatchLoop = 0, kBatchGroup, kBatchUmma };
-struct BatchRoute { int kind, BN; };
-
-// The estimates behind the choice (us).  Grouped kernel: rounds of two CTAs per SM, 1.5 us and 0.6 us per stage of a group of warps.
-// Tensor-core kernel: rounds of one CTA per SM, k-blocks of 0.25 to 0.42 us (64 to 256 columns) or the tile's drain, whichever is
-// longer, a copy of operands that TMA cannot read in place, 4 us around it.  Entry by entry: the plan's prediction less the
-// microsecond that consecutive launches overlap.
-BatchRoute batch_route(const Shape& s, const Config& c, const Machine& m, int64_t batch, bool group_ok, bool umma_ok, const BatchOperand& a,
-                       const BatchOperand& b, bool tma_store)
-{
-    BatchRoute best = {kBatchLoop, 0};
-    double us = (double)batch * std::max(1.5, c.predicted_us - 1.0);
-    if (group_ok) {
-        const double rounds = (double)ceil_div(batch * ceil_div(s.M, 64) * ceil_div(s.N, 64), 2 * (int64_t)m.n_sm);
-        const double chain = c.family == ADAPT_FAM_SIMT ? 1.0 : (double)ceil_div(s.K, 2 * kClusterKS);
-        const double t = 3.0 + rounds * (1.5 + 0.6 * chain);
-        if (t < us) { us = t; best = {kBatchGroup, 0}; }
-    }
-    if (umma_ok) {
-        const double copies = ((a.copy ? (double)a.entries * a.outer * (a.inner + a.pitch) : 0.0) + (b.copy ? (double)b.entries * b.outer * (b.inner + b.pitch) : 0.0)) * 2.0;
-        const double traffic = 2.0 * ((double)a.entries * s.M * s.K + (double)b.entries * s.K * s.N + (double)batch * s.M * s.N);
-        for (int BN : {64, 128, 256}) {
-            if (BN > 64 && s.N <= BN / 2) continue;
-            const int64_t units = batch * ceil_div(s.M, 128) * ceil_div(s.N, BN);
-            const double rounds = (double)ceil_div(units, m.n_sm);
-            const double t_kb = BN == 64 ? 0.25 : BN == 128 ? 0.30 : 0.42;
-            const double kb = 2.0 * std::min<double>(128.0, (double)s.M) * BN / 1024.0;
-            const double drain = tma_store ? 0.25 + 0.0275 * kb : 1.4 + 0.031 * kb;
-            const double t = std::max(rounds * std::max((double)ceil_div(s.K, 64) * t_kb, drain), traffic / 5.5e6) + 4.0 +
-                             (copies > 0 ? 0.5 + copies / 5.5e6 : 0.0);
-            if (t < us) { us = t; best = {kBatchUmma, BN}; }
-        }
-    }
-    return best;
-}
-
+// The entries of one launch.  *done stays false, with nothing enqueued, when the workspace cannot hold the copies (or would have to
+// grow inside a stream capture) or the driver does not take a tensor map: the caller then has the other routes.
 adapt_status_t launch_batch_umma(State& S, const Shape& s, int BN, const BatchOperand& a, const BatchOperand& b, void* C, int64_t sc, int64_t batch,
-                                 bool tma_store, cudaStream_t stream)
+                                 bool tma_store, cudaStream_t stream, bool* done)
 {
     const bool a_mn = s.layoutA == ADAPT_COL_MAJOR, b_mn = s.layoutB == ADAPT_ROW_MAJOR;
+    const int a_box = umma_a_box_rows(s, 1, 0, false);
+    const int64_t kb_total = ceil_div(s.K, kUmmaBK);
+    const int b_box_k = b_mn && kb_total == 1 ? (int)std::min<int64_t>(64, round_up(s.K, 8)) : 64;
+    const int stages = umma_deepest_ring(BN, 1, a_box, true, S.machine.smem_bytes, a_box == 128 ? 8 : kUmmaMaxStages);
+    if (stages < 2) return ADAPT_OK;
     void* ws = nullptr;
-    adapt_status_t r = get_workspace(S, stream, a.bytes + b.bytes, &ws);
-    if (r != ADAPT_OK) return r;
+    if (a.copy || b.copy) {
+        const adapt_status_t r = try_workspace(S, stream, a.bytes() + b.bytes(), &ws);
+        if (r != ADAPT_OK || !ws) return r;
+    }
     uint8_t* w8 = (uint8_t*)ws;
-    const void* pa = a.copy ? w8 : a.src;
-    const void* pb = b.copy ? w8 + a.bytes : b.src;
-    if (a.copy && b.copy) r = launch_pad2(S, a.src, w8, a.entries * a.outer, a.inner, a.pitch, b.src, w8 + a.bytes, b.entries * b.outer, b.inner, b.pitch, stream);
+    uint8_t* wb = w8 + a.bytes();
+    TmapPackT<4> maps;
+    memset(&maps, 0, sizeof(maps));
+    if (!encode_map3(S, &maps.a[0], a.copy ? w8 : a.src, s.dtype, a.pitch, a.outer, a.pitch, a.entries, a.entry_stride, 64, a_mn ? 64 : a_box) ||
+        !encode_map3(S, &maps.b[0], b.copy ? wb : b.src, s.dtype, b.pitch, b.outer, b.pitch, b.entries, b.entry_stride, 64, b_mn ? b_box_k : BN) ||
+        (tma_store && !encode_map3(S, &maps.c[0], C, s.dtype, s.N, s.M, s.N, batch, sc, 64, 32)))
+        return ADAPT_OK;
+    *done = true;
+    adapt_status_t r = ADAPT_OK;
+    if (a.copy && b.copy) r = launch_pad2(S, a.src, w8, a.entries * a.outer, a.inner, a.pitch, b.src, wb, b.entries * b.outer, b.inner, b.pitch, stream);
     else if (a.copy) r = launch_pad(S, a.src, w8, a.entries * a.outer, a.inner, a.pitch, stream);
-    else if (b.copy) r = launch_pad(S, b.src, w8 + a.bytes, b.entries * b.outer, b.inner, b.pitch, stream);
+    else if (b.copy) r = launch_pad(S, b.src, wb, b.entries * b.outer, b.inner, b.pitch, stream);
     if (r != ADAPT_OK) return r;
     UmmaParams p;
     memset(&p, 0, sizeof(p));
     p.M = (int)s.M; p.N = (int)s.N; p.K = (int)s.K;
     p.P_m = (int)ceil_div(s.M, 128); p.P_n = (int)ceil_div(s.N, BN); p.P_k = 1;
-    p.kb_total = p.kb_per_split = (int)ceil_div(s.K, kUmmaBK);
+    p.kb_total = p.kb_per_split = (int)kb_total;
     p.tiles_per_entry = p.P_m * p.P_n;
     p.num_units = (int)(batch * p.tiles_per_entry);
     p.a_entry = a.entries > 1 ? 1 : 0;
     p.b_entry = b.entries > 1 ? 1 : 0;
     p.c_entry = sc;
     p.dtype = s.dtype;
-    const int a_box = umma_a_box_rows(s, 1, 0, false);
-    const int b_box_k = b_mn && p.kb_total == 1 ? (int)std::min<int64_t>(64, round_up(s.K, 8)) : 64;
-    p.stages = umma_deepest_ring(BN, 1, a_box, true, S.machine.smem_bytes, a_box == 128 ? 8 : kUmmaMaxStages);
-    if (p.stages < 2) return fail(ADAPT_ERR_UNSUPPORTED, "no room for two stages%s");
+    p.stages = stages;
     p.a_tx_bytes = a_box * kUmmaBK * 2;
     p.b_tx_bytes = b_mn ? BN * b_box_k * 2 : BN * kUmmaBK * 2;
     p.idesc = umma_idesc(s.dtype, a_mn, b_mn, 128, BN);
@@ -1481,11 +1469,6 @@ adapt_status_t launch_batch_umma(State& S, const Shape& s, int BN, const BatchOp
     p.ncls_log2 = 3;
     p.ep = no_epilogue();
     p.status = S.d_status;
-    TmapPackT<4> maps;
-    memset(&maps, 0, sizeof(maps));
-    if ((r = encode_map3(S, &maps.a[0], pa, s.dtype, a.pitch, a.outer, a.pitch, a.entries, a.entry_stride, 64, a_mn ? 64 : a_box)) != ADAPT_OK) return r;
-    if ((r = encode_map3(S, &maps.b[0], pb, s.dtype, b.pitch, b.outer, b.pitch, b.entries, b.entry_stride, 64, b_mn ? b_box_k : BN)) != ADAPT_OK) return r;
-    if (tma_store && (r = encode_map3(S, &maps.c[0], C, s.dtype, s.N, s.M, s.N, batch, sc, 64, 32)) != ADAPT_OK) return r;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)std::min(p.num_units, S.machine.n_sm), 1, 1);
@@ -1503,11 +1486,11 @@ adapt_status_t launch_batch_umma(State& S, const Shape& s, int BN, const BatchOp
     return ADAPT_OK;
 }
 
-// A strided batch in one launch (and a copy of unaligned operands).  *done stays false when the batch is to run entry by entry:
-// forced plans of the tensor-core and warp-level families, entries that depend on one another (an output that overlaps any input
-// of the batch), arguments that the single call refuses, copies beyond the workspace limit, large entries.
+// A strided batch in as few launches as its copies allow.  Returns in *done the entries enqueued, from the first on; the others are to
+// run entry by entry: forced plans of the tensor-core and warp-level families, entries that depend on one another (an output that
+// overlaps any input of the batch), arguments that the single call refuses, large entries.
 adapt_status_t run_strided_batch(State& S, Plan* pl, const void* A, int64_t sa, const void* B, int64_t sb, void* C, int64_t sc,
-                                 int64_t batch, cudaStream_t stream, bool* done)
+                                 int64_t batch, cudaStream_t stream, int64_t* done)
 {
     const Shape& s = pl->s;
     if (!S.inited || pl->noop || pl->zero_fill || !A || !B || !C || (((uintptr_t)A | (uintptr_t)B | (uintptr_t)C) & 1)) return ADAPT_OK;
@@ -1522,12 +1505,22 @@ adapt_status_t run_strided_batch(State& S, Plan* pl, const void* A, int64_t sa, 
     const BatchOperand a(A, a_rm ? s.K : s.M, a_rm ? s.M : s.K, batch, sa), b(B, b_rm ? s.N : s.K, b_rm ? s.K : s.N, batch, sb);
     const bool tma_store = ((uintptr_t)C & 31) == 0 && s.N % 16 == 0 && sc % 16 == 0;
     const bool group_ok = c.family == ADAPT_FAM_CLUSTER || (c.family == ADAPT_FAM_SIMT && group_eligible(s, c));
-    const bool umma_ok = pl->selected && (S.machine.family_mask & (1u << ADAPT_FAM_UMMA_1CTA)) && a.ok && b.ok &&
-                         (int64_t)(a.bytes + b.bytes) <= S.machine.workspace_limit;
-    const BatchRoute route = batch_route(s, c, S.machine, batch, group_ok, umma_ok, a, b, tma_store);
+    const bool umma_ok = pl->selected && (S.machine.family_mask & (1u << ADAPT_FAM_UMMA_1CTA));
+    BatchRoute route = batch_route(s, c, S.machine, batch, group_ok, umma_ok, a, b, tma_store);
+    if (route.kind == kBatchUmma) {
+        while (*done < batch) {
+            const int64_t n = std::min(route.chunk, batch - *done);
+            bool launched = false;
+            const adapt_status_t r = launch_batch_umma(S, s, route.BN, a.part(*done, n), b.part(*done, n), (unsigned short*)C + *done * sc, sc, n,
+                                                       tma_store, stream, &launched);
+            if (r != ADAPT_OK) return r;
+            if (!launched) break;
+            *done += n;
+        }
+        if (*done > 0) return ADAPT_OK;
+        route = batch_route(s, c, S.machine, batch, group_ok, false, a, b, tma_store);
+    }
     if (route.kind == kBatchLoop) return ADAPT_OK;
-    *done = true;
-    if (route.kind == kBatchUmma) return launch_batch_umma(S, s, route.BN, a, b, C, sc, batch, tma_store, stream);
     GroupParams p;
     Config one = c;
     if (c.family == ADAPT_FAM_CLUSTER) one.cluster = 1;      // the entries fill the machine: no pieces
@@ -1540,6 +1533,7 @@ adapt_status_t run_strided_batch(State& S, Plan* pl, const void* A, int64_t sa, 
     p.sa = sa; p.sb = sb; p.sc = sc;
     CUDA_TRY(launch_group(p, a_rm, !b_rm, stream));
     S.launches.fetch_add(1, std::memory_order_relaxed);
+    *done = batch;
     return ADAPT_OK;
 }
 
@@ -1551,12 +1545,12 @@ extern "C" adapt_status_t adapt_matmul_strided_batch(adapt_handle_t plan, const 
     if (batch < 0 || stride_a < 0 || stride_b < 0 || stride_c < 0) return fail(ADAPT_ERR_INVALID_ARG, "negative batch count or stride%s");
     if (!plan) return fail(ADAPT_ERR_INVALID_ARG, "null plan%s");
     if (batch > 1 && !plan->noop && stride_c < plan->s.M * plan->s.N) return fail(ADAPT_ERR_INVALID_ARG, "outputs of the batch overlap%s");
+    int64_t done = 0;
     if (batch > 1) {
-        bool done = false;
         const adapt_status_t r = run_strided_batch(st(), plan, A, stride_a, B, stride_b, C, stride_c, batch, (cudaStream_t)cuda_stream, &done);
-        if (done || r != ADAPT_OK) return r;
+        if (r != ADAPT_OK) return r;
     }
-    for (int64_t i = 0; i < batch; ++i) {
+    for (int64_t i = done; i < batch; ++i) {
         const adapt_status_t r = adapt_matmul(plan, (const unsigned short*)A + i * stride_a, (const unsigned short*)B + i * stride_b,
                                               (unsigned short*)C + i * stride_c, cuda_stream);
         if (r != ADAPT_OK) return r;
