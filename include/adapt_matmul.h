@@ -253,7 +253,13 @@ adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t* plans, co
  *
  * adapt_matmul_strided_batch:  `batch` GEMMs of the plan's shape on operands stride_a, stride_b, stride_c ELEMENTS apart
  * (a stride of 0 shares that input across the batch; stride_c must be at least M * N).  The result is the one of the entries run in
- * batch order; entries that do not depend on one another (no output overlaps an input) share one launch where that is faster. */
+ * batch order, up to the rounding of the fp32 sums: entries that do not depend on one another (no output overlaps an input) share
+ * launches where that is faster, and the tiles of such a launch are chosen for the batch, so the order in which an entry's products are
+ * added can differ from adapt_matmul's on that entry and depends on the batch count, the strides and the alignment of the pointers (the
+ * same call gives the same bits every time).  A plan whose configuration was asked for (adapt_matmul_plan_forced, or a plan-table
+ * line that is not what the library would choose) keeps that configuration, and every entry has the bits of adapt_matmul.  Unaligned
+ * operands may be copied through the stream's workspace, 64 MB of entries at a time; where that workspace cannot be had the batch runs
+ * without the copies.  Launches on the tensor-core kernel encode two or three tensor maps per call. */
 adapt_status_t adapt_addmm(adapt_handle_t plan, const void* A, const void* B, const void* D, int d_is_vector,
                            float alpha, float beta, void* C, void* cuda_stream);
 adapt_status_t adapt_matmul_strided_batch(adapt_handle_t plan, const void* A, int64_t stride_a, const void* B, int64_t stride_b,

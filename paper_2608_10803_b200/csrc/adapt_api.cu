@@ -69,6 +69,7 @@ struct adapt_plan_s {
     Shape s;
     Config c;
     bool selected = false;    // the plan adapt_matmul_plan returns for its shape (not a forced-key plan)
+    std::atomic<int> model_pick{-1};   // is its configuration the model's choice (a table's may be another)?  -1: not looked yet
     bool noop = false;        // M == 0 or N == 0
     bool zero_fill = false;   // K == 0
     std::mutex mu;            // guards the tensor-map slots
@@ -329,6 +330,7 @@ extern "C" adapt_handle_t adapt_matmul_plan(int64_t M, int64_t N, int64_t K, ada
     }
     Plan* p = make_plan(S, s, nullptr);
     if (!p) return nullptr;
+    p->model_pick.store(1, std::memory_order_relaxed);
     insert_selected(S, s, p);
     return p;
 }
@@ -1486,9 +1488,27 @@ adapt_status_t launch_batch_umma(State& S, const Shape& s, int BN, const BatchOp
     return ADAPT_OK;
 }
 
+// Is the plan's configuration the one the model picks for its shape?  A forced key or a line of a plan table asks for exactly its
+// configuration; a table line that records the model's pick asks for nothing else than no table would.
+bool is_model_pick(State& S, Plan* pl)
+{
+    int known = pl->model_pick.load(std::memory_order_relaxed);
+    if (known < 0) {
+        std::vector<Config> cands;
+        if (pl->selected) {
+            std::lock_guard<std::mutex> lock(S.mu);
+            enumerate_configs(pl->s, S.machine, S.calib, &cands);
+        }
+        known = !cands.empty() && pack_tiling_key(pl->s, cands[0]) == pack_tiling_key(pl->s, pl->c) ? 1 : 0;
+        pl->model_pick.store(known, std::memory_order_relaxed);
+    }
+    return known != 0;
+}
+
 // A strided batch in as few launches as its copies allow.  Returns in *done the entries enqueued, from the first on; the others are to
-// run entry by entry: forced plans of the tensor-core and warp-level families, entries that depend on one another (an output that
-// overlaps any input of the batch), arguments that the single call refuses, large entries.
+// run entry by entry: entries that depend on one another (an output that overlaps any input of the batch), arguments that the single
+// call refuses, large entries.  A plan whose configuration was asked for (a forced key, a plan table) keeps it: its tiles may share a
+// launch, but they are the plan's tiles with the plan's pieces of the k range.
 adapt_status_t run_strided_batch(State& S, Plan* pl, const void* A, int64_t sa, const void* B, int64_t sb, void* C, int64_t sc,
                                  int64_t batch, cudaStream_t stream, int64_t* done)
 {
@@ -1504,8 +1524,9 @@ adapt_status_t run_strided_batch(State& S, Plan* pl, const void* A, int64_t sa, 
     const bool a_rm = s.layoutA == ADAPT_ROW_MAJOR, b_rm = s.layoutB == ADAPT_ROW_MAJOR;
     const BatchOperand a(A, a_rm ? s.K : s.M, a_rm ? s.M : s.K, batch, sa), b(B, b_rm ? s.N : s.K, b_rm ? s.K : s.N, batch, sb);
     const bool tma_store = ((uintptr_t)C & 31) == 0 && s.N % 16 == 0 && sc % 16 == 0;
-    const bool group_ok = c.family == ADAPT_FAM_CLUSTER || (c.family == ADAPT_FAM_SIMT && group_eligible(s, c));
-    const bool umma_ok = pl->selected && (S.machine.family_mask & (1u << ADAPT_FAM_UMMA_1CTA));
+    const bool free_choice = is_model_pick(S, pl);
+    const bool group_ok = group_eligible(s, c) || (free_choice && c.family == ADAPT_FAM_CLUSTER);
+    const bool umma_ok = free_choice && (S.machine.family_mask & (1u << ADAPT_FAM_UMMA_1CTA));
     BatchRoute route = batch_route(s, c, S.machine, batch, group_ok, umma_ok, a, b, tma_store);
     if (route.kind == kBatchUmma) {
         while (*done < batch) {
@@ -1523,7 +1544,7 @@ adapt_status_t run_strided_batch(State& S, Plan* pl, const void* A, int64_t sa, 
     if (route.kind == kBatchLoop) return ADAPT_OK;
     GroupParams p;
     Config one = c;
-    if (c.family == ADAPT_FAM_CLUSTER) one.cluster = 1;      // the entries fill the machine: no pieces
+    if (free_choice && c.family == ADAPT_FAM_CLUSTER) one.cluster = 1;      // the entries fill the machine: no pieces
     GroupItem it;
     const int chain = group_item(s, one, A, B, C, &it);
     group_clear(p);

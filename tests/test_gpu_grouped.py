@@ -168,3 +168,66 @@ def test_list_of_short_k_plans_that_a_table_cut_into_pieces(tmp_path, pieces):
     for x, y, s in zip(alone, listed, shapes):
         assert torch.equal(x.view(torch.int16), y.view(torch.int16)), s
     ab.adapt_shutdown()
+
+
+def strided_and_alone(plan, M, N, K, dtype, batch, offset=0, seed=31):
+    """The same batch in one call and entry by entry, with non-integer operands; launches of the one call."""
+    A = offset_operand(batch * M, K, seed, dtype, offset)
+    B = offset_operand(batch * K, N, seed + 1, dtype, offset)
+    one, many = (torch.full((batch * M * N,), float("nan"), dtype=A.dtype, device="cuda") for _ in range(2))
+    for e in range(batch):
+        ab.adapt_matmul(plan, A.data_ptr() + 2 * e * M * K, B.data_ptr() + 2 * e * K * N, many.data_ptr() + 2 * e * M * N, stream())
+    before = ab.adapt_launch_count()
+    ab.adapt_matmul_strided_batch(plan, A.data_ptr(), M * K, B.data_ptr(), K * N, one.data_ptr(), M * N, batch, stream())
+    launches = ab.adapt_launch_count() - before
+    torch.cuda.synchronize()
+    ab.adapt_poll_device_status(stream())
+    return A, B, one, many, launches
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("table", [False, True])
+def test_strided_batch_keeps_a_configuration_that_was_asked_for(tmp_path, table, offset):
+    """Every kind of candidate, forced or named by a plan table: the bits of the entries alone."""
+    M, N, K, batch, dt = 96, 200, 1000, 12, ab.F16
+    init()
+    kinds = {}
+    for c in ab.adapt_plan_candidates(M, N, K, dt):
+        kinds.setdefault((c.family, c.cluster, c.P_k > 1, c.fused, c.srcA, c.srcB), c)
+    assert {c.cluster for c in kinds.values() if c.family == ab.FAM_CLUSTER} == {1, 2, 4, 8, 16}
+    for c in kinds.values():
+        if table:
+            ab.adapt_shutdown()
+            init()
+            plan, = installed_plans(tmp_path, [(M, N, K, dt)], lambda x: x.tiling_key == c.tiling_key)
+        else:
+            plan = ab.adapt_matmul_plan_forced(M, N, K, dt, 0, 0, c.tiling_key)
+        assert ab.adapt_plan_info(plan).tiling_key == c.tiling_key
+        if table and c.tiling_key == ab.adapt_plan_candidates(M, N, K, dt)[0].tiling_key:
+            continue                                                    # what the library would choose itself
+        _, _, one, many, launches = strided_and_alone(plan, M, N, K, dt, batch, offset)
+        assert torch.equal(one.view(torch.int16), many.view(torch.int16)), (ab.FAMILY_NAMES[c.family], c.cluster, c.P_k, c.BN)
+        assert launches == 1 or c.family != ab.FAM_CLUSTER
+    if table:
+        ab.adapt_shutdown()
+
+
+@pytest.mark.parametrize("shape", [(96, 200, 1000, 12, 1), (130, 77, 259, 200, 2), (128, 256, 512, 160, 1), (513, 96, 64, 100, 1)])
+@pytest.mark.parametrize("dtype", [ab.F16, ab.BF16])
+def test_strided_batch_of_a_chosen_plan_rounds_once_and_repeats(shape, dtype):
+    """One or two launches, every element within one rounding of the 16-bit result (and an fp32 sum's error), the same bits again."""
+    M, N, K, batch, most = shape
+    init()
+    plan = ab.adapt_matmul_plan(M, N, K, dtype)
+    A, B, one, many, launches = strided_and_alone(plan, M, N, K, dtype, batch)
+    assert launches <= most
+    again = strided_and_alone(plan, M, N, K, dtype, batch)[2]
+    assert torch.equal(one.view(torch.int16), again.view(torch.int16))
+    a, b = A.view(batch, M, K).double(), B.view(batch, K, N).double()
+    want, scale = torch.bmm(a, b), torch.bmm(a.abs(), b.abs())
+    # fp32 products are exact; a sum of K of them in any order, truncated at each step, is within K 2^-23 of the sum of magnitudes; then one
+    # rounding to 16 bits
+    half_ulp = 2.0 ** -11 if dtype == ab.F16 else 2.0 ** -8
+    bound = half_ulp * want.abs() + (K * 2.0 ** -23) * 1.01 * scale + 2.0 ** -25
+    for got in (one, many):
+        assert bool(((got.view(batch, M, N).double() - want).abs() <= bound).all())
