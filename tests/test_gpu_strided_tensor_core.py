@@ -42,23 +42,29 @@ def expect_entries(A, sa, B, sb, C, sc, M, N, K, dtype, entries):
 @pytest.mark.parametrize("offset", [0, 1])
 @pytest.mark.parametrize("strides", [(8, 16), (64, 0), (16, 520), (40, 24), (3, 5)])
 def test_strided_batch_of_entries_that_overlap_one_another(strides, offset):
-    """Inputs closer together than an entry is long (sliding windows)."""
+    """Inputs closer together than an entry is long (sliding windows); read in place where rows and strides are 16-byte multiples."""
     init()
-    M, N, K, batch, dt = 130, 96, 200, 90, ab.F16
+    M, N, K, batch, dt = 200, 264, 328, 120, ab.F16
+    plan = ab.adapt_matmul_plan(M, N, K, dt)
+    assert ab.adapt_plan_info(plan).family in (ab.FAM_UMMA_1CTA, ab.FAM_UMMA_2CTA)
     sa, sb = strides
     A, B = integers((batch - 1) * sa + M * K + offset, 5)[offset:], integers((batch - 1) * sb + K * N + offset, 6)[offset:]
     C = torch.full((batch * M * N,), float("nan"), dtype=torch.float16, device="cuda")
     st = torch.cuda.current_stream().cuda_stream
-    ab.adapt_matmul_strided_batch(ab.adapt_matmul_plan(M, N, K, dt), A.data_ptr(), sa, B.data_ptr(), sb, C.data_ptr(), M * N, batch, st)
+    before = ab.adapt_launch_count()
+    ab.adapt_matmul_strided_batch(plan, A.data_ptr(), sa, B.data_ptr(), sb, C.data_ptr(), M * N, batch, st)
+    launches = ab.adapt_launch_count() - before
     torch.cuda.synchronize()
     ab.adapt_poll_device_status(st)
+    # in place: one launch; overlapping entries are not copied as a whole, so the others run one by one
+    assert (launches == 1) == (offset == 0 and sa % 8 == 0 and sb % 8 == 0)
     expect_entries(A, sa, B, sb, C, M * N, M, N, K, dt, range(0, batch, 7))
 
 
 def test_copies_of_unaligned_entries_are_held_in_parts():
     """More copied bytes than are held at a time: several launches, a bounded workspace."""
     init()
-    M, N, K, batch, dt = 300, 77, 1003, 700, ab.F16
+    M, N, K, batch, dt = 370, 737, 98, 700, ab.F16
     A, B = integers(batch * M * K, 7), integers(batch * K * N, 8)
     C = torch.full((batch * M * N,), float("nan"), dtype=torch.float16, device="cuda")
     stream = torch.cuda.Stream()
@@ -68,7 +74,7 @@ def test_copies_of_unaligned_entries_are_held_in_parts():
     ab.adapt_matmul_strided_batch(plan, A.data_ptr(), M * K, B.data_ptr(), K * N, C.data_ptr(), M * N, batch, stream.cuda_stream)
     torch.cuda.synchronize()
     ab.adapt_poll_device_status(stream.cuda_stream)
-    copied = 2 * batch * (M * 1008 + K * 80)                       # rows at a pitch of whole 32 bytes
+    copied = 2 * batch * (M * 112 + K * 752)                       # rows at a pitch of whole 32 bytes
     assert 2 * (copied >> 26) <= ab.adapt_launch_count() - before <= 2 * (copied >> 26) + 4
     assert free - torch.cuda.mem_get_info()[0] <= 96 << 20         # 64 MB, an eighth more and the allocator's rounding
     expect_entries(A, M * K, B, K * N, C, M * N, M, N, K, dt, [0, 1, 63, 64, 100, 101, batch - 2, batch - 1])
@@ -78,16 +84,21 @@ def test_strided_batch_in_a_capture_on_a_stream_without_a_workspace():
     """The plan by itself needs no workspace, so the batch can be captured without a call before it; the copy of all entries, which
     would need one, is not an option there."""
     init()
-    M, N, K, batch, dt = 130, 77, 259, 200, ab.F16
+    M, N, K, batch, dt = 100, 201, 130, 200, ab.F16
     plan = ab.adapt_matmul_plan(M, N, K, dt)
     assert ab.adapt_plan_info(plan).workspace_bytes == 0
     A, B = integers(batch * M * K, 9), integers(batch * K * N, 10)
     C = torch.full((batch * M * N,), float("nan"), dtype=torch.float16, device="cuda")
+    args = (plan, A.data_ptr(), M * K, B.data_ptr(), K * N, C.data_ptr(), M * N, batch)
+    before = ab.adapt_launch_count()
+    ab.adapt_matmul_strided_batch(*args, torch.cuda.current_stream().cuda_stream)
+    assert ab.adapt_launch_count() - before == 2                   # the copy and the tensor-core kernel
+    C.fill_(float("nan"))
     side = torch.cuda.Stream()
     torch.cuda.synchronize()
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph, stream=side):
-        ab.adapt_matmul_strided_batch(plan, A.data_ptr(), M * K, B.data_ptr(), K * N, C.data_ptr(), M * N, batch, side.cuda_stream)
+        ab.adapt_matmul_strided_batch(*args, side.cuda_stream)
     graph.replay()
     torch.cuda.synchronize()
     ab.adapt_poll_device_status(side.cuda_stream)
