@@ -229,14 +229,16 @@ adapt_status_t adapt_matmul_noalloc(int64_t M, int64_t N, int64_t K, adapt_dtype
  * - Small calls whose plans are of the one-launch family, or of the CUDA-core family with a short K (as adapt_matmul_plan
  *   returned them), leave together in one grouped launch per 64 calls, data type and pair of layouts.  A call that reads or
  *   overwrites what a collected one writes, or overwrites what it reads, makes the collected ones leave first.
- * - From eight calls on the launches are spread over cuda_stream and up to three internal streams between a fork from and a
- *   join to it (work queued on cuda_stream before the call comes first, work queued after it comes last), so that the launch
- *   gaps and the tail of one GEMM fill with the next one's work.  A launch whose output overlaps a buffer that an earlier one
- *   still reads or writes on another stream, or whose inputs overlap such an output, waits for that stream first.  Option
- *   "batch_streams" (adapt_set_option; 1 to 4, default 4) sets the number of streams; with 1 everything runs on cuda_stream.
+ * - From eight calls on the launches are spread over up to four internal streams, and cuda_stream itself for launches that need no
+ *   workspace, between a fork from and a join to cuda_stream (work queued on cuda_stream before the call comes first, work queued
+ *   after it comes last), so that the launch gaps and the tail of one GEMM fill with the next one's work.  A launch whose output
+ *   overlaps a buffer that an earlier one still reads or writes on another stream, or whose inputs overlap such an output, waits for
+ *   that stream first.  Option "batch_streams" (adapt_set_option; 1 to 4, default 4) sets the number of internal streams; with 1
+ *   everything runs on cuda_stream.
  * The internal streams keep workspaces of their own.  Once a batch has run (workspaces grown, tensor maps of its pointers
  * cached) the same batch only launches kernels and records and waits for events, so it can be captured into a CUDA graph
- * through cuda_stream and replayed. */
+ * through cuda_stream and replayed; a batch of fewer than eight calls, or with "batch_streams" 1, has to have run on that same stream if
+ * it needs a workspace. */
 adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t* plans, const void* const* A,
                                   const void* const* B, void* const* C, void* cuda_stream);
 

@@ -146,14 +146,14 @@ struct State {
     std::atomic<int> map_cache{1};         // 0: every call encodes its maps afresh (measurement of the miss cost)
     int log = 0;
     int shuffle_k = 0;                 // ShuffleK analogue (ADAPT_SHUFFLE_K=1): rotated k-block order per tile; measured, off by default
-    // adapt_matmul_batch: up to four internal streams (lanes) between a fork from and a join to the caller's stream
+    // adapt_matmul_batch: internal streams between a fork from and a join to the caller's stream
     struct BatchLanes {
-        cudaStream_t s[4] = {nullptr, nullptr, nullptr, nullptr};
-        cudaEvent_t fork = nullptr, join[4] = {nullptr, nullptr, nullptr, nullptr}, cross[4] = {nullptr, nullptr, nullptr, nullptr};
+        cudaStream_t s[kBatchInternalMax] = {};
+        cudaEvent_t fork = nullptr, cross[kBatchLanesMax] = {};        // cross: recorded on a lane for another one (or the join) to wait for
         bool ready = false;
     } lanes;
     std::mutex batch_mu;               // one batch at a time uses the lanes
-    int batch_lanes = 4;               // "batch_streams" option (1 to 4): 1 = the calls of a batch run one after the other on the caller's stream
+    int batch_lanes = 4;               // "batch_streams" option (1 to 4 internal streams; 1 = everything runs on the caller's stream)
     int prefetch = 1;                  // L2 prefetch of a kernel's first operands ahead of its dependency wait (ADAPT_PREFETCH=0 turns it off)
     bool class_promo128 = true;        // 128-byte L2 promotion for the strided class views (ADAPT_CLASS_PROMO128=0: 256 as for dense operands)
 };
@@ -799,11 +799,8 @@ extern "C" void adapt_shutdown(void)
         }
         S.pipes.clear();
         if (S.lanes.ready) {
-            for (int l = 0; l < 4; ++l) {
-                cudaStreamDestroy(S.lanes.s[l]);
-                cudaEventDestroy(S.lanes.join[l]);
-                cudaEventDestroy(S.lanes.cross[l]);
-            }
+            for (cudaStream_t s : S.lanes.s) cudaStreamDestroy(s);
+            for (cudaEvent_t e : S.lanes.cross) cudaEventDestroy(e);
             cudaEventDestroy(S.lanes.fork);
             S.lanes = State::BatchLanes();
         }
@@ -1360,6 +1357,18 @@ adapt_status_t run_plan(State& S, Plan* pl, const void* A, const void* B, void* 
     return fail(ADAPT_ERR_UNSUPPORTED, "unknown kernel family%s");
 }
 
+// Does adapt_matmul on these operands use the workspace of its stream?
+bool needs_workspace(const Plan* pl, const void* A, const void* B)
+{
+    if (pl->noop || pl->zero_fill) return false;
+    const Config& c = pl->c;
+    if (c.family == ADAPT_FAM_CLUSTER) return false;
+    if (c.P_k > 1 && !c.fused) return true;
+    if (c.family == ADAPT_FAM_SIMT || c.family == ADAPT_FAM_SKINNY) return false;
+    if (c.streamk || (((uintptr_t)A | (uintptr_t)B) & 15) != 0) return true;
+    return c.srcA == ADAPT_SRC_PAD_COPY || c.srcB != ADAPT_SRC_TMA || (c.srcA == ADAPT_SRC_TMA_CLASSES && class_tiles_copy_a(pl->s));
+}
+
 bool overlaps(const void* a, size_t an, const void* b, size_t bn)
 {
     const uintptr_t a0 = (uintptr_t)a, b0 = (uintptr_t)b;
@@ -1725,29 +1734,30 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
     }
     // Small calls (plans of the one-launch and CUDA-core families, as adapt_matmul_plan returned them) leave in grouped launches.
     auto grouped = [&](const Plan* pl) { return pl && pl->selected && !pl->noop && !pl->zero_fill && group_eligible(pl->s, pl->c); };
-    int64_t singles = 0;
-    for (int64_t i = 0; i < count; ++i) singles += grouped(plans[i]) ? 0 : 1;
-    // Lane 0 is the caller's stream, the others are internal streams between a fork from and a join to it, used from eight
-    // calls on and no more of them than there are launches to overlap.
-    const int NL = count < 8 ? 1 : (int)std::max<int64_t>(1, std::min<int64_t>(S.batch_lanes, singles + (singles < count ? 1 : 0)));
+    auto workspace = [&](int64_t i) { return plans[i] && needs_workspace(plans[i], A[i], B[i]); };
+    int64_t singles = 0, with_workspace = 0;
+    for (int64_t i = 0; i < count; ++i) {
+        if (grouped(plans[i])) continue;
+        ++singles;
+        with_workspace += workspace(i) ? 1 : 0;
+    }
+    // Lane 0 is the caller's stream, the others are internal streams between a fork from and a join to it.
+    const int NL = 1 + batch_internal_lanes(count, singles, with_workspace, S.batch_lanes);
     std::unique_lock<std::mutex> batch_lock(S.batch_mu, std::defer_lock);
     State::BatchLanes& L = S.lanes;
-    BatchOps ops = {S, plans, A, B, C, {user, nullptr, nullptr, nullptr}};
+    BatchOps ops = {S, plans, A, B, C, {user}};
     if (NL > 1) {
         batch_lock.lock();
         if (!L.ready) {
-            for (int l = 0; l < 4; ++l) {
-                CUDA_TRY(cudaStreamCreateWithFlags(&L.s[l], cudaStreamNonBlocking));
-                CUDA_TRY(cudaEventCreateWithFlags(&L.join[l], cudaEventDisableTiming));
-                CUDA_TRY(cudaEventCreateWithFlags(&L.cross[l], cudaEventDisableTiming));
-            }
+            for (cudaStream_t& s : L.s) CUDA_TRY(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+            for (cudaEvent_t& e : L.cross) CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
             CUDA_TRY(cudaEventCreateWithFlags(&L.fork, cudaEventDisableTiming));
             L.ready = true;
         }
         CUDA_TRY(cudaEventRecord(L.fork, user));
         for (int l = 1; l < NL; ++l) {
-            ops.stream[l] = L.s[l];
-            CUDA_TRY(cudaStreamWaitEvent(L.s[l], L.fork, 0));
+            ops.stream[l] = L.s[l - 1];
+            CUDA_TRY(cudaStreamWaitEvent(ops.stream[l], L.fork, 0));
         }
     }
     auto call_of = [&](int64_t i) -> BatchCall {
@@ -1762,6 +1772,7 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
         k.unsound = !A[i] || !B[i] || !C[i] || (((uintptr_t)A[i] | (uintptr_t)B[i] | (uintptr_t)C[i]) & 1) != 0 || (k.c.lo < k.a.hi && k.a.lo < k.c.hi) ||
                     (k.c.lo < k.b.hi && k.b.lo < k.c.hi);
         k.groupable = grouped(pl);
+        k.workspace = workspace(i);
         k.alone = pl->c.streamk != 0;
         k.us = pl->c.predicted_us;
         return k;
@@ -1769,7 +1780,7 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
     const adapt_status_t status = run_batch(count, NL, call_of, ops);
     // join, also after an error: the caller's stream continues after whatever was queued
     for (int l = 1; l < NL; ++l) {
-        if (cudaEventRecord(L.join[l], L.s[l]) == cudaSuccess) (void)cudaStreamWaitEvent(user, L.join[l], 0);
+        if (cudaEventRecord(L.cross[l], ops.stream[l]) == cudaSuccess) (void)cudaStreamWaitEvent(user, L.cross[l], 0);
     }
     return status;
 }

@@ -24,10 +24,21 @@ struct BatchCall {
     Range a, b, c;              // what it reads (A, B) and writes (C)
     bool unsound;               // null, misaligned or overlapping operands: most likely refused, so the calls before it leave first
     bool groupable;             // may join a grouped launch
+    bool workspace;             // needs the workspace of the stream it runs on
     bool alone;                 // nothing may run beside it (stream-K: its CTAs wait for one another and must all be resident)
     double us;                  // predicted time
 };
-constexpr int kBatchLanesMax = 4;
+constexpr int kBatchInternalMax = 4;                        // internal streams
+constexpr int kBatchLanesMax = 1 + kBatchInternalMax;       // ... and the caller's
+
+// Internal streams for a list of `count` calls of which `singles` are launched by themselves, `with_workspace` of them over a workspace:
+// none for a short list, else no more than `limit` and no more than there are launches to overlap (the caller's stream takes part).
+inline int batch_internal_lanes(int64_t count, int64_t singles, int64_t with_workspace, int limit)
+{
+    if (count < 8 || limit < 2) return 0;
+    const int64_t launches = singles + (singles < count ? 1 : 0);
+    return (int)std::max<int64_t>(0, std::min<int64_t>(std::min(limit, kBatchInternalMax), std::max(with_workspace, launches - 1)));
+}
 
 // The calls 0 .. count-1 of call_of(i), with the result of running them in that order.
 //
@@ -35,7 +46,9 @@ constexpr int kBatchLanesMax = 4;
 // collected, and another only launched past the collected ones, while none of its buffers meets theirs in a way that order would
 // matter.
 //
-// Lanes are streams that run beside each other.  A launch goes to the lane with the least predicted work queued, so that the
+// Lanes are streams that run beside each other; lane 0 is the caller's stream.  A call that needs a workspace goes to one of the others
+// where there are any: theirs are kept from list to list, whatever stream the caller names, so a list that has run once runs without
+// growing one on every stream, also in a capture on a stream that has not been used before.  A launch goes to the lane with the least predicted work queued, so that the
 // launch gaps and the tail of one call fill with the next call's work.  A launch whose output overlaps what another lane still reads
 // or writes, or whose inputs overlap what it writes, first waits for that lane; a lane remembers the buffers of its last 16 calls,
 // and when that memory is full all other lanes are made to wait for it.
@@ -47,12 +60,12 @@ adapt_status_t run_batch(int64_t count, int lanes, CallOf call_of, Ops& ops)
 {
     constexpr size_t kLaneMemory = 32;
     std::vector<Range> reads[kBatchLanesMax], writes[kBatchLanesMax];
-    double queued[kBatchLanesMax] = {0.0, 0.0, 0.0, 0.0};
+    double queued[kBatchLanesMax] = {};
 
     // Chooses the lane of a launch that reads and writes the given buffers and makes it wait for the lanes it depends on.
-    auto enter = [&](const Range* rd, size_t n_rd, const Range* wr, size_t n_wr, bool alone, int* out) -> adapt_status_t {
-        int lane = 0;
-        for (int l = 1; l < lanes; ++l) if (queued[l] < queued[lane]) lane = l;
+    auto enter = [&](const Range* rd, size_t n_rd, const Range* wr, size_t n_wr, bool alone, bool workspace, int* out) -> adapt_status_t {
+        int lane = workspace && lanes > 1 ? 1 : 0;
+        for (int l = lane + 1; l < lanes; ++l) if (queued[l] < queued[lane]) lane = l;
         *out = lane;
         for (int o = 0; o < lanes; ++o) {
             if (o == lane) continue;
@@ -85,7 +98,7 @@ adapt_status_t run_batch(int64_t count, int lanes, CallOf call_of, Ops& ops)
     auto flush = [&]() -> adapt_status_t {
         if (group.empty()) return ADAPT_OK;
         int lane = 0;
-        adapt_status_t r = enter(group_reads.data(), group_reads.size(), group_writes.data(), group_writes.size(), false, &lane);
+        adapt_status_t r = enter(group_reads.data(), group_reads.size(), group_writes.data(), group_writes.size(), false, false, &lane);
         if (r == ADAPT_OK) r = ops.group(group, lane);
         if (r == ADAPT_OK) leave(lane, group_reads.data(), group_reads.size(), group_writes.data(), group_writes.size(), group_us);
         group.clear();
@@ -110,7 +123,7 @@ adapt_status_t run_batch(int64_t count, int lanes, CallOf call_of, Ops& ops)
         }
         const Range rd[2] = {k.a, k.b};
         int lane = 0;
-        if ((status = enter(rd, 2, &k.c, 1, k.alone, &lane)) != ADAPT_OK) break;
+        if ((status = enter(rd, 2, &k.c, 1, k.alone, k.workspace, &lane)) != ADAPT_OK) break;
         if ((status = ops.single(i, lane)) != ADAPT_OK) break;
         leave(lane, rd, 2, &k.c, 1, k.us);
         if (k.alone)

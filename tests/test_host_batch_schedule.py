@@ -1,13 +1,12 @@
 """The order of the launches of a list, compiled on its own and run over random lists on simulated streams: two calls of which one writes
 what the other reads or writes are ordered as in the list, every call before a failing one is launched, and nothing runs beside a call
-that must be alone."""
+that must be alone, and a call that needs a workspace is kept off the caller's stream where there are others."""
 import os
 
 from test_host_group_plan import build_and_run
 
 PROGRAM = r"""
 #include <cstdio>
-#include <cstdlib>
 #include <random>
 #include "batch_schedule.h"
 using namespace adapt;
@@ -18,12 +17,13 @@ struct Ops {
     std::vector<std::vector<char>> lane;                // per lane: the calls that come before whatever it runs next
     std::vector<std::vector<char>> before;              // per launched call: the calls that come before it
     std::vector<int> launched;
-    int waits = 0, largest = 0;
+    int waits = 0, largest = 0, misplaced = 0;
     std::vector<BatchCall> call;
     void run(int64_t i, int l) { before[i] = lane[l]; ++launched[i]; }
     adapt_status_t single(int64_t i, int l)
     {
         if (i == failing) return ADAPT_ERR_NOMEM;
+        misplaced += call[i].workspace && lane.size() > 1 && l == 0;
         run(i, l);
         lane[l][i] = 1;
         return ADAPT_OK;
@@ -69,6 +69,7 @@ int main()
             k.alone = !k.groupable && pick(12) == 0;
             k.us = 1 + pick(20);
             k.unsound = pick(60) == 0;
+            k.workspace = !k.groupable && pick(2) == 0;
             if (i == failing && (!k.groupable || k.unsound)) o.failing = i;
             o.call.push_back(k);
         }
@@ -83,7 +84,7 @@ int main()
                 if (order) ok &= o.before[j][i] != 0, ++ordered;
                 if (x.alone || y.alone) ok &= o.before[j][i] || o.before[i][j];
             }
-        ok &= o.largest <= 8 * kGroupMax;
+        ok &= o.largest <= 8 * kGroupMax && o.misplaced == 0;
         waits += o.waits;
         grouped += o.largest > 1;
         failures += o.failing >= 0;
@@ -92,6 +93,16 @@ int main()
             return 1;
         }
     }
+    // internal streams: none for short lists or when switched off, never more than launches to overlap, one at least for any workspace
+    for (int64_t count = 2; count < 40; ++count)
+        for (int64_t singles = 0; singles <= count; ++singles)
+            for (int64_t ws = 0; ws <= singles; ++ws)
+                for (int limit = 1; limit <= 4; ++limit) {
+                    const int n = batch_internal_lanes(count, singles, ws, limit);
+                    const int64_t launches = singles + (singles < count);
+                    if (n < 0 || n > kBatchInternalMax || n > limit || (n > 0 && (count < 8 || limit < 2)) || n > std::max(ws, launches - 1) ||
+                        (count >= 8 && limit >= 2 && ws > 0 && n == 0)) return 2;
+                }
     printf("%ld waits, %ld lists with groups, %ld failing lists, %ld ordered pairs\n", waits, grouped, failures, ordered);
     return !(waits > 3000 && grouped > 1000 && failures > 150 && ordered > 10000);
 }
