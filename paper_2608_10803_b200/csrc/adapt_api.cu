@@ -602,14 +602,15 @@ static UmmaKernel umma_lookup_batch(int BN, bool a_mn, bool b_mn)
 }
 
 // fused split-K instantiations (1-CTA tiles; the k splits of a tile are one cluster)
+template <bool EPI>
 static UmmaKernel umma_lookup_fused(int BN, bool a_mn, bool b_mn)
 {
 #define ADAPT_PICK(bn)                                                                         \
     if (BN == bn) {                                                                            \
-        if (!a_mn && !b_mn) return (const void*)umma_gemm_kernel<bn, false, false, 1, 0, true>; \
-        if (!a_mn && b_mn) return (const void*)umma_gemm_kernel<bn, false, true, 1, 0, true>;   \
-        if (a_mn && !b_mn) return (const void*)umma_gemm_kernel<bn, true, false, 1, 0, true>;   \
-        return (const void*)umma_gemm_kernel<bn, true, true, 1, 0, true>;                       \
+        if (!a_mn && !b_mn) return (const void*)umma_gemm_kernel<bn, false, false, 1, 0, true, false, EPI>; \
+        if (!a_mn && b_mn) return (const void*)umma_gemm_kernel<bn, false, true, 1, 0, true, false, EPI>;   \
+        if (a_mn && !b_mn) return (const void*)umma_gemm_kernel<bn, true, false, 1, 0, true, false, EPI>;   \
+        return (const void*)umma_gemm_kernel<bn, true, true, 1, 0, true, false, EPI>;                       \
     }
     ADAPT_PICK(64)
     ADAPT_PICK(128)
@@ -669,22 +670,26 @@ static UmmaKernel launch_map_umma_plain(int family, int BN, bool a_mn, bool b_mn
     return family == ADAPT_FAM_UMMA_1CTA ? umma_lookup<1, EPI>(BN, a_mn, b_mn) : umma_lookup<2, EPI>(BN, a_mn, b_mn);
 }
 
-// epi: the instantiation that adds beta * D itself (fused kernels take it at run time; k classes as k splits have none)
-static UmmaKernel launch_map_umma(int family, int BN, bool a_mn, bool b_mn, int mode = 0, bool fused = false, bool epi = false)
+template <bool EPI>
+static UmmaKernel launch_map_umma_fused(int family, int BN, bool a_mn, bool b_mn, int mode)
 {
-    if (fused) {
-        if (family != ADAPT_FAM_UMMA_1CTA) return nullptr;
-        if (mode == 0) return umma_lookup_fused(BN, a_mn, b_mn);
-        if (mode == 1) {
-            if (BN == 64) return (const void*)umma_gemm_kernel<64, false, true, 1, 1, true>;
-            if (BN == 128) return (const void*)umma_gemm_kernel<128, false, true, 1, 1, true>;
-            if (BN == 256) return (const void*)umma_gemm_kernel<256, false, true, 1, 1, true>;
-            return nullptr;
-        }
-        if (BN == 128) return (const void*)umma_gemm_kernel<128, false, true, 1, 3, true>;
-        if (BN == 256) return (const void*)umma_gemm_kernel<256, false, true, 1, 3, true>;
+    if (family != ADAPT_FAM_UMMA_1CTA) return nullptr;
+    if (mode == 0) return umma_lookup_fused<EPI>(BN, a_mn, b_mn);
+    if (mode == 1) {
+        if (BN == 64) return (const void*)umma_gemm_kernel<64, false, true, 1, 1, true, false, EPI>;
+        if (BN == 128) return (const void*)umma_gemm_kernel<128, false, true, 1, 1, true, false, EPI>;
+        if (BN == 256) return (const void*)umma_gemm_kernel<256, false, true, 1, 1, true, false, EPI>;
         return nullptr;
     }
+    if (BN == 128) return (const void*)umma_gemm_kernel<128, false, true, 1, 3, true, false, EPI>;
+    if (BN == 256) return (const void*)umma_gemm_kernel<256, false, true, 1, 3, true, false, EPI>;
+    return nullptr;
+}
+
+// epi: the instantiation that adds beta * D itself (unfused k classes as k splits have none)
+static UmmaKernel launch_map_umma(int family, int BN, bool a_mn, bool b_mn, int mode = 0, bool fused = false, bool epi = false)
+{
+    if (fused) return epi ? launch_map_umma_fused<true>(family, BN, a_mn, b_mn, mode) : launch_map_umma_fused<false>(family, BN, a_mn, b_mn, mode);
     return epi ? launch_map_umma_plain<true>(family, BN, a_mn, b_mn, mode) : launch_map_umma_plain<false>(family, BN, a_mn, b_mn, mode);
 }
 
@@ -724,21 +729,10 @@ extern "C" adapt_status_t adapt_init(int device)
         for (int fam = ADAPT_FAM_UMMA_1CTA; fam <= ADAPT_FAM_UMMA_2CTA; ++fam)
             for (int mode = 0; mode < 3; ++mode)
                 for (int BN : {64, 128, 256, 80, 144, 208})
-                    for (int v = 0; v < (mode == 0 ? 4 : 1); ++v) {
-                        UmmaKernel k = launch_map_umma(fam, BN, (v & 1) != 0, mode != 0 || (v & 2) != 0, mode, false, epi != 0);
+                    for (int v = 0; v < (mode == 0 ? 8 : 2); ++v) {       // bit 0: fused; layouts of plain tiles
+                        UmmaKernel k = launch_map_umma(fam, BN, (v & 2) != 0, mode != 0 || (v & 4) != 0, mode, (v & 1) != 0, epi != 0);
                         if (k) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
                     }
-    for (int BN : {64, 128, 256}) {
-        for (int a = 0; a < 2; ++a)
-            for (int b = 0; b < 2; ++b)
-                CUDA_TRY(cudaFuncSetAttribute(launch_map_umma(ADAPT_FAM_UMMA_1CTA, BN, a != 0, b != 0, 0, true),
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
-        CUDA_TRY(cudaFuncSetAttribute(launch_map_umma(ADAPT_FAM_UMMA_1CTA, BN, false, true, 1, true),
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
-        if (BN != 64)
-            CUDA_TRY(cudaFuncSetAttribute(launch_map_umma(ADAPT_FAM_UMMA_1CTA, BN, false, true, 2, true),
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
-    }
     for (int fam = ADAPT_FAM_UMMA_1CTA; fam <= ADAPT_FAM_UMMA_2CTA; ++fam)
         for (int BN : {64, 128, 256})
             for (int a = 0; a < 2; ++a)
@@ -1314,7 +1308,7 @@ adapt_status_t run_simt(State& S, Plan* pl, const void* A, const void* B, void* 
     p.C = (unsigned short*)C;
     p.partial = (float*)ws;
     dim3 grid((unsigned)(ceil_div(s.M, 64) * ceil_div(s.N, 64)), (unsigned)P_k, 1);
-    CUDA_TRY(launch_pdl(simt_gemm_kernel, grid, dim3(256), 0, stream, (const unsigned short*)A, (const unsigned short*)B, p));
+    CUDA_TRY(launch_pdl(p.ep.D ? simt_gemm_kernel<true> : simt_gemm_kernel<false>, grid, dim3(256), 0, stream, (const unsigned short*)A, (const unsigned short*)B, p));
     S.launches.fetch_add(1, std::memory_order_relaxed);
     CUDA_TRY(cudaGetLastError());
     if (partials) return launch_reduce(S, (const float*)ws, C, s.M, s.N, P_k, s.dtype, stream, epi);
@@ -2052,7 +2046,7 @@ extern "C" adapt_status_t adapt_matmul_noalloc(int64_t M, int64_t N, int64_t K, 
     p.partial = scratch;
     const int64_t tiles = ceil_div(M, 64) * ceil_div(N, 64);
     dim3 grid((unsigned)tiles, (unsigned)pk, 1);
-    CUDA_TRY(launch_pdl(simt_gemm_kernel, grid, dim3(256), 0, stream, (const unsigned short*)A, (const unsigned short*)B, p));
+    CUDA_TRY(launch_pdl(simt_gemm_kernel<false>, grid, dim3(256), 0, stream, (const unsigned short*)A, (const unsigned short*)B, p));
     CUDA_TRY(cudaGetLastError());
     const int64_t work = M * (Np / 4);
     const int groups = reduce_groups(work, (int)pk, 148);

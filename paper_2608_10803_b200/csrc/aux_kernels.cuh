@@ -300,7 +300,9 @@ struct SimtParams {
 };
 
 // One 64 x 64 tile at (m0, n0), k split `split`; sA and sB are 16 x 68 floats of shared memory each.
+// EPI: beta * D is added here (an instantiation of its own: the test at run time made 1000 x 1000 x 4 without a D 6 % slower).
 typedef float SimtStage[16][64 + 4];
+template <bool EPI>
 __device__ __forceinline__ void simt_tile_body(const unsigned short* __restrict__ A, const unsigned short* __restrict__ B, const SimtParams& p,
                                                int m0, int n0, int split, SimtStage& sA, SimtStage& sB)
 {
@@ -374,18 +376,19 @@ __device__ __forceinline__ void simt_tile_body(const unsigned short* __restrict_
         for (int j = 0; j < 4; ++j) {
             const int n = n0 + tx * 4 + j;
             if (n >= p.N) continue;
-            if (p.P_k == 1) p.C[(int64_t)m * p.N + n] = float_to_16(fused_add(p.ep, acc[i][j], m, n, p.N, p.dtype), p.dtype);
+            if (p.P_k == 1) p.C[(int64_t)m * p.N + n] = float_to_16(EPI ? fused_add(p.ep, acc[i][j], m, n, p.N, p.dtype) : acc[i][j], p.dtype);
             else p.partial[((int64_t)split * p.M + m) * p.Np + n] = acc[i][j];
         }
     }
 }
 
+template <bool EPI>
 __global__ void __launch_bounds__(256)
 simt_gemm_kernel(const unsigned short* __restrict__ A, const unsigned short* __restrict__ B, const SimtParams p)
 {
     __shared__ SimtStage sA, sB;
     pdl_launch_dependents();
-    simt_tile_body(A, B, p, (int)(blockIdx.x / p.P_n) * 64, (int)(blockIdx.x % p.P_n) * 64, (int)blockIdx.y, sA, sB);
+    simt_tile_body<EPI>(A, B, p, (int)(blockIdx.x / p.P_n) * 64, (int)(blockIdx.x % p.P_n) * 64, (int)blockIdx.y, sA, sB);
 }
 
 // ---- measurement and self-test kernels ---------------------------------------------------------------

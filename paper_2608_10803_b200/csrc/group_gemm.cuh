@@ -51,7 +51,7 @@ group_gemm_kernel(const __grid_constant__ GroupParams p)
         q.Np = 0; q.dtype = BF16 ? 1 : 0; q.prefetch = 0;
         q.C = C; q.partial = nullptr; q.ep.D = nullptr;
         SimtStage* sm = reinterpret_cast<SimtStage*>(s_dyn);
-        simt_tile_body(A, B, q, m0, n0, 0, sm[0], sm[1]);
+        simt_tile_body<false>(A, B, q, m0, n0, 0, sm[0], sm[1]);
         return;
     }
     ClusterParams q;

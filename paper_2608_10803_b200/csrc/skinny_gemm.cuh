@@ -145,7 +145,8 @@ __device__ __forceinline__ void stage_small(const SkinnyParams& p, unsigned shor
 
 // KC: streamed operand k-contiguous.  BF16: element type.  ALIGNED: every 8-element group of the
 // streamed operand this kernel loads starts on a 16-byte boundary.
-template <bool KC, bool BF16, bool ALIGNED>
+// EPI: the kernel adds beta * D itself (an instantiation of its own: the test at run time made 16 x 4096 x 512 without a D 4 % slower).
+template <bool KC, bool BF16, bool ALIGNED, bool EPI>
 __global__ void __launch_bounds__(kSkinnyThreads, 2)
 skinny_gemm_kernel(const SkinnyParams p)
 {
@@ -255,7 +256,7 @@ skinny_gemm_kernel(const SkinnyParams p)
             for (int w = 0; w < WK; ++w) sum += s_out[(w * warps_r + w0) * (16 * 64) + s * 64 + rr];
             if (p.P_k == 1) {
                 // the streamed side is n or m
-                const float out = fused_add(p.ep, sum, p.n_streamed ? s : r, p.n_streamed ? r : s, p.N, BF16 ? 1 : 0);
+                const float out = EPI ? fused_add(p.ep, sum, p.n_streamed ? s : r, p.n_streamed ? r : s, p.N, BF16 ? 1 : 0) : sum;
                 p.C[(int64_t)s * p.out_ss + (int64_t)r * p.out_sr] = float_to_16(out, BF16 ? 1 : 0);
             } else {
                 p.partial[(int64_t)split * p.part_slab + (int64_t)s * p.part_ss + (int64_t)r * p.part_sr] = sum;
@@ -314,7 +315,7 @@ skinny_gemm_kernel(const SkinnyParams p)
                 const float sum = acc[0][i] + acc[1][i];
                 if (p.P_k == 1) {
                     // the streamed side is n or m
-                    const float out = fused_add(p.ep, sum, p.n_streamed ? s : rr, p.n_streamed ? rr : s, p.N, BF16 ? 1 : 0);
+                    const float out = EPI ? fused_add(p.ep, sum, p.n_streamed ? s : rr, p.n_streamed ? rr : s, p.N, BF16 ? 1 : 0) : sum;
                     p.C[(int64_t)s * p.out_ss + (int64_t)rr * p.out_sr] = float_to_16(out, BF16 ? 1 : 0);
                 } else {
                     p.partial[(int64_t)split * p.part_slab + (int64_t)s * p.part_ss + (int64_t)rr * p.part_sr] = sum;
@@ -326,11 +327,11 @@ skinny_gemm_kernel(const SkinnyParams p)
 
 typedef void (*SkinnyKernel)(const SkinnyParams);
 
-template <bool KC>
+template <bool KC, bool EPI>
 inline SkinnyKernel skinny_pick(bool bf16, bool aligned)
 {
-    if (bf16) return aligned ? skinny_gemm_kernel<KC, true, true> : skinny_gemm_kernel<KC, true, false>;
-    return aligned ? skinny_gemm_kernel<KC, false, true> : skinny_gemm_kernel<KC, false, false>;
+    if (bf16) return aligned ? skinny_gemm_kernel<KC, true, true, EPI> : skinny_gemm_kernel<KC, true, false, EPI>;
+    return aligned ? skinny_gemm_kernel<KC, false, true, EPI> : skinny_gemm_kernel<KC, false, false, EPI>;
 }
 
 // Host launcher: maps (M, N, K, layouts) onto the canonical form above.
@@ -377,7 +378,9 @@ inline adapt_status_t launch_skinny(const Shape& s, const Config& c, const void*
     // every group this kernel loads starts at Str + row * ld + (multiple of 8)
     const bool aligned = (p.ld % 8 == 0) && ((uintptr_t)p.Str % 16 == 0);
     dim3 grid((unsigned)ceil_div(p.R, p.BNs), (unsigned)c.P_k, 1);
-    SkinnyKernel k = kc ? skinny_pick<true>(s.dtype != 0, aligned) : skinny_pick<false>(s.dtype != 0, aligned);
+    const bool bf16 = s.dtype != 0;
+    SkinnyKernel k = p.ep.D ? (kc ? skinny_pick<true, true>(bf16, aligned) : skinny_pick<false, true>(bf16, aligned))
+                            : (kc ? skinny_pick<true, false>(bf16, aligned) : skinny_pick<false, false>(bf16, aligned));
     if (launch_pdl(k, grid, dim3(kSkinnyThreads, 1, 1), 0, stream, p) != cudaSuccess) return ADAPT_ERR_CUDA;
     return ADAPT_OK;
 }

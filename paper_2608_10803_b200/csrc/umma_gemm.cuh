@@ -317,7 +317,7 @@ __device__ __forceinline__ void epilogue_add(const ReduceEpilogue& e, uint32_t (
 // dimension is the entry.
 //
 // EPI: the kernel adds beta * D itself (instantiations of their own: the test alone, on top of the halo tiles' code, made
-// 20000 x 20001 x 12 without a D 5 % slower).  The fused reduction's output loop takes p.ep at run time.
+// 20000 x 20001 x 12 without a D 5 % slower, and the fused reduction's output loop 1 %: 512 x 1024 x 4096 on 128 columns 14.03 -> 14.22 us).
 template <int BN, bool A_MN, bool B_MN, int CG, int MODE, bool FUSE = false, bool SK = false, bool EPI = false>
 __global__ void __launch_bounds__(kUmmaThreads, 1)
 umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams p)
@@ -337,7 +337,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
     // units of the shifted rows instead of columns, so they compute 16 columns more than they own (see
     // the epilogue); they use 16 row classes, since rows 16 apart share their offset from such a boundary
     constexpr bool HALO = A_CLS && (BN % 64 != 0);
-    static_assert(!EPI || (!FUSE && !SK && MODE != 3), "kernels that store the 16-bit output from their own accumulator");
+    static_assert(!EPI || (!SK && (FUSE || MODE != 3)), "kernels that store the 16-bit output");
     static_assert(BN % 64 == 0 || (A_CLS && (BN - 16) % 64 == 0), "BN is a multiple of 64, plus 16 halo columns for class tiles");
     // row classes of a class tile (rows NCLS*128*g + j + NCLS*i): 8, or for halo tiles as many as C's rows need to share
     // their offset from a 32-byte boundary (16 for an odd N, 8, 4 or 2 for an even one: p.ncls_log2)
@@ -931,7 +931,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                         sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
                     }
                     const int n = n0 + 4 * g;
-                    if (p.ep.D) {
+                    if (EPI) {
                         const int m = row_base + row_step * rr;
                         sum.x = fused_add(p.ep, sum.x, m, n, p.N, p.dtype);
                         if (n + 1 < p.N) sum.y = fused_add(p.ep, sum.y, m, n + 1, p.N, p.dtype);
