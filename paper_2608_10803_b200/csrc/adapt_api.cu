@@ -1669,44 +1669,30 @@ struct BatchOps {
         CUDA_TRY(cudaStreamWaitEvent(stream[lane], S.lanes.cross[other], 0));
         return ADAPT_OK;
     }
-    // Independent calls: one launch per kGroupMax calls, data type and pair of layouts.
+    // Bit 0: dtype, 1: A row-major, 2: B column-major.
+    static int variant(const Shape& s)
+    {
+        return (s.dtype != 0 ? 1 : 0) | (s.layoutA == ADAPT_ROW_MAJOR ? 2 : 0) | (s.layoutB == ADAPT_COL_MAJOR ? 4 : 0);
+    }
     adapt_status_t group(const std::vector<int64_t>& calls, int lane)
     {
-        struct Entry { GroupItem item; int chain, variant; };
-        std::vector<Entry> entries;
+        struct Entry { GroupItem item; int chain; } entry[kGroupMax];
+        size_t n = 0;
         for (int64_t i : calls) {
-            const Shape& s = plans[i]->s;
-            Entry e;
-            e.chain = group_item(s, plans[i]->c, A[i], B[i], C[i], &e.item);
-            e.variant = (s.dtype != 0 ? 1 : 0) | (s.layoutA == ADAPT_ROW_MAJOR ? 2 : 0) | (s.layoutB == ADAPT_COL_MAJOR ? 4 : 0);
-            entries.push_back(e);
+            entry[n].chain = group_item(plans[i]->s, plans[i]->c, A[i], B[i], C[i], &entry[n].item);
+            ++n;
         }
         // longest chains first: what starts last is short
-        std::stable_sort(entries.begin(), entries.end(), [](const Entry& x, const Entry& y) { return x.chain > y.chain; });
+        std::stable_sort(entry, entry + n, [](const Entry& x, const Entry& y) { return x.chain > y.chain; });
+        const Shape& s = plans[calls[0]]->s;
         GroupParams p;
+        group_clear(p);
+        for (size_t j = 0; j < n; ++j) group_add(p, entry[j].item, entry[j].chain);
         p.prefetch = S.prefetch;
+        p.dtype = s.dtype;
         p.sa = p.sb = p.sc = 0;
-        for (int variant = 0; variant < 8; ++variant) {     // bit 0: dtype, 1: A row-major, 2: B column-major
-            group_clear(p);
-            auto launch = [&]() -> adapt_status_t {
-                if (p.count == 0) return ADAPT_OK;
-                p.dtype = variant & 1;
-                CUDA_TRY(launch_group(p, (variant & 2) != 0, (variant & 4) != 0, stream[lane]));
-                S.launches.fetch_add(1, std::memory_order_relaxed);
-                group_clear(p);
-                return ADAPT_OK;
-            };
-            for (const Entry& e : entries) {
-                if (e.variant != variant) continue;
-                group_add(p, e.item, e.chain);
-                if (p.count == kGroupMax) {
-                    const adapt_status_t r = launch();
-                    if (r != ADAPT_OK) return r;
-                }
-            }
-            const adapt_status_t r = launch();
-            if (r != ADAPT_OK) return r;
-        }
+        CUDA_TRY(launch_group(p, s.layoutA == ADAPT_ROW_MAJOR, s.layoutB == ADAPT_COL_MAJOR, stream[lane]));
+        S.launches.fetch_add(1, std::memory_order_relaxed);
         return ADAPT_OK;
     }
 };
@@ -1766,6 +1752,7 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
         k.unsound = !A[i] || !B[i] || !C[i] || (((uintptr_t)A[i] | (uintptr_t)B[i] | (uintptr_t)C[i]) & 1) != 0 || (k.c.lo < k.a.hi && k.a.lo < k.c.hi) ||
                     (k.c.lo < k.b.hi && k.b.lo < k.c.hi);
         k.groupable = grouped(pl);
+        k.variant = BatchOps::variant(s);
         k.workspace = workspace(i);
         k.alone = pl->c.streamk != 0;
         k.us = pl->c.predicted_us;

@@ -24,10 +24,12 @@ struct BatchCall {
     Range a, b, c;              // what it reads (A, B) and writes (C)
     bool unsound;               // null, misaligned or overlapping operands: most likely refused, so the calls before it leave first
     bool groupable;             // may join a grouped launch
+    int variant;                // ... of this data type and pair of layouts (0 .. kBatchVariants - 1)
     bool workspace;             // needs the workspace of the stream it runs on
     bool alone;                 // nothing may run beside it (stream-K: its CTAs wait for one another and must all be resident)
     double us;                  // predicted time
 };
+constexpr int kBatchVariants = 8;
 constexpr int kBatchInternalMax = 4;                        // internal streams
 constexpr int kBatchLanesMax = 1 + kBatchInternalMax;       // ... and the caller's
 
@@ -42,9 +44,9 @@ inline int batch_internal_lanes(int64_t count, int64_t singles, int64_t with_wor
 
 // The calls 0 .. count-1 of call_of(i), with the result of running them in that order.
 //
-// Groupable calls are collected and leave together in grouped launches; the others are launched as they come.  A call is only
-// collected, and another only launched past the collected ones, while none of its buffers meets theirs in a way that order would
-// matter.
+// Groupable calls are collected per variant, up to kGroupMax of one, and leave together in one grouped launch; the others are launched
+// as they come.  A call is only collected, and another only launched past the collected ones, while none of its buffers meets theirs
+// in a way that order would matter.
 //
 // Lanes are streams that run beside each other; lane 0 is the caller's stream.  A call that needs a workspace goes to one of the others
 // where there are any: theirs are kept from list to list, whatever stream the caller names, so a list that has run once runs without
@@ -53,7 +55,8 @@ inline int batch_internal_lanes(int64_t count, int64_t singles, int64_t with_wor
 // or writes, or whose inputs overlap what it writes, first waits for that lane; a lane remembers the buffers of its last 16 calls,
 // and when that memory is full all other lanes are made to wait for it.
 //
-// Ops: adapt_status_t single(int64_t i, int lane), group(const std::vector<int64_t>& calls, int lane), and wait(int lane, int other):
+// Ops: adapt_status_t single(int64_t i, int lane), group(const std::vector<int64_t>& calls, int lane) with calls of one variant, independent
+// of one another, and wait(int lane, int other):
 // `lane` continues after everything queued on `other`.
 template <class CallOf, class Ops>
 adapt_status_t run_batch(int64_t count, int lanes, CallOf call_of, Ops& ops)
@@ -92,33 +95,49 @@ adapt_status_t run_batch(int64_t count, int lanes, CallOf call_of, Ops& ops)
         writes[lane].insert(writes[lane].end(), wr, wr + n_wr);
     };
 
-    std::vector<int64_t> group;                         // the calls collected so far, independent of one another
-    std::vector<Range> group_reads, group_writes;
-    double group_us = 0.0;
-    auto flush = [&]() -> adapt_status_t {
-        if (group.empty()) return ADAPT_OK;
+    struct Pending {                                    // the calls of one variant collected so far; those of all variants are independent
+        std::vector<int64_t> calls;
+        std::vector<Range> reads, writes;
+        double us = 0.0;
+    } pending[kBatchVariants];
+    auto flush = [&](Pending& g) -> adapt_status_t {
+        if (g.calls.empty()) return ADAPT_OK;
         int lane = 0;
-        adapt_status_t r = enter(group_reads.data(), group_reads.size(), group_writes.data(), group_writes.size(), false, false, &lane);
-        if (r == ADAPT_OK) r = ops.group(group, lane);
-        if (r == ADAPT_OK) leave(lane, group_reads.data(), group_reads.size(), group_writes.data(), group_writes.size(), group_us);
-        group.clear();
-        group_reads.clear();
-        group_writes.clear();
-        group_us = 0.0;
+        adapt_status_t r = enter(g.reads.data(), g.reads.size(), g.writes.data(), g.writes.size(), false, false, &lane);
+        if (r == ADAPT_OK) r = ops.group(g.calls, lane);
+        if (r == ADAPT_OK) leave(lane, g.reads.data(), g.reads.size(), g.writes.data(), g.writes.size(), g.us);
+        g.calls.clear();
+        g.reads.clear();
+        g.writes.clear();
+        g.us = 0.0;
         return r;
+    };
+    auto flush_all = [&]() -> adapt_status_t {          // every variant leaves, also after one that failed; the first error
+        adapt_status_t first = ADAPT_OK;
+        for (Pending& g : pending) {
+            const adapt_status_t r = flush(g);
+            if (first == ADAPT_OK) first = r;
+        }
+        return first;
+    };
+    auto meets_pending = [&](const BatchCall& k) -> bool {
+        for (const Pending& g : pending)
+            if (!g.calls.empty() && (hits(g.writes, k.a) || hits(g.writes, k.b) || hits(g.writes, k.c) || hits(g.reads, k.c))) return true;
+        return false;
     };
 
     adapt_status_t status = ADAPT_OK;
     for (int64_t i = 0; i < count && status == ADAPT_OK; ++i) {
         const BatchCall k = call_of(i);
-        if ((k.unsound || hits(group_writes, k.a) || hits(group_writes, k.b) || hits(group_writes, k.c) || hits(group_reads, k.c)) && (status = flush()) != ADAPT_OK) break;
+        if ((k.unsound || meets_pending(k)) && (status = flush_all()) != ADAPT_OK) break;
         if (k.groupable && !k.unsound) {
-            group.push_back(i);
-            group_reads.push_back(k.a);
-            group_reads.push_back(k.b);
-            group_writes.push_back(k.c);
-            group_us += 0.25 * k.us;
-            if (group.size() >= kGroupMax) status = flush();
+            Pending& g = pending[k.variant];
+            g.calls.push_back(i);
+            g.reads.push_back(k.a);
+            g.reads.push_back(k.b);
+            g.writes.push_back(k.c);
+            g.us += 0.25 * k.us;
+            if (g.calls.size() >= kGroupMax) status = flush(g);
             continue;
         }
         const Range rd[2] = {k.a, k.b};
@@ -131,7 +150,7 @@ adapt_status_t run_batch(int64_t count, int lanes, CallOf call_of, Ops& ops)
                 if (o != lane) status = ops.wait(o, lane);
     }
     // the calls still collected come before the one that failed: they leave in any case, and the first error is the result
-    const adapt_status_t r = flush();
+    const adapt_status_t r = flush_all();
     return status != ADAPT_OK ? status : r;
 }
 

@@ -231,3 +231,22 @@ def test_strided_batch_of_a_chosen_plan_rounds_once_and_repeats(shape, dtype):
     bound = half_ulp * want.abs() + (K * 2.0 ** -23) * 1.01 * scale + 2.0 ** -25
     for got in (one, many):
         assert bool(((got.view(batch, M, N).double() - want).abs() <= bound).all())
+
+
+def test_alternating_types_and_layouts_fill_their_launches():
+    """Calls of four variants in turn: one launch per 64 calls of a variant."""
+    init()
+    M, N, K = 24, 40, 56
+    variants = [(ab.F16, 0, 0), (ab.BF16, 0, 0), (ab.F16, 0, 1), (ab.BF16, 1, 0)]
+    plans = [ab.adapt_matmul_plan(M, N, K, *v) for v in variants]
+    X = [[synth.draw_operand(r, c, ("integer", -4, 4), 40 + j, v[0], "cuda") for j, (r, c) in enumerate(((M, K), (K, N)))] for v in variants]
+    C = torch.zeros((512, M, N), dtype=torch.float16, device="cuda")
+    before = ab.adapt_launch_count()
+    ab.adapt_matmul_batch([plans[i % 4] for i in range(512)], *([X[i % 4][j].data_ptr() for i in range(512)] for j in (0, 1)),
+                          [C[i].data_ptr() for i in range(512)], stream())
+    torch.cuda.synchronize()
+    assert ab.adapt_launch_count() - before == 8
+    for i in (0, 1, 2, 3, 255, 510, 511):
+        dt, lA, lB = variants[i % 4]
+        _, want = og.gemm(synth.bits(X[i % 4][0]).reshape(-1), synth.bits(X[i % 4][1]).reshape(-1), M, N, K, dt, lA, lB)
+        assert np.array_equal(C[i].view(torch.int16).cpu().numpy().view(np.uint16).reshape(want.shape), want), i

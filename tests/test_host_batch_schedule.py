@@ -17,7 +17,7 @@ struct Ops {
     std::vector<std::vector<char>> lane;                // per lane: the calls that come before whatever it runs next
     std::vector<std::vector<char>> before;              // per launched call: the calls that come before it
     std::vector<int> launched;
-    int waits = 0, largest = 0, misplaced = 0;
+    int waits = 0, largest = 0, misplaced = 0, groups = 0, mixed = 0;
     std::vector<BatchCall> call;
     void run(int64_t i, int l) { before[i] = lane[l]; ++launched[i]; }
     adapt_status_t single(int64_t i, int l)
@@ -31,6 +31,8 @@ struct Ops {
     adapt_status_t group(const std::vector<int64_t>& calls, int l)
     {
         largest = std::max<int>(largest, (int)calls.size());
+        ++groups;
+        for (int64_t i : calls) mixed += call[i].variant != call[calls[0]].variant;
         for (int64_t i : calls) run(i, l);
         for (int64_t i : calls) lane[l][i] = 1;
         return ADAPT_OK;
@@ -52,7 +54,7 @@ int main()
     long waits = 0, grouped = 0, failures = 0, ordered = 0;
     for (int trial = 0; trial < 2000; ++trial) {
         const int count = 1 + pick(trial % 3 ? 40 : 200), lanes = 1 + pick(kBatchLanesMax), buffers = 8 + pick(trial % 5 ? 30 : 600);
-        const int small = pick(101), failing = pick(3) ? -1 : pick(count);
+        const int small = pick(101), variants = 1 + pick(kBatchVariants), failing = pick(3) ? -1 : pick(count);
         Ops o;
         o.count = count;
         o.failing = -1;
@@ -66,6 +68,7 @@ int main()
             k.b = range();
             do k.c = range(); while (meet(k.c, k.a) || meet(k.c, k.b));
             k.groupable = pick(100) < small;
+            k.variant = pick(variants);
             k.alone = !k.groupable && pick(12) == 0;
             k.us = 1 + pick(20);
             k.unsound = pick(60) == 0;
@@ -84,12 +87,34 @@ int main()
                 if (order) ok &= o.before[j][i] != 0, ++ordered;
                 if (x.alone || y.alone) ok &= o.before[j][i] || o.before[i][j];
             }
-        ok &= o.largest <= 8 * kGroupMax && o.misplaced == 0;
+        ok &= o.largest <= kGroupMax && o.misplaced == 0 && o.mixed == 0;
         waits += o.waits;
         grouped += o.largest > 1;
         failures += o.failing >= 0;
         if (!ok) {
             printf("trial %d: %d calls on %d lanes, failing %lld, status %d\n", trial, count, lanes, (long long)o.failing, (int)status);
+            return 1;
+        }
+    }
+    // calls that do not depend on one another: one launch per kGroupMax of a variant, however the variants alternate
+    for (int variants = 1; variants <= kBatchVariants; ++variants) {
+        const int count = 3 * kGroupMax * variants - 1;
+        Ops o;
+        o.count = count;
+        o.failing = -1;
+        o.lane.assign(2, std::vector<char>(count, 0));
+        o.before.resize(count);
+        o.launched.assign(count, 0);
+        for (int i = 0; i < count; ++i) {
+            BatchCall k = {};
+            const uintptr_t at = 64 * (1 + i);
+            k.a = {at, at + 8}; k.b = {at + 8, at + 16}; k.c = {at + 16, at + 24};
+            k.groupable = true;
+            k.variant = i % variants;
+            o.call.push_back(k);
+        }
+        if (run_batch(count, 2, [&](int64_t i) { return o.call[i]; }, o) != ADAPT_OK || o.groups != 3 * variants) {
+            printf("%d calls of %d variants left in %d launches\n", count, variants, o.groups);
             return 1;
         }
     }
