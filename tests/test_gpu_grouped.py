@@ -250,3 +250,28 @@ def test_alternating_types_and_layouts_fill_their_launches():
         dt, lA, lB = variants[i % 4]
         _, want = og.gemm(synth.bits(X[i % 4][0]).reshape(-1), synth.bits(X[i % 4][1]).reshape(-1), M, N, K, dt, lA, lB)
         assert np.array_equal(C[i].view(torch.int16).cpu().numpy().view(np.uint16).reshape(want.shape), want), i
+
+
+@pytest.mark.parametrize("dtype", [ab.F16, ab.BF16])
+@pytest.mark.parametrize("shape", [(65, 33, 70), (17, 130, 63), (100, 64, 8), (64, 200, 400), (130, 264, 328)])
+def test_special_values_stay_in_their_rows_columns_and_entries(shape, dtype):
+    """Infinities and NaN at the ends of rows and k ranges, in lists and strided batches, aligned and not: only the outputs that they
+    belong to are touched, and those as the arithmetic gives them."""
+    M, N, K = shape
+    init()
+    batch = 24
+    A, B = (synth.draw_operand(batch * r, c, ("integer", 1, 3), seed, dtype, "cuda").view(batch, r, c) for r, c, seed in ((M, K, 81), (K, N, 82)))
+    for e in range(0, batch, 3):
+        A[e, M - 1, K - 1], A[e, 0, 0], B[e, K - 1, N - 1], A[e, 5, K // 2] = float("inf"), float("-inf"), float("inf"), float("nan")
+    want = torch.bmm(A.double(), B.double()).to(A.dtype)                # small integers: exact before the one rounding
+    plan = ab.adapt_matmul_plan(M, N, K, dtype)
+    for offset in (0, 1):
+        a, b = (torch.empty(x.numel() + offset, dtype=A.dtype, device="cuda")[offset:].copy_(x.reshape(-1)) for x in (A, B))
+        listed, strided = (torch.full((batch, M, N), 7.0, dtype=A.dtype, device="cuda") for _ in range(2))
+        ab.adapt_matmul_batch([plan] * batch, [a.data_ptr() + 2 * e * M * K for e in range(batch)], [b.data_ptr() + 2 * e * K * N for e in range(batch)],
+                              [listed[e].data_ptr() for e in range(batch)], stream())
+        ab.adapt_matmul_strided_batch(plan, a.data_ptr(), M * K, b.data_ptr(), K * N, strided.data_ptr(), M * N, batch, stream())
+        torch.cuda.synchronize()
+        ab.adapt_poll_device_status(stream())
+        for got in (listed, strided):
+            assert torch.equal(torch.isnan(got), torch.isnan(want)) and torch.equal(torch.where(torch.isnan(got), 0.0, got.float()), torch.where(torch.isnan(want), 0.0, want.float()))
