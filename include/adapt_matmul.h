@@ -260,7 +260,7 @@ adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t* plans, co
  * added can differ from adapt_matmul's on that entry and depends on the batch count, the strides and the alignment of the pointers (the
  * same call gives the same bits every time).  A plan whose configuration was asked for (adapt_matmul_plan_forced, or a plan-table
  * line that is not what the library would choose) keeps that configuration, and every entry has the bits of adapt_matmul.  Unaligned
- * operands may be copied through the stream's workspace, 64 MB of entries at a time; where that workspace cannot be had the batch runs
+ * operands may be copied through the stream's workspace, 256 MB of entries at a time; where that workspace cannot be had the batch runs
  * without the copies.  Launches on the tensor-core kernel encode two or three tensor maps per call. */
 adapt_status_t adapt_addmm(adapt_handle_t plan, const void* A, const void* B, const void* D, int d_is_vector,
                            float alpha, float beta, void* C, void* cuda_stream);

@@ -49,7 +49,7 @@ int main()
         if (!ok && bad++ < 10) printf("trial %d: %lld x %lld x %lld, %lld entries: kind %d, %lld at a time\n", trial, (long long)s.M, (long long)s.N, (long long)s.K, (long long)batch, r.kind, (long long)r.chunk);
     }
     printf("%d on the tensor-core kernel (%d in several launches), %d grouped, %d entry by entry\n", tensor, several, grouped, loops);
-    return bad || tensor < 300 || several < 50 || grouped < 20;
+    return bad || tensor < 300 || several < 30 || grouped < 20;
 }
 """
 
