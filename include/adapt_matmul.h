@@ -105,7 +105,8 @@ typedef struct adapt_plan_info_s {
     int32_t taxonomy_class;   /* adapt_class_t */
     int32_t family;           /* adapt_family_t */
     int32_t BM, BN, BK;       /* CTA (or CTA-pair) tile: the paper's m1, n1, k1 */
-    int32_t stages;           /* depth of the shared-memory ring (Multi-Buffer / Preloading depth) */
+    int32_t stages;           /* depth of the shared-memory ring (Multi-Buffer / Preloading depth); one-launch family with one CTA per tile
+                                 and K > 64: of the ring that each of the tile's two groups of warps has */
     int32_t P_m, P_n, P_k;    /* task counts along M, N, K (Table 1) */
     int32_t cluster;          /* CTAs per cluster (2 for the 2-CTA family) */
     int32_t srcA, srcB;       /* adapt_source_t */

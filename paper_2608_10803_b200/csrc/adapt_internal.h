@@ -92,10 +92,12 @@ struct Calib {
     double skinny_pass_us = 4.4;        // one 64-row pass over one staged chunk when the streamed rows are k-contiguous
     double skinny_step_unaligned_us = 2.52;   // one 16-k step of a warp when the streamed rows are unaligned
     double skinny_mac_rate = 30e12;     // MAC/s ceiling of the warp-level kernel (small side padded to 16)
-    // one-launch cluster kernel (64 x 64 tiles, k split over a cluster); least-squares fit over 180 timed
-    // configurations of 2,000-sweep shapes: 3.7 + 0.95 stages + 0.8 (cluster > 1) + crowd (1.6 + 0.44 stages) us
-    double cluster_fixed_us = 0.75;     // beyond the launch: barrier set-up, first trip to memory, rounding and store of the tile
-    double cluster_stage_us = 0.76;     // one 64-k stage: copy issue, shift pass, MMAs, each behind a CTA-wide barrier
+    // one-launch cluster kernel (64 x 64 tiles, k split over a cluster): fitted on timed configurations of the kernel as it was when every
+    // stage had an mbarrier and a shift pass of its own.  It has become faster since (64 x 64 x 1024 by one CTA 19.0 -> 9.6 us,
+    // 256^3 4.9 -> 4.4), so these constants overstate it: a small problem whose best tcgen05 plan is predicted a few per cent
+    // faster may be better off here
+    double cluster_fixed_us = 0.75;     // beyond the launch: first trip to memory, rounding and store of the tile
+    double cluster_stage_us = 0.76;     // one 64-k stage
     double cluster_reduce_us = 1.1;     // cluster barriers + reading the partial tiles of the peers
     double cluster_crowd_us = 1.25, cluster_crowd_stage_us = 0.44;   // per CTA per SM beyond one per two SMs
     double cluster_wave_us = 5.5;       // each further round of clusters
@@ -222,6 +224,9 @@ inline int cluster_smem_bytes(int ring) { return ring * kClusterStageBytes; }
 constexpr int kClusterSeqRing = 3;
 inline int cluster_seq_ring(int chain) { return std::max(1, std::min(kClusterSeqRing, chain)); }
 inline int cluster_seq_smem_bytes(int ring) { return 2 * ring * kClusterStageBytes; }
+// ... which is how a plan without pieces is launched from K = 65 on, the groups taking alternate stages.
+inline bool cluster_two_groups(int64_t K, int cluster) { return cluster == 1 && K > kClusterKS; }
+inline int cluster_alone_ring(int64_t K) { return cluster_seq_ring((int)std::min<int64_t>(kClusterSeqRing, (K + 2 * kClusterKS - 1) / (2 * kClusterKS))); }
 // Clusters of a size the machine runs at a time with one CTA per SM (a cluster is placed inside one GPC, so
 // the larger sizes leave SMs unused): what cudaOccupancyMaxActiveClusters reports on a B200 for this kernel
 // with its deepest ring (148, 74, 33, 15, 7), scaled to other SM counts.  With two CTAs per SM (rings of up

@@ -570,7 +570,7 @@ static bool legal_cluster(const Shape& s, const Machine& m, Config& c)
     if ((int64_t)c.P_m * c.P_n * c.cluster > 2 * (int64_t)m.n_sm) return false;
     if (c.stages != cluster_ring(s.K, c.cluster, (int64_t)c.P_m * c.P_n, m.n_sm)) return false;
     c.persistent = 0;
-    c.smem_bytes = cluster_smem_bytes(c.stages);
+    c.smem_bytes = cluster_two_groups(s.K, c.cluster) ? cluster_seq_smem_bytes(cluster_alone_ring(s.K)) : cluster_smem_bytes(c.stages);
     return true;
 }
 
@@ -830,7 +830,9 @@ void fill_info(const Shape& s, const Config& c, adapt_plan_info_t* o)
     o->M = s.M; o->N = s.N; o->K = s.K;
     o->dtype = s.dtype; o->layoutA = s.layoutA; o->layoutB = s.layoutB;
     o->taxonomy_class = c.cls; o->family = c.family;
-    o->BM = c.BM; o->BN = c.BN; o->BK = c.BK; o->stages = c.stages;
+    o->BM = c.BM; o->BN = c.BN; o->BK = c.BK;
+    // (the key keeps the depth of the cluster form; a tile that one CTA computes alone is launched with another ring)
+    o->stages = c.family == ADAPT_FAM_CLUSTER && cluster_two_groups(s.K, c.cluster) ? cluster_alone_ring(s.K) : c.stages;
     o->P_m = c.P_m; o->P_n = c.P_n; o->P_k = c.P_k; o->cluster = c.cluster;
     o->srcA = c.srcA; o->srcB = c.srcB; o->grid = c.grid; o->fused = c.fused; o->streamk = c.streamk; o->reserved = 0;
     o->workspace_bytes = c.workspace_bytes;

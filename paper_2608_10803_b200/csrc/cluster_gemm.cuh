@@ -22,8 +22,8 @@
 //
 // What bounds it: the dependent chain of a stage (wait, shift, barrier, ldmatrix, MMAs), and for many tiles the shared-memory
 // port (copy in, shift, ldmatrix).  Per-thread copy groups and no shifted stages beside the raw ones, against an mbarrier per
-// stage that every thread's copies arrived on and a separate shifted buffer: 256 x 256 x 256 (CS = 4) 5.4 -> 4.6 us; two groups
-// of warps against eight warps on one stage: 64 x 64 x 1024 by one CTA 12.7 -> 9.6 us.
+// stage that every thread's copies arrived on and a separate shifted buffer: 256 x 256 x 256 (CS = 4) 4.92 -> 4.38 us, 64 x 1024 x 1024
+// 7.45 -> 6.02 us; with two groups of warps in place of eight warps on one stage as well, 64 x 64 x 1024 by one CTA 19.0 -> 9.6 us.
 #pragma once
 
 #include <cstdint>
@@ -506,8 +506,8 @@ inline adapt_status_t launch_cluster(const Shape& s, const Config& c, const void
     p.P_n = c.P_n;
     p.CS = c.cluster;
     p.k_per_cta = (int)round_up(ceil_div(s.K, c.cluster), 16);
-    const bool seq = c.cluster == 1 && s.K > kClusterKS;
-    p.ring = seq ? cluster_seq_ring((int)ceil_div(s.K, 2 * kClusterKS)) : c.stages;
+    const bool seq = cluster_two_groups(s.K, c.cluster);
+    p.ring = seq ? cluster_alone_ring(s.K) : c.stages;
     p.prefetch = prefetch;
     p.aligned = (rows_aligned16(A, p.lda) ? 1 : 0) | (rows_aligned16(B, p.ldb) ? 2 : 0);
     p.ep = epi ? *epi : no_epilogue();

@@ -209,6 +209,15 @@ def test_cluster_family_is_offered_for_small_grids_only_and_its_key_round_trips(
     assert pick.family == ab.FAM_CLUSTER and pick.workspace_bytes == 0
 
 
+def test_ring_of_a_tile_without_pieces_is_reported_as_launched():
+    """Two groups of warps take alternate stages of 64 k values from K = 65 on, with up to three stages each; the key stays loadable."""
+    for K in (1, 64, 65, 128, 129, 256, 300, 384, 385, 1000, 5000):
+        c = next(c for c in ab.adapt_plan_candidates(70, 90, K, ab.F16) if c.family == ab.FAM_CLUSTER and c.cluster == 1)
+        assert c.stages == (1 if K <= 64 else min(3, -(-K // 128))), K
+        forced = ab.adapt_plan_info(ab.adapt_matmul_plan_forced(70, 90, K, ab.F16, ab.ROW_MAJOR, ab.ROW_MAJOR, c.tiling_key))
+        assert (forced.tiling_key, forced.stages) == (c.tiling_key, c.stages)
+
+
 def test_split_k_is_chosen_for_small_mn_large_k_and_not_for_large_mn():
     small = ab.adapt_plan_info(ab.adapt_matmul_plan(256, 256, 262144, ab.BF16))
     assert small.P_k > 1 and small.taxonomy_class in (2, 3)
