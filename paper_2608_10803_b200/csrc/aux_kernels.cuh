@@ -217,7 +217,7 @@ regroup_a_kernel(const unsigned short* __restrict__ A, unsigned short* __restric
 // A small output with many splits leaves most of the chip idle while each thread walks its splits batch by batch (one trip to L2
 // per eight): there the splits are shared by `groups` threads (a power of two), each adding a run of consecutive splits in
 // ascending order; the runs' sums are then added in ascending order too.  The order depends on the shape only.
-// (256 x 256 x 262144, P_k = 64: eight batches 59.5 us for the call, one batch 55.2 us; 34 x 21 x 34323: 16.5 and 11.4 us.)
+// (256 x 256 x 262144, P_k = 64: eight batches 67.7 us for the call, one batch 63.1 us; 34 x 21 x 34323: 17.3 and 11.6 us.)
 __global__ void __launch_bounds__(256)
 splitk_reduce_kernel(const float* __restrict__ partial, unsigned short* __restrict__ C,
                      int M, int N, int Np, int P_k, int dtype, const ReduceEpilogue ep, int groups)

@@ -1,12 +1,12 @@
 // Many small GEMMs in ONE launch: the lists of adapt_matmul_batch and the entries of adapt_matmul_strided_batch.
 //
 // A GEMM of a few microseconds is mostly launch, first trip to memory and drain; one launch each leaves the chip idle
-// between them (48 layers of 16 .. 1024 a side: 97 us on four streams, two microseconds a call, for 16 MB of operands).
+// between them (48 layers of 16 .. 1024 a side: 108 us on four streams, two microseconds a call, for 16 MB of operands).
 // Here the 64 x 64 tiles of all entries run side by side, one per CTA.  An entry keeps the arithmetic of its own plan:
 //   pieces > 0: the one-launch cluster kernel's tiles.  The CTA walks the plan's pieces of the k range and adds
 //               their sums in the same order: the bits of the call made alone, where each piece has a CTA of its own.
-//               (Clusters of four CTAs with the pieces spread over them took 53 us for those 48 layers, one CTA per tile 40 us:
-//               the exchange of the partial tiles cost more than the shorter chains saved.)
+//               (With a tile of one group of warps, clusters of four CTAs with the pieces spread over them took 53 us for those
+//               48 layers, one CTA per tile 40 us: the exchange of the partial tiles cost more than the shorter chains saved.)
 //   pieces = 0: the CUDA-core kernel's tiles (a few 16-k steps).
 // The list travels in the kernel's parameters, so nothing is copied to the device and the launch can be captured.
 #pragma once
@@ -17,12 +17,12 @@
 
 namespace adapt {
 
-// What bounds it: for a list with a deep entry the chain of that entry's stages (0.33 us per aligned 64 k values and group of
-// warps, 0.6 off 16-byte boundaries), else the shared-memory port.  The deepest entries come first and the ring is no deeper
-// than the list needs.  48 layers of 16 .. 1024 a side: 97 us one launch each on four streams, 31 us (21 us without the one
-// layer that keeps a launch of its own); 96 products of 128 x 128 x 64: 266 us one launch each, 4.4 us.
+// What bounds it: latency with two CTAs per SM.  Those 48 layers take 31.0 us, 21.7 for the 47 that share the launch and 8.7 for the one
+// with a launch of its own (each by itself); the 762 tiles are 2.6 rounds of CTAs whose longest chain is 8 stages (0.33 us per aligned 64 k
+// values and group of warps, 0.6 off 16-byte boundaries).  Profiled: 13.7 warps per SM (128 registers a thread), issue slots 35 % used,
+// stalls on fixed latencies and shared memory, DRAM 4 %.  The deepest entries come first and the ring is no deeper than the list needs.
 // SHORT: every item has K <= 64 in one piece (one stage): no two-group tiles, so fewer registers and three CTAs per SM instead of two
-// (96 products of 128 x 128 x 64: 6.6 us with the general kernel, 4.4 with this one).
+// (96 products of 128 x 128 x 64 in one launch: 6.6 us with the general kernel, 4.4 with this one, 266 as 96 launches).
 template <bool A_KC, bool B_KC, bool BF16, bool SHORT>
 __global__ void __launch_bounds__(kClusterThreads, SHORT ? 3 : 2)
 group_gemm_kernel(const __grid_constant__ GroupParams p)
