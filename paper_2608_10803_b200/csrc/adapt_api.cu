@@ -1055,7 +1055,7 @@ adapt_status_t launch_reduce(State& S, const float* partial, void* C, int64_t M,
     const int64_t work = M * (Np / 4);
     const int groups = reduce_groups(work, P_k, S.machine.n_sm);
     const int blocks = (int)std::min<int64_t>(ceil_div(work, 256 / groups), (int64_t)S.machine.n_sm * 8);
-    CUDA_TRY(launch_pdl(splitk_reduce_kernel, dim3(blocks), dim3(256), 0, stream, (const float*)partial, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)P_k, (int)dtype, ep, groups));
+    CUDA_TRY(launch_pdl(groups > 1 ? splitk_reduce_kernel<true> : splitk_reduce_kernel<false>, dim3(blocks), dim3(256), 0, stream, (const float*)partial, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)P_k, (int)dtype, ep, groups));
     S.launches.fetch_add(1, std::memory_order_relaxed);
     CUDA_TRY(cudaGetLastError());
     return ADAPT_OK;
@@ -2038,7 +2038,7 @@ extern "C" adapt_status_t adapt_matmul_noalloc(int64_t M, int64_t N, int64_t K, 
     const int64_t work = M * (Np / 4);
     const int groups = reduce_groups(work, (int)pk, 148);
     const int blocks = (int)std::min<int64_t>(ceil_div(work, 256 / groups), 148 * 8);
-    CUDA_TRY(launch_pdl(splitk_reduce_kernel, dim3(blocks), dim3(256), 0, stream, (const float*)scratch, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)pk, (int)dtype, no_epilogue(), groups));
+    CUDA_TRY(launch_pdl(groups > 1 ? splitk_reduce_kernel<true> : splitk_reduce_kernel<false>, dim3(blocks), dim3(256), 0, stream, (const float*)scratch, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)pk, (int)dtype, no_epilogue(), groups));
     CUDA_TRY(cudaGetLastError());
     st().launches.fetch_add(2, std::memory_order_relaxed);
     return ADAPT_OK;

@@ -218,11 +218,14 @@ regroup_a_kernel(const unsigned short* __restrict__ A, unsigned short* __restric
 // per eight): there the splits are shared by `groups` threads (a power of two), each adding a run of consecutive splits in
 // ascending order; the runs' sums are then added in ascending order too.  The order depends on the shape only.
 // (256 x 256 x 262144, P_k = 64: eight batches 67.7 us for the call, one batch 63.1 us; 34 x 21 x 34323: 17.3 and 11.6 us.)
+// SHARED: groups > 1 (the other outputs are not charged for it: 365 x 3136 x 4672 in three splits 23.1 us, 23.6 with the one kernel).
+template <bool SHARED>
 __global__ void __launch_bounds__(256)
 splitk_reduce_kernel(const float* __restrict__ partial, unsigned short* __restrict__ C,
-                     int M, int N, int Np, int P_k, int dtype, const ReduceEpilogue ep, int groups)
+                     int M, int N, int Np, int P_k, int dtype, const ReduceEpilogue ep, int groups_shared)
 {
-    __shared__ float4 s_sum[256];
+    __shared__ float4 s_sum[SHARED ? 256 : 1];
+    const int groups = SHARED ? groups_shared : 1;
     pdl_launch_dependents();
     pdl_wait();
     const int quads = Np >> 2;                              // columns in fours
@@ -249,7 +252,7 @@ splitk_reduce_kernel(const float* __restrict__ partial, unsigned short* __restri
                     if (p0 + j < p_end) { acc.x += v[j].x; acc.y += v[j].y; acc.z += v[j].z; acc.w += v[j].w; }
             }
         }
-        if (groups > 1) {
+        if (SHARED) {
             __syncthreads();                                // the sums of the step before have been read
             s_sum[threadIdx.x] = acc;
             __syncthreads();
