@@ -1317,7 +1317,7 @@ adapt_status_t run_simt(State& S, Plan* pl, const void* A, const void* B, void* 
 
 adapt_status_t run_cluster(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi = nullptr)
 {
-    if (launch_cluster(pl->s, pl->c, A, B, C, stream, S.prefetch, epi) != ADAPT_OK) return fail(ADAPT_ERR_CUDA, "cluster kernel launch failed%s");
+    if (launch_cluster(pl->s, pl->c, A, B, C, S.machine.n_sm, stream, S.prefetch, epi) != ADAPT_OK) return fail(ADAPT_ERR_CUDA, "cluster kernel launch failed%s");
     S.launches.fetch_add(1, std::memory_order_relaxed);
     CUDA_TRY(cudaGetLastError());
     return ADAPT_OK;

@@ -220,6 +220,11 @@ constexpr int kClusterKS = 64;          // k values per stage
 constexpr int kClusterStageBytes = 2 * 64 * 144;
 constexpr int kClusterMaxRing = 6;
 inline int cluster_smem_bytes(int ring) { return ring * kClusterStageBytes; }
+// Shared memory that no two CTAs of an SM can have: what a cluster's CTAs ask for when all clusters run at once with an SM per CTA.
+// With less, two CTAs of a cluster share an SM while others idle, and each stage's chain takes longer (364 x 18 x 5002, six clusters of
+// 16: 11.5 us, 8.4 with an SM per CTA; 78 x 357 x 2547, twelve of 8: 11.8 and 8.8).
+constexpr int kClusterAloneBytes = 7 * kClusterStageBytes;
+static_assert(2 * kClusterAloneBytes > 228 * 1024, "more than half of an SM's shared memory");
 // A tile of one CTA: two groups of warps with a ring each, of `chain` stages at most (three: two CTAs per SM).
 constexpr int kClusterSeqRing = 3;
 inline int cluster_seq_ring(int chain) { return std::max(1, std::min(kClusterSeqRing, chain)); }
@@ -235,6 +240,10 @@ inline int64_t cluster_slots(int cluster, int n_sm)
 {
     const int64_t b200 = cluster == 1 ? 148 : cluster == 2 ? 74 : cluster == 4 ? 33 : cluster == 8 ? 15 : 7;
     return std::max<int64_t>(1, b200 * n_sm / 148);
+}
+inline int cluster_launch_bytes(int ring, int cluster, int64_t tiles, int n_sm)
+{
+    return cluster > 1 && tiles <= cluster_slots(cluster, n_sm) ? std::max(kClusterAloneBytes, cluster_smem_bytes(ring)) : cluster_smem_bytes(ring);
 }
 inline int cluster_ctas_per_sm(int ring, int smem_limit) { return std::max(1, std::min(2, smem_limit / cluster_smem_bytes(ring))); }
 // Depth of the raw ring: as deep as the CTA's k range needs, up to 6 stages when the tiles' clusters all run

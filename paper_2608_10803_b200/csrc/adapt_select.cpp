@@ -570,7 +570,8 @@ static bool legal_cluster(const Shape& s, const Machine& m, Config& c)
     if ((int64_t)c.P_m * c.P_n * c.cluster > 2 * (int64_t)m.n_sm) return false;
     if (c.stages != cluster_ring(s.K, c.cluster, (int64_t)c.P_m * c.P_n, m.n_sm)) return false;
     c.persistent = 0;
-    c.smem_bytes = cluster_two_groups(s.K, c.cluster) ? cluster_seq_smem_bytes(cluster_alone_ring(s.K)) : cluster_smem_bytes(c.stages);
+    c.smem_bytes = cluster_two_groups(s.K, c.cluster) ? cluster_seq_smem_bytes(cluster_alone_ring(s.K))
+                                                      : cluster_launch_bytes(c.stages, c.cluster, (int64_t)c.P_m * c.P_n, m.n_sm);
     return true;
 }
 

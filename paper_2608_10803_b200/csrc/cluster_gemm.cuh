@@ -454,12 +454,12 @@ inline ClusterKernel cluster_pick(bool a_kc, bool b_kc, bool bf16)
     return b_kc ? cluster_gemm_kernel<false, true, false, SEQ> : cluster_gemm_kernel<false, false, false, SEQ>;
 }
 
-// Once per device: the deepest ring needs more than the default dynamic shared memory.
+// Once per device: the launches need more than the default dynamic shared memory.
 inline cudaError_t cluster_set_attributes()
 {
     for (int v = 0; v < 8; ++v) {
         const ClusterKernel split = cluster_pick<false>(v & 1, v & 2, v & 4), alone = cluster_pick<true>(v & 1, v & 2, v & 4);
-        cudaError_t e = cudaFuncSetAttribute(split, cudaFuncAttributeMaxDynamicSharedMemorySize, cluster_smem_bytes(kClusterMaxRing));
+        cudaError_t e = cudaFuncSetAttribute(split, cudaFuncAttributeMaxDynamicSharedMemorySize, kClusterAloneBytes);
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(split, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // clusters of 16
         if (e != cudaSuccess) return e;
@@ -469,14 +469,14 @@ inline cudaError_t cluster_set_attributes()
     return cudaSuccess;
 }
 
-// Largest cluster size (16, 8, 4, 2, 1) of which the device runs at least one cluster with the deepest ring.
+// Largest cluster size (16, 8, 4, 2, 1) of which the device runs at least one cluster with an SM per CTA.
 inline int cluster_max_size()
 {
     for (int cs = 16; cs > 1; cs >>= 1) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)cs, 1, 1);
         cfg.blockDim = dim3(kClusterThreads, 1, 1);
-        cfg.dynamicSmemBytes = (size_t)cluster_smem_bytes(kClusterMaxRing);
+        cfg.dynamicSmemBytes = (size_t)kClusterAloneBytes;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = (unsigned)cs;
@@ -493,7 +493,7 @@ inline int cluster_max_size()
 
 // Host launcher.  c.cluster = CS; c.stages = depth of the raw ring; the grid is CS CTAs per tile, the cluster spans blockIdx.x.
 inline adapt_status_t launch_cluster(const Shape& s, const Config& c, const void* A, const void* B, void* C,
-                                     cudaStream_t stream, int prefetch = 1, const ReduceEpilogue* epi = nullptr)
+                                     int n_sm, cudaStream_t stream, int prefetch = 1, const ReduceEpilogue* epi = nullptr)
 {
     ClusterParams p;
     p.A = (const unsigned short*)A;
@@ -515,7 +515,7 @@ inline adapt_status_t launch_cluster(const Shape& s, const Config& c, const void
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)((int64_t)c.P_m * c.P_n * c.cluster), 1, 1);
     cfg.blockDim = dim3(kClusterThreads, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)(seq ? cluster_seq_smem_bytes(p.ring) : cluster_smem_bytes(p.ring));
+    cfg.dynamicSmemBytes = (size_t)(seq ? cluster_seq_smem_bytes(p.ring) : cluster_launch_bytes(p.ring, c.cluster, (int64_t)c.P_m * c.P_n, n_sm));
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     pdl_attribute(&attr[0]);

@@ -69,3 +69,29 @@ def build_and_run(tmp_path, program):
 def test_every_groupable_configuration_gets_a_kernel_that_holds_it(tmp_path):
     r = build_and_run(tmp_path, PROGRAM)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+def test_clusters_that_all_fit_get_an_sm_per_cta(tmp_path):
+    """Shared memory of a cluster launch: more than half of an SM's where all clusters run at once with an SM per CTA, never less than
+    the ring, never more than a CTA may have."""
+    r = build_and_run(tmp_path, r"""
+#include <cstdio>
+#include "adapt_internal.h"
+using namespace adapt;
+int main()
+{
+    const Machine m;
+    int alone = 0, shared = 0;
+    for (int cs : {1, 2, 4, 8, 16})
+        for (int64_t tiles = 1; tiles * cs <= 2 * m.n_sm; ++tiles)
+            for (int ring = 1; ring <= kClusterMaxRing; ++ring) {
+                const int bytes = cluster_launch_bytes(ring, cs, tiles, m.n_sm);
+                const bool fits = cs > 1 && tiles <= cluster_slots(cs, m.n_sm);
+                if (bytes < cluster_smem_bytes(ring) || bytes > m.smem_bytes || (2 * (bytes + 1024) > 228 * 1024) != fits) return 1;
+                alone += fits;
+                shared += !fits;
+            }
+    return alone == 0 || shared == 0;
+}
+""")
+    assert r.returncode == 0, r.stdout + r.stderr
