@@ -1113,8 +1113,21 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
 
     // the plan's fused reduction stands unless a fallback changed the tiling (then: partials in the workspace)
     const bool fused = c.fused != 0 && p.P_k == c.P_k && !(c.srcB == ADAPT_SRC_TMA_CLASSES && !kclsB);
-    // a fused add runs where the 16-bit output is stored: here, or with unfused k splits in the reduction kernel
-    const bool partials = p.P_k > 1 && !fused;
+    // 16-bit C through TMA stores: whole 32-byte sectors (halo tiles shift theirs)
+    const bool tma_store = p.P_k == 1 && !kclsB && (halo ? ((uintptr_t)C & 15) == 0 : (((uintptr_t)C & 31) == 0 && s.N % 16 == 0));
+    // A fused add runs where the 16-bit output is stored: here, or with unfused k splits in the reduction kernel.  A small output of
+    // one row of tiles whose threads would store it themselves goes through fp32 sums and the reduction kernel too: the few warps that
+    // drain it would wait for D pass after pass (16 x 30001 x 200 with a bias 17.9 us, 14.7 that way; 70 x 9999 x 64 12.0 and 10.5; but
+    // 100 x 17097 x 85, 1.7 million outputs, 12.3 and 15.2, and 12048 x 38 x 739 13.8 and 15.8).  Without the workspace for that (it must not grow in a capture) the kernel adds D all the same.
+    bool sums_out = epi && p.P_k == 1 && !fused && !tma_store && s.M <= 128 && s.M * s.N <= (int64_t)768 << 10;
+    if (sums_out) {
+        void* probe = nullptr;
+        const adapt_status_t r = try_workspace(S, stream, szA + szB + (size_t)round_up(s.M * partial_pitch(s.N) * 4, 256), &probe);
+        if (r != ADAPT_OK) return r;
+        sums_out = probe != nullptr;
+    }
+    p.force_partial = sums_out ? 1 : 0;
+    const bool partials = (p.P_k > 1 && !fused) || sums_out;
     p.ep = epi && !partials ? *epi : no_epilogue();
     const size_t szP = partials ? (size_t)round_up((int64_t)p.P_k * s.M * partial_pitch(s.N) * 4, 256) : 0;
     // stream-K stands unless a fallback changed the tiling; one fp32 partial tile per CTA
@@ -1183,7 +1196,7 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
     p.part_hint = (p.P_k > 1 && szP <= ((size_t)100 << 20)) ? 1 : 0;
     memset(p.c_sigma, 0, sizeof(p.c_sigma));
     memset(p.c_extent, 0, sizeof(p.c_extent));
-    if (p.P_k == 1 && !kclsB && (halo ? ((uintptr_t)C & 15) == 0 : (((uintptr_t)C & 31) == 0 && s.N % 16 == 0))) {
+    if (tma_store && !sums_out) {
         if (classesA) {
             if ((r = cached_class_maps(S, pl, kMapC, C, s.M, s.N, 32, ncls, 32, true, maps.c, p.c_sigma, p.c_extent)) != ADAPT_OK)
                 return r;

@@ -55,6 +55,7 @@ struct UmmaParams {
     int c_mode;                      // 16-bit output: 0 = stores by the epilogue threads (any N, any alignment),
                                      // 1 = TMA stores through the maps of C (rows of C, or of the tile's row class,
                                      //     start on 32-byte boundaries; class tiles with 16 halo columns shift them there)
+    int force_partial;               // write the fp32 sums also with P_k = 1 (the reduction kernel adds D)
     int shuffle_k;                   // ShuffleK (Table 2): a tile starts its k range at a k-block that depends on the tile, so the CTAs of a wave
                                      // do not all ask for the same k slice of a shared operand at the same moment (plain tiles only)
     int prefetch;                    // ask L2 for the first unit's operand boxes before waiting for the kernel ahead on the stream
@@ -247,29 +248,40 @@ __device__ __forceinline__ void store_run16(unsigned short* dst, int count, cons
     }
 }
 
-// r[i] = alpha * r[i] + beta * D[row][n + i] for the columns below `end` (AddMM, in fp32 before the cast); a row that does not
-// exist (!row_ok) is left alone.  A row of D is read as 16-byte pieces where they are aligned and whole: a thread owns 32
-// consecutive columns, two whole sectors when N % 16 == 0; a bias is the same address for all lanes.
+// r[i] = alpha * r[i] + beta * D[row][n + i] for the columns below `end` (AddMM, in fp32 before the cast; beyond `end` anything, never
+// stored); a row that does not exist (!row_ok) is left alone.  A thread owns 8 or 32 consecutive columns of a row of D (two whole sectors
+// when N % 16 == 0) and reads them as the 16-byte chunks that hold them, whatever the row's alignment (a chunk that holds an existing byte
+// is always readable); a bias is the same address for all lanes.
 // Adding D here instead of in the reduction kernel saves the trip of the fp32 sums through memory (2048 x 4096 x 4096 with a
-// bias: 33 MB out and back and a launch).
+// bias: 33 MB out and back and a launch).  Rows of D off 16-byte boundaries read element by element cost more than that trip:
+// 100 x 17097 x 85 with a matrix D 17.1 us, 15.2 through the reduction kernel, 13.4 in chunks; 2048 x 2050 x 2048 59.0, 41.1, 35.1.
 template <int COUNT>
 __device__ __forceinline__ void epilogue_add(const ReduceEpilogue& e, uint32_t (&r)[COUNT], int row, int n, int end, int N, bool row_ok, int dtype)
 {
     if (!row_ok) return;
-    const unsigned short* d = e.D + (e.d_is_vector ? (int64_t)n : (int64_t)row * N + n);
-    const bool whole = (reinterpret_cast<uintptr_t>(d) & 15) == 0;
+    const uintptr_t d = reinterpret_cast<uintptr_t>(e.D + (e.d_is_vector ? (int64_t)n : (int64_t)row * N + n));
+    const int sh = (int)(d & 15), bytes = 2 * min(COUNT, end - n);
+    const uint4* q = reinterpret_cast<const uint4*>(d - sh);
+    uint32_t w[COUNT / 2 + 4];
 #pragma unroll
-    for (int c = 0; c < COUNT; c += 8) {
-        unsigned short v[8];
-        if (whole && n + c + 8 <= end) {
-            *reinterpret_cast<uint4*>(v) = *reinterpret_cast<const uint4*>(d + c);
-        } else {
+    for (int j = 0; j <= COUNT / 8; ++j) {
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (16 * j - sh < bytes) v = q[j];
+        w[4 * j] = v.x; w[4 * j + 1] = v.y; w[4 * j + 2] = v.z; w[4 * j + 3] = v.w;
+    }
+    if (sh != 0) {                                          // to the start of the chunk: two words, one word, two bytes
+        const uint32_t sel = 0x3210u + 0x1111u * (uint32_t)(sh & 3);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = n + c + i < end ? d[c + i] : (unsigned short)0;
-        }
+        for (int k = 0; k <= COUNT / 2 + 1; ++k) w[k] = sh & 8 ? w[k + 2] : w[k];
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-            r[c + i] = __float_as_uint(fmaf(e.beta, load16_as_float(&v[i], dtype), e.alpha * __uint_as_float(r[c + i])));
+        for (int k = 0; k <= COUNT / 2; ++k) w[k] = sh & 4 ? w[k + 1] : w[k];
+#pragma unroll
+        for (int k = 0; k < COUNT / 2; ++k) w[k] = __byte_perm(w[k], w[k + 1], sel);
+    }
+#pragma unroll
+    for (int i = 0; i < COUNT; ++i) {
+        const unsigned short h = (unsigned short)(i & 1 ? w[i / 2] >> 16 : w[i / 2] & 0xFFFFu);
+        r[i] = __float_as_uint(fmaf(e.beta, load16_as_float(&h, dtype), e.alpha * __uint_as_float(r[i])));
     }
 }
 
@@ -760,9 +772,24 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
         bool ok = true;
         uint8_t* stg = stage_out + (warp - 2) * kUmmaWarpStagingBytes + lane * kUmmaStageRowBytes;   // this thread's staging row
         unsigned short* srow = reinterpret_cast<unsigned short*>(stg);
+        // EPI: asks L2 for this thread's row of D in the CTA's it-th tile, one tile ahead of its use: the passes of a tile read a line of
+        // D each, one trip to memory after the other otherwise (20000 x 20001 x 12: 626 -> 509 us; not a bias, which is in L2 after
+        // the first row of tiles: 331 -> 365)
+        auto prefetch_d = [&](int it) {
+            WorkItem w;
+            if (p.ep.d_is_vector || (!FUSE && !B_CLS && (it & 1) != half) || !next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w)) return;
+            const int r = (A_CLS ? (w.mb >> NSH) * (128 * CG * NCLS) + (w.mb & (NCLS - 1)) + NCLS * 128 * (int)cta_rank : w.mb * (128 * CG) + (int)cta_rank * 128) +
+                          (A_CLS ? NCLS : 1) * (q * 32 + lane);
+            if (r >= p.M) return;
+            const unsigned short* d = p.ep.D + (int64_t)r * p.N;
+#pragma unroll 1
+            for (int n = w.nb * TILE_N; n < min(p.N, w.nb * TILE_N + BN); n += 64) ptx::prefetch_l2(d + n);
+        };
+        if (EPI) prefetch_d(0);
         for (int it = 0; ok; ++it, ++seq) {
             WorkItem w;
             if (!next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w)) break;
+            if (EPI) prefetch_d(it + 1);
             const uintptr_t c_base = reinterpret_cast<uintptr_t>(p.C) + (BATCH ? 2ull * (uintptr_t)(w.entry * p.c_entry) : 0);
             const int unit = w.unit, mb = w.mb, nb = w.nb, split = w.split;
             (void)unit;
@@ -912,7 +939,6 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                 // lane walking the ranks serialised P_k of them (pair tiles hit the same wall: 0.8 us per k-block)
                 __syncwarp();
                 if (lane < p.P_k) ptx::mbar_arrive_cluster(xfull_bar, (uint32_t)lane);
-                if (!ptx::mbar_wait_cluster(xfull_bar, xphase, abort_flag)) { ok = false; break; }
                 // rows and 4-column groups of this tile that exist; rank r takes the r-th share of them
                 const int rows_here = A_CLS ? min(128, (p.M - row_base + row_step - 1) / row_step) : min(128, p.M - row_base);
                 const int tile_cols = min(TILE_N, p.N - n0);
@@ -922,8 +948,25 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                 const int e_end = min(total, ((int)my_rank + 1) * per);
                 const uint32_t x_addr = ptx::smem_u32(X);
                 unsigned short* c16 = reinterpret_cast<unsigned short*>(p.C);
-                for (int e = (int)my_rank * per + (warp - 2) * 32 + lane; e < e_end; e += kUmmaEpilogueWarps * 32) {
+                const int e_first = (int)my_rank * per + (warp - 2) * 32 + lane;
+                // EPI: the four elements of D of a group, loaded while the group before it is added (the first ones while the ranks meet)
+                auto load_d = [&](int e) -> uint2 {
+                    if (e >= e_end) return make_uint2(0u, 0u);
+                    const int rr = e / groups, n = n0 + 4 * (e - rr * groups);
+                    const uintptr_t d = reinterpret_cast<uintptr_t>(p.ep.D + (p.ep.d_is_vector ? (int64_t)n : (int64_t)(row_base + row_step * rr) * p.N + n));
+                    const int sh = (int)(d & 7);                         // the one or two aligned 8-byte chunks that hold them
+                    const unsigned long long* q = reinterpret_cast<const unsigned long long*>(d - sh);
+                    unsigned long long v = q[0] >> (8 * sh);
+                    if (sh != 0 && 8 - sh < 2 * min(4, p.N - n)) v |= q[1] << (64 - 8 * sh);
+                    return make_uint2((uint32_t)v, (uint32_t)(v >> 32));
+                };
+                uint2 d_next = make_uint2(0u, 0u);
+                if (EPI) d_next = load_d(e_first);
+                if (!ptx::mbar_wait_cluster(xfull_bar, xphase, abort_flag)) { ok = false; break; }
+                for (int e = e_first; e < e_end; e += kUmmaEpilogueWarps * 32) {
                     const int rr = e / groups, g = e - rr * groups;
+                    const uint2 d4 = d_next;
+                    if (EPI) d_next = load_d(e + kUmmaEpilogueWarps * 32);
                     const uint32_t a = x_addr + (uint32_t)((rr * p.x_pitch + 4 * g) * 4);
                     float4 sum = ptx::ld_cluster_f4(a, 0u);
                     for (int rk = 1; rk < p.P_k; ++rk) {
@@ -932,11 +975,12 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                     }
                     const int n = n0 + 4 * g;
                     if (EPI) {
-                        const int m = row_base + row_step * rr;
-                        sum.x = fused_add(p.ep, sum.x, m, n, p.N, p.dtype);
-                        if (n + 1 < p.N) sum.y = fused_add(p.ep, sum.y, m, n + 1, p.N, p.dtype);
-                        if (n + 2 < p.N) sum.z = fused_add(p.ep, sum.z, m, n + 2, p.N, p.dtype);
-                        if (n + 3 < p.N) sum.w = fused_add(p.ep, sum.w, m, n + 3, p.N, p.dtype);
+                        const unsigned short h[4] = {(unsigned short)(d4.x & 0xFFFFu), (unsigned short)(d4.x >> 16), (unsigned short)(d4.y & 0xFFFFu),
+                                                     (unsigned short)(d4.y >> 16)};
+                        sum.x = fmaf(p.ep.beta, load16_as_float(&h[0], p.dtype), p.ep.alpha * sum.x);
+                        sum.y = fmaf(p.ep.beta, load16_as_float(&h[1], p.dtype), p.ep.alpha * sum.y);
+                        sum.z = fmaf(p.ep.beta, load16_as_float(&h[2], p.dtype), p.ep.alpha * sum.z);
+                        sum.w = fmaf(p.ep.beta, load16_as_float(&h[3], p.dtype), p.ep.alpha * sum.w);
                     }
                     unsigned short* dst = c16 + (size_t)(row_base + row_step * rr) * p.N + n;
                     if (n + 4 <= p.N && (reinterpret_cast<uintptr_t>(dst) & 7) == 0) {
@@ -951,7 +995,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                 // done reading every rank's partial: each may overwrite it for its next tile
                 __syncwarp();
                 if (lane < p.P_k) ptx::mbar_arrive_cluster(xempty_bar, (uint32_t)lane);
-            } else if (p.P_k == 1) {
+            } else if (p.P_k == 1 && !p.force_partial) {
                 // 16-bit output, any N and any base alignment.  A thread converts 64 columns of its row
                 // and stages them in shared memory shifted by the row's misalignment in C, so that
                 // 16-byte aligned chunks of a staged row are 16-byte aligned chunks of C.  The warp then
