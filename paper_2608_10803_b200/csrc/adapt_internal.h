@@ -94,7 +94,7 @@ struct Calib {
     double skinny_mac_rate = 30e12;     // MAC/s ceiling of the warp-level kernel (small side padded to 16)
     // one-launch cluster kernel (64 x 64 tiles, k split over a cluster): fitted on timed configurations of the kernel as it was when every
     // stage had an mbarrier and a shift pass of its own.  It has become faster since (64 x 64 x 1024 by one CTA 19.0 -> 9.6 us,
-    // 256^3 5.42 -> 4.60), so these constants overstate it: a small problem whose best tcgen05 plan is predicted a few per cent
+    // 256^3 5.42 -> 3.97), so these constants overstate it: a small problem whose best tcgen05 plan is predicted a few per cent
     // faster may be better off here
     double cluster_fixed_us = 0.75;     // beyond the launch: first trip to memory, rounding and store of the tile
     double cluster_stage_us = 0.76;     // one 64-k stage

@@ -217,7 +217,7 @@ regroup_a_kernel(const unsigned short* __restrict__ A, unsigned short* __restric
 // A small output with many splits leaves most of the chip idle while each thread walks its splits batch by batch (one trip to L2
 // per eight): there the splits are shared by `groups` threads (a power of two), each adding a run of consecutive splits in
 // ascending order; the runs' sums are then added in ascending order too.  The order depends on the shape only.
-// (256 x 256 x 262144, P_k = 64: eight batches 67.7 us for the call, one batch 63.1 us; 34 x 21 x 34323: 17.3 and 11.6 us.)
+// (256 x 256 x 262144, P_k = 64: eight batches 67.9 us for the call, one batch 63.5 us; 34 x 21 x 34323: 17.3 and 11.6 us.)
 // SHARED: groups > 1 (the other outputs are not charged for it: 365 x 3136 x 4672 in three splits 23.1 us, 23.6 with the one kernel).
 template <bool SHARED>
 __global__ void __launch_bounds__(256)

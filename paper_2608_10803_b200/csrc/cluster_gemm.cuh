@@ -22,8 +22,8 @@
 //
 // What bounds it: the dependent chain of a stage (wait, shift, barrier, ldmatrix, MMAs), and for many tiles the shared-memory
 // port (copy in, shift, ldmatrix).  Per-thread copy groups and no shifted stages beside the raw ones, against an mbarrier per
-// stage that every thread's copies arrived on and a separate shifted buffer: 256 x 256 x 256 (CS = 4) 5.42 -> 4.60 us, 64 x 1024 x 1024
-// 7.16 -> 5.78 us; with two groups of warps in place of eight warps on one stage as well, 64 x 64 x 1024 by one CTA 19.0 -> 9.6 us.
+// stage that every thread's copies arrived on and a separate shifted buffer: 256 x 256 x 256 (CS = 4) 5.42 -> 4.60 us (3.97 with
+// an SM per CTA), 64 x 1024 x 1024 7.16 -> 5.78 us; with two groups of warps in place of eight warps on one stage as well, 64 x 64 x 1024 by one CTA 19.0 -> 9.6 us.
 #pragma once
 
 #include <cstdint>

@@ -1,7 +1,7 @@
 // Many small GEMMs in ONE launch: the lists of adapt_matmul_batch and the entries of adapt_matmul_strided_batch.
 //
 // A GEMM of a few microseconds is mostly launch, first trip to memory and drain; one launch each leaves the chip idle
-// between them (48 layers of 16 .. 1024 a side: 108 us on four streams, two microseconds a call, for 16 MB of operands).
+// between them (48 layers of 16 .. 1024 a side: 110 us on four streams, two microseconds a call, for 16 MB of operands).
 // Here the 64 x 64 tiles of all entries run side by side, one per CTA.  An entry keeps the arithmetic of its own plan:
 //   pieces > 0: the one-launch cluster kernel's tiles.  The CTA walks the plan's pieces of the k range and adds
 //               their sums in the same order: the bits of the call made alone, where each piece has a CTA of its own.
