@@ -114,3 +114,35 @@ def test_addmm_of_infinities_nan_and_the_types_largest_values(shape, dtype):
         ab.adapt_addmm(plan, A.data_ptr(), B.data_ptr(), finite.data_ptr(), False, 1.0, 0.0, zero.data_ptr(), st)
         torch.cuda.synchronize()
         assert same_values(synth.bits(zero), synth.bits(plain))
+
+
+@pytest.mark.parametrize("vector", [False, True])
+def test_small_output_goes_through_the_sums_or_not_with_the_same_result(vector):
+    """One row of tiles that its threads store (rows of C off 32-byte boundaries): two launches over the workspace, and in a capture on a
+    stream without one, where it must not grow, the kernel adds D itself."""
+    M, N, K, dtype = 128, 5608, 256, ab.F16
+    init()
+    plan = ab.adapt_matmul_plan(M, N, K, dtype)
+    info = ab.adapt_plan_info(plan)
+    assert info.family in (ab.FAM_UMMA_1CTA, ab.FAM_UMMA_2CTA) and info.P_k == 1 and info.workspace_bytes == 0
+    A, B, D = (synth.draw_operand(1, n, ("integer", -4, 4), seed, dtype, "cuda").reshape(-1) for n, seed in ((M * K, 71), (K * N, 72), (M * N, 73)))
+    d = D[:N] if vector else D
+    _, want = og.addmm_rows(synth.bits(A), synth.bits(B), synth.bits(d), M, N, K, dtype, 0.5, 3.0)
+    C = torch.full((M, N), float("nan"), dtype=A.dtype, device="cuda")
+    args = (plan, A.data_ptr(), B.data_ptr(), d.data_ptr(), vector, 0.5, 3.0, C.data_ptr())
+    before = ab.adapt_launch_count()
+    ab.adapt_addmm(*args, torch.cuda.current_stream().cuda_stream)
+    assert ab.adapt_launch_count() - before == 2
+    torch.cuda.synchronize()
+    assert np.array_equal(synth.bits(C).reshape(want.shape), want)
+    C.fill_(float("nan"))
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph, before = torch.cuda.CUDAGraph(), ab.adapt_launch_count()
+    with torch.cuda.graph(graph, stream=side):
+        ab.adapt_addmm(*args, side.cuda_stream)
+    assert ab.adapt_launch_count() - before == 1
+    graph.replay()
+    torch.cuda.synchronize()
+    ab.adapt_poll_device_status(side.cuda_stream)
+    assert np.array_equal(synth.bits(C).reshape(want.shape), want)
