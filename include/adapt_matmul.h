@@ -67,7 +67,7 @@ typedef enum {
 /* Kernel families of the variant library. */
 typedef enum {
     ADAPT_FAM_UMMA_1CTA = 0,  /* tcgen05 128 x BN tiles, TMEM accumulators, TMA ring; P_k > 1 adds split-K */
-    ADAPT_FAM_UMMA_2CTA = 1,  /* cta_group::2, 256 x BN tile on an SM pair */
+    ADAPT_FAM_UMMA_2CTA = 1,  /* cta_group::2, 256 x BN or 512 x 256 tile on an SM pair */
     ADAPT_FAM_SKINNY = 2,     /* warp-level kernel for M <= 16 or N <= 16, streams the large operand once */
     ADAPT_FAM_SIMT = 3,       /* CUDA-core tile kernel: legal for every shape and alignment */
     ADAPT_FAM_CLUSTER = 4     /* small problems in one launch: 64 x 64 tiles on mma.sync, any alignment, the k range

@@ -24,6 +24,7 @@
 #include "batch_schedule.h"
 #include "batch_route.h"
 #include "umma_gemm.cuh"
+#include "tall_gemm.cuh"
 
 using namespace adapt;
 
@@ -419,7 +420,7 @@ extern "C" int64_t adapt_map_encode_count(void) { return st().map_encodes.load()
 extern "C" void adapt_set_map_cache(int enabled) { st().map_cache.store(enabled ? 1 : 0); }
 // the model's calibration constants by name (the fields of Calib that are plain doubles)
 #define ADAPT_CALIB_FIELDS(X) X(launch_us) X(prologue_launch_us) X(hbm_bw) X(l2_bw_per_sm) X(tensor_flops) X(eta_mma_bn128) X(eta_mma_bn64) \
-    X(eta_2cta) X(mem_latency_us) X(hbm_latency_us) X(hbm_latency_views_us) X(umma_fixed_us) X(epi_tile_fixed_us) X(epi_us_per_kb) \
+    X(eta_2cta) X(eta_tall) X(tall_tile_us) X(mem_latency_us) X(hbm_latency_us) X(hbm_latency_views_us) X(umma_fixed_us) X(epi_tile_fixed_us) X(epi_us_per_kb) \
     X(pair_drain_factor) X(epi_partial_fixed_us) X(epi_partial_us_per_kb) X(epi_tile_fixed_unaligned_us) X(epi_us_per_kb_unaligned) \
     X(thread_store_exposed) X(thread_store_exposed_pair) X(simt_flops) X(simt_fixed_us) X(simt_step_us) X(halo_edge_tile_us) X(simt_bw_eff) \
     X(skinny_bw_eff_aligned) X(skinny_bw_eff_unaligned) X(skinny_fixed_us) X(skinny_pass_us) X(skinny_step_unaligned_us) X(skinny_mac_rate) \
@@ -693,6 +694,17 @@ static UmmaKernel launch_map_umma(int family, int BN, bool a_mn, bool b_mn, int 
     return epi ? launch_map_umma_plain<true>(family, BN, a_mn, b_mn, mode) : launch_map_umma_plain<false>(family, BN, a_mn, b_mn, mode);
 }
 
+// tall pair tiles: plain ones in every layout, and of one row class
+static UmmaKernel launch_map_tall(bool a_mn, bool b_mn, bool classes, bool epi)
+{
+#define ADAPT_PICK(cls, a, b) if (classes == cls && a_mn == a && b_mn == b) \
+        return epi ? (const void*)tall_gemm_kernel<a, b, cls, true> : (const void*)tall_gemm_kernel<a, b, cls, false>;
+    ADAPT_PICK(false, false, false) ADAPT_PICK(false, false, true) ADAPT_PICK(false, true, false) ADAPT_PICK(false, true, true)
+    ADAPT_PICK(true, false, true)
+#undef ADAPT_PICK
+    return nullptr;
+}
+
 // ---------------------------------------------------------------------------------------------
 // init / shutdown
 // ---------------------------------------------------------------------------------------------
@@ -743,6 +755,10 @@ extern "C" adapt_status_t adapt_init(int device)
     for (int BN : {64, 128, 256})
         for (int v = 0; v < 4; ++v)
             CUDA_TRY(cudaFuncSetAttribute(umma_lookup_batch(BN, (v & 1) != 0, (v & 2) != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
+    for (int v = 0; v < 16; ++v) {
+        UmmaKernel k = launch_map_tall((v & 1) != 0, (v & 2) != 0, (v & 4) != 0, (v & 8) != 0);
+        if (k) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
+    }
     // clusters of 2, 4, 8 CTAs of the tcgen05 kernel (one CTA per SM) that the device runs at a time
     for (int i = 0; i < 3; ++i) {
         cudaLaunchConfig_t cfg;
@@ -1061,6 +1077,55 @@ adapt_status_t launch_reduce(State& S, const float* partial, void* C, int64_t M,
     return ADAPT_OK;
 }
 
+// Tall pair tiles: the schedule and the launch; p holds what both kernels need.
+adapt_status_t launch_tall(State& S, const Shape& s, const UmmaParams& p, const CUtensorMap* mapA, const CUtensorMap& mapB, const CUtensorMap* mapC, bool a_mn, bool b_mn,
+                           bool classes, cudaStream_t stream)
+{
+    const int slots = S.machine.n_sm / 2;
+    TallParams q;
+    q.M = p.M; q.N = p.N; q.kb_total = p.kb_total;
+    q.work = tall_schedule(s.M, p.P_n, classes, slots);
+    q.dtype = p.dtype; q.idesc = p.idesc; q.c_hint = p.c_hint; q.prefetch = p.prefetch; q.ep = p.ep; q.status = p.status;
+    for (int j = 0; j < 8; ++j) q.a_sigma[j] = p.a_sigma[j];
+    TmapPackT<0> pack0;
+    TmapPackT<1> pack1;
+    void* args[2] = {nullptr, &q};
+    size_t arg_bytes[2] = {sizeof(pack0), sizeof(q)};
+    if (classes) {
+        memset(&pack1, 0, sizeof(pack1));
+        memcpy(pack1.a, mapA, 8 * sizeof(CUtensorMap));
+        memcpy(pack1.c, mapC, 8 * sizeof(CUtensorMap));
+        pack1.b[0] = mapB;
+        args[0] = &pack1;
+        arg_bytes[0] = sizeof(pack1);
+    } else {
+        memset(&pack0, 0, sizeof(pack0));
+        pack0.a[0] = mapA[0];
+        pack0.b[0] = mapB;
+        pack0.c[0] = mapC[0];
+        args[0] = &pack0;
+    }
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(2 * std::min(q.work.big + q.work.halves, slots)), 1, 1);
+    cfg.blockDim = dim3(kUmmaThreads, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)tall_smem_bytes();
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    pdl_attribute(&attr[1]);
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    UmmaKernel k = launch_map_tall(a_mn, b_mn, classes, q.ep.D != nullptr);
+    if (!k) return fail(ADAPT_ERR_UNSUPPORTED, "no compiled kernel for this tiling key%s");
+    CUDA_TRY(launch_exc(&cfg, k, args, arg_bytes, 2));
+    S.launches.fetch_add(1, std::memory_order_relaxed);
+    return ADAPT_OK;
+}
+
 adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi = nullptr)
 {
     const Shape& s = pl->s;
@@ -1097,6 +1162,9 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
     memset(p.b_sigma, 0, sizeof(p.b_sigma));
     p.cls_kc = (int)Kc;
     p.M = (int)s.M; p.N = (int)s.N; p.K = (int)s.K;
+    // tall tiles store whole 32-byte sectors and add D in 16-byte chunks: with a C or D off those boundaries their plan runs on 256-row
+    // pair tiles
+    const bool tall = c.BM == 512 && ((uintptr_t)C & 31) == 0 && (!epi || ((uintptr_t)epi->D & 15) == 0);
     p.P_m = c.P_m;
     // a plan made for k-class views that has to fall back to a copy of B (unaligned pointer) uses plain tiles
     p.P_n = (c.srcB == ADAPT_SRC_TMA_CLASSES && !kclsB) ? (int)ceil_div(s.N, c.BN) : c.P_n;
@@ -1221,7 +1289,7 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
     if (p.a_shift_any) p.a_shift_any = 1;
     p.dtype = s.dtype;
     // the plan's ring depth assumed its own A box; a fallback to copies may need a shallower ring
-    p.stages = c.stages;
+    p.stages = c.BM == 512 ? umma_deepest_ring(c.BN, cg, 128, true, S.machine.smem_bytes) : c.stages;
     const int fused_bytes = fused ? umma_fused_bytes(c.BN, a_box_rows) : 0;
     p.x_rows = a_box_rows;
     p.x_pitch = umma_fused_pitch(c.BN);
@@ -1253,6 +1321,10 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
     if (const char* e = getenv("ADAPT_TRACE_CTA")) p.trace_cta = atoi(e);
 #endif
 
+    if (tall) {
+        r = launch_tall(S, s, p, maps.a, maps.b[0], maps.c, a_mn, b_mn, classesA, stream);
+        return r;
+    }
     UmmaKernel k = streamk ? launch_map_umma_sk(c.family, c.BN, a_mn, b_mn)
                            : launch_map_umma(c.family, c.BN, a_mn, b_mn, classesA ? 1 : (kclsB ? 2 : 0), fused, p.ep.D != nullptr);
     if (!k) return fail(ADAPT_ERR_UNSUPPORTED, "no compiled kernel for this tiling key%s");

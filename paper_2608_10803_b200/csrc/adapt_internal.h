@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "adapt_matmul.h"
+#include "tall_plan.h"
 
 namespace adapt {
 
@@ -68,6 +69,9 @@ struct Calib {
     double eta_mma_bn128 = 0.518;        // relative tensor efficiency at BN = 128 (0.29 us per 128 x 128 x 64 block)
     double eta_mma_bn64 = 0.324;         // ... at BN = 64 (A-operand smem reads dominate)
     double eta_2cta = 1.0;              // pair tiles share B: no extra tensor cost
+    double eta_tall = 1.35;             // tall pair tiles: a quarter less operand traffic per flop (1000 x 8192 x 1024: one wave, 17.6 us, 18.6 on
+                                        // 256-row pair tiles; 10000 x 1024 x 1024: 23.0 and 23.5)
+    double tall_tile_us = 0.3;          // ... what a tile's drain does not hide
     double mem_latency_us = 1.0;        // TMA issue -> data visible (sets Delta_dep with few stages)
     double hbm_latency_us = 1.04;        // the same under a full HBM stream of a dense operand (128 x 128256 x 4096: 5 stages of 32 KB, 0.41 us each)
     double hbm_latency_views_us = 1.6;  // ... through the strided class views (79457 x 196 x 8325 with 3 stages: 0.75 us per stage)
@@ -270,6 +274,11 @@ inline StreamK streamk_schedule(int64_t tiles, int64_t slots, int64_t kblocks)
     k.rem = k.sk_tiles * kblocks - k.q0 * slots;
     return k;
 }
+// Tall pair tiles (tall_gemm.cuh): 512 x 256 outputs per SM pair, four stages of 256 rows of A and 128 columns of B per CTA.
+constexpr int kTallStages = 4;
+constexpr int kTallStageBytes = (256 + 128) * 64 * 2;
+constexpr int kTallBoxBytes = 4096;       // staging of one epilogue warp: a TMA store box of 32 rows of 64 columns
+
 constexpr int kUmmaFlagBytes = 4096;     // head of every workspace: stream-K flag words (one per CTA), zeroed when the workspace is allocated
 constexpr int kSkinnyKChunk = 512;   // k values the warp-level kernel stages per chunk; its k splits are whole chunks
 constexpr int kUmmaBarrierBytes = 1024;  // keeps the epilogue staging 1024-byte aligned (swizzled TMA boxes)
@@ -290,6 +299,7 @@ inline int umma_smem_bytes(int BN, int cluster, int stages, int a_rows, bool sta
     const int read_end = (stages - 1) * stage + 128 * 64 * 2;
     return std::max(used, read_end) + 1024;
 }
+inline int tall_smem_bytes() { return kTallStages * kTallStageBytes + kUmmaBarrierBytes + kUmmaEpilogueWarps * kTallBoxBytes + 1024; }
 // Deepest ring that fits (0 if not even two stages do).  Only a kernel that writes the 16-bit C itself
 // (P_k = 1) needs the epilogue staging; one that writes fp32 partials spends that space on stages.
 inline int umma_deepest_ring(int BN, int cluster, int a_rows, bool staging, int smem_limit, int cap = kUmmaMaxStages, int fused_bytes = 0)

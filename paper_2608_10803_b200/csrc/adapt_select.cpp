@@ -88,6 +88,7 @@ bool unpack_tiling_key(uint64_t k, Shape* s, Config* c)
     c->cls = (int)((k >> 62) & 3);
     c->family = (int)((k >> 59) & 7);
     c->BM = (int)((k >> 54) & 31) * 16;
+    if (c->BM == 0) c->BM = 512;                                    // tall pair tiles: 32 in five bits
     c->BN = (int)((k >> 48) & 63) * 16;
     c->BK = 16 << (int)((k >> 46) & 3);
     c->stages = (int)((k >> 42) & 15);
@@ -221,6 +222,10 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
     const int64_t slots = c.fused ? umma_cluster_slots(m, c.P_k) : m.n_sm / c.cluster;
     const int64_t Q = ceil_div(units, slots);
     c.grid = c.streamk ? (int)(slots * c.cluster) : (int)(std::min(units, slots) * (c.fused ? c.P_k : c.cluster));
+    const bool tall = c.BM == 512;
+    double tall_waves = 0.0;
+    const TallWork work = tall_schedule(s.M, c.P_n, c.srcA == ADAPT_SRC_TMA_CLASSES, slots, &tall_waves);
+    if (tall) c.grid = (int)(std::min<int64_t>(work.big + work.halves, slots) * c.cluster);
 
     const double MK = (double)s.M * s.K, KN = (double)s.K * s.N, MN = (double)s.M * s.N;
     // HBM traffic: operands once, plus re-reads of B when it cannot stay in L2 across m-groups.
@@ -234,7 +239,7 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
 
     // per-SM stage: each CTA loads its 128 rows of A and its share of the BN columns of B
     const double bn_per_cta = (double)c.BN / c.cluster;
-    const double a_rows = umma_a_box_rows(s, c.cluster, umma_row_classes(s, c.srcA, c.BN), kclasses);
+    const double a_rows = tall ? 256.0 : umma_a_box_rows(s, c.cluster, umma_row_classes(s, c.srcA, c.BN), kclasses);
     const double stage_bytes = 2.0 * c.BK * (a_rows + (double)round_up((int64_t)bn_per_cta, 64));
     // One SM pulls operands that other SMs also use from L2 at l2_bw_per_sm (a little less through
     // the strided row-class views); a stream that comes from HBM and is used once is bounded by the
@@ -248,8 +253,8 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
     double eta = c.BN >= 256 ? 1.0
                : c.BN >= 128 ? cal.eta_mma_bn128 + (1.0 - cal.eta_mma_bn128) * (c.BN - 128) / 128.0
                              : cal.eta_mma_bn64 + (cal.eta_mma_bn128 - cal.eta_mma_bn64) * (c.BN - 64) / 64.0;
-    if (c.cluster == 2) eta *= cal.eta_2cta;
-    const double tP = 2.0 * 128.0 * c.BN * c.BK / (cal.tensor_flops / m.n_sm * eta) * 1e6;
+    if (c.cluster == 2) eta *= tall ? cal.eta_tall : cal.eta_2cta;
+    const double tP = 2.0 * (tall ? 256.0 : 128.0) * c.BN * c.BK / (cal.tensor_flops / m.n_sm * eta) * 1e6;
     // Drain of one tile (the paper's T_drain: FixPipe cast and write).  With two or more TMEM
     // accumulators it overlaps the next tile's main loop, so a tile costs max(L * II, T_drain).
     // 16-bit tiles leave through TMA stores when C's rows are 16-byte aligned, or when class tiles with
@@ -258,7 +263,7 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
     const bool halo = c.BN % 64 != 0;
     const int own_n = halo ? c.BN - 16 : c.BN;
     // rows of a tile that exist (short M: the rest is neither stored by the threads nor by TMA)
-    const double rows_valid = std::min(128.0, (double)s.M / ((double)c.P_m * c.cluster));
+    const double rows_valid = tall ? 256.0 : std::min(128.0, (double)s.M / ((double)c.P_m * c.cluster));
     const double out_tile_kb = (c.P_k > 1 ? 4.0 : 2.0) * rows_valid * own_n / 1024.0;
     double t_drain;
     if (c.fused) t_drain = cal.fused_reduce_us + 4.0 * rows_valid * c.BN / cal.dsmem_bw_per_sm * 1e6;   // exchange + reduce + store, per tile
@@ -295,6 +300,7 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
                                            : std::max((double)L * ii + t_fixed, t_drain);
         // Eq. 14 with the drain overlapped: one fill, Q tiles back to back, the last drain exposed
         pipe = tM + (double)Q * t_tile + tP + t_drain;
+        if (tall) pipe = tM + tall_waves * std::max((double)L * ii + 2.0 * t_fixed + cal.tall_tile_us, t_drain) + tP + t_drain;   // no spare accumulator: the ends of a tile show
         if (c.streamk) {
             // whole waves as above; the leftover tiles' k-blocks shared evenly by all slots, then the owners' fix-up
             // While a slot works on its share of the leftover tiles it is at a k position of its own: nothing it loads is
@@ -451,13 +457,19 @@ static bool legal_umma(const Shape& s, const Machine& m, Config& c)
         if (c.BN != 64 && c.BN != 128 && c.BN != 256 && !halo_bn) return false;
         if (halo_bn && (c.srcA != ADAPT_SRC_TMA_CLASSES || s.N % 16 == 0 || s.M < 16)) return false;
     } else {
-        if (c.BM != 256 || c.cluster != 2) return false;
+        if ((c.BM != 256 && c.BM != 512) || c.cluster != 2) return false;
+        if (c.BM == 512) {
+            // tall tiles: both accumulators are one tile's halves; C leaves in whole 32-byte sectors; at least one row
+            // of whole tiles, and B's boxes have all their 64 k rows
+            if (c.BN != 256 || c.stages != kTallStages || c.P_k != 1 || c.streamk || c.fused || s.N % 16 != 0) return false;
+            if (s.K <= 64 || c.srcB == ADAPT_SRC_TMA_CLASSES || s.M <= (c.srcA == ADAPT_SRC_TMA_CLASSES ? 2048 : 256)) return false;
+        }
         const bool halo_bn = c.BN == 144 || c.BN == 208;                  // pair class tiles: 128 / 192 owned + 16 halo columns
         if (c.BN != 128 && c.BN != 256 && !halo_bn) return false;
         if (halo_bn && (c.srcA != ADAPT_SRC_TMA_CLASSES || s.N % 16 == 0 || s.M < 32)) return false;
     }
     if (c.BN % 16 != 0 || c.BN > 256) return false;                 // UMMA shape rule for M = 128/256
-    if (2 * c.BN > m.tmem_cols) return false;                       // at least two accumulator buffers in TMEM
+    if (2 * c.BN > m.tmem_cols) return false;                       // at least two accumulator buffers in TMEM (tall tiles: two halves)
     if (c.stages < 1 || c.stages > kUmmaMaxStages) return false;
     if (c.streamk) {
         // plain tiles, one split, not fused; needs leftover tiles and at least two k-blocks per slot in the shared part
@@ -471,6 +483,7 @@ static bool legal_umma(const Shape& s, const Machine& m, Config& c)
         if (c.srcB == ADAPT_SRC_TMA_CLASSES && c.BN == 64) return false;
     }
     c.smem_bytes = umma_smem_bytes(c.BN, c.cluster, c.stages, a_rows_box, c.P_k == 1, c.fused ? umma_fused_bytes(c.BN, a_rows_box) : 0);
+    if (c.BM == 512) c.smem_bytes = tall_smem_bytes();
     if (c.smem_bytes > m.smem_bytes) return false;
     // in class mode the k index of a tile is shifted by up to 7 elements
     // k-class mode splits the blocks of one class; in row-class mode the k index is shifted by up to 7
@@ -508,7 +521,8 @@ static bool legal_umma(const Shape& s, const Machine& m, Config& c)
     if (c.srcA == ADAPT_SRC_PAD_COPY && tma_friendly(innerA(s)) && !kclasses) return false;    // nothing to pad
     if (c.srcB == ADAPT_SRC_PAD_COPY && tma_friendly(innerB(s))) return false;
     const int ncls = umma_row_classes(s, c.srcA, c.BN);
-    c.P_m = classes ? (int)(ncls * ceil_div(s.M, ncls * c.BM)) : (int)ceil_div(s.M, c.BM);   // class tiles: 8 per 1024 rows (pair tiles: per 2048), 16 per 2048
+    const int64_t bm = std::min(c.BM, 256);                         // tall tiles are counted in their halves
+    c.P_m = classes ? (int)(ncls * ceil_div(s.M, ncls * bm)) : (int)ceil_div(s.M, bm);   // class tiles: 8 per 1024 rows (pair tiles: per 2048), 16 per 2048
     c.P_n = (int)ceil_div(s.N, kclasses ? c.BN - 8 : (c.BN % 64 ? c.BN - 16 : c.BN));
     if ((int64_t)c.P_m * c.P_n * c.P_k > (int64_t)1 << 30) return false;
     if (c.streamk) {
@@ -665,6 +679,12 @@ void enumerate_configs(const Shape& s, const Machine& m, const Calib& cal, std::
                     c.stages = st; c.P_k = pk; c.srcA = srcA; c.srcB = srcB;
                     if (st >= 2 && finalize(s, m, cal, c)) out->push_back(c);
                 }
+                if (pk == 1 && cluster == 2 && BN == 256) {               // both accumulators on one tile of 512 rows
+                    Config c;
+                    c.family = fam; c.BM = 512; c.BN = BN; c.BK = 64; c.cluster = cluster;
+                    c.stages = kTallStages; c.P_k = 1; c.srcA = srcA; c.srcB = srcB;
+                    if (finalize(s, m, cal, c)) out->push_back(c);
+                }
                 // one split, the leftover wave shared by all slots (stream-K)
                 if (pk == 1) {
                     Config c;
@@ -726,6 +746,10 @@ void enumerate_configs(const Shape& s, const Machine& m, const Calib& cal, std::
                 d.family = ADAPT_FAM_UMMA_2CTA; d.BM = 256; d.BN = BN; d.BK = 64; d.cluster = 2;
                 d.stages = deepest; d.P_k = pk; d.srcA = ADAPT_SRC_TMA_CLASSES; d.srcB = srcB;
                 if (deepest >= 2 && finalize(s, m, cal, d)) out->push_back(d);
+                if (pk == 1 && BN == 256) {
+                    d.BM = 512; d.stages = kTallStages;
+                    if (finalize(s, m, cal, d)) out->push_back(d);
+                }
             }
         }
     }
