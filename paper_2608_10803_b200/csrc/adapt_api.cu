@@ -427,7 +427,7 @@ extern "C" void adapt_set_map_cache(int enabled) { st().map_cache.store(enabled 
     X(cluster_fixed_us) X(cluster_stage_us) X(cluster_reduce_us) X(cluster_crowd_us) X(cluster_crowd_stage_us) X(cluster_wave_us) \
     X(cluster_bw_eff) X(streamk_fixup_us) X(streamk_peer_us) X(fused_reduce_us) X(fused_wave_us) X(reduce_launch_us) X(dsmem_bw_per_sm) \
     X(copy_bw_eff) X(hbm_bw_per_sm) X(class_view_sm_eff) X(class_tile_fixed_us) X(class_tile_fixed_unaligned_us) X(pair_class_tile_us) X(kclass_view_sm_eff) \
-    X(kclass_unit_fixed_us) X(kclass_tile_drain_us) X(oob_box_penalty) X(reduce_batch_us) X(class_split_bw_eff) \
+    X(kclass_unit_fixed_us) X(kclass_tile_drain_us) X(oob_box_penalty) X(l2_reread_cost) X(reduce_batch_us) X(class_split_bw_eff) \
     X(class_split_bw_eff_per_log2m) X(class_split_fused_bw_eff) X(regroup_bw_eff) X(class_view_bw_eff)
 
 static double* calib_field(Calib& c, const char* name)
@@ -991,6 +991,29 @@ adapt_status_t cached_map(State& S, Plan* pl, int which, const void* base, int64
     return ADAPT_OK;
 }
 
+// 3D map over the fp32 split-K partials [P_k][M][Np], boxes of 32 x 32: rows past M and columns past the pitch are not stored.  Cached with
+// the maps of C; false if the driver does not take this geometry.
+bool cached_partial_map(State& S, Plan* pl, float* base, int64_t M, int64_t Np, int64_t P_k, CUtensorMap* out)
+{
+    std::lock_guard<std::mutex> lock(pl->mu);
+    if (S.map_cache.load(std::memory_order_relaxed) != 0)
+        for (const MapSlot& sl : pl->maps[kMapC])
+            if (sl.matches(base, Np, P_k, M, 32, 32, 1)) { *out = sl.map[0]; return true; }
+    S.map_encodes.fetch_add(1, std::memory_order_relaxed);
+    const cuuint64_t gdim[3] = {(cuuint64_t)Np, (cuuint64_t)M, (cuuint64_t)P_k};
+    const cuuint64_t gstride[2] = {(cuuint64_t)Np * 4, (cuuint64_t)(M * Np) * 4};
+    const cuuint32_t box[3] = {32, 32, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    if (S.encode(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, gdim, gstride, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                 CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return false;
+    MapSlot& sl = take_slot(pl, kMapC);
+    sl.map.assign(1, *out);
+    sl.ptr = base; sl.pitch = Np; sl.inner = P_k; sl.outer = M;
+    sl.box_inner = 32; sl.box_outer = 32; sl.count = 1;
+    return true;
+}
+
 // Per-class maps of a row-major matrix (rows x cols, 16-byte aligned base): class j holds the rows with
 // row % ncls == j, which all start the same distance sigma_j (elements) after an `align`-byte boundary
 // (ncls * cols * 2 is a multiple of `align`: ncls = 8 for 16 bytes, 16 for 32).  Map j: base rounded down
@@ -1310,6 +1333,11 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
         p.b_tx_bytes = b_mn ? ((bn_cta + 63) / 64) * 64 * b_box_k * 2 : bn_cta * kUmmaBK * 2;
     }
     p.idesc = umma_idesc(s.dtype, a_mn, b_mn, 128 * cg, c.BN);
+    // Partials of plain tiles leave through TMA where the ring holds a CTA's whole fp32 tile (and the driver takes their geometry), from 65 rows
+    // on: 112 x 368 x 21632 13.4 -> 12.7 us, 82 x 21 x 218664 25.9 -> 25.1, 300 x 4096 x 4096 22.0 -> 20.5, but 64 x 224 x 39808 11.5 -> 11.7 and
+    // 32 x 144 x 35648 11.2 -> 11.3 (few rows are few stores)
+    p.part_tma = partials && !classesA && !kclsB && a_box_rows > 64 && (int64_t)p.stages * (p.a_tx_bytes + (int64_t)round_up(c.BN / cg, 64) * 64 * 2) >= (int64_t)c.BN * 512 &&
+                 cached_partial_map(S, pl, partial, s.M, partial_pitch(s.N), p.P_k, &maps.c[0]) ? 1 : 0;
     p.C = C;
     p.partial = partial;
     p.Np = (int)partial_pitch(s.N);

@@ -339,7 +339,11 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
         const double b_bytes = 2.0 * KN * rB * (kclasses ? c.BN / (c.BN - 8.0) : 1.0);
         t_b_extra = b_bytes / bw * (1.0 / std::max(eff, 0.3) - 1.0) * 1e6;
     }
-    const double t_hbm = c.hbm_bytes / bw * 1e6 + t_b_extra - c.t_pro_us - c.t_epi_us;
+    double t_hbm = c.hbm_bytes / bw * 1e6 + t_b_extra - c.t_pro_us - c.t_epi_us;
+    // a long contraction of a few tiles streams both operands; each further tile that reads a row block from L2 slows that stream a little
+    // (256 x 256 x 262144 in 64 splits: 52.0 us on one 256 x 256 pair tile, 55.8 on two 128 x 256 tiles that both read B)
+    if (c.P_k > 1 && !c.fused && !kclasses && c.srcA != ADAPT_SRC_TMA_CLASSES)
+        t_hbm *= 1.0 + cal.l2_reread_cost * std::min(1.0, (MK * c.P_n + KN * c.P_m) / (MK + KN) - 1.0);
     c.t_main_us = std::max(pipe, t_hbm);
     // boxes of B that lie wholly beyond N are fetched all the same (zero fill): a tile narrower than BN pays
     // for them in TMA work the terms above do not see (61370 x 32 x 85272: BN 128 -> 64 is 20 % faster)

@@ -202,6 +202,12 @@ __device__ __forceinline__ void tma_store_3d(const void* tmap, uint32_t src, int
                  ::"l"(tmap), "r"(src), "r"(x), "r"(y), "r"(z)
                  : "memory");
 }
+__device__ __forceinline__ void tma_store_3d_hint(const void* tmap, uint32_t src, int x, int y, int z, uint64_t policy)
+{
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group.L2::cache_hint [%0, {%2, %3, %4}], [%1], %5;"
+                 ::"l"(tmap), "r"(src), "r"(x), "r"(y), "r"(z), "l"(policy)
+                 : "memory");
+}
 // One 32-byte store (a whole sector); p must be 32-byte aligned.
 __device__ __forceinline__ void st_global_v8_hint(void* p, const uint32_t* r, uint64_t policy)
 {

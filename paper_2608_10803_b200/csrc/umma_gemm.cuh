@@ -64,6 +64,7 @@ struct UmmaParams {
                                      //     neighbouring column blocks of the same rows, and a CTA's consecutive class tiles share their maps)
     int c_hint;                      // TMA stores of C carry an evict-first L2 policy
     int part_hint;                   // fp32 partials are stored with an evict-last L2 policy (they fit in L2)
+    int part_tma;                    // the partials of a CTA's last unit leave through TMA stores (c[0] is their map), staged in its ring
     int c_sigma[16];                 // halo class tiles: shift (elements) of C's row class j against its 32-byte aligned base
     int c_extent[16];                // ... and the elements of a shifted row of that class that lie in whole 32-byte units
     // stream-K (SK kernels): the first sk_tiles tiles are cut into k-block ranges shared evenly by all slots (a slot is a
@@ -429,7 +430,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
         if (first_unit < p.num_units) decode_unit(p, first_unit, mb0, nb0, sp0);
         ptx::prefetch_tensormap(&maps.a[A_CLS ? (mb0 & (NCLS - 1)) : 0]);
         ptx::prefetch_tensormap(&maps.b[(B_SPLIT || B_CLS) ? (sp0 & 7) : 0]);
-        if (p.c_mode != 0) ptx::prefetch_tensormap(&maps.c[A_CLS ? (mb0 & (NCLS - 1)) : 0]);
+        if (p.c_mode != 0 || p.part_tma) ptx::prefetch_tensormap(&maps.c[A_CLS ? (mb0 & (NCLS - 1)) : 0]);
     }
     if (warp == 1) {
         ptx::tmem_alloc<CG>(tmem_slot, TMEM_COLS);
@@ -1267,6 +1268,11 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                         }
                     }
                 }
+                // The partials of the CTA's last unit are staged in the ring: no load is to come and the MMAs have read all of it (their
+                // commit is what this warp has waited for).  One box of 32 rows x 32 columns per warp and 32 columns, all of them in flight.
+                // The drain of a long contraction is not hidden by anything: stored by the threads, 32 rows of 32 bytes an instruction, a
+                // 128 x 256 tile took about 7 us (256 x 256 x 262144 on pair tiles in 64 splits: 53.0 us, 49.6 now).
+                const bool by_tma = !B_CLS && !B_SPLIT && !A_CLS && p.part_tma && unit + unit_step >= p.num_units;
 #pragma unroll 1
                 for (int c0 = 0; !B_CLS && !B_SPLIT && c0 < TILE_N; c0 += 32) {
                     if (n0 + c0 >= p.N) break;                       // uniform across the warp
@@ -1274,6 +1280,21 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                     uint32_t r[32];
                     ptx::tmem_ld_32x32(t_row + (uint32_t)c0, r);
                     ptx::tmem_ld_wait();
+                    if (by_tma) {
+                        if (row_base + 32 * q >= p.M) continue;      // no row of this warp exists (uniform)
+                        uint8_t* box = gen_base + (size_t)((c0 >> 5) * 4 + q) * 4096;
+#pragma unroll
+                        for (int c = 0; c < 8; ++c)
+                            *reinterpret_cast<uint4*>(box + lane * 128 + ((c ^ (lane & 7)) << 4)) = make_uint4(r[4 * c], r[4 * c + 1], r[4 * c + 2], r[4 * c + 3]);
+                        ptx::fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            if (p.part_hint) ptx::tma_store_3d_hint(&maps.c[0], ptx::smem_u32(box), n0 + c0, row_base + 32 * q, split, part_policy);
+                            else ptx::tma_store_3d(&maps.c[0], ptx::smem_u32(box), n0 + c0, row_base + 32 * q, split);
+                            ptx::bulk_commit();
+                        }
+                        continue;
+                    }
                     if (!row_ok) continue;
                     const int col = n0 + c0;
                     float* prow = p.partial + ((size_t)split * p.M + row) * p.Np + col;
