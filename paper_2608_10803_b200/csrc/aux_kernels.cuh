@@ -222,12 +222,17 @@ regroup_a_kernel(const unsigned short* __restrict__ A, unsigned short* __restric
 template <bool SHARED>
 __global__ void __launch_bounds__(256)
 splitk_reduce_kernel(const float* __restrict__ partial, unsigned short* __restrict__ C,
-                     int M, int N, int Np, int P_k, int dtype, const ReduceEpilogue ep, int groups_shared)
+                     int M, int N, int Np, int P_k, int dtype, const ReduceEpilogue ep, int groups_shared, int prologue)
 {
     __shared__ float4 s_sum[SHARED ? 256 : 1];
     const int groups = SHARED ? groups_shared : 1;
-    pdl_launch_dependents();
     pdl_wait();
+    // The next kernel is let in now, not first thing: while the GEMM in front of this one still runs, what starts early finds room on the few SMs
+    // without a GEMM CTA only, and all of a regrouping or re-pitching kernel that had started there ran there, beside a hundred idle SMs
+    // (34 x 102 x 35284, 112 k-class splits, in a row: 26.0 -> 13.1 us).  A call that has such a prologue (the next one will most likely be of its
+    // kind) lets the next kernel in at the end: its CTAs then spread over empty SMs, with the L1 they live on (76 x 371 x 37184 33.2 -> 27.0 us, 30.0 when
+    // let in here; 288 x 214 x 36999 40.4 -> 33.7, 40.0; without a prologue 4 x 2688 x 1728 7.7 -> 7.5, 8.6 at the end).
+    if (!prologue) pdl_launch_dependents();
     const int quads = Np >> 2;                              // columns in fours
     const int64_t total = (int64_t)M * quads;
     const int64_t slab = (int64_t)M * Np;
@@ -284,6 +289,7 @@ splitk_reduce_kernel(const float* __restrict__ partial, unsigned short* __restri
                 if (n + j < N) dst[j] = float_to_16(a[j], dtype);
         }
     }
+    if (prologue) pdl_launch_dependents();
 }
 
 // ---- CUDA-core tile GEMM: 64 x 64 tile, 256 threads, 4 x 4 outputs per thread ---------------------
