@@ -68,12 +68,13 @@ def test_k_ranges(K, dtype):
 @pytest.mark.parametrize("lB", [0, 1])
 @pytest.mark.parametrize("addmm", [None, "bias", "matrix"])
 def test_layouts_edges_and_fused_add(lA, lB, addmm):
-    for M, N, K in [(257, 16, 80), (264, 144, 328), (512, 512, 264), (776, 240, 392), (1288, 1040, 136)]:
+    # (a matrix D: tall tiles from K = 1024 on)
+    for M, N, K in [(257, 16, 80), (264, 144, 328), (512, 512, 264), (776, 240, 392), (1288, 1040, 136), (300, 272, 1032), (1288, 528, 1096)]:
         check(M, N, K, ab.BF16 if lA else ab.F16, lA, lB, addmm)
 
 
 # row classes: K off 16-byte boundaries; an odd number of 2048-row groups, a last group of a few rows
-@pytest.mark.parametrize("shape", [(2056, 256, 203), (4096, 272, 131), (4500, 688, 333), (6150, 64, 517), (9000, 48, 75)])
+@pytest.mark.parametrize("shape", [(2056, 256, 203), (4096, 272, 131), (4500, 688, 333), (6150, 64, 517), (9000, 48, 75), (4500, 80, 1037)])
 @pytest.mark.parametrize("addmm", [None, "matrix"])
 def test_row_classes(shape, addmm):
     M, N, K = shape
