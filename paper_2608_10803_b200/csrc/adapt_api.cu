@@ -1791,14 +1791,13 @@ struct BatchOps {
     }
     adapt_status_t group(const std::vector<int64_t>& calls, int lane)
     {
-        struct Entry { GroupItem item; int chain; } entry[kGroupMax];
+        GroupEntry entry[kGroupMax];
         size_t n = 0;
         for (int64_t i : calls) {
             entry[n].chain = group_item(plans[i]->s, plans[i]->c, A[i], B[i], C[i], &entry[n].item);
             ++n;
         }
-        // longest chains first: what starts last is short
-        std::stable_sort(entry, entry + n, [](const Entry& x, const Entry& y) { return x.chain > y.chain; });
+        group_order(entry, n, S.machine.n_sm);
         const Shape& s = plans[calls[0]]->s;
         GroupParams p;
         group_clear(p);

@@ -55,6 +55,7 @@ struct ClusterParams {
     int P_n;                     // tiles along n
     int CS;                      // CTAs per cluster = pieces of the k range
     int k_per_cta;               // k values per CTA, a multiple of 16
+    int share_log2, q;           // two-group tiles: the tile's pieces are shared by 2^share_log2 CTAs of a cluster, of which this is the q-th
     int ring;                    // raw stages in flight per CTA (1..kClusterMaxRing)
     int prefetch;                // L2 prefetch of the ring's stages ahead of the dependency wait
     int aligned;                 // bit 0: every row of A starts on a 16-byte boundary, bit 1: every row of B
@@ -105,7 +106,9 @@ __device__ __forceinline__ float4 cl_load4(uint32_t local_addr, uint32_t rank)
 // A_KC: A is row-major (k contiguous); B_KC: B is column-major (k contiguous).
 //
 // SEQ: one CTA takes all CS pieces of the tile's k range, in two groups of warps; else it takes the piece of its cluster rank.
-template <bool A_KC, bool B_KC, bool BF16, bool SEQ>
+// SHARED: with share = 2^share_log2 > 1 CTAs to a SEQ tile, group g of CTA q takes the pieces q + share * g + 2 * share * i (i = 0, or 0 and 1) and keeps
+// their sums apart; they meet in shared memory and are added over the cluster in the order of a tile of one CTA: even pieces, odd pieces, both.
+template <bool A_KC, bool B_KC, bool BF16, bool SEQ, bool SHARED = false>
 __device__ __forceinline__ void cluster_tile_body(const ClusterParams& p, int m0, int n0, unsigned char* s_dyn)
 {
     constexpr int ROW = kClusterPitch * 2, OPND = 64 * ROW, STAGE = 2 * OPND;
@@ -122,18 +125,20 @@ __device__ __forceinline__ void cluster_tile_body(const ClusterParams& p, int m0
     // ---- this group's stages: the first k value, the values of k left in its piece, and how both move on
     const uint32_t rank = !SEQ && p.CS > 1 ? cl_rank() : 0u;
     const int pieces = SEQ ? p.CS : 1;
+    const int share_log2 = SHARED ? p.share_log2 : 0, share = 1 << share_log2, q_of_tile = SHARED ? p.q : 0;
     const bool by_stage = !SEQ || pieces == 1;                          // one piece: SEQ groups take alternate stages
     const int step_k = SEQ && by_stage ? 2 * kClusterKS : kClusterKS;
     const int spp = by_stage ? 1 : (p.k_per_cta + kClusterKS - 1) / kClusterKS;        // stages of a whole piece
-    const int jump_k = 2 * p.k_per_cta - (spp - 1) * kClusterKS;        // from the last stage of a piece to the piece after next
-    int next_piece = SEQ ? (by_stage ? 0 : grp * p.k_per_cta) : (int)rank * p.k_per_cta;
+    const int jump_k = 2 * share * p.k_per_cta - (spp - 1) * kClusterKS;        // from the last stage of a piece to this group's next one
+    int next_piece = SEQ ? (by_stage ? 0 : ((grp << share_log2) + q_of_tile) * p.k_per_cta) : (int)rank * p.k_per_cta;
     const int k_begin = next_piece + (SEQ && by_stage ? grp * kClusterKS : 0);
     auto left_of = [&](int k) -> int { return min(p.K - k, p.k_per_cta); };             // ... of a piece that starts at k
     const int left0 = SEQ && by_stage ? p.K - k_begin : left_of(k_begin);
     auto stages_of = [&](int g) -> int {
         if (by_stage) { const int l = SEQ ? p.K - g * kClusterKS : left0; return l > 0 ? (l + step_k - 1) / step_k : 0; }
-        const int n = (pieces - g + 1) / 2, last = pieces - 1;          // pieces g, g + 2, ...; the very last one may be short
-        return (last & 1) == g ? (n - 1) * spp + (p.K - last * p.k_per_cta + kClusterKS - 1) / kClusterKS : n * spp;
+        const int first = (g << share_log2) + q_of_tile;                // first, first + 2 * share, ...; the very last piece may be short
+        const int n = (pieces - first + 2 * share - 1) >> (share_log2 + 1), last = first + (n - 1) * 2 * share;
+        return last == pieces - 1 ? (n - 1) * spp + (p.K - last * p.k_per_cta + kClusterKS - 1) / kClusterKS : n * spp;
     };
     const int n_stages = stages_of(grp);
     const bool al_a = p.aligned & 1, al_b = p.aligned & 2;
@@ -193,7 +198,7 @@ __device__ __forceinline__ void cluster_tile_body(const ClusterParams& p, int m0
         int move = step_k;
         if (!by_stage && is_left <= 0) {                                // on to this group's next piece
             move = jump_k;
-            is_next += 2 * p.k_per_cta;
+            is_next += 2 * share * p.k_per_cta;
             is_left = left_of(is_next);
         }
         src_a += unit_a * move;
@@ -301,13 +306,15 @@ __device__ __forceinline__ void cluster_tile_body(const ClusterParams& p, int m0
         if (++slot == S) slot = 0;
         left -= step_k;
         if (!by_stage && left <= 0) {
+            if (!SHARED || share == 1 || s + 1 < n_stages || n_stages <= spp) {     // (shared tiles: a second piece stays in acc)
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+                for (int i = 0; i < 2; ++i)
 #pragma unroll
-                for (int j = 0; j < NJ; ++j)
+                    for (int j = 0; j < NJ; ++j)
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) { tot[i][j][e] += acc[i][j][e]; acc[i][j][e] = 0.f; }
-            next_piece += 2 * p.k_per_cta;
+                        for (int e = 0; e < 4; ++e) { tot[i][j][e] += acc[i][j][e]; acc[i][j][e] = 0.f; }
+            }
+            next_piece += 2 * share * p.k_per_cta;
             left = left_of(next_piece);
         }
     }
@@ -346,6 +353,58 @@ __device__ __forceinline__ void cluster_tile_body(const ClusterParams& p, int m0
         }
     };
 
+    // four neighbouring outputs, rounded and stored
+    auto store4 = [&](int m, int n, const float (&o)[4]) {
+        unsigned short* dst = p.C + (int64_t)m * p.N + n;
+        unsigned short h[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) h[j] = n + j < p.N ? float_to_16(finish(o[j], m, n + j), BF16 ? 1 : 0) : 0;
+        if (n + 4 <= p.N && (reinterpret_cast<uintptr_t>(dst) & 7) == 0) {
+            *reinterpret_cast<uint2*>(dst) = make_uint2((uint32_t)h[0] | ((uint32_t)h[1] << 16), (uint32_t)h[2] | ((uint32_t)h[3] << 16));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (n + j < p.N) dst[j] = h[j];
+        }
+    };
+
+    if (SHARED && share > 1) {
+        // piece q + share * g + 2 * share * i of this CTA is buffer g + 2 i: the sums of a group's first piece are in tot, a second one's in acc
+        auto put = [&](int buffer, const float (&v)[2][NJ][4]) {
+            float* s = reinterpret_cast<float*>(s_dyn + buffer * kClusterStageBytes);
+#pragma unroll
+            for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+                for (int nj = 0; nj < NJ; ++nj)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        *reinterpret_cast<float2*>(&s[(m_w + 16 * mi + g + 8 * h) * kClusterCPitch + n_w + 8 * nj + 2 * t]) = make_float2(v[mi][nj][2 * h], v[mi][nj][2 * h + 1]);
+        };
+        __syncthreads();
+        put(grp, tot);
+        if (n_stages > spp) put(grp + 2, acc);
+        cl_sync();
+        const uint32_t base_rank = cl_rank() - (uint32_t)p.q;
+        const int rows_mine = kClusterTile >> p.share_log2;
+        for (int e = tid; e < rows_mine * 16; e += kClusterThreads) {
+            const int row = p.q * rows_mine + (e >> 4), col = (e & 15) * 4;
+            const int m = m0 + row, n = n0 + col;
+            if (m >= p.M || n >= p.N) continue;
+            float4 sum[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+            const uint32_t addr = ptx::smem_u32(s_dyn) + (uint32_t)(row * kClusterCPitch + col) * 4u;
+            for (int pc0 = 0; pc0 < pieces; pc0 += 4) {        // four remote reads in flight (pieces: 4, 8 or 16)
+                float4 v[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = cl_load4(addr + (uint32_t)(((pc0 + j) >> p.share_log2) * kClusterStageBytes), base_rank + (uint32_t)((pc0 + j) & (share - 1)));
+#pragma unroll
+                for (int j = 0; j < 4; ++j) { sum[j & 1].x += v[j].x; sum[j & 1].y += v[j].y; sum[j & 1].z += v[j].z; sum[j & 1].w += v[j].w; }
+            }
+            const float o[4] = {sum[0].x + sum[1].x, sum[0].y + sum[1].y, sum[0].z + sum[1].z, sum[0].w + sum[1].w};
+            store4(m, n, o);
+        }
+        cl_sync();                                             // no CTA leaves while a peer still reads its sums
+        return;
+    }
     if (SEQ) {
         // The two groups' sums: each group adds and stores half of its warps' rows (the 16 x 32 blocks mi = group) and hands the other
         // half over through shared memory.  With nothing on the second group's side the first one stores all.
@@ -414,18 +473,8 @@ __device__ __forceinline__ void cluster_tile_body(const ClusterParams& p, int m0
             for (int q = 0; q < 4; ++q)
                 if (q0 + q < p.CS) { sum[q & 1].x += v[q].x; sum[q & 1].y += v[q].y; sum[q & 1].z += v[q].z; sum[q & 1].w += v[q].w; }
         }
-        unsigned short* dst = p.C + (int64_t)m * p.N + n;
         const float o[4] = {sum[0].x + sum[1].x, sum[0].y + sum[1].y, sum[0].z + sum[1].z, sum[0].w + sum[1].w};
-        unsigned short h[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) h[j] = n + j < p.N ? float_to_16(finish(o[j], m, n + j), BF16 ? 1 : 0) : 0;
-        if (n + 4 <= p.N && (reinterpret_cast<uintptr_t>(dst) & 7) == 0) {
-            *reinterpret_cast<uint2*>(dst) = make_uint2((uint32_t)h[0] | ((uint32_t)h[1] << 16), (uint32_t)h[2] | ((uint32_t)h[3] << 16));
-        } else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (n + j < p.N) dst[j] = h[j];
-        }
+        store4(m, n, o);
     }
     // no CTA may leave while a peer still reads its partial tile
     cl_sync();
@@ -507,6 +556,7 @@ inline adapt_status_t launch_cluster(const Shape& s, const Config& c, const void
     p.CS = c.cluster;
     p.k_per_cta = (int)round_up(ceil_div(s.K, c.cluster), 16);
     const bool seq = cluster_two_groups(s.K, c.cluster);
+    p.share_log2 = p.q = 0;
     p.ring = seq ? cluster_alone_ring(s.K) : c.stages;
     p.prefetch = prefetch;
     p.aligned = (rows_aligned16(A, p.lda) ? 1 : 0) | (rows_aligned16(B, p.ldb) ? 2 : 0);

@@ -5,8 +5,8 @@
 // Here the 64 x 64 tiles of all entries run side by side, one per CTA.  An entry keeps the arithmetic of its own plan:
 //   pieces > 0: the one-launch cluster kernel's tiles.  The CTA walks the plan's pieces of the k range and adds
 //               their sums in the same order: the bits of the call made alone, where each piece has a CTA of its own.
-//               (With a tile of one group of warps, clusters of four CTAs with the pieces spread over them took 53 us for those
-//               48 layers, one CTA per tile 40 us: the exchange of the partial tiles cost more than the shorter chains saved.)
+//               The tiles with the longest chains are shared by two or four CTAs of a cluster (group_share).  (Clusters of four for
+//               every tile, the pieces of one group of warps spread over them, took 53 us for those 48 layers, one CTA per tile 40 us.)
 //   pieces = 0: the CUDA-core kernel's tiles (a few 16-k steps).
 // The list travels in the kernel's parameters, so nothing is copied to the device and the launch can be captured.
 #pragma once
@@ -17,27 +17,31 @@
 
 namespace adapt {
 
+enum { kGroupPlain = 0, kGroupShort, kGroupShared };
+
 // What bounds it: latency with two CTAs per SM.  Those 48 layers take 31.0 us, 21.7 for the 47 that share the launch and 8.7 for the one
 // with a launch of its own (each by itself); the 762 tiles are 2.6 rounds of CTAs whose longest chain is 8 stages (0.33 us per aligned 64 k
 // values and group of warps, 0.6 off 16-byte boundaries).  Profiled: 13.7 warps per SM (128 registers a thread), issue slots 35 % used,
 // stalls on fixed latencies and shared memory, DRAM 4 %.  The deepest entries come first and the ring is no deeper than the list needs.
-// SHORT: every item has K <= 64 in one piece (one stage): no two-group tiles, so fewer registers and three CTAs per SM instead of two
+// FORM kGroupShort: every item has K <= 64 in one piece (one stage): no two-group tiles, so fewer registers and three CTAs per SM instead of two
 // (96 products of 128 x 128 x 64 in one launch: 6.6 us with the general kernel, 4.4 with this one, 266 as 96 launches).
-template <bool A_KC, bool B_KC, bool BF16, bool SHORT>
-__global__ void __launch_bounds__(kClusterThreads, SHORT ? 3 : 2)
+// kGroupShared: clusters, with the tiles of some items shared by several CTAs (an instantiation of its own: the other lists' tiles took 4 % longer with
+// this code beside theirs).
+template <bool A_KC, bool B_KC, bool BF16, int FORM>
+__global__ void __launch_bounds__(kClusterThreads, FORM == kGroupShort ? 3 : 2)
 group_gemm_kernel(const __grid_constant__ GroupParams p)
 {
     extern __shared__ __align__(128) unsigned char s_dyn[];
     pdl_launch_dependents();
     const int t_all = (int)blockIdx.x;
-    int lo = 0, hi = p.count - 1;                           // the first item whose tiles end beyond this one
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (t_all < p.item[mid].tile_end) hi = mid; else lo = mid + 1;
+    GroupPlace at;
+    const bool work = group_place(p, t_all, at);
+    if (FORM == kGroupShared && !work) {                    // a CTA that only fills a cluster
+        if (t_all < p.sync_ctas) { cl_sync(); cl_sync(); }  // ... of shared tiles: both of their barriers
+        return;
     }
-    const GroupItem& it = p.item[lo];
-    const int local = t_all - (lo > 0 ? p.item[lo - 1].tile_end : 0);
-    const int entry = local / it.tiles, tile = local - entry * it.tiles;
+    const GroupItem& it = p.item[at.item];
+    const int entry = at.entry, tile = at.tile;
     const int m0 = (tile / it.P_n) * kClusterTile, n0 = (tile % it.P_n) * kClusterTile;
     const unsigned short* A = it.A + entry * p.sa;
     const unsigned short* B = it.B + entry * p.sb;
@@ -64,30 +68,32 @@ group_gemm_kernel(const __grid_constant__ GroupParams p)
     q.k_per_cta = it.k_per_piece;
     q.ring = p.ring;
     q.prefetch = p.prefetch;
+    q.share_log2 = it.share_log2; q.q = at.q;
     q.aligned = (rows_aligned16(A, q.lda) ? 1 : 0) | (rows_aligned16(B, q.ldb) ? 2 : 0);
     q.ep.D = nullptr;
-    cluster_tile_body<A_KC, B_KC, BF16, !SHORT>(q, m0, n0, s_dyn);
+    cluster_tile_body<A_KC, B_KC, BF16, FORM != kGroupShort, FORM == kGroupShared>(q, m0, n0, s_dyn);
 }
 
 typedef void (*GroupKernel)(const GroupParams);
 
-template <bool SHORT>
+template <int FORM>
 inline GroupKernel group_pick(bool a_kc, bool b_kc, bool bf16)
 {
     if (bf16) {
-        if (a_kc) return b_kc ? group_gemm_kernel<true, true, true, SHORT> : group_gemm_kernel<true, false, true, SHORT>;
-        return b_kc ? group_gemm_kernel<false, true, true, SHORT> : group_gemm_kernel<false, false, true, SHORT>;
+        if (a_kc) return b_kc ? group_gemm_kernel<true, true, true, FORM> : group_gemm_kernel<true, false, true, FORM>;
+        return b_kc ? group_gemm_kernel<false, true, true, FORM> : group_gemm_kernel<false, false, true, FORM>;
     }
-    if (a_kc) return b_kc ? group_gemm_kernel<true, true, false, SHORT> : group_gemm_kernel<true, false, false, SHORT>;
-    return b_kc ? group_gemm_kernel<false, true, false, SHORT> : group_gemm_kernel<false, false, false, SHORT>;
+    if (a_kc) return b_kc ? group_gemm_kernel<true, true, false, FORM> : group_gemm_kernel<true, false, false, FORM>;
+    return b_kc ? group_gemm_kernel<false, true, false, FORM> : group_gemm_kernel<false, false, false, FORM>;
 }
 
 inline cudaError_t group_set_attributes()
 {
     for (int v = 0; v < 8; ++v) {
-        cudaError_t e = cudaFuncSetAttribute(group_pick<false>(v & 1, v & 2, v & 4), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             cluster_seq_smem_bytes(kClusterSeqRing));
-        if (e != cudaSuccess) return e;
+        for (GroupKernel k : {group_pick<kGroupPlain>(v & 1, v & 2, v & 4), group_pick<kGroupShared>(v & 1, v & 2, v & 4)}) {
+            const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, cluster_seq_smem_bytes(kClusterSeqRing));
+            if (e != cudaSuccess) return e;
+        }
     }
     return cudaSuccess;
 }
@@ -98,17 +104,24 @@ inline cudaError_t launch_group(GroupParams& p, bool a_kc, bool b_kc, cudaStream
     const GroupForm form = group_form(p);
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)p.item[p.count - 1].tile_end, 1, 1);
+    cfg.gridDim = dim3((unsigned)group_grid(p), 1, 1);
     cfg.blockDim = dim3(kClusterThreads, 1, 1);
     cfg.dynamicSmemBytes = (size_t)form.smem_bytes;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     pdl_attribute(&attr[0]);
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = kGroupCluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = p.sync_ctas > 0 ? 2 : 1;
     void* args[1] = {&p};
     const size_t bytes[1] = {sizeof(p)};
-    return launch_exc(&cfg, (const void*)(form.short_k ? group_pick<true>(a_kc, b_kc, p.dtype != 0) : group_pick<false>(a_kc, b_kc, p.dtype != 0)), args, bytes, 1);
+    const bool bf16 = p.dtype != 0;
+    const GroupKernel k = p.sync_ctas > 0 ? group_pick<kGroupShared>(a_kc, b_kc, bf16) : form.short_k ? group_pick<kGroupShort>(a_kc, b_kc, bf16)
+                                                                                                     : group_pick<kGroupPlain>(a_kc, b_kc, bf16);
+    return launch_exc(&cfg, (const void*)k, args, bytes, 1);
 }
 
 }  // namespace adapt

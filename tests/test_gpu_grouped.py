@@ -57,6 +57,35 @@ def test_grouped_list_gives_the_bits_of_single_calls(layouts, offset):
     assert {1, 4, 8} <= pieces
 
 
+@pytest.mark.parametrize("layouts", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("dtype", [ab.F16, ab.BF16])
+def test_tiles_shared_by_several_ctas_give_the_bits_of_single_calls(layouts, dtype):
+    """Short lists whose longest k chains are shared by two CTAs (four pieces) or four (eight, sixteen), beside tiles that are not; ragged
+    last pieces, odd numbers of shared tiles, tiles of one row and column, and a list that only holds shared tiles."""
+    init()
+    lists = [[(84, 39, 1014), (20, 30, 40)], [(504, 209, 576), (100, 100, 100), (30, 7, 20)], [(64, 64, 1024), (65, 63, 1000), (17, 763, 618), (105, 845, 611), (1, 1, 500)],
+             [(38, 48, 787), (48, 38, 808), (1, 70, 790)], [(64, 128, 1008), (16, 200, 520), (129, 1, 400), (300, 200, 50), (10, 10, 65), (33, 65, 130), (7, 9, 11), (40, 342, 267)]]
+    seen = set()
+    for k, shapes in enumerate(lists):
+        calls = []
+        for i, (M, N, K) in enumerate(shapes):
+            p = ab.adapt_matmul_plan(M, N, K, dtype, *layouts)
+            assert ab.adapt_plan_info(p).family in (ab.FAM_CLUSTER, ab.FAM_SIMT), (M, N, K)
+            seen.add(ab.adapt_plan_info(p).cluster)
+            A, B = offset_operand(M, K, 900 + 2 * i, dtype, i % 3), offset_operand(K, N, 901 + 2 * i, dtype, k % 2)
+            calls.append((p, A, B) + tuple(torch.full((M * N,), float("nan"), dtype=A.dtype, device="cuda") for _ in range(2)))
+        for p, A, B, C1, _ in calls:
+            ab.adapt_matmul(p, A.data_ptr(), B.data_ptr(), C1.data_ptr(), stream())
+        launches = ab.adapt_launch_count()
+        ab.adapt_matmul_batch([c[0] for c in calls], *([c[j].data_ptr() for c in calls] for j in (1, 2, 4)), stream())
+        assert ab.adapt_launch_count() - launches == 1
+        torch.cuda.synchronize()
+        ab.adapt_poll_device_status(stream())
+        for (_, _, _, C1, C2), shape in zip(calls, shapes):
+            assert torch.equal(C1.view(torch.int16), C2.view(torch.int16)), shape
+    assert {1, 4, 8, 16} <= seen
+
+
 def test_grouped_list_keeps_the_order_of_dependent_calls():
     """Calls that read what an earlier call of the list wrote, overwrite what it read, or write the same output."""
     init()

@@ -95,3 +95,78 @@ int main()
 }
 """)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+SHARED = r"""
+#include <cstdio>
+#include <map>
+#include <random>
+#include <vector>
+#include "group_plan.h"
+using namespace adapt;
+
+int main()
+{
+    std::mt19937 rng(7);
+    int bad = 0, shared_lists = 0, fillers = 0;
+    for (int trial = 0; trial < 3000; ++trial) {
+        const int n = 1 + rng() % (trial % 3 ? 6 : 64);
+        std::vector<GroupEntry> e(n);
+        for (GroupEntry& x : e) {
+            const int pieces[] = {0, 1, 1, 2, 4, 4, 8, 16};
+            x.item = GroupItem();
+            x.item.pieces = (short)pieces[rng() % 8];
+            x.item.k_per_piece = x.item.pieces ? 16 * (1 + rng() % 12) : 0;
+            x.item.tiles = 1 + rng() % 30;
+            x.item.K = x.item.pieces * x.item.k_per_piece;
+            const int spp = (x.item.k_per_piece + 63) / 64;
+            x.chain = x.item.pieces <= 1 ? 1 + rng() % 3 : x.item.pieces / 2 * spp;
+            x.item.M = x.chain;                                     // (kept to compare with)
+        }
+        group_order(e.data(), n, 148);
+        int64_t ctas = 0, shared = 0;
+        for (const GroupEntry& x : e) {
+            const int share = 1 << x.item.share_log2;
+            ctas += x.item.tiles * share;
+            shared += share > 1;
+            // no more than two pieces for a group of warps of a shared tile, and the chain that is left holds them
+            if (share > 1 ? x.item.pieces > 4 * share || x.item.pieces < 2 * share || x.chain >= x.item.M || x.chain < x.item.pieces / (2 * share) : x.chain != x.item.M) ++bad;
+        }
+        if (shared && ctas > 4 * 148) ++bad;
+        GroupParams p;
+        group_clear(p);
+        for (GroupEntry& x : e) group_add(p, x.item, x.chain);
+        const int grid = group_grid(p);
+        shared_lists += p.sync_ctas > 0;
+        if (p.sync_ctas % kGroupCluster || (p.sync_ctas && grid % kGroupCluster)) ++bad;
+        std::map<std::pair<int, int>, std::vector<int>> who;       // (item, tile) -> CTAs in order of q
+        for (int cta = 0; cta < grid; ++cta) {
+            GroupPlace w;
+            if (!group_place(p, cta, w)) { ++fillers; continue; }
+            std::vector<int>& v = who[{w.item, w.tile}];
+            if ((int)v.size() != w.q || w.entry != 0 || w.tile >= p.item[w.item].tiles) ++bad;
+            v.push_back(cta);
+            // the CTAs of a shared tile wait at two cluster barriers, and so do all of their cluster; no others do
+            if ((p.item[w.item].share_log2 > 0) != (cta < p.sync_ctas)) ++bad;
+        }
+        int tiles = 0;
+        for (int i = 0; i < p.count; ++i) tiles += p.item[i].tiles;
+        if ((int)who.size() != tiles) ++bad;
+        for (auto& kv : who) {
+            const int share = 1 << p.item[kv.first.first].share_log2;
+            if ((int)kv.second.size() != share || kv.second.back() - kv.second[0] != share - 1) ++bad;
+            if (share > 1 && kv.second[0] / kGroupCluster != kv.second.back() / kGroupCluster) ++bad;
+            // buffers of the pieces' sums: two per piece of a group of warps, inside the rings
+            if (share > 1 && p.item[kv.first.first].pieces / share * kClusterStageBytes > group_form(p).smem_bytes) ++bad;
+        }
+        if (group_form(p).short_k && p.sync_ctas) ++bad;
+    }
+    printf("%d lists with shared tiles, %d CTAs without work, %d wrong\n", shared_lists, fillers, bad);
+    return bad || shared_lists < 500 || fillers < 100;
+}
+"""
+
+
+def test_shared_tiles_get_their_ctas_in_one_cluster(tmp_path):
+    r = build_and_run(tmp_path, SHARED)
+    assert r.returncode == 0, r.stdout + r.stderr
