@@ -128,7 +128,7 @@ typedef struct adapt_plan_info_s {
 } adapt_plan_info_t;
 
 /* TilingKey bit layout (Section 3.2 asks only for "a compact 64-bit key"; the fields are this
- * library's): [63:62] taxonomy class, [61:59] family, [58:54] BM/16, [53:48] BN/16,
+ * library's): [63:62] taxonomy class, [61:59] family, [58:54] BM/16 (0: 512), [53:48] BN/16,
  * [47:46] log2(BK/16), [45:42] stages, [41:32] P_k, [31] persistent tile loop,
  * [30:29] srcA, [28:27] srcB, [26] dtype, [25] layoutA, [24] layoutB, [23:22] log2(cluster) mod 4,
  * [21] log2(cluster) / 4, [20] fused in-cluster split-K reduction, [19] stream-K, [18:0] zero. */
