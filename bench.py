@@ -719,6 +719,7 @@ def validate_model(args):
     import numpy as np
     import torch
     from paper_2608_10803_b200 import binding as ab
+    from paper_2608_10803_b200 import calibrate
     from paper_2608_10803_b200 import synth
     ab.adapt_init(0)
     st = torch.cuda.current_stream().cuda_stream
@@ -758,8 +759,7 @@ def validate_model(args):
             torch.cuda.synchronize()
             times.append(e0.elapsed_time(e1) / reps * 1e3)
         for cand, t in zip(cands, times):
-            cand_rows.append((c.M, c.N, c.K, c.dtype, ab.FAMILY_NAMES[cand.family], cand.BN, cand.stages, cand.P_k, cand.cluster, cand.fused,
-                              cand.streamk, cand.srcA, cand.srcB, cand.predicted_us, cand.t_pro_us, cand.t_main_us, cand.t_epi_us, t))
+            cand_rows.append(calibrate.table_row((c.M, c.N, c.K, c.dtype), cand, t))
         best = int(np.argmin(times))
         hits += int(best == 0 or times[0] <= 1.02 * times[best])
         exact += int(best == 0)
@@ -779,9 +779,7 @@ def validate_model(args):
     print(json.dumps(out))
     if args.dump_candidates:
         with open(args.dump_candidates, "w") as f:
-            f.write("M,N,K,dtype,family,BN,stages,P_k,cluster,fused,streamk,srcA,srcB,pred_us,t_pro,t_main,t_epi,time_us\n")
-            for r in cand_rows:
-                f.write(",".join(f"{x:.3f}" if isinstance(x, float) else str(x) for x in r) + "\n")
+            f.writelines(",".join(r) + "\n" for r in [calibrate.COLUMNS] + cand_rows)
     if args.dump:
         with open(args.dump, "w") as f:
             f.write("M,N,K,candidates,picked_us,best_us,predicted_us\n")

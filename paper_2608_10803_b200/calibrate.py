@@ -34,7 +34,24 @@ GROUPS = 40
 NAMES = {0: "plain P_k=1", 1: "plain P_k=1 + prologue", 2: "plain split-K", 3: "plain split-K + prologue", 4: "plain fused split-K",
          5: "plain stream-K", 6: "row classes P_k=1", 7: "row classes split-K", 8: "row classes fused", 9: "halo class tiles",
          10: "k-class accumulators", 11: "k classes as splits", 12: "k classes fused", 13: "warp-level P_k=1", 14: "warp-level split-K",
-         15: "CUDA-core P_k=1", 16: "CUDA-core split-K", 17: "one-launch cluster of 1", 18: "one-launch cluster > 1"}
+         15: "CUDA-core P_k=1", 16: "CUDA-core split-K", 17: "one-launch cluster of 1", 18: "one-launch cluster > 1",
+         36: "tall pair tiles", 37: "tall pair tiles + prologue", 38: "tall pair tiles, row classes"}
+
+# The columns of a table of timed configurations: what ``bench.py --dump-candidates`` writes, one line per configuration.
+COLUMNS = ("M,N,K,dtype,family,BM,BN,stages,P_k,cluster,fused,streamk,srcA,srcB,pred_us,t_pro,t_main,t_epi,time_us").split(",")
+
+
+def table_row(shape, info, time_us):
+    """One line of the table: a candidate (``adapt_plan_candidates``) of (M, N, K, dtype) and its measured time."""
+    values = {"family": list(FAMILY_ID)[info.family], "pred_us": info.predicted_us, "t_pro": info.t_pro_us, "t_main": info.t_main_us,
+              "t_epi": info.t_epi_us, "time_us": time_us}
+    values.update(zip(("M", "N", "K", "dtype"), shape))
+    return [f"{v:.3f}" if isinstance(v, float) else str(v) for v in (values[c] if c in values else getattr(info, c) for c in COLUMNS)]
+
+
+def tile_rows(row) -> int:
+    """BM of a table line; tables written before there were tall pair tiles have no such column, and one BM per family."""
+    return int(row["BM"]) if row.get("BM") else {"umma_1cta": 128, "umma_2cta": 256, "skinny": 16}.get(row["family"], 64)
 
 
 def group_of(row) -> int:
@@ -48,6 +65,8 @@ def group_of(row) -> int:
     if fam == "cluster":
         return 17 if cluster == 1 else 18
     pro = src_a == 1 or src_b == 1
+    if tile_rows(row) == 512:
+        return 38 if src_a == 3 else (37 if pro else 36)
     if src_b == 3:
         g = 10 if bn == 64 else (12 if fused else 11)
     elif src_a == 3:
@@ -73,7 +92,7 @@ class TimedSet:
             with open(path, newline="") as f:
                 for r in csv.DictReader(f):
                     shape = (int(r["M"]), int(r["N"]), int(r["K"]), int(r["dtype"]))
-                    cfg = (FAMILY_ID[r["family"]], int(r["BN"]), int(r["stages"]), int(r["P_k"]), int(r["cluster"]), int(r["fused"]),
+                    cfg = (FAMILY_ID[r["family"]], tile_rows(r), int(r["BN"]), int(r["stages"]), int(r["P_k"]), int(r["cluster"]), int(r["fused"]),
                            int(r["streamk"]), int(r["srcA"]), int(r["srcB"]))
                     t = float(r["time_us"])
                     d = self.shapes.setdefault(shape, {})
@@ -86,7 +105,7 @@ class TimedSet:
             best = min(timed.values())
             pick_pred, pick_t = float("inf"), None
             for c in ab.adapt_plan_candidates(M, N, K, dt):
-                t = timed.get((c.family, c.BN, c.stages, c.P_k, c.cluster, c.fused, c.streamk, c.srcA, c.srcB))
+                t = timed.get((c.family, c.BM, c.BN, c.stages, c.P_k, c.cluster, c.fused, c.streamk, c.srcA, c.srcB))
                 if t is None:
                     continue
                 if c.predicted_us < pick_pred:
@@ -191,7 +210,7 @@ def main():
         f = math.exp(sums[g] / counts[g]) if counts[g] >= 20 else 1.0
         out.append(current[g] * f)
         if counts[g]:
-            name = NAMES.get(g % 20, "?") + (" (pair tiles)" if g >= 20 else "")
+            name = NAMES[g] if g in NAMES else NAMES.get(g % 20, "?") + " (pair tiles)"
             print(f"group {g:2d} {name:32s} n={counts[g]:6d} measured/predicted {f:.3f} -> factor {out[-1]:.3f}")
     print("group_bias = {" + ", ".join(f"{x:.3f}" for x in out) + "};")
 

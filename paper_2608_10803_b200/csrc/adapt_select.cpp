@@ -122,7 +122,7 @@ static int64_t innerB(const Shape& s) { return s.layoutB == ADAPT_ROW_MAJOR ? s.
 static int64_t outerB(const Shape& s) { return s.layoutB == ADAPT_ROW_MAJOR ? s.K : s.N; }
 
 // Group of a configuration for the last calibration factor: kernel family, tiling mode, and which extra launches
-// (prologue, reduction) or in-kernel exchanges (fused reduction, stream-K) it has.  Pair tiles: + 20.
+// (prologue, reduction) or in-kernel exchanges (fused reduction, stream-K) it has.  Pair tiles: + 20, tall ones from 36 on.
 int calib_group(const Config& c)
 {
     const bool pro = c.srcA == ADAPT_SRC_PAD_COPY || c.srcB == ADAPT_SRC_PAD_COPY;
@@ -133,6 +133,7 @@ int calib_group(const Config& c)
         case ADAPT_FAM_CLUSTER: return c.cluster == 1 ? 17 : 18;
         default: break;
     }
+    if (c.BM == 512) return c.srcA == ADAPT_SRC_TMA_CLASSES ? 38 : (pro ? 37 : 36);
     if (c.srcB == ADAPT_SRC_TMA_CLASSES) g = c.BN == 64 ? 10 : (c.fused ? 12 : 11);
     else if (c.srcA == ADAPT_SRC_TMA_CLASSES) g = c.BN % 64 ? 9 : (c.fused ? 8 : (c.P_k == 1 ? 6 : 7));
     else if (c.fused) g = 4;
