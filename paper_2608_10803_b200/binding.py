@@ -21,7 +21,7 @@ LIB_PATH = os.path.join(_HERE, "libadaptmm.so")
 
 EXPORTS = [
     "adapt_init", "adapt_shutdown", "adapt_matmul_plan", "adapt_matmul", "adapt_matmul_host", "adapt_last_error",
-    "adapt_last_error_message", "adapt_status_string", "adapt_plan_info", "adapt_plan_candidates",
+    "adapt_last_error_message", "adapt_status_string", "adapt_plan_info", "adapt_plan_info_call", "adapt_plan_candidates",
     "adapt_matmul_plan_forced", "adapt_classify", "adapt_model_read_volume", "adapt_model_write_volume",
     "adapt_model_pipeline", "adapt_poll_device_status", "adapt_plan_cache_size", "adapt_launch_count",
     "adapt_matmul_noalloc", "adapt_matmul_batch", "adapt_matmul_repeat", "adapt_measure_dispatch",
@@ -108,6 +108,8 @@ def load():
     lib.adapt_status_string.argtypes = [i32]
     lib.adapt_plan_info.restype = i32
     lib.adapt_plan_info.argtypes = [vp, ctypes.POINTER(PlanInfo)]
+    lib.adapt_plan_info_call.restype = i32
+    lib.adapt_plan_info_call.argtypes = [vp, vp, vp, i32, ctypes.POINTER(PlanInfo)]
     lib.adapt_plan_candidates.restype = i32
     lib.adapt_plan_candidates.argtypes = [i64, i64, i64, i32, i32, i32, ctypes.POINTER(PlanInfo), i32]
     lib.adapt_classify.restype = i32
@@ -326,6 +328,13 @@ def adapt_selftest_wait_expiry(limit_ns: int, stream: int = 0):
 def adapt_plan_info(plan) -> PlanInfo:
     info = PlanInfo()
     _check(load().adapt_plan_info(plan, ctypes.byref(info)))
+    return info
+
+
+def adapt_plan_info_call(plan, C_ptr: int, D_ptr: int = 0, d_is_vector: bool = False) -> PlanInfo:
+    """What a call that writes C and adds D (0: none) runs: the plan's configuration, or its second one where C or D rule out tall tiles."""
+    info = PlanInfo()
+    _check(load().adapt_plan_info_call(plan, C_ptr, D_ptr, 1 if d_is_vector else 0, ctypes.byref(info)))
     return info
 
 

@@ -177,6 +177,8 @@ void enumerate_configs(const Shape& s, const Machine& m, const Calib& cal, std::
 
 // Rebuild the full Config a key describes for this shape; false if it is not legal.
 bool config_from_key(const Shape& s, uint64_t key, const Machine& m, const Calib& cal, Config* out);
+// 256-row pair tiles over the operand sources of a configuration of tall ones, without a split.
+Config short_counterpart(const Shape& s, const Machine& m, const Calib& cal, const Config& tall);
 
 void fill_info(const Shape& s, const Config& c, adapt_plan_info_t* out);
 

@@ -837,6 +837,19 @@ void enumerate_configs(const Shape& s, const Machine& m, const Calib& cal, std::
     });
 }
 
+Config short_counterpart(const Shape& s, const Machine& m, const Calib& cal, const Config& tall)
+{
+    Machine all = m;
+    all.family_mask |= 1u << ADAPT_FAM_UMMA_2CTA;
+    all.workspace_limit = INT64_MAX;                                // no larger than the tall plan's, which is there
+    Config c;
+    c.family = tall.family; c.BM = 256; c.BN = tall.BN; c.BK = tall.BK; c.cluster = tall.cluster; c.P_k = 1;
+    c.srcA = tall.srcA; c.srcB = tall.srcB;
+    c.stages = umma_deepest_ring(c.BN, c.cluster, 128, true, m.smem_bytes, 8);
+    finalize(s, all, cal, c);                                       // legal wherever the tall tiles are
+    return c;
+}
+
 bool config_from_key(const Shape& s, uint64_t key, const Machine& m, const Calib& cal, Config* out)
 {
     Shape flags;
