@@ -54,7 +54,8 @@ struct TallItem {
     bool two;
 };
 
-// The it-th item of a slot: its whole tiles, then its share of the single blocks.
+// The it-th item of a slot: its whole tiles, then its share of the single blocks.  (A single block behind the whole tile of a slot, where
+// another slot had none: 1771 x 4736 x 6288, 57 tiles and 19 single blocks on 74 pairs, 100 us instead of 62 with zero operands.)
 template <bool CLS>
 ADAPT_HOST_DEVICE bool tall_item(const TallWork& p, int slot, int n_slots, int it, TallItem& w)
 {
@@ -65,11 +66,17 @@ ADAPT_HOST_DEVICE bool tall_item(const TallWork& p, int slot, int n_slots, int i
     if (w.two) {
         t = slot + it * n_slots;
     } else {
-        int first = slot - p.big % n_slots;                    // the slots without a tile in the last wave come first
-        if (first < 0) first += n_slots;
-        h = first + (it - mine) * n_slots;
+        // two for each slot without a tile in the last wave (which the others spend on a whole tile), then one for every slot in turn
+        const int last = p.big % n_slots, free_slots = last ? n_slots - last : 0;
+        const int first = slot < last ? slot + free_slots : slot - last;
+        int j = it - mine;
+        w.acc = j & 1;
+        if (last && slot >= last) {
+            h = first + j * free_slots;
+            j -= 2;
+        }
+        if (j >= 0) h = 2 * free_slots + first + j * n_slots;
         if (h >= p.halves) return false;
-        w.acc = (it - mine) & 1;
         t = p.big + (h >> 1);
         if (h >= p.split) {                                    // the odd rows
             const int o = h - p.split;

@@ -64,6 +64,44 @@ def test_tall_tiles_cover_the_output_once(tmp_path):
     assert r.returncode == 0, r.stdout + r.stderr
 
 
+BALANCE = r"""
+#include <cstdio>
+#include "adapt_internal.h"
+using namespace adapt;
+
+template <bool CLS>
+int check(int64_t M, int P_n, int slots)
+{
+    double waves = 0, longest = 0;
+    const TallWork w = tall_schedule(M, P_n, CLS, slots, &waves);
+    const int grid = std::min(w.big + w.halves, slots);
+    for (int slot = 0; slot < grid; ++slot) {
+        TallItem t;
+        double len = 0;
+        for (int it = 0; tall_item<CLS>(w, slot, grid, it, t); ++it) len += t.two ? 1.0 : 0.5;
+        longest = std::max(longest, len);
+    }
+    if (longest == waves) return 0;
+    printf("M %lld P_n %d slots %d classes %d: %.1f waves, longest slot %.1f\n", (long long)M, P_n, slots, (int)CLS, waves, longest);
+    return 1;
+}
+
+int main()
+{
+    int bad = 0;
+    for (int slots : {74, 66, 5, 1})
+        for (int P_n = 1; P_n <= 100; ++P_n)
+            for (int64_t M = 300; M < 20000; M += 419) bad += check<false>(M, P_n, slots) + check<true>(M, P_n, slots);
+    return bad != 0;
+}
+"""
+
+
+def test_longest_slot_is_what_the_model_counts(tmp_path):
+    r = build_and_run(tmp_path, BALANCE)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr
+
+
 @pytest.fixture
 def tall_preferred():
     """The model made to take tall tiles wherever they are legal and compute-bound, whatever its constants."""
