@@ -232,7 +232,8 @@ adapt_status_t adapt_matmul_noalloc(int64_t M, int64_t N, int64_t K, adapt_dtype
  *   or overwrites what a collected one writes, or overwrites what it reads, makes the collected ones leave first.
  * - From eight calls on the launches are spread over up to four internal streams, and cuda_stream itself for launches that need no
  *   workspace, between a fork from and a join to cuda_stream (work queued on cuda_stream before the call comes first, work queued
- *   after it comes last), so that the launch gaps and the tail of one GEMM fill with the next one's work.  A launch whose output
+ *   after it comes last), so that the launch gaps and the tail of one GEMM fill with the next one's work (two launches without a
+ *   workspace stay on cuda_stream where that would hide less than the events cost).  A launch whose output
  *   overlaps a buffer that an earlier one still reads or writes on another stream, or whose inputs overlap such an output, waits for
  *   that stream first.  Option "batch_streams" (adapt_set_option; 1 to 4, default 4) sets the number of internal streams; with 1
  *   everything runs on cuda_stream.

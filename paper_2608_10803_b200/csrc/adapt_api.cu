@@ -1842,15 +1842,19 @@ struct BatchOps {
     {
         return (s.dtype != 0 ? 1 : 0) | (s.layoutA == ADAPT_ROW_MAJOR ? 2 : 0) | (s.layoutB == ADAPT_COL_MAJOR ? 4 : 0);
     }
+    size_t entries(const int64_t* calls, size_t n, GroupEntry* entry) const
+    {
+        for (size_t j = 0; j < n; ++j) {
+            const int64_t i = calls[j];
+            entry[j].chain = group_item(plans[i]->s, plans[i]->c, A[i], B[i], C[i], &entry[j].item);
+        }
+        group_order(entry, n, S.machine.n_sm);
+        return n;
+    }
     adapt_status_t group(const std::vector<int64_t>& calls, int lane)
     {
         GroupEntry entry[kGroupMax];
-        size_t n = 0;
-        for (int64_t i : calls) {
-            entry[n].chain = group_item(plans[i]->s, plans[i]->c, A[i], B[i], C[i], &entry[n].item);
-            ++n;
-        }
-        group_order(entry, n, S.machine.n_sm);
+        const size_t n = entries(calls.data(), calls.size(), entry);
         const Shape& s = plans[calls[0]]->s;
         GroupParams p;
         group_clear(p);
@@ -1883,17 +1887,29 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
     auto grouped = [&](const Plan* pl) { return pl && pl->selected && !pl->noop && !pl->zero_fill && group_eligible(pl->s, pl->c); };
     auto config = [&](int64_t i) -> const Config& { return call_config(S, plans[i], C[i], nullptr, false); };
     auto workspace = [&](int64_t i) { return plans[i] && needs_workspace(plans[i], config(i), A[i], B[i]); };
-    int64_t singles = 0, with_workspace = 0;
+    int64_t singles = 0, with_workspace = 0, single = 0, small[kBatchVariants] = {}, first[kGroupMax];
     for (int64_t i = 0; i < count; ++i) {
-        if (grouped(plans[i])) continue;
+        if (grouped(plans[i])) {
+            if (i - singles < kGroupMax) first[i - singles] = i;
+            ++small[BatchOps::variant(plans[i]->s)];
+            continue;
+        }
         ++singles;
+        single = i;
         with_workspace += workspace(i) ? 1 : 0;
     }
+    int64_t grouped_launches = 0;
+    for (int64_t n : small) grouped_launches += ceil_div(n, kGroupMax);
+    BatchOps ops = {S, plans, A, B, C, {user}};
+    double hidden_us = 0.0;
+    if (count >= 8 && singles == 1 && grouped_launches == 1 && with_workspace == 0 && plans[single]) {
+        GroupEntry entry[kGroupMax];
+        hidden_us = batch_hidden_us(entry, ops.entries(first, (size_t)(count - 1), entry), S.machine.n_sm, config(single).predicted_us);
+    }
     // Lane 0 is the caller's stream, the others are internal streams between a fork from and a join to it.
-    const int NL = 1 + batch_internal_lanes(count, singles, with_workspace, S.batch_lanes);
+    const int NL = 1 + batch_internal_lanes(count, singles, with_workspace, S.batch_lanes, grouped_launches, hidden_us);
     std::unique_lock<std::mutex> batch_lock(S.batch_mu, std::defer_lock);
     State::BatchLanes& L = S.lanes;
-    BatchOps ops = {S, plans, A, B, C, {user}};
     if (NL > 1) {
         batch_lock.lock();
         if (!L.ready) {

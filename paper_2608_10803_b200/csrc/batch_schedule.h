@@ -33,16 +33,35 @@ constexpr int kBatchVariants = 8;
 constexpr int kBatchInternalMax = 4;                        // internal streams
 constexpr int kBatchLanesMax = 1 + kBatchInternalMax;       // ... and the caller's
 
-// Internal streams for a list of `count` calls of which `singles` are launched by themselves, `with_workspace` of them over a workspace:
-// none for a short list, nor for two launches without a workspace (the events of a fork and a join cost what the overlap brings: 48 layers of
-// 16 .. 1024 a side, a grouped launch and one by itself, 31.0 us on two streams, 29.5 on one), else no more than `limit` and no more than there
-// are launches to overlap (the caller's stream takes part).
-inline int batch_internal_lanes(int64_t count, int64_t singles, int64_t with_workspace, int limit)
+// What a second stream has to hide of a list of two launches (us) to be worth the events of its fork and join.
+constexpr double kBatchForkUs = 4.0;
+
+// Internal streams for a list of `count` calls of which `singles` are launched by themselves, `with_workspace` of them over a workspace, and the
+// others in `grouped` launches: none for a short list, nor for two launches in all without a workspace of which a second stream would hide less than
+// kBatchForkUs, else no more than `limit` and no more than there are calls to overlap (the caller's stream takes part).
+inline int batch_internal_lanes(int64_t count, int64_t singles, int64_t with_workspace, int limit, int64_t grouped = 1, double hidden_us = 0.0)
 {
     if (count < 8 || limit < 2) return 0;
-    const int64_t launches = singles + (singles < count ? 1 : 0);
-    if (with_workspace == 0 && launches <= 2) return 0;
-    return (int)std::max<int64_t>(0, std::min<int64_t>(std::min(limit, kBatchInternalMax), std::max(with_workspace, launches - 1)));
+    if (with_workspace == 0 && singles + (singles < count ? grouped : 0) <= 2 && hidden_us < kBatchForkUs) return 0;
+    const int64_t apart = singles + (singles < count ? 1 : 0);         // the grouped launches follow one another
+    return (int)std::max<int64_t>(0, std::min<int64_t>(std::min(limit, kBatchInternalMax), std::max(with_workspace, apart - 1)));
+}
+
+// What a second stream hides of a grouped launch of these entries (in group_order) and a call of `single_us`.  The launch leaves SMs idle while its
+// longest chain runs: about 2 us a stage, against 3.3 us for what a CTA slot (two per SM) has to do on average.  A long call covers the launch's start
+// and end.  Measured over 140 such lists of 8 to 48 calls, 128 to 1500 a side, time on two streams over time on one: where this says 4 us or more (23 lists)
+// 0.68 to 1.01, 0.90 on average (15 calls to 1500 and 4096 x 4096 x 4096: 138.8 -> 107.2 us); elsewhere 1.035 on average, one stream being faster by more
+// than 5 % in 51 lists (23 calls to 256 and 20000 x 64 x 64: 15.5 and 17.7) and slower in 15.
+inline double batch_hidden_us(const GroupEntry* e, size_t n, int n_sm, double single_us)
+{
+    double work = 0.0;
+    int longest = 0;
+    for (size_t j = 0; j < n; ++j) {
+        work += (double)(e[j].item.tiles << e[j].item.share_log2) * e[j].chain;
+        longest = std::max(longest, e[j].chain);
+    }
+    const double idle = 2.0 * longest - 3.3 * work / (2.0 * n_sm);
+    return std::max(std::min(idle, single_us), 0.05 * single_us);
 }
 
 // The calls 0 .. count-1 of call_of(i), with the result of running them in that order.

@@ -137,3 +137,51 @@ int main()
 def test_lists_keep_their_order_on_any_number_of_streams(tmp_path):
     r = build_and_run(tmp_path, PROGRAM)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+LANES = r"""
+#include <cstdio>
+#include "batch_schedule.h"
+using namespace adapt;
+
+static int bad = 0;
+static void check(bool ok, const char* what) { if (!ok) { printf("%s\n", what); ++bad; } }
+
+int main()
+{
+    // one launch or two on the caller's stream; a second one where it hides something, or where there are more launches than two
+    check(batch_internal_lanes(48, 0, 0, 4, 1, 0.0) == 0, "a grouped launch alone");
+    check(batch_internal_lanes(48, 1, 0, 4, 1, 0.0) == 0 && batch_internal_lanes(48, 1, 0, 4, 1, kBatchForkUs - 0.1) == 0, "two launches, nothing to hide");
+    check(batch_internal_lanes(48, 1, 0, 4, 1, kBatchForkUs) == 1, "two launches, one hides the other");
+    check(batch_internal_lanes(300, 1, 0, 4, 5, 0.0) == 1 && batch_internal_lanes(48, 1, 0, 4, 2, 0.0) == 1, "several grouped launches and one call");
+    check(batch_internal_lanes(48, 1, 1, 4, 1, 0.0) == 1 && batch_internal_lanes(8, 2, 2, 4, 1, 0.0) == 2, "a call with a workspace");
+    check(batch_internal_lanes(48, 1, 0, 1, 5, 99.0) == 0 && batch_internal_lanes(7, 1, 1, 4, 1, 99.0) == 0, "switched off, or a short list");
+    // lists of more launches: as many streams as there are calls launched by themselves, however many launches the small calls take
+    for (int64_t count = 8; count < 40; ++count)
+        for (int64_t singles = 0; singles <= count; ++singles)
+            for (int64_t ws = 0; ws <= singles; ++ws)
+                for (int limit = 2; limit <= 4; ++limit)
+                    for (int64_t grouped = 1; grouped <= 4; ++grouped) {
+                        const int64_t launches = singles + (singles < count ? grouped : 0);
+                        if (ws == 0 && launches <= 2) continue;
+                        const int64_t want = std::min<int64_t>(limit, std::max(ws, singles + (singles < count) - 1));
+                        check(batch_internal_lanes(count, singles, ws, limit, grouped, 0.0) == want, "streams of a longer list");
+                    }
+    // a long chain among short ones, busy SMs, a long call
+    GroupEntry e[2];
+    for (GroupEntry& x : e) x.item = GroupItem();
+    e[0].item.tiles = 40; e[0].chain = 12;
+    e[1].item.tiles = 400; e[1].chain = 2;
+    check(batch_hidden_us(e, 2, 148, 20.0) > kBatchForkUs && batch_hidden_us(e, 2, 148, 3.0) < kBatchForkUs, "SMs idle beside a long chain");
+    e[1].item.tiles = 1200;
+    check(batch_hidden_us(e, 2, 148, 20.0) < kBatchForkUs && batch_hidden_us(e, 2, 148, 90.0) > kBatchForkUs, "busy SMs");
+    e[0].item.share_log2 = 2; e[0].chain = 3;
+    check(batch_hidden_us(e, 2, 148, 20.0) < kBatchForkUs, "a shared chain");
+    return bad;
+}
+"""
+
+
+def test_lists_get_the_streams_that_their_launches_can_use(tmp_path):
+    r = build_and_run(tmp_path, LANES)
+    assert r.returncode == 0, r.stdout + r.stderr
