@@ -1100,16 +1100,15 @@ adapt_status_t launch_pad2(State& S, const void* srcA, void* dstA, int64_t outer
     return ADAPT_OK;
 }
 
-// prologue: the call re-pitched or regrouped an operand first
 adapt_status_t launch_reduce(State& S, const float* partial, void* C, int64_t M, int64_t N, int P_k, int dtype, cudaStream_t stream,
-                             const ReduceEpilogue* epi = nullptr, bool prologue = false)
+                             const ReduceEpilogue* epi = nullptr, int release = kReleaseFirst)
 {
     const ReduceEpilogue ep = epi ? *epi : no_epilogue();
     const int64_t Np = partial_pitch(N);
     const int64_t work = M * (Np / 4);
     const int groups = reduce_groups(work, P_k, S.machine.n_sm);
     const int blocks = (int)std::min<int64_t>(ceil_div(work, 256 / groups), (int64_t)S.machine.n_sm * 8);
-    CUDA_TRY(launch_pdl(groups > 1 ? splitk_reduce_kernel<true> : splitk_reduce_kernel<false>, dim3(blocks), dim3(256), 0, stream, (const float*)partial, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)P_k, (int)dtype, ep, groups, prologue ? 1 : 0));
+    CUDA_TRY(launch_pdl(groups > 1 ? splitk_reduce_kernel<true> : splitk_reduce_kernel<false>, dim3(blocks), dim3(256), 0, stream, (const float*)partial, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)P_k, (int)dtype, ep, groups, release));
     S.launches.fetch_add(1, std::memory_order_relaxed);
     CUDA_TRY(cudaGetLastError());
     return ADAPT_OK;
@@ -1402,8 +1401,9 @@ adapt_status_t run_umma(State& S, Plan* pl, const Config& c, const void* A, cons
     }
     CUDA_TRY(launch_exc(&cfg, k, args, arg_bytes, 2));
     S.launches.fetch_add(1, std::memory_order_relaxed);
-    if (partials) return launch_reduce(S, partial, C, s.M, s.N, p.P_k, s.dtype, stream, epi, padA || padB || kclsB);
-    return ADAPT_OK;
+    if (!partials) return ADAPT_OK;
+    const int release = padA || padB || kclsB ? kReleaseAtEnd : (cg == 1 && p.P_m == 1 && !classesA) ? kReleaseAfterWait : kReleaseFirst;
+    return launch_reduce(S, partial, C, s.M, s.N, p.P_k, s.dtype, stream, epi, release);
 }
 
 adapt_status_t run_simt(State& S, const Shape& s, const Config& c, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi)
@@ -2223,7 +2223,7 @@ extern "C" adapt_status_t adapt_matmul_noalloc(int64_t M, int64_t N, int64_t K, 
     const int64_t work = M * (Np / 4);
     const int groups = reduce_groups(work, (int)pk, 148);
     const int blocks = (int)std::min<int64_t>(ceil_div(work, 256 / groups), 148 * 8);
-    CUDA_TRY(launch_pdl(groups > 1 ? splitk_reduce_kernel<true> : splitk_reduce_kernel<false>, dim3(blocks), dim3(256), 0, stream, (const float*)scratch, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)pk, (int)dtype, no_epilogue(), groups, 0));
+    CUDA_TRY(launch_pdl(groups > 1 ? splitk_reduce_kernel<true> : splitk_reduce_kernel<false>, dim3(blocks), dim3(256), 0, stream, (const float*)scratch, (unsigned short*)C, (int)M, (int)N, (int)Np, (int)pk, (int)dtype, no_epilogue(), groups, (int)kReleaseFirst));
     CUDA_TRY(cudaGetLastError());
     st().launches.fetch_add(2, std::memory_order_relaxed);
     return ADAPT_OK;

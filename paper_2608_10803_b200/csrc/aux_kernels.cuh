@@ -219,20 +219,27 @@ regroup_a_kernel(const unsigned short* __restrict__ A, unsigned short* __restric
 // ascending order; the runs' sums are then added in ascending order too.  The order depends on the shape only.
 // (256 x 256 x 262144, P_k = 64: eight batches 67.9 us for the call, one batch 63.5 us; 34 x 21 x 34323: 17.3 and 11.6 us.)
 // SHARED: groups > 1 (the other outputs are not charged for it: 365 x 3136 x 4672 in three splits 23.1 us, 23.6 with the one kernel).
+// When the reduction lets the next kernel in, by what ran in front of it.
+//   At its end: calls that re-pitched or regrouped an operand (the next one will most likely be of their kind).  While the GEMM still runs, what starts
+//     early finds room on the few SMs without a GEMM CTA only, and all of a regrouping or re-pitching kernel that had started there ran there, beside
+//     a hundred idle SMs (34 x 102 x 35284, 112 k-class splits, in a row: 26.0 -> 13.1 us).  Let in at the end its CTAs spread over empty SMs, with
+//     the L1 they live on: 44 k-class shapes 0.81 of the time of the first form, 0.91 when let in after the wait.
+//   After its wait for the GEMM: plain 1-CTA tiles, one row of them (matrix-vector and other streaming calls): 143 shapes of up to 128 rows 0.983 of the
+//     time (1 x 4416 x 1024 7.70 -> 6.97, 4 x 2688 x 1728 7.7 -> 7.5; at worst 1 x 13312 x 1984 14.65 -> 15.16); at the end 1.09.
+//   First thing: everything else.  More rows of 1-CTA tiles 1.000, pair tiles 0.999 (153 x 8832 x 15808 65.2 -> 70.9 let in after the wait), row
+//     classes 1.000 (1132 x 48 x 10417 15.5 -> 16.6); the warp-level and the CUDA-core kernel leave room on their SMs.
+enum { kReleaseFirst = 0, kReleaseAfterWait, kReleaseAtEnd };
+
 template <bool SHARED>
 __global__ void __launch_bounds__(256)
 splitk_reduce_kernel(const float* __restrict__ partial, unsigned short* __restrict__ C,
-                     int M, int N, int Np, int P_k, int dtype, const ReduceEpilogue ep, int groups_shared, int prologue)
+                     int M, int N, int Np, int P_k, int dtype, const ReduceEpilogue ep, int groups_shared, int release)
 {
     __shared__ float4 s_sum[SHARED ? 256 : 1];
     const int groups = SHARED ? groups_shared : 1;
+    if (release == kReleaseFirst) pdl_launch_dependents();
     pdl_wait();
-    // The next kernel is let in now, not first thing: while the GEMM in front of this one still runs, what starts early finds room on the few SMs
-    // without a GEMM CTA only, and all of a regrouping or re-pitching kernel that had started there ran there, beside a hundred idle SMs
-    // (34 x 102 x 35284, 112 k-class splits, in a row: 26.0 -> 13.1 us).  A call that has such a prologue (the next one will most likely be of its
-    // kind) lets the next kernel in at the end: its CTAs then spread over empty SMs, with the L1 they live on (76 x 371 x 37184 33.2 -> 27.0 us, 30.0 when
-    // let in here; 288 x 214 x 36999 40.4 -> 33.7, 40.0; without a prologue 4 x 2688 x 1728 7.7 -> 7.5, 8.6 at the end).
-    if (!prologue) pdl_launch_dependents();
+    if (release == kReleaseAfterWait) pdl_launch_dependents();
     const int quads = Np >> 2;                              // columns in fours
     const int64_t total = (int64_t)M * quads;
     const int64_t slab = (int64_t)M * Np;
@@ -289,7 +296,7 @@ splitk_reduce_kernel(const float* __restrict__ partial, unsigned short* __restri
                 if (n + j < N) dst[j] = float_to_16(a[j], dtype);
         }
     }
-    if (prologue) pdl_launch_dependents();
+    if (release == kReleaseAtEnd) pdl_launch_dependents();
 }
 
 // ---- CUDA-core tile GEMM: 64 x 64 tile, 256 threads, 4 x 4 outputs per thread ---------------------
