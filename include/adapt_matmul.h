@@ -319,7 +319,7 @@ int64_t adapt_map_encode_count(void);
  *               amount that depends on the tile, so that the CTAs of a wave do not all ask for the same k slice of a shared
  *               operand at once.  The order is a function of the tile, so results stay reproducible, but they may differ
  *               in the last bit from those with the option off (another summation order).  Plain tiles only; a plan of 512 x 256
- *               plain tiles runs another configuration meanwhile (adapt_plan_info_call).
+ *               plain tiles runs 256 x 256 ones meanwhile (adapt_plan_info_call).
  *   "prefetch"  (default 1): L2 prefetch of a kernel's first operand boxes ahead of its wait for the kernel before it.
  *   "batch_streams" (default 4): internal streams of adapt_matmul_batch, 1 to 4 (see there). */
 adapt_status_t adapt_set_option(const char* name, int value);
@@ -353,10 +353,8 @@ const char* adapt_status_string(adapt_status_t s);
 adapt_status_t adapt_plan_info(adapt_handle_t plan, adapt_plan_info_t* out);
 /* The configuration a call of the plan runs that writes C and adds D (addresses only, nothing is read; D null: adapt_matmul).  It is the
  * plan's own but for a plan of 512 x 256 pair tiles whose call these do not serve: C off a 32-byte boundary, D off a 16-byte one, a matrix D
- * (d_is_vector == 0) with K < 1024, or option "shuffle_k" on a plan without row classes.  Such a call runs the best candidate on other tiles (a
- * plan forced, or loaded, with a key that is not the model's choice: 256 x 256 pair tiles).  Where that configuration needs a larger workspace than
- * the plan and the stream has not got it in a capture, or it cannot be allocated, the call runs 256 x 256 pair tiles without it, whose sums
- * may differ in the last bit. */
+ * (d_is_vector == 0) with K < 1024, or option "shuffle_k" on a plan without row classes.  Such a call runs 256 x 256 pair tiles over the same
+ * operand sources. */
 adapt_status_t adapt_plan_info_call(adapt_handle_t plan, const void* C, const void* D, int d_is_vector, adapt_plan_info_t* out);
 
 /* Every legal configuration for the shape with its predicted time (Eq. 6's search

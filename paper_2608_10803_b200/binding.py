@@ -332,7 +332,7 @@ def adapt_plan_info(plan) -> PlanInfo:
 
 
 def adapt_plan_info_call(plan, C_ptr: int, D_ptr: int = 0, d_is_vector: bool = False) -> PlanInfo:
-    """What a call that writes C and adds D (0: none) runs: the plan's configuration, or its second one where C or D rule out tall tiles."""
+    """What a call that writes C and adds D (0: none) runs: the plan's configuration, or 256-row pair tiles where C or D rule out tall ones."""
     info = PlanInfo()
     _check(load().adapt_plan_info_call(plan, C_ptr, D_ptr, 1 if d_is_vector else 0, ctypes.byref(info)))
     return info

@@ -71,8 +71,7 @@ struct adapt_plan_s {
     Config c;
     bool selected = false;    // the plan adapt_matmul_plan returns for its shape (not a forced-key plan)
     std::atomic<int> model_pick{-1};   // is its configuration the model's choice (a table's may be another)?  -1: not looked yet
-    Config other;             // tall pair tiles: the configuration of calls whose buffers these cannot serve (call_config)
-    std::atomic<bool> other_known{false};
+    Config other;             // a plan of tall pair tiles: the configuration of calls that these cannot serve (call_config)
     bool noop = false;        // M == 0 or N == 0
     bool zero_fill = false;   // K == 0
     std::mutex mu;            // guards the tensor-map slots
@@ -209,17 +208,6 @@ bool valid_shape(int64_t M, int64_t N, int64_t K, int dtype, int lA, int lB)
     return true;
 }
 
-// The second configuration of a plan of tall tiles that the model chose: the best of its candidates on other tiles.
-void remember_other(Plan* p, const std::vector<Config>& cands)
-{
-    for (const Config& k : cands)
-        if (k.BM != 512) {
-            p->other = k;
-            p->other_known.store(true, std::memory_order_release);
-            return;
-        }
-}
-
 Plan* make_plan(State& S, const Shape& s, const uint64_t* forced_key)
 {
     Plan* p = new Plan();
@@ -232,6 +220,7 @@ Plan* make_plan(State& S, const Shape& s, const uint64_t* forced_key)
             fail(ADAPT_ERR_UNSUPPORTED, "tiling key is not legal for this shape%s");
             return nullptr;
         }
+        if (p->c.BM == 512) p->other = short_counterpart(s, S.machine, S.calib, p->c);
         return p;
     }
     std::vector<Config> cands;
@@ -242,7 +231,7 @@ Plan* make_plan(State& S, const Shape& s, const uint64_t* forced_key)
         return nullptr;
     }
     p->c = cands[0];
-    if (p->c.BM == 512) remember_other(p, cands);
+    if (p->c.BM == 512) p->other = short_counterpart(s, S.machine, S.calib, p->c);
     if (S.log) {
         fprintf(stderr, "[adapt] plan %lldx%lldx%lld dt%d: fam %d class %d tile %dx%dx%d st %d P_k %d src %d/%d pred %.2f us (%zu candidates)\n",
                 (long long)s.M, (long long)s.N, (long long)s.K, s.dtype, p->c.family, p->c.cls, p->c.BM, p->c.BN, p->c.BK,
@@ -1163,9 +1152,23 @@ adapt_status_t launch_tall(State& S, const Shape& s, const UmmaParams& p, const 
     return ADAPT_OK;
 }
 
-adapt_status_t run_umma(State& S, Plan* pl, const Config& c, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi)
+// The configuration of a call that writes C and adds D (null: none): the plan's, but for tall tiles that cannot serve it.  They store whole 32-byte
+// sectors, add D in 16-byte chunks and have one order of k; and a matrix D over a short k range makes trips to memory that nothing hides
+// (64179 x 576 x 896: 106 us, 108.8 on tall tiles; 5366 x 16320 x 1920: 322 and 287).  Such a call runs 256-row pair tiles, also where the model would
+// take another configuration if there were no tall ones: with C 16 bytes off, 55 shapes whose best other candidate cuts k took 1.06 times as long on it,
+// 12 with 1-CTA tiles 1.03 (three with stream-K 0.88); with a matrix D and K < 1024 it was the same configuration for all of 70 shapes.
+const Config& call_config(const State& S, const Plan* pl, const void* C, const void* D, bool d_is_vector)
+{
+    const Config& c = pl->c;
+    if (c.BM != 512) return c;
+    const bool reorder = S.shuffle_k && c.srcA != ADAPT_SRC_TMA_CLASSES;
+    return ((uintptr_t)C & 31) == 0 && ((uintptr_t)D & 15) == 0 && (!D || d_is_vector || pl->s.K >= 1024) && !reorder ? c : pl->other;
+}
+
+adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi = nullptr)
 {
     const Shape& s = pl->s;
+    const Config& c = call_config(S, pl, C, epi ? epi->D : nullptr, epi && epi->d_is_vector);
     const bool b_mn = s.layoutB == ADAPT_ROW_MAJOR;       // N contiguous
     // class tiles read A through per-row-class maps: in place when its base is 16-byte aligned (whatever K
     // is), else over a re-pitched copy; the k-class views of B need an aligned base, else B is copied
@@ -1406,9 +1409,10 @@ adapt_status_t run_umma(State& S, Plan* pl, const Config& c, const void* A, cons
     return launch_reduce(S, partial, C, s.M, s.N, p.P_k, s.dtype, stream, epi, release);
 }
 
-adapt_status_t run_simt(State& S, const Shape& s, const Config& c, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi)
+adapt_status_t run_simt(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi = nullptr)
 {
-    const int P_k = c.P_k;
+    const Shape& s = pl->s;
+    const int P_k = pl->c.P_k;
     const bool partials = P_k > 1;
     const size_t szP = partials ? (size_t)round_up((int64_t)P_k * s.M * partial_pitch(s.N) * 4, 256) : 0;
     void* ws = nullptr;
@@ -1435,16 +1439,18 @@ adapt_status_t run_simt(State& S, const Shape& s, const Config& c, const void* A
     return ADAPT_OK;
 }
 
-adapt_status_t run_cluster(State& S, const Shape& s, const Config& c, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi)
+adapt_status_t run_cluster(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi = nullptr)
 {
-    if (launch_cluster(s, c, A, B, C, S.machine.n_sm, stream, S.prefetch, epi) != ADAPT_OK) return fail(ADAPT_ERR_CUDA, "cluster kernel launch failed%s");
+    if (launch_cluster(pl->s, pl->c, A, B, C, S.machine.n_sm, stream, S.prefetch, epi) != ADAPT_OK) return fail(ADAPT_ERR_CUDA, "cluster kernel launch failed%s");
     S.launches.fetch_add(1, std::memory_order_relaxed);
     CUDA_TRY(cudaGetLastError());
     return ADAPT_OK;
 }
 
-adapt_status_t run_skinny(State& S, const Shape& s, const Config& c, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi)
+adapt_status_t run_skinny(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi = nullptr)
 {
+    const Shape& s = pl->s;
+    const Config& c = pl->c;
     const size_t szP = c.P_k > 1 ? (size_t)round_up((int64_t)c.P_k * s.M * partial_pitch(s.N) * 4, 256) : 0;
     void* ws = nullptr;
     adapt_status_t r = get_workspace(S, stream, szP, &ws);
@@ -1457,81 +1463,23 @@ adapt_status_t run_skinny(State& S, const Shape& s, const Config& c, const void*
     return ADAPT_OK;
 }
 
-// Is the plan's configuration the one the model picks for its shape?  A forced key or a line of a plan table asks for exactly its
-// configuration; a table line that records the model's pick asks for nothing else than no table would.
-bool is_model_pick(State& S, Plan* pl)
-{
-    int known = pl->model_pick.load(std::memory_order_relaxed);
-    if (known < 0) {
-        std::vector<Config> cands;
-        if (pl->selected) {
-            std::lock_guard<std::mutex> lock(S.mu);
-            enumerate_configs(pl->s, S.machine, S.calib, &cands);
-        }
-        known = !cands.empty() && pack_tiling_key(pl->s, cands[0]) == pack_tiling_key(pl->s, pl->c) ? 1 : 0;
-        pl->model_pick.store(known, std::memory_order_relaxed);
-    }
-    return known != 0;
-}
-
-// The configuration of a call that writes C and adds D (null: none): the plan's, but for tall tiles that cannot serve it.  They store whole 32-byte
-// sectors, add D in 16-byte chunks and have one order of k; and a matrix D over a short k range makes trips to memory that nothing hides
-// (64179 x 576 x 896: 106 us, 108.8 on tall tiles; 5366 x 16320 x 1920: 322 and 287).  Such a call takes the best configuration on other tiles, the
-// one the model would choose if there were no tall ones; a plan that asks for tall tiles by its key takes 256-row pair tiles.
-const Config& call_config(State& S, Plan* pl, const void* C, const void* D, bool d_is_vector)
-{
-    const Config& c = pl->c;
-    if (c.BM != 512) return c;
-    const bool reorder = S.shuffle_k && c.srcA != ADAPT_SRC_TMA_CLASSES;
-    if (((uintptr_t)C & 31) == 0 && ((uintptr_t)D & 15) == 0 && (!D || d_is_vector || pl->s.K >= 1024) && !reorder) return c;
-    if (!pl->other_known.load(std::memory_order_acquire)) {
-        const bool model = is_model_pick(S, pl);                // (a line of a plan table may name the model's choice)
-        std::lock_guard<std::mutex> lock(S.mu);
-        if (!pl->other_known.load(std::memory_order_relaxed)) {
-            std::vector<Config> cands;
-            if (model) enumerate_configs(pl->s, S.machine, S.calib, &cands);
-            remember_other(pl, cands);
-            if (!pl->other_known.load(std::memory_order_relaxed)) {
-                pl->other = short_counterpart(pl->s, S.machine, S.calib, c);
-                pl->other_known.store(true, std::memory_order_release);
-            }
-        }
-    }
-    return pl->other;
-}
-
 adapt_status_t run_plan(State& S, Plan* pl, const void* A, const void* B, void* C, cudaStream_t stream, const ReduceEpilogue* epi)
 {
-    const Shape& s = pl->s;
-    const Config* c = &call_config(S, pl, C, epi ? epi->D : nullptr, epi && epi->d_is_vector);
-    Config uncut;
-    if (c != &pl->c && c->workspace_bytes > pl->c.workspace_bytes) {
-        // a second configuration over a workspace that the plan itself does not need: without it (a capture, no memory) 256-row pair tiles
-        const bool a_rm = s.layoutA == ADAPT_ROW_MAJOR, b_rm = s.layoutB == ADAPT_ROW_MAJOR;
-        const int64_t copies = (((uintptr_t)A & 15) ? round_up((a_rm ? s.M : s.K) * padded_pitch(a_rm ? s.K : s.M) * 2, 256) : 0) +
-                               (((uintptr_t)B & 15) ? round_up((b_rm ? s.K : s.N) * padded_pitch(b_rm ? s.N : s.K) * 2, 256) : 0);
-        void* probe = nullptr;
-        const adapt_status_t r = try_workspace(S, stream, (size_t)(c->workspace_bytes + copies), &probe);
-        if (r != ADAPT_OK) return r;
-        if (!probe) {
-            uncut = short_counterpart(s, S.machine, S.calib, pl->c);
-            c = &uncut;
-        }
-    }
-    switch (c->family) {
+    switch (pl->c.family) {
         case ADAPT_FAM_UMMA_1CTA:
-        case ADAPT_FAM_UMMA_2CTA: return run_umma(S, pl, *c, A, B, C, stream, epi);
-        case ADAPT_FAM_SKINNY: return run_skinny(S, s, *c, A, B, C, stream, epi);
-        case ADAPT_FAM_SIMT: return run_simt(S, s, *c, A, B, C, stream, epi);
-        case ADAPT_FAM_CLUSTER: return run_cluster(S, s, *c, A, B, C, stream, epi);
+        case ADAPT_FAM_UMMA_2CTA: return run_umma(S, pl, A, B, C, stream, epi);
+        case ADAPT_FAM_SKINNY: return run_skinny(S, pl, A, B, C, stream, epi);
+        case ADAPT_FAM_SIMT: return run_simt(S, pl, A, B, C, stream, epi);
+        case ADAPT_FAM_CLUSTER: return run_cluster(S, pl, A, B, C, stream, epi);
     }
     return fail(ADAPT_ERR_UNSUPPORTED, "unknown kernel family%s");
 }
 
-// Does adapt_matmul on these operands, with the call's configuration, use the workspace of its stream?
-bool needs_workspace(const Plan* pl, const Config& c, const void* A, const void* B)
+// Does adapt_matmul on these operands use the workspace of its stream?
+bool needs_workspace(const Plan* pl, const void* A, const void* B)
 {
     if (pl->noop || pl->zero_fill) return false;
+    const Config& c = pl->c;
     if (c.family == ADAPT_FAM_CLUSTER) return false;
     if (c.P_k > 1 && !c.fused) return true;
     if (c.family == ADAPT_FAM_SIMT || c.family == ADAPT_FAM_SKINNY) return false;
@@ -1674,6 +1622,23 @@ adapt_status_t launch_batch_umma(State& S, const Shape& s, int BN, const BatchOp
     CUDA_TRY(launch_exc(&cfg, umma_lookup_batch(BN, a_mn, b_mn), args, bytes, 2));
     S.launches.fetch_add(1, std::memory_order_relaxed);
     return ADAPT_OK;
+}
+
+// Is the plan's configuration the one the model picks for its shape?  A forced key or a line of a plan table asks for exactly its
+// configuration; a table line that records the model's pick asks for nothing else than no table would.
+bool is_model_pick(State& S, Plan* pl)
+{
+    int known = pl->model_pick.load(std::memory_order_relaxed);
+    if (known < 0) {
+        std::vector<Config> cands;
+        if (pl->selected) {
+            std::lock_guard<std::mutex> lock(S.mu);
+            enumerate_configs(pl->s, S.machine, S.calib, &cands);
+        }
+        known = !cands.empty() && pack_tiling_key(pl->s, cands[0]) == pack_tiling_key(pl->s, pl->c) ? 1 : 0;
+        pl->model_pick.store(known, std::memory_order_relaxed);
+    }
+    return known != 0;
 }
 
 // A strided batch in as few launches as its copies allow.  Returns in *done the entries enqueued, from the first on; the others are to
@@ -1885,8 +1850,7 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
     }
     // Small calls (plans of the one-launch and CUDA-core families, as adapt_matmul_plan returned them) leave in grouped launches.
     auto grouped = [&](const Plan* pl) { return pl && pl->selected && !pl->noop && !pl->zero_fill && group_eligible(pl->s, pl->c); };
-    auto config = [&](int64_t i) -> const Config& { return call_config(S, plans[i], C[i], nullptr, false); };
-    auto workspace = [&](int64_t i) { return plans[i] && needs_workspace(plans[i], config(i), A[i], B[i]); };
+    auto workspace = [&](int64_t i) { return plans[i] && needs_workspace(plans[i], A[i], B[i]); };
     int64_t singles = 0, with_workspace = 0, single = 0, small[kBatchVariants] = {}, first[kGroupMax];
     for (int64_t i = 0; i < count; ++i) {
         if (grouped(plans[i])) {
@@ -1904,7 +1868,7 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
     double hidden_us = 0.0;
     if (count >= 8 && singles == 1 && grouped_launches == 1 && with_workspace == 0 && plans[single]) {
         GroupEntry entry[kGroupMax];
-        hidden_us = batch_hidden_us(entry, ops.entries(first, (size_t)(count - 1), entry), S.machine.n_sm, config(single).predicted_us);
+        hidden_us = batch_hidden_us(entry, ops.entries(first, (size_t)(count - 1), entry), S.machine.n_sm, plans[single]->c.predicted_us);
     }
     // Lane 0 is the caller's stream, the others are internal streams between a fork from and a join to it.
     const int NL = 1 + batch_internal_lanes(count, singles, with_workspace, S.batch_lanes, grouped_launches, hidden_us);
@@ -1938,9 +1902,8 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
         k.groupable = grouped(pl);
         k.variant = BatchOps::variant(s);
         k.workspace = workspace(i);
-        const Config& c = config(i);
-        k.alone = c.streamk != 0;
-        k.us = c.predicted_us;
+        k.alone = pl->c.streamk != 0;
+        k.us = pl->c.predicted_us;
         return k;
     };
     const adapt_status_t status = run_batch(count, NL, call_of, ops);

@@ -841,7 +841,7 @@ Config short_counterpart(const Shape& s, const Machine& m, const Calib& cal, con
 {
     Machine all = m;
     all.family_mask |= 1u << ADAPT_FAM_UMMA_2CTA;
-    all.workspace_limit = INT64_MAX;                                // no larger than the tall plan's, which is there
+    all.workspace_limit = INT64_MAX;                                // (the tall plan's, which is there)
     Config c;
     c.family = tall.family; c.BM = 256; c.BN = tall.BN; c.BK = tall.BK; c.cluster = tall.cluster; c.P_k = 1;
     c.srcA = tall.srcA; c.srcB = tall.srcB;

@@ -1,5 +1,4 @@
-"""Plans of tall pair tiles as the library picks them: calls whose buffers the tall tiles cannot serve run the plan's second configuration, also in
-lists and captures."""
+"""Plans of tall pair tiles: calls whose buffers the tall tiles cannot serve run 256-row pair tiles, in one launch, also in lists and captures."""
 import pytest
 import torch
 
@@ -12,14 +11,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.fixture(autouse=True)
-def tall_preferred():
-    """The model made to take tall tiles for the long products of this file, whatever its constants."""
+def options():
     init()
-    old = ab.adapt_get_calibration("eta_tall")
-    ab.adapt_set_calibration("eta_tall", 3.0)
     yield
     ab.adapt_set_option("shuffle_k", 0)
-    ab.adapt_set_calibration("eta_tall", old)
 
 
 def stream():
@@ -40,8 +35,8 @@ class Call:
     """Operands of one call, C (and D) a number of elements off an allocation's start."""
 
     def __init__(self, M, N, K, dtype, lA=0, lB=0, c_off=0, addmm=None, d_off=0):
-        self.plan = ab.adapt_matmul_plan(M, N, K, dtype, lA, lB)
-        assert ab.adapt_plan_info(self.plan).BM == 512, (M, N, K, lA, lB)
+        tall = next(c for c in ab.adapt_plan_candidates(M, N, K, dtype, lA, lB) if c.BM == 512)
+        self.plan = ab.adapt_matmul_plan_forced(M, N, K, dtype, lA, lB, tall.tiling_key)
         self.A, self.B = integers(M * K, 1, dtype), integers(K * N, 2, dtype)
         self.flat = torch.full((M * N + 128,), float("nan"), dtype=self.A.dtype, device="cuda")
         self.at = 64 + c_off
@@ -77,63 +72,51 @@ def launches(call, st):
     return ab.adapt_launch_count() - before
 
 
-# second configurations: pair and 1-CTA tiles in splits, stream-K, uncut tiles in place and over a copy, row classes uncut and in splits, and a split over
-# a copy in place of row classes
-SHAPES = [(1207, 4416, 8704), (407, 3248, 3848), (3401, 5552, 7632), (5372, 16320, 896), (3623, 3616, 1219), (3367, 2608, 4955), (3749, 2704, 8389), (2491, 2080, 8573)]
+# in place, a short k range, over a copy, of row classes
+SHAPES = [(1207, 4416, 2048), (5372, 4096, 896), (3623, 3616, 1219), (3367, 2608, 2955)]
+
+
+def copies(call):
+    return int(call.info.srcA == 1 or call.info.srcB == 1)
 
 
 @pytest.mark.parametrize("shape", SHAPES)
 @pytest.mark.parametrize("addmm", [None, "bias", "matrix"])
-def test_unaligned_output_runs_the_second_configuration(shape, addmm):
+def test_unaligned_output(shape, addmm):
     for c_off in (8, 1):
         call = Call(*shape, ab.BF16, c_off=c_off, addmm=addmm)
-        i = call.info
-        best = next(c for c in ab.adapt_plan_candidates(*shape, ab.BF16) if c.BM != 512)
-        assert i.tiling_key == best.tiling_key
-        assert launches(call, stream()) == 1 + (i.P_k > 1 and not i.fused) + (i.srcA == 1 or i.srcB == 1)
+        assert call.info.BM == 256 and launches(call, stream()) == 1 + copies(call)
         call.check()
 
 
 @pytest.mark.parametrize("lA,lB", [(0, 0), (0, 1), (1, 0), (1, 1)])
 def test_unaligned_or_short_added_matrix_and_reordered_k(lA, lB):
-    for addmm, d_off, shape in [("bias", 1, (1208, 4416, 8704)), ("matrix", 4, (1208, 4416, 8704)), ("matrix", 0, (5376, 16320, 896))]:
+    for addmm, d_off, shape in [("bias", 1, (1208, 4416, 2048)), ("matrix", 4, (1208, 4416, 2048)), ("matrix", 0, (5376, 4096, 896))]:
         call = Call(*shape, ab.F16, lA, lB, addmm=addmm, d_off=d_off)
-        assert call.info.BM != 512
+        assert call.info.BM == 256
         call.run(stream())
         call.check()
-    call = Call(1208, 4416, 8704, ab.F16, lA, lB)
+    call = Call(1208, 4416, 2048, ab.F16, lA, lB)
     assert call.info.BM == 512
     call.run(stream())
     call.check()
     ab.adapt_set_option("shuffle_k", 1)
-    assert ab.adapt_plan_info_call(call.plan, call.C.data_ptr()).BM != 512
+    assert ab.adapt_plan_info_call(call.plan, call.C.data_ptr()).BM == 256
     call.run(stream())
     call.check()
 
 
-def test_capture_without_the_second_configurations_workspace():
-    """The plan needs no workspace, so a call of it can be captured on any stream: where the k splits of the second configuration have none, 256-row
-    tiles without a split run."""
-    call = Call(1207, 4416, 8704, ab.BF16, c_off=8)
-    assert ab.adapt_plan_info(call.plan).workspace_bytes == 0 and call.info.P_k > 1 and call.info.workspace_bytes > 0
-    assert launches(call, stream()) == 2
-    call.check()
-    call.C.fill_(float("nan"))
+def test_capture_and_lists():
+    """No workspace that the plan does not need: such a call can be captured on any stream, and goes into a list as the plan's other calls do."""
+    call = Call(1207, 4416, 2048, ab.BF16, c_off=8)
     side = torch.cuda.Stream()
     torch.cuda.synchronize()
-    graph, before = torch.cuda.CUDAGraph(), ab.adapt_launch_count()
+    graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph, stream=side):
-        call.run(side.cuda_stream)
-    assert ab.adapt_launch_count() - before == 1
+        assert launches(call, side.cuda_stream) == 1
     graph.replay()
     call.check()
-
-
-def test_lists_of_such_calls():
-    """On the library's streams: second configurations with a workspace, or whose CTAs wait for one another, beside other calls."""
     calls = [Call(*s, ab.BF16, c_off=o) for s in SHAPES for o in (8, 0)]
-    for _ in range(2):
-        ab.adapt_matmul_batch([c.plan for c in calls], [c.A.data_ptr() for c in calls], [c.B.data_ptr() for c in calls], [c.C.data_ptr() for c in calls], stream())
-        for c in calls:
-            c.check()
-            c.C.fill_(float("nan"))
+    ab.adapt_matmul_batch([c.plan for c in calls], [c.A.data_ptr() for c in calls], [c.B.data_ptr() for c in calls], [c.C.data_ptr() for c in calls], stream())
+    for c in calls:
+        c.check()

@@ -102,59 +102,38 @@ def test_longest_slot_is_what_the_model_counts(tmp_path):
     assert r.returncode == 0, r.stdout[-2000:] + r.stderr
 
 
-@pytest.fixture
-def tall_preferred():
-    """The model made to take tall tiles wherever they are legal and compute-bound, whatever its constants."""
-    adapt_build.build()
-    ab.load()
-    old = ab.adapt_get_calibration("eta_tall")
-    ab.adapt_set_calibration("eta_tall", 3.0)
-    yield
-    ab.adapt_set_option("shuffle_k", 0)
-    ab.adapt_set_calibration("eta_tall", old)
-
-
 C, D, D_OFF = 1 << 20, 1 << 30, (1 << 30) + 8          # addresses, never followed
 
 
-# (others: 4 splits, 7 splits, uncut tiles over a copy, in place, of row classes)
-@pytest.mark.parametrize("M,N,K", [(1203, 4416, 8704), (413, 4736, 8960), (5366, 16320, 901), (8192, 4096, 1024), (8192, 2048, 4093)])
-def test_second_configuration_is_the_best_on_other_tiles(tall_preferred, M, N, K):
-    plan = ab.adapt_matmul_plan(M, N, K, ab.BF16)
-    key = ab.adapt_plan_info(plan).tiling_key
-    assert ab.adapt_plan_info(plan).BM == 512
-    other = next(c for c in ab.adapt_plan_candidates(M, N, K, ab.BF16) if c.BM != 512)
-    first, second = {(C, 0, False), (C, D, True), (C + 32, D + 16, True)}, {(C + 16, 0, False), (C + 2, D, True), (C, D_OFF, True), (C, D_OFF, False)}
-    (first if K >= 1024 else second).add((C, D, False))
-    for call in first:
-        assert ab.adapt_plan_info_call(plan, *call).tiling_key == key, call
-    for call in second:
-        assert ab.adapt_plan_info_call(plan, *call).tiling_key == other.tiling_key, call
-    ab.adapt_set_option("shuffle_k", 1)                 # (row classes have no such order)
-    assert ab.adapt_plan_info_call(plan, C).tiling_key == (key if ab.adapt_plan_info(plan).srcA == 3 else other.tiling_key)
+@pytest.fixture(autouse=True)
+def library():
+    adapt_build.build()
+    ab.load()
+    yield
+    ab.adapt_set_option("shuffle_k", 0)
 
 
-def test_second_configuration_of_a_forced_key_keeps_its_tiles_and_sources(tall_preferred):
-    for M, N, K, lA, lB in [(1203, 4416, 8704, 0, 0), (300, 272, 80, 1, 1), (4501, 688, 333, 0, 0), (1001, 688, 333, 0, 0)]:
-        tall = next(c for c in ab.adapt_plan_candidates(M, N, K, ab.F16, lA, lB) if c.BM == 512)
-        plan = ab.adapt_matmul_plan_forced(M, N, K, ab.F16, lA, lB, tall.tiling_key)
-        assert ab.adapt_plan_info_call(plan, C).tiling_key == tall.tiling_key
-        i = ab.adapt_plan_info_call(plan, C + 2)
-        assert (i.family, i.BM, i.BN, i.P_k, i.srcA, i.srcB, i.fused, i.streamk) == (ab.FAM_UMMA_2CTA, 256, 256, 1, tall.srcA, tall.srcB, 0, 0)
-        assert any(c.tiling_key == i.tiling_key for c in ab.adapt_plan_candidates(M, N, K, ab.F16, lA, lB))
+# in place, a short k range, over copies, of row classes; plans of the model's choice, and by their keys
+@pytest.mark.parametrize("M,N,K,lA,lB", [(8192, 8192, 8192, 0, 0), (5366, 16320, 896, 0, 0), (8193, 4096, 2048, 1, 1), (5366, 16320, 2901, 0, 0), (12288, 688, 16991, 0, 0), (300, 272, 80, 1, 1)])
+def test_calls_that_tall_tiles_cannot_serve_run_256_row_tiles_over_the_same_sources(M, N, K, lA, lB):
+    cands = ab.adapt_plan_candidates(M, N, K, ab.BF16, lA, lB)
+    tall = next(c for c in cands if c.BM == 512)
+    plans = [ab.adapt_matmul_plan_forced(M, N, K, ab.BF16, lA, lB, tall.tiling_key)]
+    if cands[0].BM == 512:
+        plans.append(ab.adapt_matmul_plan(M, N, K, ab.BF16, lA, lB))
+    assert len(plans) == 1 + (M > 300)
+    served, others = {(C, 0, False), (C, D, True), (C + 32, D + 16, True)}, {(C + 16, 0, False), (C + 2, D, True), (C, D_OFF, True), (C, D_OFF, False)}
+    (served if K >= 1024 else others).add((C, D, False))
+    def runs_short(plan, call):
+        i = ab.adapt_plan_info_call(plan, *call)
+        assert any(c.tiling_key == i.tiling_key for c in cands)
+        return (i.family, i.BM, i.BN, i.P_k, i.srcA, i.srcB, i.fused, i.streamk) == (ab.FAM_UMMA_2CTA, 256, 256, 1, tall.srcA, tall.srcB, 0, 0)
 
-
-def test_second_configuration_of_a_loaded_plan(tall_preferred, tmp_path):
-    M, N, K = 1205, 4416, 8704
-    cands = ab.adapt_plan_candidates(M, N, K, ab.BF16)
-    assert cands[0].BM == 512
-    path = tmp_path / "table.txt"
-    ab.adapt_matmul_plan(M, N, K, ab.BF16)
-    ab.adapt_plan_table_save(str(path))
-    line = [x for x in path.read_text().splitlines() if f"{M} {N} {K}" in x.replace(",", " ")]
-    assert len(line) == 1
-    path.write_text("\n".join([path.read_text().splitlines()[0]] + [line[0].replace(str(M), str(M + 1), 1)]) + "\n")
-    assert ab.adapt_plan_table_load(str(path)) == 1
-    plan = ab.adapt_matmul_plan(M + 1, N, K, ab.BF16)
-    other = next(c for c in ab.adapt_plan_candidates(M + 1, N, K, ab.BF16) if c.BM != 512)
-    assert ab.adapt_plan_info(plan).BM == 512 and ab.adapt_plan_info_call(plan, C + 4).tiling_key == other.tiling_key
+    for plan in plans:
+        for call in served:
+            assert ab.adapt_plan_info_call(plan, *call).tiling_key == tall.tiling_key, call
+        for call in others:
+            assert runs_short(plan, call), call
+        ab.adapt_set_option("shuffle_k", 1)             # (row classes have no such order)
+        assert runs_short(plan, (C, 0, False)) == (tall.srcA != 3)
+        ab.adapt_set_option("shuffle_k", 0)
