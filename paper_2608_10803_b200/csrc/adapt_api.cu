@@ -423,7 +423,7 @@ extern "C" int64_t adapt_map_encode_count(void) { return st().map_encodes.load()
 extern "C" void adapt_set_map_cache(int enabled) { st().map_cache.store(enabled ? 1 : 0); }
 // the model's calibration constants by name (the fields of Calib that are plain doubles)
 #define ADAPT_CALIB_FIELDS(X) X(launch_us) X(prologue_launch_us) X(hbm_bw) X(l2_bw_per_sm) X(tensor_flops) X(eta_mma_bn128) X(eta_mma_bn64) \
-    X(eta_2cta) X(eta_tall) X(tall_tile_us) X(mem_latency_us) X(hbm_latency_us) X(hbm_latency_views_us) X(umma_fixed_us) X(epi_tile_fixed_us) X(epi_us_per_kb) \
+    X(eta_2cta) X(eta_tall) X(eta_tall_half) X(tall_tile_us) X(tall_beside_streamk) X(mem_latency_us) X(hbm_latency_us) X(hbm_latency_views_us) X(umma_fixed_us) X(epi_tile_fixed_us) X(epi_us_per_kb) \
     X(pair_drain_factor) X(epi_partial_fixed_us) X(epi_partial_us_per_kb) X(epi_tile_fixed_unaligned_us) X(epi_us_per_kb_unaligned) \
     X(thread_store_exposed) X(thread_store_exposed_pair) X(simt_flops) X(simt_fixed_us) X(simt_step_us) X(halo_edge_tile_us) X(simt_bw_eff) \
     X(skinny_bw_eff_aligned) X(skinny_bw_eff_unaligned) X(skinny_fixed_us) X(skinny_pass_us) X(skinny_step_unaligned_us) X(skinny_mac_rate) \

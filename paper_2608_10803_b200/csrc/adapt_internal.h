@@ -69,9 +69,16 @@ struct Calib {
     double eta_mma_bn128 = 0.518;        // relative tensor efficiency at BN = 128 (0.29 us per 128 x 128 x 64 block)
     double eta_mma_bn64 = 0.324;         // ... at BN = 64 (A-operand smem reads dominate)
     double eta_2cta = 1.0;              // pair tiles share B: no extra tensor cost
-    double eta_tall = 1.35;             // tall pair tiles: a quarter less operand traffic per flop (1000 x 8192 x 1024: one wave, 17.6 us, 18.6 on
-                                        // 256-row pair tiles; 10000 x 1024 x 1024: 23.0 and 23.5)
-    double tall_tile_us = 0.3;          // ... what a tile's drain does not hide
+    // Tall pair tiles: relative tensor efficiency of whole tiles, of single blocks (they bring B for half the rows), and what a tile's drain does not
+    // hide.  Fitted on 420 shapes whose best tall and best other configuration are predicted within 0.72 .. 1.12 of each other, both timed in turn
+    // with random operands: the pick costs 1.0 % over the better of the two on average (1.8 with one efficiency of 1.35 for all of a tile's work); it takes a
+    // tall configuration that is more than 3 % slower on 31 of them (69) and passes over one that is as much faster on 21 (9).  9000 shapes of another
+    // seed: 64 picks go from split-K, stream-K and 1-CTA tiles to tall ones, to 0.89 of their time, one of the 58 that stay after the next line's rule being
+    // more than 3 % slower; 120 of the 198 picks that left the single efficiency's choice run 0.954 of its time (13 more than 3 % longer).
+    double eta_tall = 1.3;
+    double eta_tall_half = 1.1;
+    double tall_tile_us = 0.5;
+    double tall_beside_streamk = 1.3;   // their time over the model's where stream-K is the best other configuration
     double mem_latency_us = 1.0;        // TMA issue -> data visible (sets Delta_dep with few stages)
     double hbm_latency_us = 1.04;        // the same under a full HBM stream of a dense operand (128 x 128256 x 4096: 5 stages of 32 KB, 0.41 us each)
     double hbm_latency_views_us = 1.6;  // ... through the strided class views (79457 x 196 x 8325 with 3 stages: 0.75 us per stage)
@@ -124,7 +131,8 @@ struct Calib {
     double kclass_view_sm_eff = 0.605;   // per-SM rate through the k-class views of B relative to l2_bw_per_sm (272 x 67839 x 6046: 48 KB per 0.75 us)
     double kclass_unit_fixed_us = 1.65;  // per unit of a k class run as a k split (1 x 80711 x 221: 18 units of one k-block in 37 us)
     double kclass_tile_drain_us = 2.5;  // drain of a tile with eight class accumulators (29 x 58492 x 94: 8 tile rounds in 35 us)
-    double l2_reread_cost = 0.08;       // long contractions: what a second reading of all operands from L2 adds to the stream's time
+    double l2_reread_cost = 0.08;       // long contractions: what a second reading of all operands from L2 adds to the stream's time (it moved
+                                        // twelve of 18000 picks, near ties, to 0.93 .. 1.14 of their time, 0.997 on average)
     double oob_box_penalty = 0.05;      // main-loop cost of one B box per stage that lies wholly beyond N
     double reduce_batch_us = 0.8;       // split-K reduction: one batch of eight slabs (13 x 420 x 43580: P_k 72 -> 24 saves 13 us)
     double class_split_bw_eff = 0.873;   // HBM rate through the k-class views of B with full-width tiles (classes as k splits) at M = 1 ...

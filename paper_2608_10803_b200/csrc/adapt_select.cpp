@@ -224,14 +224,13 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
     const int64_t Q = ceil_div(units, slots);
     c.grid = c.streamk ? (int)(slots * c.cluster) : (int)(std::min(units, slots) * (c.fused ? c.P_k : c.cluster));
     const bool tall = c.BM == 512;
-    double tall_waves = 0.0;
-    const TallWork work = tall_schedule(s.M, c.P_n, c.srcA == ADAPT_SRC_TMA_CLASSES, slots, &tall_waves);
+    const TallWork work = tall_schedule(s.M, c.P_n, c.srcA == ADAPT_SRC_TMA_CLASSES, slots);
     if (tall) c.grid = (int)(std::min<int64_t>(work.big + work.halves, slots) * c.cluster);
 
     const double MK = (double)s.M * s.K, KN = (double)s.K * s.N, MN = (double)s.M * s.N;
     // HBM traffic: operands once, plus re-reads of B when it cannot stay in L2 across m-groups.
     double rB = 1.0, rA = 1.0;
-    const int64_t rows_per_group = (int64_t)kGroupM * c.BM;
+    const int64_t rows_per_group = (int64_t)kGroupM * std::min(c.BM, 256);      // (eight tall tiles: as many rows as sixteen of 256)
     if (2.0 * KN > kL2Bytes) rB = (double)ceil_div(s.M, rows_per_group);
     if (rB > 1.0 && 2.0 * MK <= kL2Bytes) {          // alternatively A stays resident and B streams once
         rB = 1.0;
@@ -301,7 +300,14 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
                                            : std::max((double)L * ii + t_fixed, t_drain);
         // Eq. 14 with the drain overlapped: one fill, Q tiles back to back, the last drain exposed
         pipe = tM + (double)Q * t_tile + tP + t_drain;
-        if (tall) pipe = tM + tall_waves * std::max((double)L * ii + 2.0 * t_fixed + cal.tall_tile_us, t_drain) + tP + t_drain;   // no spare accumulator: the ends of a tile show
+        if (tall) {
+            // no spare accumulator: the ends of a tile show.  A single block brings its share of B for half the rows: a 256-row tile's k-blocks
+            const double tM_half = std::max(stage_bytes * 2.0 / 3.0 / sm_rate * 1e6, mem_bound ? tM : cal.mem_latency_us / (c.stages - 1));
+            const double tP_half = 0.5 * tP * cal.eta_tall / cal.eta_tall_half;
+            const double t_whole = std::max((double)L * ii + 2.0 * t_fixed + cal.tall_tile_us, t_drain);
+            const double t_half = std::max((double)L * std::max(tM_half, tP_half) + t_fixed, 0.5 * t_drain);
+            pipe = tM + tall_length(work, slots, t_whole, t_half) + tP + t_drain;
+        }
         if (c.streamk) {
             // whole waves as above; the leftover tiles' k-blocks shared evenly by all slots, then the owners' fix-up
             // While a slot works on its share of the leftover tiles it is at a k position of its own: nothing it loads is
@@ -828,6 +834,15 @@ void enumerate_configs(const Shape& s, const Machine& m, const Calib& cal, std::
         c.srcA = c.srcB = ADAPT_SRC_LSU;
         if (finalize(s, m, cal, c)) out->push_back(c);
     }
+    // Where the best other configuration is stream-K, a long product whose last wave would be mostly idle, the model has tall tiles too short: the
+    // clock that the power cap leaves does not rise while pairs idle.  The six of 9000 shapes that went from stream-K to tall tiles, predicted 0.81 .. 0.95
+    // of its time, took 1.09 .. 1.21 (6668 x 2112 x 13504: 296 and 357 us).
+    const Config* other = nullptr;
+    for (const Config& c : *out)
+        if (c.BM != 512 && (!other || c.predicted_us < other->predicted_us)) other = &c;
+    if (other && other->streamk)
+        for (Config& c : *out)
+            if (c.BM == 512) c.predicted_us *= cal.tall_beside_streamk;
     // argmin of Eq. 6 with a deterministic tie-break: time, then fewer splits, then smaller
     // workspace, then enumeration order (stable sort keeps it)
     std::stable_sort(out->begin(), out->end(), [](const Config& a, const Config& b) {

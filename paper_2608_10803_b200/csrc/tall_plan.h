@@ -21,7 +21,17 @@ struct TallWork {
     int big;                             // tiles computed as such; the rest as their 256-row halves,
     int split;                           // this many,
     int halves;                          // ... and these with the blocks of the odd rows
+    int last, free_slots;                // slots with a whole tile in the last wave, and without (none: 0, 0)
 };
+
+// The length of a schedule whose whole tiles take t_tile and whose single blocks take t_half: whole waves, then the blocks, first on the slots
+// without a tile in the last wave (two in a tile's time).
+inline double tall_length(const TallWork& w, int64_t slots, double t_tile, double t_half)
+{
+    const int64_t last = w.big % slots, room = last ? 2 * (slots - last) : 0, more = w.halves > room ? w.halves - room : 0;
+    const bool twos = last && 2 * w.halves > room;                   // some slot has two blocks in the last wave's time
+    return (double)(w.big / slots) * t_tile + (last ? (twos && 2.0 * t_half > t_tile ? 2.0 * t_half : t_tile) : 0.0) + (double)((more + slots - 1) / slots) * t_half;
+}
 
 // The tiles that do not fill a whole wave of slots (SM pairs) are cut when all the halves then fit one wave of half the length: they
 // bring B twice, but 2048 x 14336 x 4096, 224 tiles on 74 pairs, takes 3.5 waves instead of 4.
@@ -39,11 +49,10 @@ inline TallWork tall_schedule(int64_t M, int64_t P_n, bool classes, int64_t slot
     w.big = (int)(cut ? tiles - rest : tiles);
     w.split = (int)(cut ? 2 * rest : 0);
     w.halves = (int)(w.split + single);
-    if (waves) {
-        // whole waves, then the halves, first on the slots without a tile in the last wave (two in a tile's time)
-        const int64_t last = w.big % slots, room = last ? 2 * (slots - last) : 0, more = w.halves > room ? w.halves - room : 0;
-        *waves = (double)(w.big / slots + (last ? 1 : 0)) + 0.5 * (double)((more + slots - 1) / slots);
-    }
+    const int64_t n_slots = w.big + w.halves < slots ? w.big + w.halves : slots;
+    w.last = n_slots ? (int)(w.big % n_slots) : 0;
+    w.free_slots = w.last ? (int)(n_slots - w.last) : 0;
+    if (waves) *waves = tall_length(w, slots, 1.0, 0.5);
     return w;
 }
 
@@ -67,15 +76,14 @@ ADAPT_HOST_DEVICE bool tall_item(const TallWork& p, int slot, int n_slots, int i
         t = slot + it * n_slots;
     } else {
         // two for each slot without a tile in the last wave (which the others spend on a whole tile), then one for every slot in turn
-        const int last = p.big % n_slots, free_slots = last ? n_slots - last : 0;
-        const int first = slot < last ? slot + free_slots : slot - last;
+        const int first = slot < p.last ? slot + p.free_slots : slot - p.last;
         int j = it - mine;
         w.acc = j & 1;
-        if (last && slot >= last) {
-            h = first + j * free_slots;
+        if (p.last && slot >= p.last) {
+            h = first + j * p.free_slots;
             j -= 2;
         }
-        if (j >= 0) h = 2 * free_slots + first + j * n_slots;
+        if (j >= 0) h = 2 * p.free_slots + first + j * n_slots;
         if (h >= p.halves) return false;
         t = p.big + (h >> 1);
         if (h >= p.split) {                                    // the odd rows

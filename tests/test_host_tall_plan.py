@@ -137,3 +137,16 @@ def test_calls_that_tall_tiles_cannot_serve_run_256_row_tiles_over_the_same_sour
         ab.adapt_set_option("shuffle_k", 1)             # (row classes have no such order)
         assert runs_short(plan, (C, 0, False)) == (tall.srcA != 3)
         ab.adapt_set_option("shuffle_k", 0)
+
+
+@pytest.mark.parametrize("M,N,K", [(16384, 16384, 4096), (40000, 16384, 4096), (8192, 8192, 8192), (6000, 14336, 4096)])
+def test_both_pair_tiles_are_charged_the_same_readings_of_b(M, N, K):
+    """Eight rows of tall tiles to a raster group are as many rows of A as sixteen of 256."""
+    pair = {c.BM: c for c in ab.adapt_plan_candidates(M, N, K, ab.BF16) if c.family == ab.FAM_UMMA_2CTA and c.BN == 256 and c.P_k == 1 and not c.streamk}
+    assert pair[512].hbm_bytes == pair[256].hbm_bytes
+
+
+@pytest.mark.parametrize("M,N,K,lB", [(6668, 2112, 13504, 1), (5889, 2496, 9408, 0), (966, 10048, 16000, 0), (958, 15424, 12928, 0)])
+def test_stream_k_is_not_given_up_for_a_mostly_idle_wave_of_tall_tiles(M, N, K, lB):
+    cands = ab.adapt_plan_candidates(M, N, K, ab.F16, 0, lB)
+    assert cands[0].streamk and [c.predicted_us for c in cands] == sorted(c.predicted_us for c in cands)
