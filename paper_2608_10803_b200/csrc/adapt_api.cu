@@ -1811,7 +1811,7 @@ struct BatchOps {
     {
         for (size_t j = 0; j < n; ++j) {
             const int64_t i = calls[j];
-            entry[j].chain = group_item(plans[i]->s, plans[i]->c, A[i], B[i], C[i], &entry[j].item);
+            entry[j] = group_entry(plans[i]->s, plans[i]->c, A[i], B[i], C[i]);
         }
         group_order(entry, n, S.machine.n_sm);
         return n;

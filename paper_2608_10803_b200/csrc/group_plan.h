@@ -114,39 +114,77 @@ ADAPT_HOST_DEVICE bool group_place(const GroupParams& p, int cta, GroupPlace& w)
     return cta < it.tile_end && w.entry < p.entries;
 }
 
-// An entry of a list, and the stages one group of warps of its tiles walks.
-struct GroupEntry { GroupItem item; int chain; };
+// What sharing the tiles of a list is weighed with (us): a stage of a group of warps on aligned rows, what the shift of an operand adds whose rows are
+// not on 16-byte boundaries (a whole tile's rows of it), the rest of a CTA's life, the exchange of a shared tile, and a round of further CTAs (two per SM).
+constexpr double kGroupStageUs = 0.5, kGroupShiftUs = 0.4, kGroupTileUs = 1.5, kGroupExchangeUs = 0.3, kGroupRoundUs = 3.5;
 
-// Shares the tiles of an entry whose chain the launch would wait for between two CTAs (four pieces) or four (eight, sixteen), whose groups of
-// warps then walk one piece each, or two.
-inline void group_share(GroupEntry* e, double average_chain)
+// An entry of a list, and the stages one group of warps of its tiles walks.
+struct GroupEntry {
+    GroupItem item;
+    int chain;
+    double stage_us = kGroupStageUs + 2.0 * kGroupShiftUs;
+};
+inline GroupEntry group_entry(const Shape& s, const Config& c, const void* A, const void* B, void* C)
 {
-    GroupItem& it = e->item;
-    if (it.pieces < 4 || e->chain < 3 || 2 * e->chain <= average_chain) return;
-    it.share_log2 = it.pieces == 4 ? 1 : 2;
-    e->chain = it.pieces / (2 << it.share_log2) * (int)ceil_div(it.k_per_piece, kClusterKS);
+    GroupEntry e;
+    e.chain = group_item(s, c, A, B, C, &e.item);
+    const int64_t lda = s.layoutA == ADAPT_ROW_MAJOR ? s.K : s.M, ldb = s.layoutB == ADAPT_ROW_MAJOR ? s.N : s.K;
+    e.stage_us = kGroupStageUs + ((((uintptr_t)A & 15) || lda % 8) ? kGroupShiftUs * std::min(1.0, (double)s.M / 64.0) : 0.0) +
+                 ((((uintptr_t)B & 15) || ldb % 8) ? kGroupShiftUs * std::min(1.0, (double)s.N / 64.0) : 0.0);
+    return e;
 }
 
-// The order of a list's entries in the launch.  An unaligned stage takes a group of warps 1.4 us, so the tile with the most of them is what a
-// short list waits for: its tiles are shared where the chain is longer than half of what a CTA slot (two per SM) has to do on average and
-// the list stays within four CTAs per SM.  Beyond, the SMs are busy while the long chains run (the longest come first), and clusters, which
+// Tiles whose chain the launch would wait for are shared between two CTAs (four pieces) or four (eight, sixteen), whose groups of warps then walk
+// one piece each, or two: log2 of the CTAs, and the chain that is left.
+struct GroupShare { int log2, chain; };
+inline GroupShare group_share(const GroupEntry& e, double average_us)
+{
+    const GroupItem& it = e.item;
+    if (it.pieces < 4 || 2.0 * e.chain * e.stage_us <= average_us) return {0, e.chain};
+    const int log2 = it.pieces == 4 ? 1 : 2, chain = it.pieces / (2 << log2) * (int)ceil_div(it.k_per_piece, kClusterKS);
+    if ((e.chain - chain) * e.stage_us < 1.0) return {0, e.chain};
+    return {log2, chain};
+}
+
+// The order of a list's entries in the launch.  The tile with the longest chain is what a short list waits for: its tiles are shared where the chain is
+// longer than half of what a CTA slot (two per SM) has to do on average, where that takes off more than the exchange and the further CTAs
+// cost, and the list stays within four CTAs per SM.  Beyond, the SMs are busy while the long chains run (the longest come first), and clusters, which
 // start when four slots of a GPC are free, cost more than they save: 8 layers of 16 .. 1024 a side 9.7 -> 7.7 us, 24 layers 19.3 -> 11.8,
-// 15 layers with K > 256 19.4 -> 17.5, but 47 layers (1018 CTAs shared, 762 not) 20.9 -> 27.3.
+// 15 layers with K > 256 19.4 -> 17.5, but 47 layers (1018 CTAs shared, 762 not) 20.9 -> 27.3.  Of 344 lists in which sharing every
+// long chain had been the rule, this one takes 1.003 of the better of both ways on average, that one 1.010 (8 layers of 200 x 200 x 512 beside 20 small
+// ones: 9.1 us and 13.6).
 inline void group_order(GroupEntry* e, size_t n, int n_sm)
 {
-    double work = 0.0;
-    for (size_t j = 0; j < n; ++j) work += (double)e[j].item.tiles * e[j].chain;
-    int64_t ctas = 0;
-    GroupEntry as_is[kGroupMax];
+    const double slots = 2.0 * n_sm;
+    double work = 0.0, longest = 0.0, left = 0.0;
+    int64_t tiles = 0, ctas = 0;
     for (size_t j = 0; j < n; ++j) {
-        as_is[j] = e[j];
-        group_share(&e[j], work / (2.0 * n_sm));
-        ctas += (int64_t)e[j].item.tiles << e[j].item.share_log2;
+        const double us = e[j].chain * e[j].stage_us;
+        work += e[j].item.tiles * us;
+        tiles += e[j].item.tiles;
+        longest = std::max(longest, us);
     }
-    if (ctas > 4 * (int64_t)n_sm) std::copy(as_is, as_is + n, e);
-    std::stable_sort(e, e + n, [](const GroupEntry& x, const GroupEntry& y) {
-        return x.item.share_log2 != y.item.share_log2 ? x.item.share_log2 > y.item.share_log2 : x.chain > y.chain;
-    });
+    GroupShare share[kGroupMax];
+    for (size_t j = 0; j < n; ++j) {
+        share[j] = group_share(e[j], work / slots);
+        ctas += (int64_t)e[j].item.tiles << share[j].log2;
+        left = std::max(left, share[j].chain * e[j].stage_us);
+    }
+    const double busy = (work + kGroupTileUs * tiles) / slots;         // what the slots have to do in any case
+    const double saved = std::max(longest, busy) - std::max(left, busy);
+    const double rounds = (std::max((double)ctas, slots) - std::max((double)tiles, slots)) / slots;
+    if (ctas <= 4 * (int64_t)n_sm && saved > kGroupExchangeUs + kGroupRoundUs * rounds)
+        for (size_t j = 0; j < n; ++j) {
+            e[j].item.share_log2 = (short)share[j].log2;
+            e[j].chain = share[j].chain;
+        }
+    // (by keys: sorting the entries themselves is a tenth of what the host spends on a list)
+    uint32_t key[kGroupMax];
+    for (size_t j = 0; j < n; ++j) key[j] = (uint32_t)(3 - e[j].item.share_log2) << 24 | (uint32_t)(0xffff - std::min(e[j].chain, 0xffff)) << 8 | (uint32_t)j;
+    std::sort(key, key + n);
+    GroupEntry by_key[kGroupMax];
+    for (size_t j = 0; j < n; ++j) by_key[j] = e[key[j] & 0xff];
+    std::copy(by_key, by_key + n, e);
 }
 
 // The kernel of a launch: one stage with all warps on it (SHORT), or two groups of warps with a ring each.  SHORT is the body of a

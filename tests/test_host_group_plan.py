@@ -170,3 +170,65 @@ int main()
 def test_shared_tiles_get_their_ctas_in_one_cluster(tmp_path):
     r = build_and_run(tmp_path, SHARED)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+WORTH = r"""
+#include <cmath>
+#include <cstdio>
+#include <vector>
+#include "group_plan.h"
+using namespace adapt;
+
+struct Dims { int64_t M, N, K; };
+// The entries of a list as the library plans them, in launch order; bit s: some tile is shared by 2^s CTAs.
+static int shares(const std::vector<Dims>& list, uintptr_t offset = 0)
+{
+    std::vector<GroupEntry> e;
+    for (const Dims& d : list) {
+        Shape s;
+        s.M = d.M; s.N = d.N; s.K = d.K;
+        std::vector<Config> all;
+        enumerate_configs(s, Machine(), default_calib(), &all);
+        if (!group_eligible(s, all[0])) { printf("%lld x %lld x %lld is not for the grouped launch\n", (long long)d.M, (long long)d.N, (long long)d.K); return -1; }
+        e.push_back(group_entry(s, all[0], (const void*)(4096 + offset), (const void*)8192, (void*)16384));
+    }
+    group_order(e.data(), e.size(), 148);
+    int bits = 0;
+    for (const GroupEntry& x : e) bits |= 1 << x.item.share_log2;
+    return bits;
+}
+static int bad = 0;
+static void check(bool ok, const char* what) { if (!ok) { printf("%s\n", what); ++bad; } }
+
+int main()
+{
+    // the lists of the bit-for-bit test on the GPU: tiles of one, two and four CTAs
+    const std::vector<std::vector<Dims>> lists = {{{84, 39, 1014}, {20, 30, 40}}, {{504, 209, 576}, {100, 100, 100}, {30, 7, 20}},
+        {{64, 64, 1024}, {65, 63, 1000}, {17, 763, 618}, {105, 845, 611}, {1, 1, 500}}, {{38, 48, 787}, {48, 38, 808}, {1, 70, 790}},
+        {{64, 128, 1008}, {16, 200, 520}, {129, 1, 400}, {300, 200, 50}, {10, 10, 65}, {33, 65, 130}, {7, 9, 11}, {40, 342, 267}}};
+    int seen = 0;
+    for (const auto& l : lists) seen |= shares(l);
+    check(seen == 7, "tiles of one, two and four CTAs");
+    // eight layers of 16 tiles beside 20 small ones: not where four CTAs to a tile are a round more
+    auto beside = [&](int count, Dims d) { std::vector<Dims> l(20, Dims{40, 40, 40}); l.insert(l.end(), count, d); return l; };
+    for (int64_t K : {384, 500, 512}) check(shares(beside(8, {200, 200, K})) == 1, "many tiles of medium chains");
+    check(shares(beside(1, {128, 65, 500})) == (1 | 4) && shares(beside(4, {64, 64, 1024})) == (1 | 4), "long chains of a few tiles");
+    // a stage takes longer by the shift of each operand off 16-byte boundaries: its rows, its buffer, as many rows as a tile has of it
+    auto stage = [&](Dims d, uintptr_t a, uintptr_t b) {
+        Shape s;
+        s.M = d.M; s.N = d.N; s.K = d.K;
+        std::vector<Config> all;
+        enumerate_configs(s, Machine(), default_calib(), &all);
+        return group_entry(s, all[0], (const void*)a, (const void*)b, nullptr).stage_us;
+    };
+    check(stage({64, 64, 512}, 4096, 8192) == kGroupStageUs && stage({64, 64, 512}, 4098, 8192) == kGroupStageUs + kGroupShiftUs, "a buffer");
+    check(std::abs(stage({64, 63, 511}, 4096, 8192) - (kGroupStageUs + kGroupShiftUs * (1.0 + 63.0 / 64.0))) < 1e-12 && stage({16, 64, 511}, 4096, 8192) == kGroupStageUs + kGroupShiftUs / 4, "rows");
+    check(shares(std::vector<Dims>(60, Dims{130, 65, 389})) == 1, "busy SMs");
+    return bad;
+}
+"""
+
+
+def test_tiles_are_shared_where_it_pays(tmp_path):
+    r = build_and_run(tmp_path, WORTH)
+    assert r.returncode == 0, r.stdout + r.stderr
