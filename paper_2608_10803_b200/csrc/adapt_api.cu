@@ -1811,7 +1811,7 @@ struct BatchOps {
     {
         for (size_t j = 0; j < n; ++j) {
             const int64_t i = calls[j];
-            entry[j] = group_entry(plans[i]->s, plans[i]->c, A[i], B[i], C[i]);
+            group_entry(plans[i]->s, plans[i]->c, A[i], B[i], C[i], &entry[j]);
         }
         group_order(entry, n, S.machine.n_sm);
         return n;
@@ -1851,24 +1851,30 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
     // Small calls (plans of the one-launch and CUDA-core families, as adapt_matmul_plan returned them) leave in grouped launches.
     auto grouped = [&](const Plan* pl) { return pl && pl->selected && !pl->noop && !pl->zero_fill && group_eligible(pl->s, pl->c); };
     auto workspace = [&](int64_t i) { return plans[i] && needs_workspace(plans[i], A[i], B[i]); };
-    int64_t singles = 0, with_workspace = 0, single = 0, small[kBatchVariants] = {}, first[kGroupMax];
+    int64_t singles = 0, with_workspace = 0, single = 0;
     for (int64_t i = 0; i < count; ++i) {
-        if (grouped(plans[i])) {
-            if (i - singles < kGroupMax) first[i - singles] = i;
-            ++small[BatchOps::variant(plans[i]->s)];
-            continue;
-        }
+        if (grouped(plans[i])) continue;
         ++singles;
         single = i;
         with_workspace += workspace(i) ? 1 : 0;
     }
-    int64_t grouped_launches = 0;
-    for (int64_t n : small) grouped_launches += ceil_div(n, kGroupMax);
     BatchOps ops = {S, plans, A, B, C, {user}};
+    int64_t grouped_launches = 1;
     double hidden_us = 0.0;
-    if (count >= 8 && singles == 1 && grouped_launches == 1 && with_workspace == 0 && plans[single]) {
-        GroupEntry entry[kGroupMax];
-        hidden_us = batch_hidden_us(entry, ops.entries(first, (size_t)(count - 1), entry), S.machine.n_sm, plans[single]->c.predicted_us);
+    if (count >= 8 && singles == 1 && with_workspace == 0) {            // two launches, or more
+        int64_t small[kBatchVariants] = {}, others[kGroupMax], n = 0;
+        for (int64_t i = 0; i < count; ++i) {
+            if (i == single) continue;
+            if (n < kGroupMax) others[n] = i;
+            ++n;
+            ++small[BatchOps::variant(plans[i]->s)];
+        }
+        grouped_launches = 0;
+        for (int64_t k : small) grouped_launches += ceil_div(k, kGroupMax);
+        if (grouped_launches == 1 && plans[single]) {
+            GroupEntry entry[kGroupMax];
+            hidden_us = batch_hidden_us(entry, ops.entries(others, (size_t)n, entry), S.machine.n_sm, plans[single]->c.predicted_us);
+        }
     }
     // Lane 0 is the caller's stream, the others are internal streams between a fork from and a join to it.
     const int NL = 1 + batch_internal_lanes(count, singles, with_workspace, S.batch_lanes, grouped_launches, hidden_us);

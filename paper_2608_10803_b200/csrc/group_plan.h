@@ -124,14 +124,12 @@ struct GroupEntry {
     int chain;
     double stage_us = kGroupStageUs + 2.0 * kGroupShiftUs;
 };
-inline GroupEntry group_entry(const Shape& s, const Config& c, const void* A, const void* B, void* C)
+inline void group_entry(const Shape& s, const Config& c, const void* A, const void* B, void* C, GroupEntry* e)
 {
-    GroupEntry e;
-    e.chain = group_item(s, c, A, B, C, &e.item);
+    e->chain = group_item(s, c, A, B, C, &e->item);
     const int64_t lda = s.layoutA == ADAPT_ROW_MAJOR ? s.K : s.M, ldb = s.layoutB == ADAPT_ROW_MAJOR ? s.N : s.K;
-    e.stage_us = kGroupStageUs + ((((uintptr_t)A & 15) || lda % 8) ? kGroupShiftUs * std::min(1.0, (double)s.M / 64.0) : 0.0) +
+    e->stage_us = kGroupStageUs + ((((uintptr_t)A & 15) || lda % 8) ? kGroupShiftUs * std::min(1.0, (double)s.M / 64.0) : 0.0) +
                  ((((uintptr_t)B & 15) || ldb % 8) ? kGroupShiftUs * std::min(1.0, (double)s.N / 64.0) : 0.0);
-    return e;
 }
 
 // Tiles whose chain the launch would wait for are shared between two CTAs (four pieces) or four (eight, sixteen), whose groups of warps then walk
@@ -182,9 +180,9 @@ inline void group_order(GroupEntry* e, size_t n, int n_sm)
     uint32_t key[kGroupMax];
     for (size_t j = 0; j < n; ++j) key[j] = (uint32_t)(3 - e[j].item.share_log2) << 24 | (uint32_t)(0xffff - std::min(e[j].chain, 0xffff)) << 8 | (uint32_t)j;
     std::sort(key, key + n);
-    GroupEntry by_key[kGroupMax];
-    for (size_t j = 0; j < n; ++j) by_key[j] = e[key[j] & 0xff];
-    std::copy(by_key, by_key + n, e);
+    GroupEntry as_given[kGroupMax];
+    std::copy(e, e + n, as_given);
+    for (size_t j = 0; j < n; ++j) e[j] = as_given[key[j] & 0xff];
 }
 
 // The kernel of a launch: one stage with all warps on it (SHORT), or two groups of warps with a ring each.  SHORT is the body of a

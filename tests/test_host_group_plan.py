@@ -190,7 +190,8 @@ static int shares(const std::vector<Dims>& list, uintptr_t offset = 0)
         std::vector<Config> all;
         enumerate_configs(s, Machine(), default_calib(), &all);
         if (!group_eligible(s, all[0])) { printf("%lld x %lld x %lld is not for the grouped launch\n", (long long)d.M, (long long)d.N, (long long)d.K); return -1; }
-        e.push_back(group_entry(s, all[0], (const void*)(4096 + offset), (const void*)8192, (void*)16384));
+        e.emplace_back();
+        group_entry(s, all[0], (const void*)(4096 + offset), (const void*)8192, (void*)16384, &e.back());
     }
     group_order(e.data(), e.size(), 148);
     int bits = 0;
@@ -219,7 +220,9 @@ int main()
         s.M = d.M; s.N = d.N; s.K = d.K;
         std::vector<Config> all;
         enumerate_configs(s, Machine(), default_calib(), &all);
-        return group_entry(s, all[0], (const void*)a, (const void*)b, nullptr).stage_us;
+        GroupEntry e;
+        group_entry(s, all[0], (const void*)a, (const void*)b, nullptr, &e);
+        return e.stage_us;
     };
     check(stage({64, 64, 512}, 4096, 8192) == kGroupStageUs && stage({64, 64, 512}, 4098, 8192) == kGroupStageUs + kGroupShiftUs, "a buffer");
     check(std::abs(stage({64, 63, 511}, 4096, 8192) - (kGroupStageUs + kGroupShiftUs * (1.0 + 63.0 / 64.0))) < 1e-12 && stage({16, 64, 511}, 4096, 8192) == kGroupStageUs + kGroupShiftUs / 4, "rows");
