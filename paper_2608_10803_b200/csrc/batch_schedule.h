@@ -154,6 +154,11 @@ adapt_status_t run_batch(int64_t count, int lanes, CallOf call_of, Ops& ops)
         if ((k.unsound || meets_pending(k)) && (status = flush_all()) != ADAPT_OK) break;
         if (k.groupable && !k.unsound) {
             Pending& g = pending[k.variant];
+            if (g.calls.empty()) {                      // (growing them call by call is a tenth of what a list of small calls takes the host)
+                g.calls.reserve(kGroupMax);
+                g.reads.reserve(2 * kGroupMax);
+                g.writes.reserve(kGroupMax);
+            }
             g.calls.push_back(i);
             g.reads.push_back(k.a);
             g.reads.push_back(k.b);
