@@ -4,10 +4,12 @@
 // (8192^3 with zero operands, where power does not interfere, cycles per k-block: 685 in full, 587 with the MMAs alone, 638 with the loads
 // alone; six or seven stages change nothing), and with data in the operands the same traffic is the energy the power cap takes out of the
 // clock.  Here a CTA takes 256 rows and half of 256 columns: 48 KB per 1024 cycles of MMA, a quarter less per flop.
-// Measured, 256 x 256 pair tiles -> this kernel, bf16 with random operands under the power cap: 8192^3 920 -> 801 us, 16384 x 16384 x 4096
-// 2167 -> 1560, 2048 x 14336 x 4096 207 -> 183, 2048 x 4096 x 4096 59 -> 52, 4096 x 4096 x 2048 64 -> 55, 12288 x 688 x 16991 (row classes)
-// 305 -> 258; short k ranges gain little: 8192 x 4096 x 512 36.6 -> 34.6, 10000 x 1024 x 1024 23.5 -> 23.0, and row classes lose there
-// (20000 x 512 x 333: 17.1, 15.6 on 1-CTA tiles).  8192^3 with zero operands: 601 -> 523 us = 2.1 PFLOP/s.
+// Measured by itself in a row of calls, 256 x 256 pair tiles -> this kernel, bf16 with random operands under the power cap: 8192^3 920 -> 801 us,
+// 16384 x 16384 x 4096 2167 -> 1560, 2048 x 14336 x 4096 207 -> 183, 2048 x 4096 x 4096 59 -> 52, 4096 x 4096 x 2048 64 -> 55, 12288 x 688 x 16991 (row
+// classes) 305 -> 258.  A 2048-token training step of a 4096 x 4096 layer makes the fourth of these twice and the fifth once: one after the other, with
+// operands from DRAM and 64 tiles on 74 pairs, they take 193 -> 186 us in all.  Short k ranges gain little: 8192 x 4096 x 512 36.6 -> 34.6,
+// 10000 x 1024 x 1024 23.5 -> 23.0, and row classes lose there (20000 x 512 x 333: 17.1, 15.6 on 1-CTA tiles).  8192^3 with zero operands: 601 -> 523 us
+// = 2.1 PFLOP/s.  Profiled on 8192 x 8192 x 4096: tensor pipe 88 % busy (78), 3.6 GB through L2 (5.3).
 //
 // The two accumulators are the halves of one tile, so there is no spare buffer to hide the drain of a tile behind the next one's MMAs.
 // Instead the halves are a few k-blocks apart at the ends of a tile: the upper half's MMAs of the first kTallLag k-blocks are issued before
@@ -16,7 +18,7 @@
 // back, and lets the packed values leave through one TMA store box per warp (the ring takes 192 KB) beside the next tile's MMAs.
 // (Stored from the registers, 32 rows of 32 bytes an instruction, a tile took 8 us instead of 4.)
 //
-// Tiles that would leave most of the last wave idle are cut into their 256-row halves (tall_schedule).
+// Tiles that would leave most of the last wave idle are cut into their 256-row halves (tall_schedule).  k runs in one order (no rotation by tile).
 #pragma once
 
 #include "umma_gemm.cuh"
