@@ -64,7 +64,7 @@ struct TallItem {
 };
 
 // The it-th item of a slot: its whole tiles, then its share of the single blocks.  (A single block behind the whole tile of a slot, where
-// another slot had none: 1771 x 4736 x 6288, 57 tiles and 19 single blocks on 74 pairs, 100 us instead of 62 with zero operands.)
+// another slot had none: 1771 x 4736 x 6288, 57 tiles and 19 single blocks on 74 pairs, with zero operands 100 us, 77 this way.)
 template <bool CLS>
 ADAPT_HOST_DEVICE bool tall_item(const TallWork& p, int slot, int n_slots, int it, TallItem& w)
 {
