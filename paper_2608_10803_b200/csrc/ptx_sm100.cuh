@@ -70,17 +70,24 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// One lane of a converged warp, the same one every time.  A loop guarded by it as a whole is known to run in one thread: a TMA request or an MMA
+// then takes its operands from uniform registers, where one guarded by a lane number is issued through a loop over the active lanes.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t one;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(one));
+    return one != 0;
+}
+
 // Bounded wait.  Returns false when the time limit expires or another role has already given
 // up (abort flag in shared memory); the caller then leaves its loop and falls through to the
 // kernel's common exit.
 constexpr uint64_t kWaitLimitNs = 2000000000ull;   // 2 s: orders of magnitude above any legitimate wait
 __device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, volatile int* abort_flag, uint64_t limit_ns)
 {
-    if (mbar_try_wait(bar, parity)) return true;
-    uint32_t spins = 0;
     uint64_t t0 = 0;
-    while (!mbar_try_wait(bar, parity)) {
-        if ((++spins & 0xff) == 0) {
+    for (uint32_t spins = 1; !mbar_try_wait(bar, parity); ++spins) {
+        if ((spins & 0xff) == 0) {
             if (*abort_flag) return false;
             const uint64_t now = globaltimer_ns();
             if (t0 == 0) t0 = now;
@@ -92,6 +99,20 @@ __device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, v
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag)
 {
     return mbar_wait_limit(bar, parity, abort_flag, kWaitLimitNs);
+}
+
+// The same for a whole warp, with one outcome for all its lanes: what follows may elect one of them.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag)
+{
+    uint64_t t0 = 0;
+    for (uint32_t spins = 1; !__all_sync(0xffffffffu, mbar_try_wait(bar, parity)); ++spins) {
+        if ((spins & 0xff) == 0) {
+            const uint64_t now = globaltimer_ns();
+            if (t0 == 0) t0 = now;
+            if (__any_sync(0xffffffffu, *abort_flag != 0 || now - t0 > kWaitLimitNs)) { *abort_flag = 1; return false; }
+        }
+    }
+    return true;
 }
 
 // The same wait with cluster-scope acquire: for barriers that CTAs of the cluster arrive on after writing
@@ -347,6 +368,14 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr, uint32_t lbo
 {
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) |
            ((uint64_t)(sbo_bytes >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+// A descriptor from its two halves.  The start address, in units of 16 bytes, is the lowest field: no address of shared memory carries out of it, so a
+// loop moves a descriptor by adding to the low half, one instruction (the loop that issues the MMAs is bound by its instructions).
+__device__ __forceinline__ uint64_t smem_desc_join(uint32_t lo, uint32_t hi)
+{
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+    return d;
 }
 
 }  // namespace ptx

@@ -100,11 +100,10 @@ tall_gemm_kernel(const __grid_constant__ TmapPackT<CLS ? 1 : 0> maps, const __gr
     ptx::tc_fence_after();
     const uint32_t tmem_base = *tmem_slot_ptr;
 
-    // One lane per TMA request of a k-block: A's boxes of the upper half, of the lower half, then B's.
+    // The TMA requests of a k-block: A's boxes of the upper half, of the lower half, then B's.
     constexpr int A_BOXES = A_MN ? 2 : 1;                      // per half: one of 64 k x 128 rows, or two of 64 rows x 64 k
     constexpr int B_BOXES = B_MN ? 2 : 1;
     constexpr int NREQ = 2 * A_BOXES + B_BOXES;
-    constexpr uint32_t REQ_MASK = (1u << NREQ) - 1u;
     const bool is_a = lane < 2 * A_BOXES;
     const int half_of = lane / A_BOXES, ja = lane % A_BOXES, jb = lane - 2 * A_BOXES;
     auto row_of = [&](int blk) -> int {                        // this CTA's first row of a block: of A, or of the class's view
@@ -131,7 +130,8 @@ tall_gemm_kernel(const __grid_constant__ TmapPackT<CLS ? 1 : 0> maps, const __gr
 
     if (warp == 0) {
         // ------------------------------ producer -----------------------------------------------
-        if (lane < NREQ) {
+        // (one elected thread: umma_gemm.cuh's producer says why)
+        if (ptx::elect_one()) {
             int stage = 0;
             uint32_t phase = 0;
             uint32_t full_leader, afull_own;                   // cluster addresses: the leader's barriers, this CTA's own
@@ -141,27 +141,28 @@ tall_gemm_kernel(const __grid_constant__ TmapPackT<CLS ? 1 : 0> maps, const __gr
             TallItem w;
             for (int it = 0; ok && tall_item<CLS>(p.work, slot, n_slots, it, w); ++it) {
                 const int cls = CLS ? (w.blk0 & 7) : 0;
-                const int kshift = CLS ? p.a_sigma[cls] : 0;   // B's k-rows lag A's by sigma
-                const CUtensorMap* tm = is_a ? &maps.a[cls] : &maps.b[0];
+                const int kshift = CLS ? p.a_sigma[cls] : 0;       // B's k-rows lag A's by sigma
+                const CUtensorMap* tmA = &maps.a[cls];
                 const int a_bytes = w.two ? 2 * A_HALF : A_HALF;
-                const int own = is_a ? row_of(half_of ? w.blk1 : w.blk0) + (A_MN ? 64 * ja : 0)
-                                     : w.nb * 256 + (int)cta_rank * 128 + (B_MN ? 64 * jb : 0);     // this lane's rows or columns
-                const uint32_t off = is_a ? (uint32_t)(half_of * A_HALF + ja * 8192) : (uint32_t)(2 * A_HALF + jb * 8192);
-                const bool idle = is_a && half_of != 0 && !w.two;
+                const int rows[2] = {row_of(w.blk0), row_of(w.blk1)}, col = w.nb * 256 + (int)cta_rank * 128;
                 for (int kb = 0; kb < p.kb_total; ++kb) {
-                    ok = __all_sync(REQ_MASK, ptx::mbar_wait(empty_bar + 8u * stage, phase ^ 1u, abort_flag));
-                    if (!ok) break;
+                    if (!ptx::mbar_wait(empty_bar + 8u * stage, phase ^ 1u, abort_flag)) { ok = false; break; }
                     const bool heads = CLS && kb == 0 && kshift > 0;       // A's first k-block has row heads to zero: it reports to its own CTA
-                    if (lane == 0) {
-                        if (heads) ptx::mbar_arrive_expect_tx(afull_bar + 8u * stage, (uint32_t)a_bytes);
-                        if (leader) ptx::mbar_arrive_expect_tx(full_bar + 8u * stage, (uint32_t)(2 * (B_BYTES + (heads ? 0 : a_bytes))));
-                    }
-                    __syncwarp(REQ_MASK);
+                    if (heads) ptx::mbar_arrive_expect_tx(afull_bar + 8u * stage, (uint32_t)a_bytes);
+                    if (leader) ptx::mbar_arrive_expect_tx(full_bar + 8u * stage, (uint32_t)(2 * (B_BYTES + (heads ? 0 : a_bytes))));
                     const int k0 = kb * kUmmaBK;
-                    const bool mn = is_a ? A_MN : B_MN;
-                    const int k = is_a ? k0 : k0 - kshift;
-                    if (!idle) ptx::tma_load_2d_pair(smem_base + (uint32_t)stage * STAGE_BYTES + off, tm,
-                                                     (heads && is_a ? afull_own : full_leader) + 8u * stage, mn ? own : k, mn ? k : own);
+                    const uint32_t at = smem_base + (uint32_t)stage * STAGE_BYTES, fb = full_leader + 8u * stage;
+                    const uint32_t ab = heads ? afull_own + 8u * stage : fb;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (h == 1 && !w.two) break;
+#pragma unroll
+                        for (int j = 0; j < A_BOXES; ++j)
+                            ptx::tma_load_2d_pair(at + (uint32_t)(h * A_HALF + j * 8192), tmA, ab, A_MN ? rows[h] + 64 * j : k0, A_MN ? k0 : rows[h]);
+                    }
+#pragma unroll
+                    for (int j = 0; j < B_BOXES; ++j)
+                        ptx::tma_load_2d_pair(at + (uint32_t)(2 * A_HALF + j * 8192), &maps.b[0], fb, B_MN ? col + 64 * j : k0 - kshift, B_MN ? k0 - kshift : col);
                     if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
             }
@@ -194,11 +195,6 @@ tall_gemm_kernel(const __grid_constant__ TmapPackT<CLS ? 1 : 0> maps, const __gr
             ptx::fence_proxy_async_smem();
             __syncwarp();
         };
-        auto wait_all = [&](uint32_t bar, uint32_t parity) -> bool {           // lane 0 waits, every lane learns the outcome
-            int ok = 1;
-            if (lane == 0) ok = ptx::mbar_wait(bar, parity, abort_flag) ? 1 : 0;
-            return __shfl_sync(0xffffffffu, ok, 0) != 0;
-        };
         int stage = 0;
         uint32_t phase = 0, aphase = 0;                        // aphase: per stage, parity of the next use of its A barriers
         TallItem w;
@@ -207,97 +203,102 @@ tall_gemm_kernel(const __grid_constant__ TmapPackT<CLS ? 1 : 0> maps, const __gr
                 for (int it = 0; tall_item<CLS>(p.work, slot, n_slots, it, w); ++it) {
                     const int sigma = p.a_sigma[w.blk0 & 7];
                     if (sigma > 0) {
-                        if (!wait_all(afull_bar + 8u * stage, (aphase >> stage) & 1u)) break;
+                        if (!ptx::mbar_wait_warp(afull_bar + 8u * stage, (aphase >> stage) & 1u, abort_flag)) break;
                         zero_row_heads(stage, sigma, w.two);
                         if (lane == 0) ptx::mbar_arrive_cluster(aready_bar + 8u * stage, 0);
                         aphase ^= 1u << stage;
                     }
                     stage = (stage + p.kb_total) % S;
                 }
-        } else if (CLS || lane == 0) {
-            constexpr uint32_t a_lbo = A_MN ? 8192u : 16u, b_lbo = B_MN ? 8192u : 16u;
+        } else {
+            // One elected thread issues the MMAs and their commits; with row classes the warp comes here together for every item.
             constexpr uint32_t a_kstep = A_MN ? 2048u : 32u, b_kstep = B_MN ? 2048u : 32u;
-            auto mma = [&](int half, int st, int acc, bool first) {            // one k-block of one half
-                const uint32_t sA = smem_base + (uint32_t)st * STAGE_BYTES + (uint32_t)(half * A_HALF);
-                const uint32_t sB = smem_base + (uint32_t)st * STAGE_BYTES + 2u * A_HALF;
+            const uint64_t a_desc = ptx::smem_desc_sw128(smem_base, A_MN ? 8192u : 16u, 1024u);
+            const uint64_t b_desc = ptx::smem_desc_sw128(smem_base + 2u * A_HALF, B_MN ? 8192u : 16u, 1024u);
+            const uint32_t a_lo = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32), b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32), idesc = p.idesc;
+            auto mma = [&](int half, int st, int acc, uint32_t more) {         // one k-block of one half; more = 0 starts its sum
+                const uint32_t off = (uint32_t)st * (uint32_t)(STAGE_BYTES >> 4), ao = a_lo + off + (uint32_t)half * (uint32_t)(A_HALF >> 4), bo = b_lo + off;
 #pragma unroll
                 for (int k16 = 0; k16 < kUmmaBK / 16; ++k16)
-                    ptx::umma_f16<2>(tmem_base + 256u * acc, ptx::smem_desc_sw128(sA + k16 * a_kstep, a_lbo, 1024u),
-                                     ptx::smem_desc_sw128(sB + k16 * b_kstep, b_lbo, 1024u), p.idesc, (!first || k16 > 0) ? 1u : 0u);
+                    ptx::umma_f16<2>(tmem_base + 256u * acc, ptx::smem_desc_join(ao + (k16 * a_kstep >> 4), a_hi), ptx::smem_desc_join(bo + (k16 * b_kstep >> 4), b_hi), idesc, k16 > 0 ? 1u : more);
             };
             uint32_t used = 0;                                 // bit h: parity of accumulator h's next use
-            for (int it = 0; tall_item<CLS>(p.work, slot, n_slots, it, w); ++it) {
-                const int sigma = CLS ? p.a_sigma[w.blk0 & 7] : 0;
-                if (sigma > 0) {
-                    if (!wait_all(afull_bar + 8u * stage, (aphase >> stage) & 1u)) break;
-                    zero_row_heads(stage, sigma, w.two);
+            const int L = p.kb_total;
+            bool heads = false;
+            // an item's k-blocks, from ring position (st, ph) on
+            auto contract = [&](int& st, uint32_t& ph) -> bool {
+                auto next = [&]() { if (++st == S) { st = 0; ph ^= 1u; } };
+                auto ready = [&]() -> bool { return ptx::mbar_wait(full_bar + 8u * st, ph, abort_flag); };      // the k-block's operands are in place
+                auto enter = [&](int acc) -> bool {            // the accumulator is free
+                    if (!ptx::mbar_wait(tempty_bar + 8u * acc, ((used >> acc) & 1u) ^ 1u, abort_flag)) return false;
+                    used ^= 1u << acc;
+                    ptx::tc_fence_after();
+                    return true;
+                };
+                if (CLS && heads && !ptx::mbar_wait(aready_bar + 8u * st, (aphase >> st) & 1u, abort_flag)) return false;       // the peer's half too
+                if (!w.two) {
+                    if (!enter(w.acc)) return false;
+                    for (int kb = 0; kb < L; ++kb) {
+                        if (!ready()) return false;
+                        mma(0, st, w.acc, kb > 0);
+                        ptx::umma_commit_2(empty_bar + 8u * st);
+                        next();
+                    }
+                    ptx::umma_commit_2(tfull_bar + 8u * w.acc);
+                    return true;
                 }
-                int done = 1;
-                if (lane == 0) {
+                // k-blocks [0, lag) and [L - lag, L): the upper half's first, then the lower half's of the same stages
+                const int lag = min(kTallLag, L), tail = max(lag, L - kTallLag);
+                auto apart = [&](int kb0, int kb1, bool begin, bool end) -> bool {
+                    const int st0 = st;
+                    if (begin && !enter(0)) return false;
+                    for (int kb = kb0; kb < kb1; ++kb) {
+                        if (!ready()) return false;
+                        mma(0, st, 0, kb > 0);
+                        next();
+                    }
+                    if (end) ptx::umma_commit_2(tfull_bar);
+                    if (begin && !enter(1)) return false;
+                    int s2 = st0;
+                    for (int kb = kb0; kb < kb1; ++kb) {
+                        mma(1, s2, 1, kb > 0);
+                        ptx::umma_commit_2(empty_bar + 8u * s2);
+                        if (++s2 == S) s2 = 0;
+                    }
+                    if (end) ptx::umma_commit_2(tfull_bar + 8u);
+                    return true;
+                };
+                if (!apart(0, lag, true, lag == L)) return false;
+                for (int kb = lag; kb < tail; ++kb) {
+                    if (!ready()) return false;
+                    mma(0, st, 0, 1u);
+                    mma(1, st, 1, 1u);
+                    ptx::umma_commit_2(empty_bar + 8u * st);
+                    next();
+                }
+                return tail == L || apart(tail, L, false, true);
+            };
+            if (!CLS) {
+                if (ptx::elect_one())
+                    for (int it = 0; tall_item<CLS>(p.work, slot, n_slots, it, w) && contract(stage, phase); ++it) {}
+            } else {
+                for (int it = 0; tall_item<CLS>(p.work, slot, n_slots, it, w); ++it) {
+                    const int sigma = p.a_sigma[w.blk0 & 7];
+                    heads = sigma > 0;
+                    if (heads) {
+                        if (!ptx::mbar_wait_warp(afull_bar + 8u * stage, (aphase >> stage) & 1u, abort_flag)) break;
+                        zero_row_heads(stage, sigma, w.two);
+                    }
+                    bool done = true;
                     int st = stage;
                     uint32_t ph = phase;
-                    auto next = [&]() { if (++st == S) { st = 0; ph ^= 1u; } };
-                    auto ready = [&](int kb) -> bool {         // the k-block's operands are in place
-                        if (sigma > 0 && kb == 0 && !ptx::mbar_wait(aready_bar + 8u * st, (aphase >> st) & 1u, abort_flag)) return false;
-                        if (!ptx::mbar_wait(full_bar + 8u * st, ph, abort_flag)) return false;
-                        ptx::tc_fence_after();
-                        return true;
-                    };
-                    auto enter = [&](int acc) -> bool {        // the accumulator is free
-                        if (!ptx::mbar_wait(tempty_bar + 8u * acc, ((used >> acc) & 1u) ^ 1u, abort_flag)) return false;
-                        used ^= 1u << acc;
-                        ptx::tc_fence_after();
-                        return true;
-                    };
-                    const int L = p.kb_total;
-                    if (!w.two) {
-                        done = enter(w.acc);
-                        for (int kb = 0; done && kb < L; ++kb) {
-                            if (!ready(kb)) { done = 0; break; }
-                            mma(0, st, w.acc, kb == 0);
-                            ptx::umma_commit_2(empty_bar + 8u * st);
-                            next();
-                        }
-                        if (done) ptx::umma_commit_2(tfull_bar + 8u * w.acc);
-                    } else {
-                        // k-blocks [0, lag) and [L - lag, L): the upper half's first, then the lower half's of the same stages
-                        const int lag = min(kTallLag, L), tail = max(lag, L - kTallLag);
-                        auto apart = [&](int kb0, int kb1, bool begin, bool end) -> bool {
-                            const int st0 = st;
-                            if (begin && !enter(0)) return false;
-                            for (int kb = kb0; kb < kb1; ++kb) {
-                                if (!ready(kb)) return false;
-                                mma(0, st, 0, kb == 0);
-                                next();
-                            }
-                            if (end) ptx::umma_commit_2(tfull_bar);
-                            if (begin && !enter(1)) return false;
-                            int s2 = st0;
-                            for (int kb = kb0; kb < kb1; ++kb) {
-                                mma(1, s2, 1, kb == 0);
-                                ptx::umma_commit_2(empty_bar + 8u * s2);
-                                if (++s2 == S) s2 = 0;
-                            }
-                            if (end) ptx::umma_commit_2(tfull_bar + 8u);
-                            return true;
-                        };
-                        done = apart(0, lag, true, lag == L);
-                        for (int kb = lag; done && kb < tail; ++kb) {
-                            if (!ready(kb)) { done = 0; break; }
-                            mma(0, st, 0, false);
-                            mma(1, st, 1, false);
-                            ptx::umma_commit_2(empty_bar + 8u * st);
-                            next();
-                        }
-                        if (done && tail < L) done = apart(tail, L, false, true);
-                    }
+                    if (ptx::elect_one()) done = contract(st, ph);
+                    if (!__all_sync(0xffffffffu, done)) break;
+                    if (heads) aphase ^= 1u << stage;
+                    const int adv = stage + L;                 // (the other lanes' copy of the ring position)
+                    phase ^= (uint32_t)((adv / S) & 1);
+                    stage = adv % S;
                 }
-                if (CLS) done = __shfl_sync(0xffffffffu, done, 0);
-                if (!done) break;
-                if (sigma > 0) aphase ^= 1u << stage;
-                const int adv = stage + p.kb_total;
-                phase ^= (uint32_t)((adv / S) & 1);
-                stage = adv % S;
             }
         }
     } else {
@@ -391,8 +392,8 @@ tall_gemm_kernel(const __grid_constant__ TmapPackT<CLS ? 1 : 0> maps, const __gr
     }
 
     // ------------------------------ common exit ----------------------------------------------
+    __syncwarp();                        // (one thread has run the producer's and the MMA issuer's loops)
     ptx::tc_fence_before();
-    __syncwarp();
     ptx::cluster_sync_all();                                   // no CTA leaves while its peer may still arrive on its barriers
     if (threadIdx.x == 0 && *abort_flag) atomicOr(p.status, 1u);
     if (warp == 1) {

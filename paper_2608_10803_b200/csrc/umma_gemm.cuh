@@ -497,14 +497,12 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
 
     if (warp == 0) {
         // ------------------------------ producer -----------------------------------------------
-        // One lane per TMA request of a k-block (A: one box, two when M-contiguous; B: one box, or one per 64
-        // columns when N-contiguous): the lanes run the loop together and issue their requests with one
-        // instruction.  A single lane issuing them one after the other spends about 0.1 us per request, which
-        // bounds a 128 x 256 tile with an N-contiguous B (five requests per k-block) at 0.5 us per k-block.
-        constexpr int NREQ_A = A_MN ? 2 : 1;
-        constexpr int NREQ = NREQ_A + (B_MN ? B_BOXES : 1);
-        constexpr uint32_t REQ_MASK = (1u << NREQ) - 1u;
-        if (lane < NREQ) {
+        // One elected thread.  What bounds this loop is its own chain of instructions before it is the loads: with a lane per request, which takes a
+        // vote and a barrier of a few lanes per k-block (200 cycles), an SM asked for a k-block every 0.26 us whether it had 16 or 32 KB, half of
+        // what it can take in; this way it asks for 24 KB every 0.11 us and for 48 KB every 0.25 (98 bytes a cycle).
+        if (ptx::elect_one()) {
+            constexpr int NREQ_A = A_MN ? 2 : 1;
+            constexpr int NREQ_B = B_MN ? B_BOXES : 1;
             int stage = 0;
             uint32_t phase = 0;
             // the byte count of a stage is signalled on the leader's barrier (pair form)
@@ -517,8 +515,6 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                 if (CG == 1) ptx::tma_load_2d(dst, tm, bar, x, y);
                 else ptx::tma_load_2d_pair(dst, tm, bar, x, y);
             };
-            const bool is_a = lane < NREQ_A;
-            const int jb = lane - NREQ_A;                                     // B box of this lane
             for (int it = 0; ok; ++it) {
                 WorkItem w;
                 if (!next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w)) break;
@@ -530,7 +526,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                 const int kshift = A_CLS ? p.a_sigma[cls] : 0;                // B's k-rows lag A's kappa by sigma
                 const CUtensorMap* tmA = &maps.a[cls];
                 const CUtensorMap* tmB = &maps.b[B_SPLIT ? (split & 7) : 0];  // k classes as splits: the class's view of B
-                if ((A_CLS || B_SPLIT) && lane == 0 && unit + unit_step < p.num_units) {
+                if ((A_CLS || B_SPLIT) && unit + unit_step < p.num_units) {
                     // the next unit may go through other maps: fetch their descriptors while this unit loads
                     int mb2, nb2, sp2;
                     decode_unit(p, unit + unit_step, mb2, nb2, sp2);
@@ -543,75 +539,56 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                     // class by class: A' columns j*Kc + 64*b .., B's class-j rows 64*b .. at shifted columns 56*nb ..
                     for (int j = 0; ok && j < 8; ++j)
                         for (int kb = kb0; kb < kb1; ++kb) {
-                            ok = __all_sync(REQ_MASK, ptx::mbar_wait(empty_bar + 8u * stage, phase ^ 1u, abort_flag));
-                            if (!ok) break;
+                            if (!ptx::mbar_wait(empty_bar + 8u * stage, phase ^ 1u, abort_flag)) { ok = false; break; }
                             const uint32_t sA = smem_base + (uint32_t)stage * STAGE_BYTES;
-                            if (lane == 0) ptx::mbar_arrive_expect_tx(full_bar + 8u * stage, (uint32_t)(p.a_tx_bytes + p.b_tx_bytes));
-                            __syncwarp(REQ_MASK);
-                            if (is_a) load(sA, tmA, full_bar + 8u * stage, j * p.cls_kc + kb * kUmmaBK, row0);
-                            else load(sA + A_BYTES, &maps.b[B_CLS ? j : 0], full_bar + 8u * stage, col0, kb * kUmmaBK);
+                            ptx::mbar_arrive_expect_tx(full_bar + 8u * stage, (uint32_t)(p.a_tx_bytes + p.b_tx_bytes));
+                            load(sA, tmA, full_bar + 8u * stage, j * p.cls_kc + kb * kUmmaBK, row0);
+                            load(sA + A_BYTES, &maps.b[B_CLS ? j : 0], full_bar + 8u * stage, col0, kb * kUmmaBK);
                             if (++stage == S) { stage = 0; phase ^= 1u; }
                         }
                 }
                 // ShuffleK: the unit's k-blocks in rotated order (the MMA warp consumes the stages in ring order and sums
                 // whatever arrives, so only the loads know; the order is a function of the tile, hence fixed)
-                const int kb_rot = (MODE == 0 && !SK && p.shuffle_k && kb1 - kb0 > 1) ? ((mb + nb) * 5) % (kb1 - kb0) : 0;
-                for (int kbi = kb0; !B_CLS && kbi < kb1; ++kbi) {
-                    const int kb = (MODE == 0 && !SK) ? kb0 + (kbi - kb0 + kb_rot) % (kb1 - kb0) : kbi;
-                    ok = __all_sync(REQ_MASK, ptx::mbar_wait(empty_bar + 8u * stage, phase ^ 1u, abort_flag));
-                    if (!ok) break;
+                int kb = kb0;
+                if (MODE == 0 && !SK && p.shuffle_k && kb1 - kb0 > 1) kb += ((mb + nb) * 5) % (kb1 - kb0);
+                for (int left = B_CLS ? 0 : kb1 - kb0; left > 0; --left) {
+                    if (!ptx::mbar_wait(empty_bar + 8u * stage, phase ^ 1u, abort_flag)) { ok = false; break; }
                     const uint32_t sA = smem_base + (uint32_t)stage * STAGE_BYTES;
                     const uint32_t sB = sA + A_BYTES;
                     const uint32_t fb = full_target + 8u * stage;
-                    if (lane == 0) {
-                        if (CG == 1) ptx::mbar_arrive_expect_tx(full_bar + 8u * stage, (uint32_t)(p.a_tx_bytes + p.b_tx_bytes));
-                        else if (A_CLS && kb == 0 && kshift > 0) {
-                            // pair tiles of one row class, a unit's first k-block with row heads to zero: each CTA's A box
-                            // reports to its own barrier (its warp 1 zeroes the heads there before the MMA); the B boxes of
-                            // both CTAs report to the leader's as always
-                            ptx::mbar_arrive_expect_tx(afull_bar + 8u * stage, (uint32_t)A_BYTES);
-                            if (leader) ptx::mbar_arrive_expect_tx(full_bar + 8u * stage, (uint32_t)(2 * p.b_tx_bytes));
-                        }
-                        else if (leader) ptx::mbar_arrive_expect_tx(full_bar + 8u * stage, (uint32_t)(2 * (A_BYTES + p.b_tx_bytes)));
-                    }
-                    __syncwarp(REQ_MASK);
-                    const int k0 = kb * kUmmaBK;
-                    // this lane's request: where it lands, through which map, at which coordinates
-                    uint32_t dst;
-                    const CUtensorMap* tm;
-                    int x, y;
-                    if (is_a) {
-                        tm = tmA;
-                        if (!A_MN) { dst = sA; x = k0 + a_k_off; y = row0; }
-                        else { dst = sA + (uint32_t)lane * 8192u; x = row0 + lane * 64; y = k0; }
+                    // pair tiles of one row class, a unit's first k-block with row heads to zero: each CTA's A box reports to its own
+                    // barrier (its warp 1 zeroes the heads there before the MMA); the B boxes of both CTAs report to the leader's as always
+                    const bool heads = A_CLS && CG == 2 && kb == 0 && kshift > 0;
+                    if (CG == 1) {
+                        ptx::mbar_arrive_expect_tx(full_bar + 8u * stage, (uint32_t)(p.a_tx_bytes + p.b_tx_bytes));
                     } else {
-                        tm = tmB;
-                        if (B_MN) { dst = sB + (uint32_t)jb * 8192u; x = col0 + jb * 64; y = k0 - kshift; }
-                        else { dst = sB; x = k0; y = col0; }
+                        if (heads) ptx::mbar_arrive_expect_tx(afull_bar + 8u * stage, (uint32_t)A_BYTES);
+                        if (leader) ptx::mbar_arrive_expect_tx(full_bar + 8u * stage, (uint32_t)(2 * (p.b_tx_bytes + (heads ? 0 : A_BYTES))));
                     }
-                    if (A_CLS && CG == 2 && is_a && kb == 0 && kshift > 0) load(dst, tm, afull_own + 8u * stage, x, y);   // this CTA's own barrier
-                    else if (BATCH) ptx::tma_load_3d(dst, tm, fb, x, y, w.entry * (is_a ? p.a_entry : p.b_entry));
-                    else load(dst, tm, fb, x, y);
+                    const int k0 = kb * kUmmaBK;
+                    const uint32_t ab = heads ? afull_own + 8u * stage : fb;
+#pragma unroll
+                    for (int j = 0; j < NREQ_A; ++j) {
+                        const int x = A_MN ? row0 + 64 * j : k0 + a_k_off, y = A_MN ? k0 : row0;
+                        if (BATCH) ptx::tma_load_3d(sA + 8192u * j, tmA, fb, x, y, w.entry * p.a_entry);
+                        else load(sA + 8192u * j, tmA, ab, x, y);
+                    }
+#pragma unroll
+                    for (int j = 0; j < NREQ_B; ++j) {
+                        const int x = B_MN ? col0 + 64 * j : k0, y = B_MN ? k0 - kshift : col0;
+                        if (BATCH) ptx::tma_load_3d(sB + 8192u * j, tmB, fb, x, y, w.entry * p.b_entry);
+                        else load(sB + 8192u * j, tmB, fb, x, y);
+                    }
+                    if (++kb == kb1) kb = kb0;
                     if (++stage == S) { stage = 0; phase ^= 1u; }
                 }
-                if (lane == 0) ADAPT_TRACE(1, unit);
+                ADAPT_TRACE(1, unit);
             }
         }
     } else if (warp == 1) {
         // ------------------------------ MMA issuer ---------------------------------------------
-        // one thread issues the MMAs; in class mode the whole warp runs the loop so that its other
-        // lanes can zero the stale leading elements of A' in the first k-block
-        // (only when some class of A is shifted: with K % 8 == 0 every sigma is zero and one lane is enough)
-        // (pair tiles of one row class: always, and the peer's warp 1 runs the forwarding loop further down)
-        const bool warp_wide = A_CLS && (p.a_shift_any != 0 || CG == 2);
-        // in class mode all 32 lanes run these loops: lane 0 waits and the outcome is broadcast, so
-        // the lanes never part ways before a __syncwarp
-        auto mma_wait = [&](uint32_t bar, uint32_t parity) -> bool {
-            if (!warp_wide) return ptx::mbar_wait(bar, parity, abort_flag);
-            int w = 1;
-            if (lane == 0) w = ptx::mbar_wait(bar, parity, abort_flag) ? 1 : 0;
-            return __shfl_sync(0xffffffffu, w, 0) != 0;
-        };
+        // One elected thread waits for operands and accumulators, issues the MMAs and their commits (a commit covers what its own thread has
+        // issued).  In class mode the warp comes here together for every unit: its other lanes help to zero the stale leading elements of A' in the first k-block.
         // Class tile whose rows are shifted: the sigma elements in front of each row of the first k-block belong to
         // the previous row of A and are zeroed before the tensor core reads them.  Rows lane, lane+32, ...: chunk 0
         // of row r (its first 8 elements) sits at r*128 + ((r & 7) << 4); one masked 16-byte read-modify-write per row.
@@ -649,7 +626,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                 if (!next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w)) break;
                 const int sigma = p.a_sigma[w.mb & (NCLS - 1)];
                 if (w.kb0 == 0 && w.kb1 > 0 && sigma > 0) {
-                    if (!mma_wait(afull_bar + 8u * stage, (aphase >> stage) & 1u)) { ok = false; break; }
+                    if (!ptx::mbar_wait_warp(afull_bar + 8u * stage, (aphase >> stage) & 1u, abort_flag)) { ok = false; break; }
                     zero_row_heads(stage, sigma);
                     if (lane == 0) ptx::mbar_arrive_cluster(aready_bar + 8u * stage, 0);
                     aphase ^= 1u << stage;
@@ -657,100 +634,80 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
                 stage = (stage + (w.kb1 - w.kb0)) % S;
             }
         }
-        if ((lane == 0 || warp_wide) && leader) {
+        if (leader) {
             int stage = 0;
             uint32_t phase = 0;
             uint32_t aphase = 0;              // pair tiles of one row class: per stage, parity of the next use of its A barriers
             int buf = 0;
             uint32_t buf_phase = 0;
+            bool heads = false;               // class mode: this unit's first k-block has row heads to zero
             // K-major operand: rows of 128 B, 8-row groups 1024 B apart, +32 B per 16-element k step.
             // MN-major operand: 64-element blocks along M/N 8192 B apart (LBO), 8-row k groups
             // 1024 B apart (SBO), +2048 B per 16-element k step.
-            const uint32_t a_lbo = A_MN ? 8192u : 16u, b_lbo = B_MN ? 8192u : 16u;
-            const uint32_t a_kstep = A_MN ? 2048u : 32u, b_kstep = B_MN ? 2048u : 32u;
-            bool ok = true;
-            for (int it = 0; ok; ++it) {
-                WorkItem w;
-                if (!next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w)) break;
-                const int unit = w.unit, mb = w.mb, nb = w.nb, split = w.split, kb0 = w.kb0, kb1 = w.kb1;
-                (void)unit; (void)nb; (void)split;
-                if (warp_wide && kb0 == 0 && kb1 > 0) {
-                    // Done here, before the wait for a free accumulator: the loads run ahead of the drain, so
-                    // in the write-bound regime this work hides behind that wait.
-                    const int sigma = p.a_sigma[mb & (NCLS - 1)];
-                    if (sigma > 0) {
-                        if (!mma_wait((A_CLS && CG == 2) ? afull_bar + 8u * stage : full_bar + 8u * stage,
-                                      (A_CLS && CG == 2) ? ((aphase >> stage) & 1u) : phase)) { ok = false; break; }
+            constexpr uint32_t a_kstep = A_MN ? 2048u : 32u, b_kstep = B_MN ? 2048u : 32u;
+            const uint64_t a_desc = ptx::smem_desc_sw128(smem_base, A_MN ? 8192u : 16u, 1024u);
+            const uint64_t b_desc = ptx::smem_desc_sw128(smem_base + (uint32_t)A_BYTES, B_MN ? 8192u : 16u, 1024u);
+            const uint32_t a_lo = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32), b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32);
+            const uint32_t idesc = p.idesc, stage_step = (uint32_t)STAGE_BYTES >> 4;
+            // a unit's k-blocks, from ring position (st, ph) on
+            auto contract = [&](const WorkItem& w, int& st, uint32_t& ph) -> bool {
+                if (!ptx::mbar_wait(tempty_bar + 8u * buf, buf_phase ^ 1u, abort_flag)) return false;
+                ptx::tc_fence_after();
+                ADAPT_TRACE(2, w.unit);
+                // pair tiles of one row class, row heads zeroed in both CTAs: the peer's warp 1 hands its half over.  The leader reads none of the
+                // peer's shared memory itself (the peer's tensor core does, after the peer's own proxy fence), so an ordinary wait is enough.
+                if (A_CLS && CG == 2 && heads) {
+                    if (!ptx::mbar_wait(aready_bar + 8u * st, (aphase >> st) & 1u, abort_flag)) return false;
+                    ptx::tc_fence_after();
+                }
+                uint32_t off = (uint32_t)st * stage_step;                  // the stage's place, in the descriptors' units
+                for (int j = 0; j < (B_CLS ? 8 : 1); ++j) {                // (k-class mode: class by class, each into its own accumulator)
+                    const uint32_t d = tmem_base + (uint32_t)(B_CLS ? 64 * j : buf * BN);
+                    uint32_t more = 0;                                     // 0: this k-block's first MMA starts the sum
+                    for (int left = w.kb1 - w.kb0; left > 0; --left, more = 1u) {
+                        // (no tcgen05 fence here: the loads' barrier orders them; the accumulator's is above)
+                        if (!ptx::mbar_wait(full_bar + 8u * st, ph, abort_flag)) return false;
+#pragma unroll
+                        for (int k16 = 0; k16 < kUmmaBK / 16; ++k16)
+                            ptx::umma_f16<CG>(d, ptx::smem_desc_join(a_lo + off + (k16 * a_kstep >> 4), a_hi), ptx::smem_desc_join(b_lo + off + (k16 * b_kstep >> 4), b_hi), idesc, k16 > 0 ? 1u : more);
+                        // free the stage (in both CTAs of a pair) once these MMAs have read it
+                        if (CG == 1) ptx::umma_commit_1(empty_bar + 8u * st);
+                        else ptx::umma_commit_2(empty_bar + 8u * st);
+                        off += stage_step;
+                        if (++st == S) { st = 0; off = 0; ph ^= 1u; }
+                    }
+                }
+                if (CG == 1) ptx::umma_commit_1(tfull_bar + 8u * buf);
+                else ptx::umma_commit_2(tfull_bar + 8u * buf);
+                ADAPT_TRACE(3, w.unit);
+                return true;
+            };
+            WorkItem w;
+            if (!A_CLS) {
+                if (ptx::elect_one())
+                    for (int it = 0; next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w) && contract(w, stage, phase); ++it)
+                        if (++buf == NBUF) { buf = 0; buf_phase ^= 1u; }
+            } else {
+                for (int it = 0; next_item<SK, B_SPLIT, BATCH>(p, unit0, unit_step, it, w); ++it) {
+                    const int sigma = w.kb0 == 0 && w.kb1 > 0 ? p.a_sigma[w.mb & (NCLS - 1)] : 0;
+                    heads = sigma > 0;
+                    if (heads) {
+                        // Done here, before the wait for a free accumulator: the loads run ahead of the drain, so
+                        // in the write-bound regime this work hides behind that wait.
+                        if (!ptx::mbar_wait_warp(CG == 2 ? afull_bar + 8u * stage : full_bar + 8u * stage, CG == 2 ? ((aphase >> stage) & 1u) : phase, abort_flag)) break;
                         zero_row_heads(stage, sigma);
                     }
-                }
-                if (!mma_wait(tempty_bar + 8u * buf, buf_phase ^ 1u)) { ok = false; break; }
-                ptx::tc_fence_after();
-                ADAPT_TRACE(2, unit);
-                const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
-                if (B_CLS) {
-                    for (int j = 0; ok && j < 8; ++j)
-                        for (int kb = kb0; kb < kb1; ++kb) {
-                            if (!mma_wait(full_bar + 8u * stage, phase)) { ok = false; break; }
-                            ptx::tc_fence_after();
-                            const uint32_t sA = smem_base + (uint32_t)stage * STAGE_BYTES;
-                            const uint32_t sB = sA + A_BYTES;
-#pragma unroll
-                            for (int k16 = 0; k16 < kUmmaBK / 16; ++k16) {
-                                const uint64_t adesc = ptx::smem_desc_sw128(sA + k16 * a_kstep, a_lbo, 1024u);
-                                const uint64_t bdesc = ptx::smem_desc_sw128(sB + k16 * b_kstep, b_lbo, 1024u);
-                                ptx::umma_f16<CG>(tmem_base + 64u * j, adesc, bdesc, p.idesc, (kb > kb0 || k16 > 0) ? 1u : 0u);
-                            }
-                            ptx::umma_commit_1(empty_bar + 8u * stage);
-                            if (++stage == S) { stage = 0; phase ^= 1u; }
-                        }
-                }
-                if (!B_CLS) {
-                    // The k-block loop proper runs in ONE lane, also when the warp came here together (class tiles): a
-                    // warp-wide loop pays a shuffle for every wait, and the MMA thread's loop is what the tensor core waits
-                    // for (pair tiles of one row class: 0.82 us per k-block with the warp-wide loop).  The other lanes step
-                    // their copy of (stage, phase) by the number of k-blocks and pick up the outcome afterwards.
-                    int done = 1;
-                    if (lane == 0) {
-                        int st = stage;
-                        uint32_t ph = phase;
-                        for (int kb = kb0; kb < kb1; ++kb) {
-                            if (A_CLS && CG == 2 && kb == 0 && p.a_sigma[mb & (NCLS - 1)] > 0) {
-                                // the unit's first k-block, row heads zeroed: this CTA's box (waited for above) and the peer's,
-                                // handed over by the peer's warp 1.  The leader reads none of the peer's shared memory itself
-                                // (the peer's tensor core does, after the peer's own proxy fence), so an ordinary wait is enough.
-                                if (!ptx::mbar_wait(aready_bar + 8u * st, (aphase >> st) & 1u, abort_flag)) { done = 0; break; }
-                            }
-                            if (!ptx::mbar_wait(full_bar + 8u * st, ph, abort_flag)) { done = 0; break; }
-                            ptx::tc_fence_after();
-                            const uint32_t sA = smem_base + (uint32_t)st * STAGE_BYTES;
-                            const uint32_t sB = sA + A_BYTES;
-#pragma unroll
-                            for (int k16 = 0; k16 < kUmmaBK / 16; ++k16) {
-                                const uint64_t adesc = ptx::smem_desc_sw128(sA + k16 * a_kstep, a_lbo, 1024u);
-                                const uint64_t bdesc = ptx::smem_desc_sw128(sB + k16 * b_kstep, b_lbo, 1024u);
-                                ptx::umma_f16<CG>(d_tmem, adesc, bdesc, p.idesc, (kb > kb0 || k16 > 0) ? 1u : 0u);
-                            }
-                            // free the stage (in both CTAs of a pair) once these MMAs have read it
-                            if (CG == 1) ptx::umma_commit_1(empty_bar + 8u * st);
-                            else ptx::umma_commit_2(empty_bar + 8u * st);
-                            if (++st == S) { st = 0; ph ^= 1u; }
-                        }
-                    }
-                    if (warp_wide) done = __shfl_sync(0xffffffffu, done, 0);
-                    if (!done) { ok = false; break; }
-                    if (A_CLS && CG == 2 && kb0 == 0 && kb1 > 0 && p.a_sigma[mb & (NCLS - 1)] > 0) aphase ^= 1u << stage;
-                    const int adv = stage + (kb1 - kb0);
+                    bool done = true;
+                    int st = stage;
+                    uint32_t ph = phase;
+                    if (ptx::elect_one()) done = contract(w, st, ph);
+                    if (!__all_sync(0xffffffffu, done)) break;
+                    if (CG == 2 && heads) aphase ^= 1u << stage;
+                    const int adv = stage + (w.kb1 - w.kb0);               // (the other lanes' copy of the ring position)
                     phase ^= (uint32_t)((adv / S) & 1);
                     stage = adv % S;
+                    if (++buf == NBUF) { buf = 0; buf_phase ^= 1u; }
                 }
-                if (!ok) break;
-                if (lane == 0) {
-                    if (CG == 1) ptx::umma_commit_1(tfull_bar + 8u * buf);
-                    else ptx::umma_commit_2(tfull_bar + 8u * buf);
-                }
-                ADAPT_TRACE(3, unit);
-                if (++buf == NBUF) { buf = 0; buf_phase ^= 1u; }
             }
         }
     } else {
@@ -1316,6 +1273,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
     }
 
     // ------------------------------ common exit ----------------------------------------------
+    __syncwarp();                        // (one thread has run the producer's and the MMA issuer's loops)
     ptx::tc_fence_before();
     if (CG == 2 || FUSE) {      // no CTA leaves while a peer may still read its shared memory or arrive on its barriers
         asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
