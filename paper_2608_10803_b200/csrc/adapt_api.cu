@@ -25,6 +25,7 @@
 #include "batch_route.h"
 #include "umma_gemm.cuh"
 #include "tall_gemm.cuh"
+#include "direct_gemm.cuh"
 
 using namespace adapt;
 
@@ -431,7 +432,9 @@ extern "C" void adapt_set_map_cache(int enabled) { st().map_cache.store(enabled 
     X(cluster_bw_eff) X(streamk_fixup_us) X(streamk_peer_us) X(fused_reduce_us) X(fused_wave_us) X(reduce_launch_us) X(dsmem_bw_per_sm) \
     X(copy_bw_eff) X(hbm_bw_per_sm) X(class_view_sm_eff) X(class_tile_fixed_us) X(class_tile_fixed_unaligned_us) X(pair_class_tile_us) X(kclass_view_sm_eff) \
     X(kclass_unit_fixed_us) X(kclass_tile_drain_us) X(oob_box_penalty) X(l2_reread_cost) X(reduce_batch_us) X(class_split_bw_eff) \
-    X(class_split_bw_eff_per_log2m) X(class_split_fused_bw_eff) X(regroup_bw_eff) X(class_view_bw_eff)
+    X(class_split_bw_eff_per_log2m) X(class_split_fused_bw_eff) X(regroup_bw_eff) X(class_view_bw_eff) \
+    X(direct_fixed_us) X(direct_latency_us) X(direct_latency_warm_us) X(direct_mma64_us) X(direct_mma128_us) X(direct_mma256_us) X(direct_exchange_us) X(direct_exchange_us_per_kb) \
+    X(direct_narrow_bw_eff) X(direct_unaligned_us) X(direct_prologue_us) X(direct_hbm_bw) X(b_piece256_eff) X(b_piece128_eff) X(epi_hidden)
 
 static double* calib_field(Calib& c, const char* name)
 {
@@ -762,6 +765,13 @@ extern "C" adapt_status_t adapt_init(int device)
         UmmaKernel k = launch_map_tall((v & 1) != 0, (v & 2) != 0, (v & 4) != 0, (v & 8) != 0);
         if (k) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes));
     }
+    for (int v = 0; v < 4; ++v)
+        for (const void* k : {direct_group_pick<kDirectGroupMax>((v & 1) != 0, (v & 2) != 0), direct_group_pick<kDirectGroupFew>((v & 1) != 0, (v & 2) != 0)})
+            CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes - kDirectStaticBytes));
+    for (int BN : {64, 128, 256})
+        for (int v = 0; v < 16; ++v)
+            CUDA_TRY(cudaFuncSetAttribute(direct_kernel(BN, (v & 1) != 0, (v & 2) != 0, (v & 4) != 0, (v & 8) != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          S.machine.smem_bytes - kDirectStaticBytes));
     // clusters of 2, 4, 8 CTAs of the tcgen05 kernel (one CTA per SM) that the device runs at a time
     for (int i = 0; i < 3; ++i) {
         cudaLaunchConfig_t cfg;
@@ -1152,6 +1162,47 @@ adapt_status_t launch_tall(State& S, const Shape& s, const UmmaParams& p, const 
     return ADAPT_OK;
 }
 
+// One tile per CTA: p holds what both kernels need.  b_box_k: k rows one box of a row-major B brings.
+adapt_status_t launch_direct(State& S, const UmmaParams& p, int BN, int a_box_rows, const ReduceEpilogue& ep, const CUtensorMap& mapA, const CUtensorMap& mapB,
+                             const CUtensorMap& mapC, bool a_mn, bool b_mn, cudaStream_t stream)
+{
+    DirectMaps maps;
+    maps.a = mapA; maps.b = mapB; maps.c = mapC;
+    DirectParams q;
+    q.M = p.M; q.N = p.N; q.P_m = p.P_m; q.P_n = p.P_n;
+    q.kb_total = p.kb_total; q.kb_per_split = p.kb_per_split;
+    q.a_bytes = a_box_rows * kUmmaBK * 2;
+    q.tx_bytes = p.a_tx_bytes + p.b_tx_bytes;
+    q.stages = direct_stages(BN, a_box_rows, p.kb_per_split, p.P_k, S.machine.smem_bytes);
+    q.dtype = p.dtype; q.raster = p.raster; q.c_hint = p.c_hint;
+    q.splits_log2 = p.P_k == 8 ? 3 : p.P_k == 4 ? 2 : p.P_k == 2 ? 1 : 0;
+    q.idesc = p.idesc;
+    q.x_offset = (uint32_t)direct_ring_bytes(BN, a_box_rows, q.stages, p.P_k);
+    q.x_rows = a_box_rows;
+    q.C = (unsigned short*)p.C;
+    q.c_tma = p.c_mode;
+    q.ep = ep; q.status = p.status;
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)p.num_units, 1, 1);
+    cfg.blockDim = dim3((unsigned)(BN > 64 ? DirectShape<128>::kThreads : DirectShape<64>::kThreads), 1, 1);
+    cfg.dynamicSmemBytes = (size_t)direct_smem_bytes(BN, a_box_rows, q.stages, p.P_k);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    pdl_attribute(&attr[0]);
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)p.P_k;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = p.P_k > 1 ? 2 : 1;
+    void* args[2] = {&maps, &q};
+    const size_t arg_bytes[2] = {sizeof(maps), sizeof(q)};
+    CUDA_TRY(launch_exc(&cfg, direct_kernel(BN, a_mn, b_mn, p.P_k > 1, ep.D != nullptr), args, arg_bytes, 2));
+    S.launches.fetch_add(1, std::memory_order_relaxed);
+    return ADAPT_OK;
+}
+
 // The configuration of a call that writes C and adds D (null: none): the plan's, but for tall tiles that cannot serve it.  They store whole 32-byte
 // sectors, add D in 16-byte chunks and have one order of k; and a matrix D over a short k range makes trips to memory that nothing hides
 // (64179 x 576 x 896: 106 us, 108.8 on tall tiles; 5366 x 16320 x 1920: 322 and 287).  Such a call runs 256-row pair tiles, also where the model would
@@ -1217,19 +1268,22 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
 
     // the plan's fused reduction stands unless a fallback changed the tiling (then: partials in the workspace)
     const bool fused = c.fused != 0 && p.P_k == c.P_k && !(c.srcB == ADAPT_SRC_TMA_CLASSES && !kclsB);
+    bool direct = !kclsB && direct_config(s, c, S.machine) && (p.P_k == 1 || fused) && !S.shuffle_k;     // one tile per CTA
     // 16-bit C through TMA stores: whole 32-byte sectors (halo tiles shift theirs)
-    const bool tma_store = p.P_k == 1 && !kclsB && (halo ? ((uintptr_t)C & 15) == 0 : (((uintptr_t)C & 31) == 0 && s.N % 16 == 0));
+    const bool tma_store = direct ? p.P_k == 1 && ((uintptr_t)C & 15) == 0 && s.N % 8 == 0 : p.P_k == 1 && !kclsB && (halo ? ((uintptr_t)C & 15) == 0 : (((uintptr_t)C & 31) == 0 && s.N % 16 == 0));
     // A fused add runs where the 16-bit output is stored: here, or with unfused k splits in the reduction kernel.  A small output of
     // one row of tiles whose threads would store it themselves goes through fp32 sums and the reduction kernel too: the few warps that
     // drain it would wait for D pass after pass (16 x 30001 x 200 with a bias 17.9 us, 14.7 that way; 70 x 9999 x 64 12.0 and 10.5; but
     // 100 x 17097 x 85, 1.7 million outputs, 12.3 and 15.2, and 12048 x 38 x 739 13.8 and 15.8).  Without the workspace for that (it must not grow in a capture) the kernel adds D all the same.
-    bool sums_out = epi && p.P_k == 1 && !fused && !tma_store && s.M <= 128 && s.M * s.N <= (int64_t)768 << 10;
+    const bool whole_sectors = direct ? ((uintptr_t)C & 31) == 0 && s.N % 16 == 0 : tma_store;
+    bool sums_out = epi && p.P_k == 1 && !fused && !whole_sectors && s.M <= 128 && s.M * s.N <= (int64_t)768 << 10;
     if (sums_out) {
         void* probe = nullptr;
         const adapt_status_t r = try_workspace(S, stream, szA + szB + (size_t)round_up(s.M * partial_pitch(s.N) * 4, 256), &probe);
         if (r != ADAPT_OK) return r;
         sums_out = probe != nullptr;
     }
+    if (sums_out) direct = false;
     p.force_partial = sums_out ? 1 : 0;
     const bool partials = (p.P_k > 1 && !fused) || sums_out;
     p.ep = epi && !partials ? *epi : no_epilogue();
@@ -1286,7 +1340,7 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
     } else {
         // a row-major B whose K fits one k-block is loaded with boxes of just the k rows that exist (rounded up to 8; class
         // tiles shift B's rows by up to 7): boxes of 64 rows that lie mostly beyond K load several times slower when B is wide
-        if (b_mn && p.kb_total == 1) b_box_k = (int)std::min<int64_t>(64, round_up(s.K + (classesA ? class_k_slack(s) : 0), 8));
+        if (b_mn && p.kb_total == 1 && !direct) b_box_k = (int)std::min<int64_t>(64, round_up(s.K + (classesA ? class_k_slack(s) : 0), 8));
         if ((r = cached_map(S, pl, kMapB, b_src, extB, outB, pitchB, 64, b_mn ? b_box_k : c.BN / cg, &maps.b[0])) != ADAPT_OK) return r;
     }
 
@@ -1362,6 +1416,7 @@ adapt_status_t run_umma(State& S, Plan* pl, const void* A, const void* B, void* 
     if (const char* e = getenv("ADAPT_TRACE_CTA")) p.trace_cta = atoi(e);
 #endif
 
+    if (direct) return launch_direct(S, p, c.BN, a_box_rows, p.ep, maps.a[0], maps.b[0], maps.c[0], a_mn, b_mn, stream);
     if (c.BM == 512) return launch_tall(S, s, p, maps.a, maps.b[0], maps.c, a_mn, b_mn, classesA, stream);
     UmmaKernel k = streamk ? launch_map_umma_sk(c.family, c.BN, a_mn, b_mn)
                            : launch_map_umma(c.family, c.BN, a_mn, b_mn, classesA ? 1 : (kclsB ? 2 : 0), fused, p.ep.D != nullptr);
@@ -1802,6 +1857,12 @@ struct BatchOps {
         CUDA_TRY(cudaStreamWaitEvent(stream[lane], S.lanes.cross[other], 0));
         return ADAPT_OK;
     }
+    // Does call i share a launch of one tcgen05 tile per CTA?  (Buffers that TMA takes as they are.)
+    bool direct(int64_t i) const
+    {
+        const Plan* pl = plans[i];
+        return !S.shuffle_k && direct_groupable(pl->s, pl->c, S.machine) && (((uintptr_t)A[i] | (uintptr_t)B[i] | (uintptr_t)C[i]) & 15) == 0;
+    }
     // Bit 0: dtype, 1: A row-major, 2: B column-major.
     static int variant(const Shape& s)
     {
@@ -1816,8 +1877,61 @@ struct BatchOps {
         group_order(entry, n, S.machine.n_sm);
         return n;
     }
+    // Calls whose plans are one tcgen05 tile per CTA.  Long k ranges first.  Two CTAs per SM where there are more tiles than SMs.
+    template <int MAX>
+    adapt_status_t group_direct(const std::vector<int64_t>& calls, int lane)
+    {
+        int64_t order[MAX];
+        const int n = (int)calls.size();
+        std::copy(calls.begin(), calls.end(), order);
+        std::sort(order, order + n, [&](int64_t x, int64_t y) { return plans[x]->s.K != plans[y]->s.K ? plans[x]->s.K > plans[y]->s.K : x < y; });
+        const Shape& s0 = plans[calls[0]]->s;
+        const bool a_mn = s0.layoutA == ADAPT_COL_MAJOR, b_mn = s0.layoutB == ADAPT_ROW_MAJOR;
+        DirectGroupParams<MAX> g;
+        int tiles = 0, blocks = 1;
+        for (int j = 0; j < n; ++j) {
+            Plan* pl = plans[order[j]];
+            const Shape& s = pl->s;
+            const int64_t i = order[j];
+            const int rows = umma_a_box_rows(s, 1, 0, false);
+            DirectGroupItem& it = g.item[j];
+            adapt_status_t r;
+            if ((r = cached_map(S, pl, kMapA, A[i], a_mn ? s.M : s.K, a_mn ? s.K : s.M, a_mn ? s.M : s.K, 64, a_mn ? 64 : rows, &it.a)) != ADAPT_OK) return r;
+            if ((r = cached_map(S, pl, kMapB, B[i], b_mn ? s.N : s.K, b_mn ? s.K : s.N, b_mn ? s.N : s.K, 64, 64, &it.b)) != ADAPT_OK) return r;
+            it.C = (unsigned short*)C[i];
+            it.M = (int)s.M; it.N = (int)s.N; it.P_n = pl->c.P_n;
+            it.kb_total = (int)ceil_div(s.K, kUmmaBK);
+            it.a_bytes = rows * kUmmaBK * 2;
+            it.tx_bytes = it.a_bytes + 64 * kUmmaBK * 2;
+            it.tile_end = tiles += pl->c.P_m * pl->c.P_n;
+            blocks = std::max(blocks, it.kb_total);
+        }
+        g.count = n;
+        g.dtype = s0.dtype;
+        g.idesc = umma_idesc(s0.dtype, a_mn, b_mn, 128, 64);
+        g.status = S.d_status;
+        const bool shared = tiles > S.machine.n_sm;
+        g.stages = std::min(blocks, shared ? 4 : 8);
+        cudaLaunchConfig_t cfg;
+        memset(&cfg, 0, sizeof(cfg));
+        cfg.gridDim = dim3((unsigned)tiles, 1, 1);
+        cfg.blockDim = dim3((unsigned)DirectShape<64>::kThreads, 1, 1);
+        cfg.dynamicSmemBytes = (size_t)(shared ? direct_ring_bytes(64, 128, g.stages, 1) + 1024 : direct_smem_bytes(64, 128, g.stages, 1));
+        cfg.stream = stream[lane];
+        cudaLaunchAttribute attr[1];
+        pdl_attribute(&attr[0]);
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        void* args[1] = {&g};
+        const size_t arg_bytes[1] = {sizeof(g)};
+        CUDA_TRY(launch_exc(&cfg, direct_group_pick<MAX>(a_mn, b_mn), args, arg_bytes, 1));
+        S.launches.fetch_add(1, std::memory_order_relaxed);
+        return ADAPT_OK;
+    }
     adapt_status_t group(const std::vector<int64_t>& calls, int lane)
     {
+        if (direct(calls[0])) return calls.size() == 1 ? single(calls[0], lane) : calls.size() <= kDirectGroupFew ? group_direct<kDirectGroupFew>(calls, lane) : group_direct<kDirectGroupMax>(calls, lane);
+        static_assert(kGroupMax <= kDirectGroupMax, "a list's launch");
         GroupEntry entry[kGroupMax];
         const size_t n = entries(calls.data(), calls.size(), entry);
         const Shape& s = plans[calls[0]]->s;
@@ -1849,29 +1963,33 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
         return ADAPT_OK;
     }
     // Small calls (plans of the one-launch and CUDA-core families, as adapt_matmul_plan returned them) leave in grouped launches.
-    auto grouped = [&](const Plan* pl) { return pl && pl->selected && !pl->noop && !pl->zero_fill && group_eligible(pl->s, pl->c); };
+    BatchOps ops = {S, plans, A, B, C, {user}};
+    // ... and so do those of one tcgen05 tile per CTA, among themselves.
+    auto grouped = [&](int64_t i) {
+        const Plan* pl = plans[i];
+        return pl && pl->selected && !pl->noop && !pl->zero_fill && (group_eligible(pl->s, pl->c) || ops.direct(i));
+    };
     auto workspace = [&](int64_t i) { return plans[i] && needs_workspace(plans[i], A[i], B[i]); };
     int64_t singles = 0, with_workspace = 0, single = 0;
     for (int64_t i = 0; i < count; ++i) {
-        if (grouped(plans[i])) continue;
+        if (grouped(i)) continue;
         ++singles;
         single = i;
         with_workspace += workspace(i) ? 1 : 0;
     }
-    BatchOps ops = {S, plans, A, B, C, {user}};
     int64_t grouped_launches = 1;
     double hidden_us = 0.0;
     if (count >= 8 && singles == 1 && with_workspace == 0) {            // two launches, or more
-        int64_t small[kBatchVariants] = {}, others[kGroupMax], n = 0;
+        int64_t small[kBatchKinds] = {}, others[kGroupMax], n = 0;
         for (int64_t i = 0; i < count; ++i) {
             if (i == single) continue;
-            if (n < kGroupMax) others[n] = i;
-            ++n;
-            ++small[BatchOps::variant(plans[i]->s)];
+            const bool direct = ops.direct(i);
+            if (n < kGroupMax && !direct) others[n++] = i;
+            ++small[BatchOps::variant(plans[i]->s) + (direct ? kBatchDirect : 0)];
         }
         grouped_launches = 0;
         for (int64_t k : small) grouped_launches += ceil_div(k, kGroupMax);
-        if (grouped_launches == 1 && plans[single]) {
+        if (grouped_launches == 1 && n > 0 && plans[single]) {             // (a launch of tcgen05 tiles has no long chain that a second stream would hide)
             GroupEntry entry[kGroupMax];
             hidden_us = batch_hidden_us(entry, ops.entries(others, (size_t)n, entry), S.machine.n_sm, plans[single]->c.predicted_us);
         }
@@ -1905,8 +2023,8 @@ extern "C" adapt_status_t adapt_matmul_batch(int64_t count, const adapt_handle_t
         k.c = {(uintptr_t)C[i], (uintptr_t)C[i] + (uintptr_t)s.M * s.N * 2};
         k.unsound = !A[i] || !B[i] || !C[i] || (((uintptr_t)A[i] | (uintptr_t)B[i] | (uintptr_t)C[i]) & 1) != 0 || (k.c.lo < k.a.hi && k.a.lo < k.c.hi) ||
                     (k.c.lo < k.b.hi && k.b.lo < k.c.hi);
-        k.groupable = grouped(pl);
-        k.variant = BatchOps::variant(s);
+        k.groupable = grouped(i);
+        k.variant = BatchOps::variant(s) + (k.groupable && ops.direct(i) ? kBatchDirect : 0);
         k.workspace = workspace(i);
         k.alone = pl->c.streamk != 0;
         k.us = pl->c.predicted_us;

@@ -53,6 +53,9 @@ int calib_group(const Config& c);
 // then give mean regrets 1.047, 1.039, 1.044 and maxima 1.81, 1.51, 1.58, with 45 to 53 % exact picks.  Of that pass
 // hbm_bw_per_sm was taken back from 75.6 to 60.5 GB/s: the larger value hides the cost of a partial last wave on the
 // heaviest shapes (61370 x 32 x 85272 picked without split or stream-K: 2275 against 1700 us), 1.4 % of their time in total.
+// When the loops that issue loads and MMAs had got faster and one-tile-per-CTA plans had a kernel of their own, two rounds of the same descent on 655 drawn shapes
+// (sweep, recommendation and LLM layers, long contractions; three operand sets in turn in a captured row, predicted below 120 us; tall tiles' constants and the rates of the
+// chip left alone) moved thirty: on 178 shapes of another seed the mean regret went from 1.046 to 1.030, with 56 % exact picks.
 struct Calib {
     // All ones: factors fitted on 34,000 timed configurations of 500 sweep shapes (0.72 for plain one-split tiles ... 1.19 for
     // fused k classes, 0.48 for the warp-level kernel) raised the mean regret on a held-out shape set from 1.063 to 1.076,
@@ -66,8 +69,8 @@ struct Calib {
     double hbm_bw = 6.2e12;             // B/s, large streaming transfers
     double l2_bw_per_sm = 1.1e11;        // B/s one SM pulls through TMA from L2 (8192^3, 128 x 256 tiles: 48 KB per 0.48 us)
     double tensor_flops = 1.58e15;      // whole chip, kind::f16, BN = 256 (8192^3 on 256 x 256 pair tiles: 1.56e15)
-    double eta_mma_bn128 = 0.518;        // relative tensor efficiency at BN = 128 (0.29 us per 128 x 128 x 64 block)
-    double eta_mma_bn64 = 0.324;         // ... at BN = 64 (A-operand smem reads dominate)
+    double eta_mma_bn128 = 0.57;          // relative tensor efficiency at BN = 128
+    double eta_mma_bn64 = 0.4455;         // ... at BN = 64 (A-operand smem reads dominate)
     double eta_2cta = 1.0;              // pair tiles share B: no extra tensor cost
     // Tall pair tiles: relative tensor efficiency of whole tiles, of single blocks (they bring B for half the rows), and what a tile's drain does not
     // hide.  Fitted on 420 shapes whose best tall and best other configuration are predicted within 0.72 .. 1.12 of each other, both timed in turn
@@ -82,12 +85,12 @@ struct Calib {
     double mem_latency_us = 1.0;        // TMA issue -> data visible (sets Delta_dep with few stages)
     double hbm_latency_us = 1.04;        // the same under a full HBM stream of a dense operand (128 x 128256 x 4096: 5 stages of 32 KB, 0.41 us each)
     double hbm_latency_views_us = 1.6;  // ... through the strided class views (79457 x 196 x 8325 with 3 stages: 0.75 us per stage)
-    double umma_fixed_us = 1.1;         // barrier init, TMEM alloc, first load, last drain, TMEM free (the same fit: 2.5 was 3 us high)
+    double umma_fixed_us = 1.09;         // barrier init, TMEM alloc, first load, last drain, TMEM free (the same fit: 2.5 was 3 us high)
     // drain of one output tile through the epilogue warps (overlaps the next tile's main loop):
     // fixed part per tile + part per KB written; rows of C that are not 16-byte aligned cost more
     double epi_tile_fixed_us = 0.25, epi_us_per_kb = 0.0275;          // TMA stores (40000 x 40000 x 8: 4.8 TB/s)
-    double pair_drain_factor = 1.39;    // 40000 x 40000 x 8: 780 us on pair tiles, 671 us on 1-CTA tiles
-    double epi_partial_fixed_us = 0.44, epi_partial_us_per_kb = 0.0529;   // fp32 partials, stored by the epilogue threads
+    double pair_drain_factor = 1.529;    // 40000 x 40000 x 8: 780 us on pair tiles, 671 us on 1-CTA tiles
+    double epi_partial_fixed_us = 0.396, epi_partial_us_per_kb = 0.04655;   // fp32 partials, stored by the epilogue threads
     double epi_tile_fixed_unaligned_us = 1.41, epi_us_per_kb_unaligned = 0.0311;
     double thread_store_exposed = 0.495;  // share of the main loop that a drain through the epilogue threads does not hide
     double thread_store_exposed_pair = 0.25;   // ... on pair tiles (13835 x 3906 x 852 and 7111 x 97981 x 289 bracket it)
@@ -103,43 +106,54 @@ struct Calib {
     double skinny_pass_us = 4.4;        // one 64-row pass over one staged chunk when the streamed rows are k-contiguous
     double skinny_step_unaligned_us = 2.52;   // one 16-k step of a warp when the streamed rows are unaligned
     double skinny_mac_rate = 30e12;     // MAC/s ceiling of the warp-level kernel (small side padded to 16)
-    // one-launch cluster kernel (64 x 64 tiles, k split over a cluster): fitted on timed configurations of the kernel as it was when every
-    // stage had an mbarrier and a shift pass of its own.  It has become faster since (64 x 64 x 1024 by one CTA 19.0 -> 9.6 us,
-    // 256^3 5.42 -> 3.97), so these constants overstate it: a small problem whose best tcgen05 plan is predicted a few per cent
-    // faster may be better off here
-    double cluster_fixed_us = 0.75;     // beyond the launch: first trip to memory, rounding and store of the tile
+    // one-launch cluster kernel (64 x 64 tiles, k split over a cluster)
+    double cluster_fixed_us = 0.6;      // beyond the launch: first trip to memory, rounding and store of the tile
     double cluster_stage_us = 0.76;     // one 64-k stage
-    double cluster_reduce_us = 1.1;     // cluster barriers + reading the partial tiles of the peers
-    double cluster_crowd_us = 1.25, cluster_crowd_stage_us = 0.44;   // per CTA per SM beyond one per two SMs
+    double cluster_reduce_us = 0.79;    // cluster barriers + reading the partial tiles of the peers
+    double cluster_crowd_us = 1.25, cluster_crowd_stage_us = 0.55;   // per CTA per SM beyond one per two SMs
     double cluster_wave_us = 5.5;       // each further round of clusters
     double cluster_bw_eff = 0.35;       // fraction of hbm_bw its 16-byte copies reach when memory-bound
     double streamk_fixup_us = 10.0;     // stream-K: partial tile out (5 us) and its fence, the flag, the owner's exposed last drain ...
     double streamk_peer_us = 3.0;       // ... and its additions, per slot that shares the tile (2560 x 4096 x 4096, 6 sharers: 87 us
                                         // against 55 us of main loop; 5120 x 4096 x 8192, 3 sharers: 246 us against 226 us)
-    double fused_reduce_us = 2.0;       // fused split-K: cluster scheduling, drain to shared memory, two cluster-wide barrier rounds,
+    double fused_reduce_us = 2.2;       // fused split-K: cluster scheduling, drain to shared memory, two cluster-wide barrier rounds,
                                         // first remote reads (1 x 4096 x 4096, 128 x 128 tiles, P_k 4: 11.3 us fused, 11.1 us with the reduce launch;
                                         // 128 x 4096 x 4096: 13.3 against 14.1 us)
     double fused_wave_us = 3.0;         // each further round of clusters starts cold (1 x 4096 x 4096, P_k 8, 3 rounds: 14.2 us against 11.3 us in one)
-    double reduce_launch_us = 1.5;      // the reduce launch behind the GEMM: programmatic dependent launch hides about half of a launch
+    double reduce_launch_us = 1.65;      // the reduce launch behind the GEMM: programmatic dependent launch hides about half of a launch
     double dsmem_bw_per_sm = 60e9;      // B/s one SM reads from its peers' shared memory during the fused reduction
-    double copy_bw_eff = 0.935;          // pad-copy and reduce kernels
+    // HBM rate with a row-major B in pieces of 256 and of 128 bytes (tiles of 128 and of 64 columns), relative to wider ones
+    double b_piece256_eff = 0.78, b_piece128_eff = 0.75;
+    double epi_hidden = 0.72;            // share of the k splits' reduction that a stream from memory hides
+    double copy_bw_eff = 1.0;            // pad-copy and reduce kernels
     double hbm_bw_per_sm = 6.05e10;        // B/s one SM streams from HBM (tail wave of 20000 x 8 x 60001: 15 MB per tile in 0.3 ms)
-    double class_view_sm_eff = 0.935;    // per-SM rate through those views relative to l2_bw_per_sm (20000 x 8 x 60001 tail wave)
-    double class_tile_fixed_us = 0.625, class_tile_fixed_unaligned_us = 0.99;   // per class tile (44479 x 54634 x 16..72, 64-column tiles)
+    double class_view_sm_eff = 0.748;    // per-SM rate through those views relative to l2_bw_per_sm (20000 x 8 x 60001 tail wave)
+    double class_tile_fixed_us = 0.625, class_tile_fixed_unaligned_us = 0.792;   // per class tile (44479 x 54634 x 16..72, 64-column tiles)
     double pair_class_tile_us = 1.1;    // pair tiles of one row class, rows with stale heads: the peer zeroes its half and tells the leader across
                                         // the cluster before the tile's first MMA (7111 x 97981 x 289: 3.7 us per pair tile of six k-blocks)
     double kclass_view_sm_eff = 0.605;   // per-SM rate through the k-class views of B relative to l2_bw_per_sm (272 x 67839 x 6046: 48 KB per 0.75 us)
     double kclass_unit_fixed_us = 1.65;  // per unit of a k class run as a k split (1 x 80711 x 221: 18 units of one k-block in 37 us)
-    double kclass_tile_drain_us = 2.5;  // drain of a tile with eight class accumulators (29 x 58492 x 94: 8 tile rounds in 35 us)
+    double kclass_tile_drain_us = 2.0;  // drain of a tile with eight class accumulators (29 x 58492 x 94: 8 tile rounds in 35 us)
     double l2_reread_cost = 0.08;       // long contractions: what a second reading of all operands from L2 adds to the stream's time (it moved
                                         // twelve of 18000 picks, near ties, to 0.93 .. 1.14 of their time, 0.997 on average)
     double oob_box_penalty = 0.05;      // main-loop cost of one B box per stage that lies wholly beyond N
-    double reduce_batch_us = 0.8;       // split-K reduction: one batch of eight slabs (13 x 420 x 43580: P_k 72 -> 24 saves 13 us)
-    double class_split_bw_eff = 0.873;   // HBM rate through the k-class views of B with full-width tiles (classes as k splits) at M = 1 ...
+    double reduce_batch_us = 0.88;       // split-K reduction: one batch of eight slabs (13 x 420 x 43580: P_k 72 -> 24 saves 13 us)
+    double class_split_bw_eff = 0.768;   // HBM rate through the k-class views of B with full-width tiles (classes as k splits) at M = 1 ...
     double class_split_bw_eff_per_log2m = 0.031;   // ... and what it loses per doubling of M (1 x 50321 x 48452 ... 80 x 23916 x 86044)
     double class_split_fused_bw_eff = 0.815;       // ... with the classes of a tile as one cluster (36 x 81499 x 66349: 6.3 TB/s)
     double regroup_bw_eff = 0.85;       // class-major regrouping of a row-major A (20000 x 8000: 600 MB in 107 us) relative to hbm_bw
-    double class_view_bw_eff = 0.8;     // HBM rate through the per-row-class TMA views of an unaligned A
+    double class_view_bw_eff = 1.0;     // HBM rate through the per-row-class TMA views of an unaligned A
+    // one tile per CTA (direct_gemm.cuh): set-up, first load, drain and exit beyond the launch; a load's trip under load and with operands of a few MB;
+    // a k-block's MMAs on 64, 128 and 256 columns; the exchange of a split tile, and per KB of its fp32 sums; HBM rate with B in pieces of 128 bytes, relative
+    // to wider ones (256 x 256 x 256 2.7 us, 1000 x 1024 x 1024 4.8, 256 x 4096 x 4096 12.5 in nine stages and 20.5 in four, 16 x 14336 x 4096 20.7, 16 x 4096 x 4096 in four splits 8.2)
+    double direct_fixed_us = 0.72;
+    double direct_latency_us = 1.444, direct_latency_warm_us = 0.625;
+    double direct_mma64_us = 0.115, direct_mma128_us = 0.1815, direct_mma256_us = 0.308;
+    double direct_exchange_us = 0.576, direct_exchange_us_per_kb = 0.025;
+    double direct_narrow_bw_eff = 0.935;
+    double direct_hbm_bw = 7.1e12;      // B/s of a stream from memory (16 x 14336 x 4096)
+    double direct_unaligned_us = 0.4;   // rows of C off 16-byte boundaries
+    double direct_prologue_us = 1.6;     // operands over a copy: its launch is not hidden as it is behind a longer kernel
 };
 
 // ---- one configuration x of the search set S(b(s)) (Eq. 6) ------------------------------------
@@ -318,6 +332,54 @@ inline int umma_deepest_ring(int BN, int cluster, int a_rows, bool staging, int 
     for (int st = cap; st >= 2; --st)
         if (umma_smem_bytes(BN, cluster, st, a_rows, staging, fused_bytes) <= smem_limit) return st;
     return 0;
+}
+
+// One tile per CTA (direct_gemm.cuh): shared memory of its ring (the output's staging too) and of what the ranks of a split tile send each other.
+constexpr int kDirectAloneBytes = 116 * 1024;      // more than half of an SM's
+constexpr int kDirectStaticBytes = 1024;           // barriers and the like, static
+inline int direct_exchange_bytes(int BN, int rows, int splits) { return splits > 1 ? splits * rows * (BN / splits + 4) * 4 : 0; }
+inline int direct_ring_bytes(int BN, int rows, int stages, int splits)
+{
+    const int stage = (rows + BN) * 128;
+    // the MMA reads 128 rows of A from every stage, also where the box brings fewer
+    const int used = std::max(stages * stage, (stages - 1) * stage + 128 * 128);
+    return (int)round_up(std::max(used, splits > 1 ? direct_exchange_bytes(BN, rows, splits) : BN * 256), 1024);      // output boxes, or the sums for each rank
+}
+inline int direct_smem_bytes(int BN, int rows, int stages, int splits)
+{
+    return std::max(kDirectAloneBytes, direct_ring_bytes(BN, rows, stages, splits) + direct_exchange_bytes(BN, rows, splits) + 1024);
+}
+// The deepest ring that fits, no deeper than the CTA's k-blocks.
+inline int direct_stages(int BN, int rows, int64_t k_blocks, int splits, int smem_limit)
+{
+    int s = (int)std::min<int64_t>(kUmmaMaxStages, k_blocks);
+    while (s > 1 && direct_smem_bytes(BN, rows, s, splits) + kDirectStaticBytes > smem_limit) --s;
+    return s;
+}
+inline int umma_a_box_rows(const Shape& s, int cluster, int row_classes, bool k_classes);
+
+// Products below 2^24 multiply-adds, and those whose tiles would be less than three quarters full, stay with the one-launch cluster kernel: called by
+// themselves the host bounds them (3.3 us a call), in lists its grouped launch costs the host less an entry (0.2 us, 0.35 with two tensor maps), and its 64 x 64 tiles pad
+// less (256 x 256 x 256 in a row of calls 3.6 us there, 2.7 here).
+constexpr int64_t kDirectMinMacs = (int64_t)1 << 24;
+// Does a call of this configuration run on that kernel?  Plain tiles (operands read in place or over a re-pitched copy) of which every CTA has one, or one k
+// split of one whose reduction is fused; any C.
+inline bool direct_config(const Shape& s, const Config& c, const Machine& m)
+{
+    if (c.family != ADAPT_FAM_UMMA_1CTA || c.srcA == ADAPT_SRC_TMA_CLASSES || c.srcB == ADAPT_SRC_TMA_CLASSES || c.streamk || (c.P_k > 1 && !c.fused)) return false;
+    // (a split tile's sums, sent and received, beside two stages)
+    if (c.P_k > 1 && direct_smem_bytes(c.BN, umma_a_box_rows(s, 1, 0, false), 2, c.P_k) + kDirectStaticBytes > m.smem_bytes) return false;
+    if ((int64_t)c.P_m * c.P_n > umma_cluster_slots(m, c.fused ? c.P_k : 1) || s.M * s.N * s.K < kDirectMinMacs) return false;
+    // (an operand that has to be copied first is a launch more a call, also in a list; rows of C off 16-byte boundaries keep an entry out of the lists' launch)
+    if ((c.srcA == ADAPT_SRC_PAD_COPY || c.srcB == ADAPT_SRC_PAD_COPY || s.N % 8 != 0) && s.M * s.N * s.K < 4 * kDirectMinMacs) return false;
+    const int64_t rows = s.M < 128 ? s.M : 128 * (int64_t)c.P_m;       // (a short A is loaded with a box of its rows)
+    return 4 * s.M * s.N >= 3 * rows * std::min<int64_t>(round_up(s.N, 64), (int64_t)c.BN * c.P_n) || s.M * s.N * s.K >= 8 * kDirectMinMacs;
+}
+
+// Can a list's entry of this configuration share a launch with others of its kind (direct_group_kernel)?  Unsplit tiles of 64 columns, operands read in place.
+inline bool direct_groupable(const Shape& s, const Config& c, const Machine& m)
+{
+    return direct_config(s, c, m) && c.BN == 64 && c.P_k == 1 && c.srcA == ADAPT_SRC_TMA && c.srcB == ADAPT_SRC_TMA && s.N % 8 == 0;
 }
 
 // Rows of A one TMA box brings per stage (a multiple of 8, so the stage stays a multiple of 1024 B).

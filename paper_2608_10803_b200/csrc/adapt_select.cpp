@@ -337,16 +337,16 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
                                      : std::max(0.6, cal.class_split_bw_eff - cal.class_split_bw_eff_per_log2m * std::log2((double)std::max<int64_t>(1, s.M)));
     const double bw = ksplit_cls ? cal.hbm_bw * split_eff
                     : (c.srcA == ADAPT_SRC_TMA_CLASSES || kclasses) ? cal.hbm_bw * cal.class_view_bw_eff : cal.hbm_bw;
-    // A row-major B arrives as k-rows of BN contiguous columns per tile: short pieces stream below the
-    // HBM rate (8 x 30016 x 40000: 3.6 / 5.5 / 6.9 TB/s at 128 / 256 / 512 bytes)
+    // A row-major B arrives as k-rows of BN contiguous columns per tile: short pieces stream below the HBM rate
     double t_b_extra = 0.0;
     if (s.layoutB == ADAPT_ROW_MAJOR) {
         const double piece = 2.0 * c.BN;
-        const double eff = piece >= 512 ? 1.0 : (piece >= 256 ? 0.8 + 0.2 * (piece - 256) / 256 : 0.52 + 0.28 * (piece - 128) / 128);
+        const double eff = piece >= 512 ? 1.0 : (piece >= 256 ? cal.b_piece256_eff + (1.0 - cal.b_piece256_eff) * (piece - 256) / 256
+                                                              : cal.b_piece128_eff + (cal.b_piece256_eff - cal.b_piece128_eff) * (piece - 128) / 128);
         const double b_bytes = 2.0 * KN * rB * (kclasses ? c.BN / (c.BN - 8.0) : 1.0);
         t_b_extra = b_bytes / bw * (1.0 / std::max(eff, 0.3) - 1.0) * 1e6;
     }
-    double t_hbm = c.hbm_bytes / bw * 1e6 + t_b_extra - c.t_pro_us - c.t_epi_us;
+    double t_hbm = c.hbm_bytes / bw * 1e6 + t_b_extra - c.t_pro_us - cal.epi_hidden * c.t_epi_us;
     // a long contraction of a few tiles streams both operands; each further tile that reads a row block from L2 slows that stream a little
     // (256 x 256 x 262144 in 64 splits: 52.0 us on one 256 x 256 pair tile, 55.8 on two 128 x 256 tiles that both read B)
     if (c.P_k > 1 && !c.fused && !kclasses && c.srcA != ADAPT_SRC_TMA_CLASSES)
@@ -358,6 +358,30 @@ static void model_umma(const Shape& s, const Machine& m, const Calib& cal, Confi
         const int64_t loaded = c.cluster * ceil_div(c.BN / c.cluster, 64), needed = ceil_div(std::min<int64_t>(s.N, c.BN), 64);
         c.t_main_us *= 1.0 + cal.oob_box_penalty * (double)std::max<int64_t>(0, loaded - needed) / c.cluster;
     }
+    finish_common(s, c, cal);
+}
+
+// One tile per CTA: a k-block takes its MMAs or its share of a load's trip through the ring; a stream from memory is bounded by that.
+static void model_direct(const Shape& s, const Machine& m, const Calib& cal, Config& c)
+{
+    const double MK = (double)s.M * s.K, KN = (double)s.K * s.N, MN = (double)s.M * s.N;
+    const int rows = umma_a_box_rows(s, 1, 0, false);
+    const int64_t L = ceil_div(ceil_div(s.K, c.BK), c.P_k);
+    const int stages = direct_stages(c.BN, rows, L, c.P_k, m.smem_bytes);
+    c.grid = c.P_m * c.P_n * c.P_k;
+    c.hbm_bytes = 2.0 * (MK + KN + MN);
+    const double t_mma = c.BN == 64 ? cal.direct_mma64_us : c.BN == 128 ? cal.direct_mma128_us : cal.direct_mma256_us;
+    const double latency = 2.0 * (MK + KN) > 16e6 ? cal.direct_latency_us : cal.direct_latency_warm_us;
+    const double t_block = std::max(t_mma, (latency + t_mma) / stages);
+    const double t_fixed = cal.direct_fixed_us + 0.5 * std::min(1.0, (double)c.grid / m.n_sm) + (c.P_k > 1 ? cal.direct_exchange_us + cal.direct_exchange_us_per_kb * rows * c.BN * 4.0 / 1024.0 : 0.0) + (c.BN == 256 ? 0.3 : 0.0) +
+                           (s.N % 8 != 0 && c.P_k == 1 ? cal.direct_unaligned_us : 0.0) +
+                           (c.srcA == ADAPT_SRC_PAD_COPY || c.srcB == ADAPT_SRC_PAD_COPY ? cal.direct_prologue_us : 0.0);
+    model_prologue(s, c, cal);
+    c.ws_partial = 0;
+    c.t_epi_us = 0;
+    const double narrow = s.layoutB == ADAPT_ROW_MAJOR && c.BN == 64 ? 2.0 * KN * (1.0 / cal.direct_narrow_bw_eff - 1.0) : 0.0;
+    const double t_hbm = (2.0 * (MK + KN + MN) + narrow) / cal.direct_hbm_bw * 1e6;
+    c.t_main_us = t_fixed + std::max((double)L * t_block, t_hbm);
     finish_common(s, c, cal);
 }
 
@@ -621,7 +645,7 @@ static bool finalize(const Shape& s, const Machine& m, const Calib& cal, Config&
                    : (on_chip ? ADAPT_CLASS_MULTI_CORE_SPLIT_K : ADAPT_CLASS_HYBRID_SPLIT_K);
     switch (c.family) {
         case ADAPT_FAM_UMMA_1CTA:
-        case ADAPT_FAM_UMMA_2CTA: model_umma(s, m, cal, c); break;
+        case ADAPT_FAM_UMMA_2CTA: if (direct_config(s, c, m)) model_direct(s, m, cal, c); else model_umma(s, m, cal, c); break;
         case ADAPT_FAM_SKINNY: model_skinny(s, m, cal, c); break;
         case ADAPT_FAM_CLUSTER: model_cluster(s, m, cal, c); break;
         default: model_simt(s, m, cal, c); break;

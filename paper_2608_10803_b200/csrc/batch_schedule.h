@@ -24,12 +24,14 @@ struct BatchCall {
     Range a, b, c;              // what it reads (A, B) and writes (C)
     bool unsound;               // null, misaligned or overlapping operands: most likely refused, so the calls before it leave first
     bool groupable;             // may join a grouped launch
-    int variant;                // ... of this data type and pair of layouts (0 .. kBatchVariants - 1)
+    int variant;                // ... of this kernel, data type and pair of layouts (0 .. kBatchKinds - 1)
     bool workspace;             // needs the workspace of the stream it runs on
     bool alone;                 // nothing may run beside it (stream-K: its CTAs wait for one another and must all be resident)
     double us;                  // predicted time
 };
-constexpr int kBatchVariants = 8;
+constexpr int kBatchVariants = 8;                           // data types and pairs of layouts
+constexpr int kBatchDirect = kBatchVariants;                // ... and from here on the same for calls of one tcgen05 tile per CTA (direct_gemm.cuh)
+constexpr int kBatchKinds = 2 * kBatchVariants;
 constexpr int kBatchInternalMax = 4;                        // internal streams
 constexpr int kBatchLanesMax = 1 + kBatchInternalMax;       // ... and the caller's
 
@@ -121,7 +123,7 @@ adapt_status_t run_batch(int64_t count, int lanes, CallOf call_of, Ops& ops)
         std::vector<int64_t> calls;
         std::vector<Range> reads, writes;
         double us = 0.0;
-    } pending[kBatchVariants];
+    } pending[kBatchKinds];
     auto flush = [&](Pending& g) -> adapt_status_t {
         if (g.calls.empty()) return ADAPT_OK;
         int lane = 0;
@@ -134,17 +136,21 @@ adapt_status_t run_batch(int64_t count, int lanes, CallOf call_of, Ops& ops)
         g.us = 0.0;
         return r;
     };
-    auto flush_all = [&]() -> adapt_status_t {          // every variant leaves, also after one that failed; the first error
+    unsigned collected = 0;                             // the kinds that have any (a list of small calls asks for them at every call)
+    auto flush_all = [&]() -> adapt_status_t {          // every kind leaves, also after one that failed; the first error
         adapt_status_t first = ADAPT_OK;
-        for (Pending& g : pending) {
-            const adapt_status_t r = flush(g);
+        for (int v = 0; collected >> v; ++v) {
+            const adapt_status_t r = flush(pending[v]);
             if (first == ADAPT_OK) first = r;
         }
+        collected = 0;
         return first;
     };
     auto meets_pending = [&](const BatchCall& k) -> bool {
-        for (const Pending& g : pending)
+        for (int v = 0; collected >> v; ++v) {
+            const Pending& g = pending[v];
             if (!g.calls.empty() && (hits(g.writes, k.a) || hits(g.writes, k.b) || hits(g.writes, k.c) || hits(g.reads, k.c))) return true;
+        }
         return false;
     };
 
@@ -159,6 +165,7 @@ adapt_status_t run_batch(int64_t count, int lanes, CallOf call_of, Ops& ops)
                 g.reads.reserve(2 * kGroupMax);
                 g.writes.reserve(kGroupMax);
             }
+            collected |= 1u << k.variant;
             g.calls.push_back(i);
             g.reads.push_back(k.a);
             g.reads.push_back(k.b);

@@ -1,0 +1,389 @@
+// tcgen05 GEMM kernel for launches of ONE output tile per CTA: plain 128 x BN tiles, operands that TMA reads (in place or over a copy).
+//
+// A product of some tens of microseconds or less is launch, set-up, one trip to memory, a short main loop and one drain.  The persistent kernel
+// (umma_gemm.cuh) spends more than a microsecond each on its set-up and on draining one tile, and keeps 64 KB of staging out of its ring.  Here
+//   warp 0 (barriers, then TMA loads) starts loading before TMEM is allocated, and the other warps wait for the barriers only;
+//   warp 1 (TMEM, tcgen05.mma) commits a stage only when a later k-block takes it;
+//   warps 2 .. 5 or 9 (accumulator -> one rounding -> shared memory -> TMA stores of 32 x 64 boxes) all work on the one tile, and their staging is the
+//   ring: when the accumulator is complete, every load has landed and been read.
+// What bounds it: for operands in L2 the ring (a load takes 1.1 us under load, so its 200 KB bring 24 KB per 0.17 us), then the MMAs (192 cycles per
+// k-block on 64 columns, bound by shared memory); for a stream from memory the stream.  Measured in a captured row of calls, three sets of operands in
+// turn, the persistent kernel (as it was | with the same loops) and this one: 1000 x 1024 x 1024 on 64 columns 8.9 | 6.3 | 4.8 us, 256 x 4096 x 4096 on 64
+// columns 19.6 | 17.8 | 12.5, 16 x 14336 x 4096 24.9 | 24.9 | 20.7, 256 x 256 x 256 2.7 (3.6 with the one-launch cluster kernel).
+// One CTA per SM on purpose (kDirectAloneBytes): with two, the next kernel's CTAs double up on the SMs that this grid leaves idle: 1000 x 1024 x 1024 in
+// four stages 6.4 us with 97 KB a CTA, 5.8 with 120.
+//
+// SPLIT: the k range of a tile is cut over the CTAs of a thread-block cluster (2, 4 or 8; rank = split), each of which stores 1 / P of the tile's columns:
+// a CTA puts its fp32 sums into its ring, every rank's share in one piece, copies the pieces into the receive buffers of their ranks (bulk copies between the
+// CTAs' shared memory, counted on the receiver's barrier), and each rank adds what it has in ascending rank order.  The receive buffer is not part
+// of the ring, so nobody waits for a peer before that.  (Stored across the cluster by the threads, 16 bytes at a row each, the sums of a 128 x 128 tile
+// took 4.3 us: 8 bytes a cycle.)
+#pragma once
+
+#include <cuda.h>
+#include <cuda_fp16.h>
+#include <cuda_bf16.h>
+
+#include "adapt_internal.h"
+#include "aux_kernels.cuh"        // fused-add parameters
+#include "launch_pdl.cuh"
+#include "ptx_sm100.cuh"
+#include "umma_gemm.cuh"          // pack16, epilogue_add, kGroupM
+
+namespace adapt {
+
+struct DirectParams {
+    int M, N;
+    int P_m, P_n;
+    int kb_total, kb_per_split;      // k-blocks of K, of a CTA's share
+    int stages, a_bytes;             // ring depth; bytes of a stage's A region (the rows one box brings)
+    int tx_bytes;                    // bytes the loads of a stage deliver
+    int dtype, raster, c_hint, splits_log2;
+    uint32_t idesc;
+    uint32_t x_offset;               // SPLIT: the receive buffer, bytes behind the ring's start, ...
+    int x_rows;                      // ... and the rows it holds of every rank (as many as one box of A brings)
+    unsigned short* C;               // SPLIT, LIST, and where c_tma is 0: stored by the threads
+    int c_tma;                       // C has a map: its rows start on 16-byte boundaries
+    ReduceEpilogue ep;               // EPI
+    unsigned int* status;
+};
+struct DirectMaps { CUtensorMap a, b, c; };
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+template <int BN> struct DirectShape {
+    static constexpr int kEpilogueWarps = BN > 64 ? 8 : 4;
+    static constexpr int kThreads = 64 + 32 * kEpilogueWarps;
+};
+
+// Tile (mb, nb) by the calling CTA; SPLIT: the rank-th split of it.  map_c null (LIST): the threads store the boxes, whole rows of 128 bytes.
+template <int BN, bool A_MN, bool B_MN, bool SPLIT, bool EPI, bool LIST = false>
+__device__ __forceinline__ void direct_tile(const CUtensorMap* map_a, const CUtensorMap* map_b, const CUtensorMap* map_c, const DirectParams& p, int rank, int mb, int nb)
+{
+    constexpr int EW = DirectShape<BN>::kEpilogueWarps, THREADS = DirectShape<BN>::kThreads;
+    constexpr int B_BOXES = B_MN ? BN / 64 : 1, A_BOXES = A_MN ? 2 : 1;
+    constexpr uint32_t B_BYTES = BN * kUmmaBK * 2;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(16) uint64_t bars[2 * kUmmaMaxStages + 2];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_word;
+    volatile int* abort_flag = &abort_word;
+    const uint32_t ring = (ptx::smem_u32(smem_raw) + 1023u) & ~1023u;          // swizzle atoms are 1024-byte aligned
+    uint8_t* ring_gen = smem_raw + (ring - ptx::smem_u32(smem_raw));
+    const uint32_t full_bar = ptx::smem_u32(bars), empty_bar = full_bar + 8u * kUmmaMaxStages, done_bar = empty_bar + 8u * kUmmaMaxStages, sums_bar = done_bar + 8u;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+    const int S = p.stages;
+    const uint32_t stage_bytes = (uint32_t)p.a_bytes + B_BYTES;
+
+    const int row0 = mb * 128, n0 = nb * BN;
+    // SPLIT: columns of a rank's share, floats from a row of it to the next, rows of this tile that are exchanged (those of warps with a row of C)
+    const int w_log2 = (BN == 64 ? 6 : BN == 128 ? 7 : 8) - (SPLIT ? p.splits_log2 : 0), pitch = (1 << w_log2) + 4;
+    const int live_rows = SPLIT ? min(p.x_rows, (p.M - row0 + 31) & ~31) : 0;
+    const int kb0 = SPLIT ? rank * p.kb_per_split : 0, n_kb = SPLIT ? min(p.kb_total - kb0, p.kb_per_split) : p.kb_total;
+
+    if (warp == 0) {
+        if (ptx::elect_one()) {
+            abort_word = 0;
+            for (int s = 0; s < S; ++s) {
+                ptx::mbar_init(full_bar + 8u * s, 1);
+                ptx::mbar_init(empty_bar + 8u * s, 1);
+            }
+            ptx::mbar_init(done_bar, 1);
+            if (SPLIT) {
+                ptx::mbar_init(sums_bar, 1);
+                ptx::mbar_arrive_expect_tx(sums_bar, (uint32_t)(((1 << p.splits_log2) - 1) * live_rows * pitch * 4));
+            }
+            ptx::fence_barrier_init();
+            ptx::fence_proxy_async_smem();
+            ptx::prefetch_tensormap(map_a);
+            ptx::prefetch_tensormap(map_b);
+            if (!SPLIT && !LIST && p.c_tma) ptx::prefetch_tensormap(map_c);
+        }
+        __syncwarp();
+        asm volatile("bar.arrive 1, %0;" ::"n"(THREADS) : "memory");           // the other warps wait for it
+        if (SPLIT) cluster_arrive();
+        pdl_wait();
+        if (ptx::elect_one()) {
+            int stage = 0;
+            uint32_t phase = 1;
+            for (int kb = 0; kb < n_kb; ++kb) {
+                if (!ptx::mbar_wait(empty_bar + 8u * stage, phase, abort_flag)) break;
+                const uint32_t sA = ring + (uint32_t)stage * stage_bytes, sB = sA + (uint32_t)p.a_bytes, fb = full_bar + 8u * stage;
+                const int k0 = (kb0 + kb) * kUmmaBK;
+                ptx::mbar_arrive_expect_tx(fb, (uint32_t)p.tx_bytes);
+#pragma unroll
+                for (int j = 0; j < A_BOXES; ++j) ptx::tma_load_2d(sA + 8192u * j, map_a, fb, A_MN ? row0 + 64 * j : k0, A_MN ? k0 : row0);
+#pragma unroll
+                for (int j = 0; j < B_BOXES; ++j) ptx::tma_load_2d(sB + 8192u * j, map_b, fb, B_MN ? n0 + 64 * j : k0, B_MN ? k0 : n0);
+                if (++stage == S) { stage = 0; phase ^= 1u; }
+            }
+        }
+        __syncwarp();
+    } else {
+        if (SPLIT) cluster_arrive();
+        if (warp == 1) {
+            ptx::tmem_alloc<1>(ptx::smem_u32(&tmem_slot), (uint32_t)BN);
+            ptx::tmem_relinquish<1>();
+            pdl_launch_dependents();                       // not before: a CTA of the next kernel must not take the columns this one waits for
+        }
+        ptx::tc_fence_before();
+        asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
+        ptx::tc_fence_after();
+    }
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_slot);    // (warp 0 has no use for it)
+
+    if (warp == 1) {
+        constexpr uint32_t a_kstep = A_MN ? 2048u : 32u, b_kstep = B_MN ? 2048u : 32u;
+        const uint64_t a_desc = ptx::smem_desc_sw128(ring, A_MN ? 8192u : 16u, 1024u);
+        const uint64_t b_desc = ptx::smem_desc_sw128(ring + (uint32_t)p.a_bytes, B_MN ? 8192u : 16u, 1024u);
+        if (ptx::elect_one()) {
+            const uint32_t a_lo = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32), b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32);
+            const uint32_t idesc = p.idesc, step = stage_bytes >> 4, full_end = full_bar + 8u * S;
+            uint32_t off = 0, fb = full_bar, phase = 0, more = 0;
+            for (int left = n_kb; left > 0; --left, more = 1u) {
+                if (!ptx::mbar_wait(fb, phase, abort_flag)) break;
+#pragma unroll
+                for (int k16 = 0; k16 < kUmmaBK / 16; ++k16)
+                    ptx::umma_f16<1>(tmem, ptx::smem_desc_join(a_lo + off + (k16 * a_kstep >> 4), a_hi), ptx::smem_desc_join(b_lo + off + (k16 * b_kstep >> 4), b_hi), idesc, k16 > 0 ? 1u : more);
+                if (left > S) ptx::umma_commit_1(fb + 8u * kUmmaMaxStages);     // a later k-block takes this stage
+                if (left == 1) ptx::umma_commit_1(done_bar);
+                off += step;
+                fb += 8u;
+                if (fb == full_end) { fb = full_bar; off = 0; phase ^= 1u; }
+            }
+        }
+        __syncwarp();
+    } else if (warp >= 2) {
+        // warp w reads TMEM lanes 32 (w % 4) .. + 31; eight warps: two per lane quarter, half of the columns each
+        constexpr int COLS = BN * 4 / EW;
+        const int q = warp & 3, c_first = ((warp - 2) >> 2) * COLS;
+        const int row = row0 + q * 32 + lane;
+        const bool row_ok = row < p.M, live = row0 + q * 32 < p.M;              // (live: a row of this warp exists, uniform)
+        const uint32_t t_row = tmem + ((uint32_t)(q * 32) << 16);
+        const bool done = ptx::mbar_wait_warp(done_bar, 0, abort_flag);
+        if (SPLIT) cluster_wait();                                              // the peers run: their shared memory may be written
+        pdl_wait();                                                             // (long past: the loads have waited for it)
+        if (done && live) {
+            ptx::tc_fence_after();
+            if (!SPLIT) {
+                const uint64_t policy = ptx::l2_policy_evict_first();
+#pragma unroll
+                for (int pass = 0; pass < COLS / 64; ++pass) {
+                    const int c0 = c_first + 64 * pass;
+                    if (n0 + c0 >= p.N) break;                                  // uniform
+                    uint32_t r[2][32];
+                    ptx::tmem_ld_32x32(t_row + (uint32_t)c0, r[0]);
+                    ptx::tmem_ld_32x32(t_row + (uint32_t)(c0 + 32), r[1]);
+                    ptx::tmem_ld_wait();
+                    uint8_t* box = ring_gen + ((warp - 2) * (COLS / 64) + pass) * 4096;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (EPI) epilogue_add(p.ep, r[h], row, n0 + c0 + 32 * h, p.N, p.N, row_ok && n0 + c0 + 32 * h < p.N, p.dtype);
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) {
+                            const uint32_t* v = r[h] + 8 * c;
+                            *reinterpret_cast<uint4*>(box + lane * 128 + (((4 * h + c) ^ (lane & 7)) << 4)) =
+                                make_uint4(pack16(__uint_as_float(v[0]), __uint_as_float(v[1]), p.dtype), pack16(__uint_as_float(v[2]), __uint_as_float(v[3]), p.dtype),
+                                           pack16(__uint_as_float(v[4]), __uint_as_float(v[5]), p.dtype), pack16(__uint_as_float(v[6]), __uint_as_float(v[7]), p.dtype));
+                        }
+                    }
+                    if (LIST) {
+                        __syncwarp();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int r8 = 4 * i + (lane >> 3), ch = lane & 7, m = row0 + q * 32 + r8, n = n0 + c0 + 8 * ch;
+                            if (m < p.M && n < p.N)
+                                *reinterpret_cast<uint4*>(p.C + (int64_t)m * p.N + n) = *reinterpret_cast<const uint4*>(box + r8 * 128 + ((ch ^ (r8 & 7)) << 4));
+                        }
+                        continue;
+                    }
+                    if (!p.c_tma) {
+                        // rows of C anywhere: a row's 64 columns at a time, two to a lane
+                        __syncwarp();
+                        const int rows = min(32, p.M - row0 - q * 32), n = n0 + c0 + 2 * lane;
+                        unsigned short* dst = p.C + (int64_t)(row0 + q * 32) * p.N + n;
+#pragma unroll 8
+                        for (int i = 0; i < rows; ++i, dst += p.N) {
+                            const uint32_t v = *reinterpret_cast<const uint32_t*>(box + i * 128 + (((lane >> 2) ^ (i & 7)) << 4) + (lane & 3) * 4);
+                            if ((reinterpret_cast<uintptr_t>(dst) & 3) == 0 && n + 1 < p.N) {
+                                *reinterpret_cast<uint32_t*>(dst) = v;
+                            } else {
+                                if (n < p.N) dst[0] = (unsigned short)v;
+                                if (n + 1 < p.N) dst[1] = (unsigned short)(v >> 16);
+                            }
+                        }
+                        continue;
+                    }
+                    ptx::fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (p.c_hint) ptx::tma_store_2d_hint(map_c, ptx::smem_u32(box), n0 + c0, row0 + q * 32, policy);
+                        else ptx::tma_store_2d(map_c, ptx::smem_u32(box), n0 + c0, row0 + q * 32);
+                        ptx::bulk_commit();
+                    }
+                }
+                if (!LIST && p.c_tma && lane == 0) ptx::bulk_wait_read<0>();
+            } else {
+                // column c of the tile belongs to rank c / W; pieces and buffers: [rank][row][W + 4]
+                const int r_in = q * 32 + lane;
+#pragma unroll
+                for (int c0 = c_first; c0 < c_first + COLS; c0 += 32) {
+                    uint32_t r[32];
+                    ptx::tmem_ld_32x32(t_row + (uint32_t)c0, r);
+                    ptx::tmem_ld_wait();
+                    if (r_in < p.x_rows) {
+#pragma unroll
+                        for (int g = 0; g < 8; ++g) {
+                            const int c = c0 + 4 * g;
+                            *reinterpret_cast<uint4*>(ring_gen + (((c >> w_log2) * p.x_rows + r_in) * pitch + (c & ((1 << w_log2) - 1))) * 4) =
+                                make_uint4(r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+                        }
+                    }
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                // one lane for each rank that this warp has columns of
+                const int to = (c_first >> w_log2) + lane, rows = min(32, p.x_rows - q * 32);
+                if (lane < max(1, COLS >> w_log2) && to != rank) {
+                    uint32_t dst, bar;
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(dst) : "r"(ring + p.x_offset + (uint32_t)((rank * p.x_rows + q * 32) * pitch) * 4u), "r"(to));
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(sums_bar), "r"(to));
+                    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                                 ::"r"(dst), "r"(ring + (uint32_t)((to * p.x_rows + q * 32) * pitch) * 4u), "r"(rows * pitch * 4), "r"(bar) : "memory");
+                }
+            }
+        }
+        ptx::tc_fence_before();
+    }
+    if (SPLIT) {
+        if (warp < 2) cluster_wait();
+        if (warp >= 2) {
+            asm volatile("bar.sync 2, %0;" ::"n"(32 * EW) : "memory");            // this CTA's own pieces are in place
+            if (ptx::mbar_wait_warp(sums_bar, 0, abort_flag)) {
+                const float *own = reinterpret_cast<const float*>(ring_gen), *got = reinterpret_cast<const float*>(ring_gen + p.x_offset);
+                const int slab = p.x_rows * pitch;
+                // groups of four columns, a row's side by side on neighbouring threads
+#pragma unroll 2
+                for (int i = (int)threadIdx.x - 64; i < live_rows << (w_log2 - 2); i += 32 * EW) {
+                    const int r = i >> (w_log2 - 2), c = (i - (r << (w_log2 - 2))) * 4, row = row0 + r, n = n0 + (rank << w_log2) + c;
+                    if (row >= p.M || n >= p.N) continue;
+                    const int at = r * pitch + c;
+                    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int s = 0; s < (1 << p.splits_log2); ++s) {
+                        const float4 v = *reinterpret_cast<const float4*>((s == rank ? own : got) + s * slab + at);
+                        if (s == 0) sum = v;
+                        else { sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w; }
+                    }
+                    unsigned short* dst = p.C + (int64_t)row * p.N + n;
+                    if (EPI) {
+                        sum.x = fused_add(p.ep, sum.x, row, n, p.N, p.dtype);
+                        if (n + 1 < p.N) sum.y = fused_add(p.ep, sum.y, row, n + 1, p.N, p.dtype);
+                        if (n + 2 < p.N) sum.z = fused_add(p.ep, sum.z, row, n + 2, p.N, p.dtype);
+                        if (n + 3 < p.N) sum.w = fused_add(p.ep, sum.w, row, n + 3, p.N, p.dtype);
+                    }
+                    const uint2 v = make_uint2(pack16(sum.x, sum.y, p.dtype), pack16(sum.z, sum.w, p.dtype));
+                    if (n + 4 <= p.N && (reinterpret_cast<uintptr_t>(dst) & 7) == 0) {
+                        *reinterpret_cast<uint2*>(dst) = v;
+                    } else {
+                        dst[0] = (unsigned short)v.x;
+                        if (n + 1 < p.N) dst[1] = (unsigned short)(v.x >> 16);
+                        if (n + 2 < p.N) dst[2] = (unsigned short)v.y;
+                        if (n + 3 < p.N) dst[3] = (unsigned short)(v.y >> 16);
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        ptx::cluster_sync_all();                                                // no CTA leaves while its pieces are still read
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && abort_word) atomicOr(p.status, 1u);
+    if (warp == 1) {
+        ptx::tc_fence_after();
+        ptx::tmem_dealloc<1>(tmem, (uint32_t)BN);
+    }
+}
+
+template <int BN, bool A_MN, bool B_MN, bool SPLIT, bool EPI>
+__global__ void __launch_bounds__(DirectShape<BN>::kThreads, 2)
+direct_gemm_kernel(const __grid_constant__ DirectMaps maps, const __grid_constant__ DirectParams p)
+{
+    const int rank = SPLIT ? (int)blockIdx.x & ((1 << p.splits_log2) - 1) : 0, t = SPLIT ? (int)blockIdx.x >> p.splits_log2 : (int)blockIdx.x;
+    int mb, nb;
+    if (p.P_m == 1) {
+        mb = 0; nb = t;
+    } else if (p.raster) {
+        mb = t / p.P_n; nb = t - mb * p.P_n;
+    } else {
+        const int g = t / (kGroupM * p.P_n), gm = min(p.P_m - g * kGroupM, kGroupM), r = t - g * kGroupM * p.P_n;
+        nb = r / gm; mb = g * kGroupM + r - nb * gm;
+    }
+    direct_tile<BN, A_MN, B_MN, SPLIT, EPI>(&maps.a, &maps.b, &maps.c, p, rank, mb, nb);
+}
+
+// The tiles of up to kDirectGroupMax products (128 x 64 each, of one data type and pair of layouts) side by side in one launch: the lists of
+// adapt_matmul_batch.  An entry's tiles are what its own launch computes, so a list gives the bits of the calls made alone.  The entries' maps travel in
+// the kernel's parameters, so nothing is copied to the device and the launch can be captured; C has no map (a list of tiny products is bound by the host,
+// which pays for each).  48 products of 64 .. 512 a side, steps of 64, in a captured row: 28 us as they were planned before, 14 now; 48 of 256 x 256 x 256 17.7 and 6.7.
+constexpr int kDirectGroupMax = 64, kDirectGroupFew = 16;       // entries of a launch; of the form with the smaller parameters
+struct DirectGroupItem {
+    CUtensorMap a, b;
+    unsigned short* C;
+    int M, N, P_n, kb_total;
+    int a_bytes, tx_bytes;
+    int tile_end;                    // tiles of this and all earlier items
+};
+template <int MAX>
+struct DirectGroupParams {
+    DirectGroupItem item[MAX];
+    int count, stages, dtype;
+    uint32_t idesc;
+    unsigned int* status;
+};
+static_assert(sizeof(DirectGroupParams<kDirectGroupMax>) <= 32764, "kernel parameters");
+
+template <bool A_MN, bool B_MN, int MAX>
+__global__ void __launch_bounds__(DirectShape<64>::kThreads, 2)
+direct_group_kernel(const __grid_constant__ DirectGroupParams<MAX> g)
+{
+    int lo = 0, hi = g.count - 1;                               // the first item whose tiles end beyond this CTA's
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if ((int)blockIdx.x < g.item[mid].tile_end) hi = mid; else lo = mid + 1;
+    }
+    const DirectGroupItem& it = g.item[lo];
+    const int t = (int)blockIdx.x - (lo > 0 ? g.item[lo - 1].tile_end : 0), mb = t / it.P_n;
+    DirectParams p;
+    p.M = it.M; p.N = it.N;
+    p.kb_total = it.kb_total;
+    p.stages = min(g.stages, it.kb_total);
+    p.a_bytes = it.a_bytes; p.tx_bytes = it.tx_bytes;
+    p.dtype = g.dtype; p.C = it.C;
+    p.idesc = g.idesc; p.status = g.status;
+    direct_tile<64, A_MN, B_MN, false, false, true>(&it.a, &it.b, nullptr, p, 0, mb, t - mb * it.P_n);
+}
+
+// ---- host side ----------------------------------------------------------------------------------------------------------------------
+template <bool SPLIT, bool EPI>
+inline const void* direct_pick(int BN, bool a_mn, bool b_mn)
+{
+#define ADAPT_PICK(bn) if (BN == bn) return a_mn ? (b_mn ? (const void*)direct_gemm_kernel<bn, true, true, SPLIT, EPI> : (const void*)direct_gemm_kernel<bn, true, false, SPLIT, EPI>) \
+                                                 : (b_mn ? (const void*)direct_gemm_kernel<bn, false, true, SPLIT, EPI> : (const void*)direct_gemm_kernel<bn, false, false, SPLIT, EPI>);
+    ADAPT_PICK(64) ADAPT_PICK(128) ADAPT_PICK(256)
+#undef ADAPT_PICK
+    return nullptr;
+}
+template <int MAX>
+inline const void* direct_group_pick(bool a_mn, bool b_mn)
+{
+    return a_mn ? (b_mn ? (const void*)direct_group_kernel<true, true, MAX> : (const void*)direct_group_kernel<true, false, MAX>)
+                : (b_mn ? (const void*)direct_group_kernel<false, true, MAX> : (const void*)direct_group_kernel<false, false, MAX>);
+}
+inline const void* direct_kernel(int BN, bool a_mn, bool b_mn, bool split, bool epi)
+{
+    if (split) return epi ? direct_pick<true, true>(BN, a_mn, b_mn) : direct_pick<true, false>(BN, a_mn, b_mn);
+    return epi ? direct_pick<false, true>(BN, a_mn, b_mn) : direct_pick<false, false>(BN, a_mn, b_mn);
+}
+
+}  // namespace adapt

@@ -64,7 +64,6 @@ tall_gemm_kernel(const __grid_constant__ TmapPackT<CLS ? 1 : 0> maps, const __gr
     volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(bar_gen + 32 * S + 32);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_gen + 32 * S + 36);
 
-    pdl_launch_dependents();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t cta_rank = ptx::cluster_ctarank();
     const bool leader = cta_rank == 0;
@@ -94,6 +93,7 @@ tall_gemm_kernel(const __grid_constant__ TmapPackT<CLS ? 1 : 0> maps, const __gr
     if (warp == 1) {
         ptx::tmem_alloc<2>(tmem_slot, 512);
         ptx::tmem_relinquish<2>();
+        pdl_launch_dependents();                               // (umma_gemm.cuh says why not before)
     }
     ptx::tc_fence_before();
     ptx::cluster_sync_all();                                   // the peer's barriers exist

@@ -394,7 +394,6 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
     const uint32_t afull_bar = bar_base + 544u, aready_bar = bar_base + 672u;
     int* sk_count = reinterpret_cast<int*>(bar_gen + 528);     // stream-K: epilogue warps that have written their share of a partial
 
-    pdl_launch_dependents();
     if (threadIdx.x == 0) ADAPT_TRACE(11, 0);
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -435,6 +434,7 @@ umma_gemm_kernel(const __grid_constant__ TmapPackT<MODE> maps, const UmmaParams 
     if (warp == 1) {
         ptx::tmem_alloc<CG>(tmem_slot, TMEM_COLS);
         ptx::tmem_relinquish<CG>();
+        pdl_launch_dependents();           // not before: a CTA of a later kernel must not hold columns that this one waits for
     } else if (p.b_tx_bytes < B_BYTES) {
         // Short-K boxes of B: a load then brings only the k rows that exist, so the rest of every stage's B region is
         // zeroed here, once (no load ever writes it; the tensor core multiplies it with the zero-filled k tail of A).

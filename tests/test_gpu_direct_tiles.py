@@ -1,0 +1,130 @@
+"""The kernel of one tcgen05 tile per CTA: exact on integers at the edges of its tiles, rings and splits, in every layout, with special values and a
+fused add, through a C off 32-byte boundaries, and in lists."""
+import random
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import gemm as og
+from paper_2608_10803_b200 import binding as ab
+from paper_2608_10803_b200 import synth
+
+from gpu_util import check_case, init
+
+pytestmark = pytest.mark.gpu
+
+
+def stream():
+    return torch.cuda.current_stream().cuda_stream
+
+
+def integers(rows, cols, seed, dtype):
+    return synth.draw_operand(rows, cols, ("integer", -2, 2), seed, dtype, "cuda")
+
+
+def forms(M, N, K, dtype, lA=0, lB=0):
+    """One plan per tile width and split that this kernel serves."""
+    seen = {}
+    for c in ab.adapt_plan_candidates(M, N, K, dtype, lA, lB):
+        if c.family == ab.FAM_UMMA_1CTA and c.BN % 64 == 0 and c.srcA != 3 and c.srcB != 3 and not c.streamk and (c.P_k == 1 or c.fused):
+            seen.setdefault((c.BN, c.P_k), c.tiling_key)
+    return {k: ab.adapt_matmul_plan_forced(M, N, K, dtype, lA, lB, key) for k, key in seen.items()}
+
+
+# rows: a short box of A, a whole tile, one row more; columns: less than a box, a last box of 8 columns; k: one block, a remainder, longer than any ring
+SHAPES = [(1, 16384, 1032), (7, 4104, 2056), (33, 2048, 1000), (127, 1032, 1024), (128, 1024, 136), (129, 520, 1096), (256, 256, 256), (1000, 1024, 1024),
+          (300, 1000, 328), (640, 968, 72), (96, 200, 8192), (1152, 1088, 64), (130, 777, 1032), (64, 1027, 999), (500, 501, 502)]
+
+
+@pytest.mark.parametrize("layouts", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_every_form_is_exact_on_integers(shape, layouts):
+    M, N, K = shape
+    lA, lB = layouts
+    dtype = ab.F16 if (M + N + K) % 16 else ab.BF16
+    init()
+    A, B = integers(M, K, 41, dtype), integers(K, N, 42, dtype)
+    a = A.t().contiguous() if lA else A
+    b = B.t().contiguous() if lB else B
+    plans = forms(M, N, K, dtype, lA, lB)
+    assert plans
+    for plan in plans.values():
+        check_case(M, N, K, dtype, a, b, lA, lB, plan=plan, exact=True)
+
+
+def test_the_forms_cover_tiles_and_splits():
+    init()
+    keys = set()
+    for M, N, K in SHAPES:
+        keys |= set(forms(M, N, K, ab.F16))
+    assert {bn for bn, _ in keys} == {64, 128, 256} and {p for _, p in keys} == {1, 2, 4, 8}
+
+
+@pytest.mark.parametrize("offset", [0, 8, 1])
+@pytest.mark.parametrize("bias", [False, True])
+@pytest.mark.parametrize("shape", [(16, 4096, 4096), (200, 520, 1024), (1000, 1024, 512), (300, 515, 1000)])
+def test_fused_add_and_output_alignment(shape, bias, offset):
+    """C on a 32-byte boundary, on a 16-byte one (offset 8) and off both (stored by the threads); D has any alignment."""
+    M, N, K = shape
+    dtype = ab.F16
+    init()
+    A, B = integers(M, K, 43, dtype), integers(K, N, 44, dtype)
+    D = torch.empty((1 if bias else M) * N + 1, dtype=A.dtype, device="cuda")[1:]
+    D.copy_(integers(1 if bias else M, N, 45, dtype).reshape(-1))
+    want, _ = og.gemm(synth.bits(A).reshape(-1), synth.bits(B).reshape(-1), M, N, K, dtype)
+    want = 0.5 * want.reshape(M, N) - 2.0 * D.reshape(-1, N).double().cpu().numpy()
+    want = want.astype(np.float16)                          # (sums of integers and halves: one rounding)
+    for plan in list(forms(M, N, K, dtype).values()) + [ab.adapt_matmul_plan(M, N, K, dtype)]:
+        C = torch.full((M * N + 16,), 7.0, dtype=A.dtype, device="cuda")
+        ab.adapt_addmm(plan, A.data_ptr(), B.data_ptr(), D.data_ptr(), bias, 0.5, -2.0, C.data_ptr() + 2 * offset, stream())
+        torch.cuda.synchronize()
+        ab.adapt_poll_device_status(stream())
+        got = C.cpu().numpy()
+        assert np.array_equal(got[offset:offset + M * N].reshape(M, N), want)
+        assert (got[:offset] == 7.0).all() and (got[offset + M * N:] == 7.0).all()
+
+
+@pytest.mark.parametrize("shape", [(100, 1024, 2048), (256, 512, 1024)])
+def test_infinities_and_nan_stay_in_their_rows_and_columns(shape):
+    M, N, K = shape
+    dtype = ab.BF16
+    init()
+    A, B = integers(M, K, 46, dtype), integers(K, N, 47, dtype)
+    A[3, 5], B[K - 1, N - 2] = float("nan"), float("inf")
+    B[:, N - 2] = B[:, N - 2].abs() + 1.0
+    A[:, K - 1] = A[:, K - 1].abs() + 1.0
+    for plan in forms(M, N, K, dtype).values():
+        C = torch.full((M, N), float("nan"), dtype=A.dtype, device="cuda")
+        ab.adapt_matmul(plan, A.data_ptr(), B.data_ptr(), C.data_ptr(), stream())
+        torch.cuda.synchronize()
+        bad = ~torch.isfinite(C)
+        expect = torch.zeros_like(bad)
+        expect[3, :] = True
+        expect[:, N - 2] = True
+        assert torch.equal(bad, expect) and torch.isnan(C[3]).all() and torch.isinf(C[4, N - 2])
+
+
+@pytest.mark.parametrize("layouts", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("count", [2, 16, 17, 90])
+def test_lists_give_the_bits_of_single_calls_in_shared_launches(count, layouts):
+    init()
+    r = random.Random(count)
+    dims = [256, 320, 384, 504, 512, 640, 1024]
+    calls = []
+    for i in range(count):
+        M, N, K = r.choice(dims), r.choice(dims), r.choice([256, 264, 512, 1000, 1024])
+        dt = ab.F16 if i % 5 else ab.BF16
+        A, B = synth.draw_operand(M, K, synth.U11, 2 * i, dt, "cuda"), synth.draw_operand(K, N, synth.U11, 2 * i + 1, dt, "cuda")
+        C1, C2 = (torch.full((M, N), float("nan"), dtype=A.dtype, device="cuda") for _ in range(2))
+        calls.append((ab.adapt_matmul_plan(M, N, K, dt, *layouts), A, B, C1, C2))
+    for p, A, B, C1, _ in calls:
+        ab.adapt_matmul(p, A.data_ptr(), B.data_ptr(), C1.data_ptr(), stream())
+    torch.cuda.synchronize()
+    launches = ab.adapt_launch_count()
+    ab.adapt_matmul_batch([c[0] for c in calls], *([c[j].data_ptr() for c in calls] for j in (1, 2, 4)), stream())
+    torch.cuda.synchronize()
+    ab.adapt_poll_device_status(stream())
+    assert count < 16 or ab.adapt_launch_count() - launches < 0.8 * count
+    for p, _, _, C1, C2 in calls:
+        assert torch.equal(C1.view(torch.int16), C2.view(torch.int16)), ab.adapt_plan_info(p).BN
