@@ -1,6 +1,7 @@
-"""ctypes binding of ``libadaptmm.so``: the same names as ``include/adapt_matmul.h``.
+"""Binding of ``libadaptmm.so``: the same names as ``include/adapt_matmul.h``.
 
-Argument marshalling only.  Every step of the GEMM path runs inside the CUDA
+Argument marshalling only, through ctypes; the calls that enqueue work go through ``_fastcall`` (``csrc/fastcall.c``) where their
+arguments are plain numbers.  Every step of the GEMM path runs inside the CUDA
 library; there is no fallback.  If the shared object is missing, ``load()``
 raises and nothing else in this module works.
 """
@@ -8,6 +9,11 @@ from __future__ import annotations
 
 import ctypes
 import os
+
+try:
+    from . import _fastcall
+except ImportError:             # another interpreter than the one it was built for: every call goes through ctypes
+    _fastcall = None
 
 F16, BF16 = 0, 1
 ROW_MAJOR, COL_MAJOR = 0, 1
@@ -157,8 +163,18 @@ def load():
     lib.adapt_plan_table_load.argtypes = [ctypes.c_char_p]
     lib.adapt_selftest_wait_expiry.restype = i32
     lib.adapt_selftest_wait_expiry.argtypes = [u64, vp]
+    if _fastcall is not None:
+        _fastcall.bind(*(ctypes.cast(f, vp).value for f in (lib.adapt_matmul, lib.adapt_addmm, lib.adapt_matmul_strided_batch)))
     _lib = lib
     return lib
+
+
+def _no_fastcall(*args):
+    return -1
+
+
+# The status of a call that enqueues work, or -1 where the arguments (or the first call of all) take it through ctypes.
+_fast_matmul, _fast_addmm, _fast_strided = (_fastcall.matmul, _fastcall.addmm, _fastcall.strided) if _fastcall is not None else (_no_fastcall,) * 3
 
 
 def _check(status):
@@ -192,18 +208,25 @@ def adapt_matmul_plan_forced(M, N, K, dtype, layoutA, layoutB, tiling_key):
 
 def adapt_matmul(plan, A_ptr: int, B_ptr: int, C_ptr: int, stream: int = 0):
     """Enqueue C = A*B.  Pointers are raw device addresses (``tensor.data_ptr()``)."""
-    _check(load().adapt_matmul(plan, A_ptr, B_ptr, C_ptr, stream))
+    status = _fast_matmul(plan, A_ptr, B_ptr, C_ptr, stream)
+    if status:
+        _check(status if status > 0 else load().adapt_matmul(plan, A_ptr, B_ptr, C_ptr, stream))
 
 
 def adapt_addmm(plan, A_ptr: int, B_ptr: int, D_ptr: int, d_is_vector: bool, alpha: float, beta: float, C_ptr: int, stream: int = 0):
     """Enqueue C = alpha * (A*B) + beta * D (D: M x N, or a row of N values when d_is_vector)."""
-    _check(load().adapt_addmm(plan, A_ptr, B_ptr, D_ptr, 1 if d_is_vector else 0, alpha, beta, C_ptr, stream))
+    vector = 1 if d_is_vector else 0
+    status = _fast_addmm(plan, A_ptr, B_ptr, D_ptr, vector, alpha, beta, C_ptr, stream)
+    if status:
+        _check(status if status > 0 else load().adapt_addmm(plan, A_ptr, B_ptr, D_ptr, vector, alpha, beta, C_ptr, stream))
 
 
 def adapt_matmul_strided_batch(plan, A_ptr: int, stride_a: int, B_ptr: int, stride_b: int, C_ptr: int, stride_c: int, batch: int,
                                stream: int = 0):
     """Enqueue `batch` GEMMs of the plan's shape on operands the given numbers of elements apart."""
-    _check(load().adapt_matmul_strided_batch(plan, A_ptr, stride_a, B_ptr, stride_b, C_ptr, stride_c, batch, stream))
+    status = _fast_strided(plan, A_ptr, stride_a, B_ptr, stride_b, C_ptr, stride_c, batch, stream)
+    if status:
+        _check(status if status > 0 else load().adapt_matmul_strided_batch(plan, A_ptr, stride_a, B_ptr, stride_b, C_ptr, stride_c, batch, stream))
 
 
 def adapt_matmul_host(plan, A_host_ptr: int, B_host_ptr: int, C_host_ptr: int, stream: int = 0):

@@ -4,23 +4,36 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libadaptmm.so")
 SOURCES = ["adapt_api.cu", "adapt_select.cpp"]
+FASTCALL, FASTCALL_SOURCE = os.path.join(HERE, "_fastcall.so"), os.path.join(CSRC, "fastcall.c")
 
 
 def _stale() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "adapt_matmul.h")]
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f != os.path.basename(FASTCALL_SOURCE)] + [os.path.join(ROOT, "include", "adapt_matmul.h")]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_fastcall(force: bool = False) -> str:
+    """The binding's calls that enqueue work, as a module of the interpreter this runs in."""
+    if not force and os.path.exists(FASTCALL) and os.path.getmtime(FASTCALL) >= os.path.getmtime(FASTCALL_SOURCE):
+        return FASTCALL
+    tmp = FASTCALL + f".{os.getpid()}.tmp"
+    subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", tmp, FASTCALL_SOURCE], check=True)
+    os.replace(tmp, FASTCALL)
+    return FASTCALL
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_fastcall(force)
     if not force and not _stale():
         return LIB
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -1,0 +1,38 @@
+"""The binding's calls that enqueue work give what ctypes gives: the library's status for plain arguments, its conversions and refusals for others."""
+import ctypes
+
+import pytest
+
+from paper_2608_10803_b200 import binding as ab
+
+ab.load()
+CALLS = [("adapt_matmul", (0, 0, 0, 0, 0)), ("adapt_addmm", (0, 0, 0, 0, 1, 1.0, 1.0, 0, 0)), ("adapt_matmul_strided_batch", (0, 0, 0, 0, 0, 0, 0, 2, 0))]
+
+
+@pytest.mark.parametrize("name,args", CALLS)
+def test_a_refused_call_raises_with_the_status_and_message_of_the_library(name, args):
+    assert getattr(ab.load(), name)(*args) == ab.ERR_INVALID_ARG
+    for form in (args, tuple(None if a == 0 and i in (0, 1, len(args) - 1) else a for i, a in enumerate(args))):
+        with pytest.raises(ab.AdaptError) as e:
+            getattr(ab, name)(*form)
+        assert e.value.status == ab.ERR_INVALID_ARG and "null" in str(e.value)
+
+
+@pytest.mark.parametrize("name,args", CALLS)
+@pytest.mark.parametrize("bad", ["x", 1.5, object(), ctypes.c_void_p(0), True])
+def test_other_arguments_are_left_to_ctypes(name, args, bad):
+    def outcome(call):
+        try:
+            return call()
+        except Exception as e:          # noqa: BLE001
+            return type(e), getattr(e, "status", None)
+
+    form = args[:1] + (bad,) + args[2:]
+    assert outcome(lambda: getattr(ab, name)(*form)) == outcome(lambda: ab._check(getattr(ab.load(), name)(*form)))
+    assert ab._fastcall is None or getattr(ab, {"adapt_matmul": "_fast_matmul", "adapt_addmm": "_fast_addmm"}.get(name, "_fast_strided"))(*form) == -1
+
+
+def test_numbers_of_the_fused_add_convert_as_in_ctypes():
+    for alpha in (1, True, 0.1, 1e300):
+        with pytest.raises(ab.AdaptError):
+            ab.adapt_addmm(0, 0, 0, 0, False, alpha, 0.0, 0)
