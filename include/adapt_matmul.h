@@ -228,8 +228,9 @@ adapt_status_t adapt_matmul_noalloc(int64_t M, int64_t N, int64_t K, adapt_dtype
  * MatMul / GroupMM operators in recommendation models (Section 6.5), whose layers issue lists of small GEMMs of different
  * shapes.  The result is the one of the calls made in order, bit for bit:
  * - Small calls whose plans are of the one-launch family, or of the CUDA-core family with a short K (as adapt_matmul_plan
- *   returned them), are collected per data type and pair of layouts and leave together, 64 in one grouped launch.  A call that reads
- *   or overwrites what a collected one writes, or overwrites what it reads, makes the collected ones leave first.
+ *   returned them), or of the tcgen05 family with no more unsplit 64-column tiles than SMs, are collected per family, data type and
+ *   pair of layouts and leave together, up to 64 in one grouped launch.  A call that reads or overwrites what a collected one writes, or
+ *   overwrites what it reads, makes the collected ones leave first.
  * - From eight calls on the launches are spread over up to four internal streams, and cuda_stream itself for launches that need no
  *   workspace, between a fork from and a join to cuda_stream (work queued on cuda_stream before the call comes first, work queued
  *   after it comes last), so that the launch gaps and the tail of one GEMM fill with the next one's work (two launches without a

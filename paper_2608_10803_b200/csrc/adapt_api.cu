@@ -768,6 +768,9 @@ extern "C" adapt_status_t adapt_init(int device)
     for (int v = 0; v < 4; ++v)
         for (const void* k : {direct_group_pick<kDirectGroupMax>((v & 1) != 0, (v & 2) != 0), direct_group_pick<kDirectGroupFew>((v & 1) != 0, (v & 2) != 0)})
             CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes - kDirectStaticBytes));
+    for (int v = 0; v < 4; ++v)
+        for (const void* k : {direct_swap_pick<false>((v & 1) != 0, (v & 2) != 0), direct_swap_pick<true>((v & 1) != 0, (v & 2) != 0)})
+            CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S.machine.smem_bytes - kDirectStaticBytes));
     for (int BN : {64, 128, 256})
         for (int v = 0; v < 16; ++v)
             CUDA_TRY(cudaFuncSetAttribute(direct_kernel(BN, (v & 1) != 0, (v & 2) != 0, (v & 4) != 0, (v & 8) != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1198,7 +1201,12 @@ adapt_status_t launch_direct(State& S, const UmmaParams& p, int BN, int a_box_ro
     cfg.numAttrs = p.P_k > 1 ? 2 : 1;
     void* args[2] = {&maps, &q};
     const size_t arg_bytes[2] = {sizeof(maps), sizeof(q)};
-    CUDA_TRY(launch_exc(&cfg, direct_kernel(BN, a_mn, b_mn, p.P_k > 1, ep.D != nullptr), args, arg_bytes, 2));
+    const void* k = direct_kernel(BN, a_mn, b_mn, p.P_k > 1, ep.D != nullptr);
+    if (direct_swaps(p.M, BN, p.P_k)) {                     // B's columns are the MMA's rows, A's rows its columns
+        k = ep.D ? direct_swap_pick<true>(a_mn, b_mn) : direct_swap_pick<false>(a_mn, b_mn);
+        q.idesc = umma_idesc(p.dtype, b_mn, a_mn, 128, (int)round_up(p.M, 16));
+    }
+    CUDA_TRY(launch_exc(&cfg, k, args, arg_bytes, 2));
     S.launches.fetch_add(1, std::memory_order_relaxed);
     return ADAPT_OK;
 }

@@ -349,10 +349,13 @@ inline int direct_smem_bytes(int BN, int rows, int stages, int splits)
 {
     return std::max(kDirectAloneBytes, direct_ring_bytes(BN, rows, stages, splits) + direct_exchange_bytes(BN, rows, splits) + 1024);
 }
+// Whole tiles of 128 columns and few rows run as the transposed product (with 128 rows it would save nothing).
+constexpr int kDirectSwapRows = 112, kDirectSwapStages = 8;
+inline bool direct_swaps(int64_t M, int BN, int splits) { return M <= kDirectSwapRows && BN == 128 && splits == 1; }
 // The deepest ring that fits, no deeper than the CTA's k-blocks.
 inline int direct_stages(int BN, int rows, int64_t k_blocks, int splits, int smem_limit)
 {
-    int s = (int)std::min<int64_t>(kUmmaMaxStages, k_blocks);
+    int s = (int)std::min<int64_t>(direct_swaps(rows, BN, splits) ? kDirectSwapStages : kUmmaMaxStages, k_blocks);
     while (s > 1 && direct_smem_bytes(BN, rows, s, splits) + kDirectStaticBytes > smem_limit) --s;
     return s;
 }

@@ -57,13 +57,19 @@ template <int BN> struct DirectShape {
     static constexpr int kThreads = 64 + 32 * kEpilogueWarps;
 };
 
+// SWAP: the transposed product, for fewer rows than a tile: B's 128 columns are the MMA's rows and the rows of A its columns (16 .. 112), so a k-block costs what its
+// rows need and not what 128 would.  The stream of a few rows' product is bound by memory only while the chip keeps its clocks: 16 x 14336 x 4096 for milliseconds on end
+// took 22.6 us with 128 rows of MMA and takes 19.2 (floor 18.0); 64 rows 23.3 and 21.7.  Eight stages are enough for such a stream, and twelve slow it: 20.6.
+//
 // Tile (mb, nb) by the calling CTA; SPLIT: the rank-th split of it.  map_c null (LIST): the threads store the boxes, whole rows of 128 bytes.
-template <int BN, bool A_MN, bool B_MN, bool SPLIT, bool EPI, bool LIST = false>
+template <int BN, bool A_MN, bool B_MN, bool SPLIT, bool EPI, bool LIST = false, bool SWAP = false>
 __device__ __forceinline__ void direct_tile(const CUtensorMap* map_a, const CUtensorMap* map_b, const CUtensorMap* map_c, const DirectParams& p, int rank, int mb, int nb)
 {
     constexpr int EW = DirectShape<BN>::kEpilogueWarps, THREADS = DirectShape<BN>::kThreads;
     constexpr int B_BOXES = B_MN ? BN / 64 : 1, A_BOXES = A_MN ? 2 : 1;
     constexpr uint32_t B_BYTES = BN * kUmmaBK * 2;
+    static_assert(!SWAP || (BN == 128 && !SPLIT && !LIST), "the transposed product: whole tiles of 128 columns");
+    const uint32_t tmem_cols = SWAP ? (p.M <= 32 ? 32u : p.M <= 64 ? 64u : 128u) : (uint32_t)BN;
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(16) uint64_t bars[2 * kUmmaMaxStages + 2];
     __shared__ uint32_t tmem_slot;
@@ -123,7 +129,7 @@ __device__ __forceinline__ void direct_tile(const CUtensorMap* map_a, const CUte
     } else {
         if (SPLIT) cluster_arrive();
         if (warp == 1) {
-            ptx::tmem_alloc<1>(ptx::smem_u32(&tmem_slot), (uint32_t)BN);
+            ptx::tmem_alloc<1>(ptx::smem_u32(&tmem_slot), tmem_cols);
             ptx::tmem_relinquish<1>();
             pdl_launch_dependents();                       // not before: a CTA of the next kernel must not take the columns this one waits for
         }
@@ -138,14 +144,17 @@ __device__ __forceinline__ void direct_tile(const CUtensorMap* map_a, const CUte
         const uint64_t a_desc = ptx::smem_desc_sw128(ring, A_MN ? 8192u : 16u, 1024u);
         const uint64_t b_desc = ptx::smem_desc_sw128(ring + (uint32_t)p.a_bytes, B_MN ? 8192u : 16u, 1024u);
         if (ptx::elect_one()) {
-            const uint32_t a_lo = (uint32_t)a_desc, a_hi = (uint32_t)(a_desc >> 32), b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32);
+            // (SWAP: the operands change places, and so do their steps from one k16 to the next)
+            constexpr uint32_t x_kstep = SWAP ? b_kstep : a_kstep, y_kstep = SWAP ? a_kstep : b_kstep;
+            const uint64_t x_desc = SWAP ? b_desc : a_desc, y_desc = SWAP ? a_desc : b_desc;
+            const uint32_t a_lo = (uint32_t)x_desc, a_hi = (uint32_t)(x_desc >> 32), b_lo = (uint32_t)y_desc, b_hi = (uint32_t)(y_desc >> 32);
             const uint32_t idesc = p.idesc, step = stage_bytes >> 4, full_end = full_bar + 8u * S;
             uint32_t off = 0, fb = full_bar, phase = 0, more = 0;
             for (int left = n_kb; left > 0; --left, more = 1u) {
                 if (!ptx::mbar_wait(fb, phase, abort_flag)) break;
 #pragma unroll
                 for (int k16 = 0; k16 < kUmmaBK / 16; ++k16)
-                    ptx::umma_f16<1>(tmem, ptx::smem_desc_join(a_lo + off + (k16 * a_kstep >> 4), a_hi), ptx::smem_desc_join(b_lo + off + (k16 * b_kstep >> 4), b_hi), idesc, k16 > 0 ? 1u : more);
+                    ptx::umma_f16<1>(tmem, ptx::smem_desc_join(a_lo + off + (k16 * x_kstep >> 4), a_hi), ptx::smem_desc_join(b_lo + off + (k16 * y_kstep >> 4), b_hi), idesc, k16 > 0 ? 1u : more);
                 if (left > S) ptx::umma_commit_1(fb + 8u * kUmmaMaxStages);     // a later k-block takes this stage
                 if (left == 1) ptx::umma_commit_1(done_bar);
                 off += step;
@@ -159,14 +168,43 @@ __device__ __forceinline__ void direct_tile(const CUtensorMap* map_a, const CUte
         constexpr int COLS = BN * 4 / EW;
         const int q = warp & 3, c_first = ((warp - 2) >> 2) * COLS;
         const int row = row0 + q * 32 + lane;
-        const bool row_ok = row < p.M, live = row0 + q * 32 < p.M;              // (live: a row of this warp exists, uniform)
+        const bool row_ok = row < p.M, live = SWAP ? n0 + q * 32 < p.N : row0 + q * 32 < p.M;      // (live: a row, SWAP: a column, of this warp exists, uniform)
         const uint32_t t_row = tmem + ((uint32_t)(q * 32) << 16);
         const bool done = ptx::mbar_wait_warp(done_bar, 0, abort_flag);
         if (SPLIT) cluster_wait();                                              // the peers run: their shared memory may be written
         pdl_wait();                                                             // (long past: the loads have waited for it)
         if (done && live) {
             ptx::tc_fence_after();
-            if (!SPLIT) {
+            if constexpr (SWAP) {
+                // a lane has a column of C; neighbours trade halves of two rows, so that each stores a pair of columns of one
+                const int n = n0 + q * 32 + lane;
+                for (int g = (warp - 2) >> 2; 8 * g < p.M; g += 2) {
+                    uint32_t r[8];
+                    __syncwarp();                                               // (the stores below are the lanes' own)
+                    ptx::tmem_ld_32x8(t_row + 8u * g, r);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 8; i += 2) {
+                        const int m = 8 * g + i;
+                        float v0 = __uint_as_float(r[i]), v1 = __uint_as_float(r[i + 1]);
+                        if (EPI && n < p.N) {
+                            if (m < p.M) v0 = fused_add(p.ep, v0, m, n, p.N, p.dtype);
+                            if (m + 1 < p.M) v1 = fused_add(p.ep, v1, m + 1, n, p.N, p.dtype);
+                        }
+                        const uint32_t h0 = cast16(v0, p.dtype), h1 = cast16(v1, p.dtype), other = __shfl_xor_sync(0xffffffffu, lane & 1 ? h0 : h1, 1);
+                        const uint32_t pair = lane & 1 ? other | (h1 << 16) : h0 | (other << 16);
+                        const int mr = m + (lane & 1), nc = n & ~1;
+                        if (mr >= p.M || nc >= p.N) continue;
+                        unsigned short* dst = p.C + (int64_t)mr * p.N + nc;
+                        if (nc + 1 < p.N && (reinterpret_cast<uintptr_t>(dst) & 3) == 0) {
+                            *reinterpret_cast<uint32_t*>(dst) = pair;
+                        } else {
+                            dst[0] = (unsigned short)pair;
+                            if (nc + 1 < p.N) dst[1] = (unsigned short)(pair >> 16);
+                        }
+                    }
+                }
+            } else if (!SPLIT) {
                 const uint64_t policy = ptx::l2_policy_evict_first();
 #pragma unroll
                 for (int pass = 0; pass < COLS / 64; ++pass) {
@@ -301,11 +339,11 @@ __device__ __forceinline__ void direct_tile(const CUtensorMap* map_a, const CUte
     if (threadIdx.x == 0 && abort_word) atomicOr(p.status, 1u);
     if (warp == 1) {
         ptx::tc_fence_after();
-        ptx::tmem_dealloc<1>(tmem, (uint32_t)BN);
+        ptx::tmem_dealloc<1>(tmem, tmem_cols);
     }
 }
 
-template <int BN, bool A_MN, bool B_MN, bool SPLIT, bool EPI>
+template <int BN, bool A_MN, bool B_MN, bool SPLIT, bool EPI, bool SWAP = false>
 __global__ void __launch_bounds__(DirectShape<BN>::kThreads, 2)
 direct_gemm_kernel(const __grid_constant__ DirectMaps maps, const __grid_constant__ DirectParams p)
 {
@@ -319,7 +357,7 @@ direct_gemm_kernel(const __grid_constant__ DirectMaps maps, const __grid_constan
         const int g = t / (kGroupM * p.P_n), gm = min(p.P_m - g * kGroupM, kGroupM), r = t - g * kGroupM * p.P_n;
         nb = r / gm; mb = g * kGroupM + r - nb * gm;
     }
-    direct_tile<BN, A_MN, B_MN, SPLIT, EPI>(&maps.a, &maps.b, &maps.c, p, rank, mb, nb);
+    direct_tile<BN, A_MN, B_MN, SPLIT, EPI, false, SWAP>(&maps.a, &maps.b, &maps.c, p, rank, mb, nb);
 }
 
 // The tiles of up to kDirectGroupMax products (128 x 64 each, of one data type and pair of layouts) side by side in one launch: the lists of
@@ -379,6 +417,12 @@ inline const void* direct_group_pick(bool a_mn, bool b_mn)
 {
     return a_mn ? (b_mn ? (const void*)direct_group_kernel<true, true, MAX> : (const void*)direct_group_kernel<true, false, MAX>)
                 : (b_mn ? (const void*)direct_group_kernel<false, true, MAX> : (const void*)direct_group_kernel<false, false, MAX>);
+}
+template <bool EPI>
+inline const void* direct_swap_pick(bool a_mn, bool b_mn)
+{
+    return a_mn ? (b_mn ? (const void*)direct_gemm_kernel<128, true, true, false, EPI, true> : (const void*)direct_gemm_kernel<128, true, false, false, EPI, true>)
+                : (b_mn ? (const void*)direct_gemm_kernel<128, false, true, false, EPI, true> : (const void*)direct_gemm_kernel<128, false, false, false, EPI, true>);
 }
 inline const void* direct_kernel(int BN, bool a_mn, bool b_mn, bool split, bool epi)
 {

@@ -1,7 +1,7 @@
 // Programmatic dependent launch: every kernel of this library is launched with the
-// programmatic-stream-serialization attribute and begins with pdl_enter().  A kernel then starts
-// as soon as all CTAs of the kernel before it on the stream have started (they signal it first
-// thing), runs its set-up (barrier init, TMEM allocation, tensor-map prefetch) while that kernel
+// programmatic-stream-serialization attribute and begins with pdl_enter() or its two halves.  A kernel
+// then starts as soon as all CTAs of the kernel before it on the stream have signalled it (first thing,
+// or once they hold their TMEM), runs its set-up (barrier init, TMEM allocation, tensor-map prefetch) while that kernel
 // drains, and touches global memory only after griddepcontrol.wait has seen it complete and its
 // writes flushed.  The data dependences between the launches of one call (copy -> GEMM -> reduce)
 // and between calls that share a workspace are therefore kept; only the launch latency overlaps.

@@ -1,6 +1,6 @@
 // tcgen05 GEMM on tall pair tiles: 512 x 256 outputs per SM pair, all 512 TMEM columns as the two accumulators of ONE tile.
 //
-// The 256 x 256 pair tile (umma_gemm.cuh) brings 32 KB per k-block and SM for 512 cycles of MMA: its loop is bound by the SM's load port
+// The 256 x 256 pair tile (umma_gemm.cuh) brings 32 KB per k-block and SM for 512 cycles of MMA: when this kernel was written, that loop was bound by its loads
 // (8192^3 with zero operands, where power does not interfere, cycles per k-block: 685 in full, 587 with the MMAs alone, 638 with the loads
 // alone; six or seven stages change nothing), and with data in the operands the same traffic is the energy the power cap takes out of the
 // clock.  Here a CTA takes 256 rows and half of 256 columns: 48 KB per 1024 cycles of MMA, a quarter less per flop.
