@@ -53,6 +53,19 @@ def test_every_form_is_exact_on_integers(shape, layouts):
         check_case(M, N, K, dtype, a, b, lA, lB, plan=plan, exact=True)
 
 
+# the ends of the MMA's column counts and of its TMEM columns, and the last rows that are computed transposed
+@pytest.mark.parametrize("layouts", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("rows", [9, 16, 17, 32, 40, 65, 104, 112, 113])
+def test_few_rows_in_tiles_of_128_columns(rows, layouts):
+    N, K, dtype = 2056, 1000 if layouts[0] == 0 else 1024, ab.BF16
+    rows = rows if layouts[0] == 0 else (rows + 7) // 8 * 8         # (the columns of a column-major A are read in place from whole 16 bytes on)
+    init()
+    A, B = integers(rows, K, 46, dtype), integers(K, N, 47, dtype)
+    plan = forms(rows, N, K, dtype, *layouts).get((128, 1))
+    assert plan is not None
+    check_case(rows, N, K, dtype, A.t().contiguous() if layouts[0] else A, B.t().contiguous() if layouts[1] else B, *layouts, plan=plan, exact=True)
+
+
 def test_the_forms_cover_tiles_and_splits():
     init()
     keys = set()
